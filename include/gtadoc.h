@@ -27,10 +27,11 @@
  *     gt_last_error.  Failures that only the GPU can detect (a full overflow
  *     list, a row count past its bound, an invalid symbol) are recorded in a
  *     device status word and reported by gt_sync / gt_result_view.  The
- *     only waits inside kernels are decoupled look-backs (the global
- *     sequence count's bucket path and the inverted index: a CTA polls the
- *     published totals of the items taken before its own); each gives up
- *     after a bounded number of polls with GT_ETIMEOUT.
+ *     only waits inside kernels are decoupled look-backs (scans, the radix
+ *     sort, the reduction of equal keys, the global sequence count's bucket
+ *     path and the inverted index: a CTA polls the published totals of the
+ *     items taken before its own); each gives up after a bounded number of
+ *     polls with GT_ETIMEOUT.
  *   - There is no CPU fallback: if no usable sm_103a device is present,
  *     gt_create fails with GT_ECUDA.
  */
@@ -355,13 +356,11 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *                   bucket path (2..3072, default 3072); fuller buckets are
  *                   sorted in global memory.
  *   "radix_items"   keys per thread of the LSD radix sort's scatter passes:
- *                   8 (default, tiles of 2048 keys) or 16 (tiles of 4096:
- *                   longer runs per digit in each tile's writes); GT_EINVAL
- *                   otherwise.  Same results.
- *   "radix_prefetch" 1: the radix sort's scatter passes (2048-key tiles) run
- *                   as a persistent kernel that copies the next tile into
- *                   shared memory asynchronously while it ranks the current
- *                   one; 0 (default): one CTA per tile.  Same results.
+ *                   8 (default): tiles of 2048 keys below 2^20 rows and of
+ *                   4096 keys from there on; 16: always tiles of 4096.
+ *                   GT_EINVAL otherwise.  Same results.
+ *   "radix_prefetch" accepted, without effect: it selected a persistent
+ *                   scatter that was slower than one CTA per tile.
  *   "file_strategy" per-file analytics (term vector, inverted index, per-file
  *                   sequence count, ranked index): 0 (default) picks top-down
  *                   for at most 64 files and bottom-up otherwise (the paper's

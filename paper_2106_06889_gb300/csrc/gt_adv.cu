@@ -20,26 +20,21 @@ namespace gt {
 namespace {
 
 // Rows of the pairs of every 3-gram: (a, b) and (a, c) of key a|b|c with its
-// count; rows past the number of 3-grams get the pad key.
+// count, after the files' last pairs (one row per file); *rows counts them all.
 __global__ void cooc_rows_kernel(const uint64_t* __restrict__ key3, const uint64_t* __restrict__ cnt3,
-                                 const int64_t* __restrict__ n3_dev, int64_t bound, uint64_t key_pad,
-                                 uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+                                 const int64_t* __restrict__ n3_dev, int32_t F, uint64_t* __restrict__ keys,
+                                 uint32_t* __restrict__ vals, int64_t* __restrict__ rows) {
   const int64_t n3 = *n3_dev;
   const uint64_t m = (uint64_t(1) << 21) - 1;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < bound; i += int64_t(gridDim.x) * blockDim.x) {
-    uint64_t k0 = key_pad, k1 = key_pad;
-    uint32_t c = 0;
-    if (i < n3) {
-      const uint64_t k = key3[i];
-      const uint64_t a = k >> 42, b = (k >> 21) & m, cw = k & m;
-      k0 = (a << 21) | b;
-      k1 = (a << 21) | cw;
-      c = uint32_t(cnt3[i]);  // below 2^32: fewer than 2^32 tokens
-    }
-    keys[2 * i] = k0;
-    keys[2 * i + 1] = k1;
-    vals[2 * i] = c;
-    vals[2 * i + 1] = c;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *rows = 2 * n3 + F;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n3; i += int64_t(gridDim.x) * blockDim.x) {
+    const uint64_t k = key3[i];
+    const uint64_t a = k >> 42, b = (k >> 21) & m, cw = k & m;
+    const uint32_t c = uint32_t(cnt3[i]);  // below 2^32: fewer than 2^32 tokens
+    keys[F + i] = (a << 21) | b;
+    keys[F + n3 + i] = (a << 21) | cw;
+    vals[F + i] = c;
+    vals[F + n3 + i] = c;
   }
 }
 
@@ -89,23 +84,22 @@ gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s) {
     const int64_t U = g->info.owned_windows;  // distinct 3-grams at most
     const int64_t n = 2 * U + d.F;
     const uint64_t key_pad = uint64_t(1) << 42;  // above every pair key
-    Buf keys(ctx, size_t(n) * 8, s), vals(ctx, size_t(n) * 4, s);
+    Buf keys(ctx, size_t(n) * 8, s), vals(ctx, size_t(n) * 4, s), rows(ctx, 8, s);
     Buf tail(ctx, size_t(d.R) * 8, s), head(ctx, size_t(d.R) * 8, s);
     {
       Phase ph(ctx, "cooc_rows", s);
       run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s);
       const int threads = 256, cap = ctx->num_sms * 16;
-      if (U > 0) {
-        cooc_rows_kernel<<<grid_for(U, threads, cap), threads, 0, s>>>(
-            static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, U, key_pad, keys.as<uint64_t>(),
-            vals.as<uint32_t>());
-        GT_LAUNCH_CHECK();
-      }
+      cooc_rows_kernel<<<grid_for(U, threads, cap), threads, 0, s>>>(
+          static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, d.F, keys.as<uint64_t>(), vals.as<uint32_t>(),
+          rows.as<int64_t>());
+      GT_LAUNCH_CHECK();
       file_last_pair_kernel<<<grid_for(d.F, threads, cap), threads, 0, s>>>(
-          d, tail.as<int32_t>(), key_pad, keys.as<uint64_t>() + 2 * U, vals.as<uint32_t>() + 2 * U);
+          d, tail.as<int32_t>(), key_pad, keys.as<uint64_t>(), vals.as<uint32_t>());
       GT_LAUNCH_CHECK();
     }
-    gt_result* out = reduce_key_rows(ctx, keys, vals, n, 43, key_pad, s, reinterpret_cast<uint32_t*>(seq->d_lens));
+    gt_result* out = reduce_key_rows(ctx, keys, vals, n, 43, key_pad, s, reinterpret_cast<uint32_t*>(seq->d_lens),
+                                     rows.as<int64_t>());
     out->deps.push_back(seq);  // the 3-gram result's buffers live until this result is freed
     return out;
   } catch (...) {

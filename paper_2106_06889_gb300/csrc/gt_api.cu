@@ -450,6 +450,8 @@ gt_result* sort_from_counts(gt_grammar* g, const uint64_t* wc, int order, cudaSt
   auto* words = static_cast<int32_t*>(rb.alloc(size_t(V) * 4));
   auto* counts = static_cast<uint64_t*>(rb.alloc(size_t(V) * 8));
   int64_t* nlen = rb.new_len_slot();
+  GT_CUDA(cudaMemcpyAsync(rb.status(), wc_status, 4, cudaMemcpyDeviceToDevice, s));
+  gt::StatusScope scope(rb.status());
   gt::Phase ph(ctx, "sort_canon", s);
   if (order == 0) {
     Buf flag(ctx, size_t(V) * 8, s), pos(ctx, size_t(V) * 8, s), sc(ctx, gt::scan_scratch_bytes(V), s);
@@ -466,14 +468,18 @@ gt_result* sort_from_counts(gt_grammar* g, const uint64_t* wc, int order, cudaSt
     count_keys_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(wc, V, N, k0.as<uint64_t>(),
                                                                         v0.as<uint32_t>());
     GT_LAUNCH_CHECK();
-    gt::radix_sort_u64(k0.as<uint64_t>(), k1.as<uint64_t>(), v0.p, v1.p, 4, V, 0, bits_for(N), rs.p, s);
+    const int kbits = bits_for(N);
+    if (!gt::radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), v0.p, v1.p, 4, V, 0, kbits, kbits, kbits, rs.p,
+                                 s)) {
+      std::swap(k0, k1);
+      std::swap(v0, v1);
+    }
     count_unkey_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(k1.as<uint64_t>(), v1.as<uint32_t>(), V, N,
                                                                          words, counts, nlen);
     GT_LAUNCH_CHECK();
   }
   rb.field_dyn("word", words, nlen);
   rb.field_dyn("count", counts, nlen);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), wc_status, 4, cudaMemcpyDeviceToDevice, s));
   return rb.finish();
 }
 

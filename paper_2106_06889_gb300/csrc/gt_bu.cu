@@ -74,18 +74,71 @@ __global__ void redge_len_kernel(const DevGrammar d, bool windows, int64_t* __re
 
 // ---- word rows: key = file << kbw | word ----
 
-__global__ void root_word_rows_kernel(const DevGrammar d, int kbw, uint64_t pad, uint64_t* __restrict__ key,
-                                      uint32_t* __restrict__ val) {
-  for (int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; j < d.root_len; j += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t s = d.sym[j];
-    if (s < d.V) {
-      const int64_t f = upper_bound_dev(d.file_off, int64_t(d.F) + 1, j) - 1;
-      key[j] = (uint64_t(f) << kbw) | uint64_t(uint32_t(s));
-      val[j] = 1u;
-    } else {
-      key[j] = pad;
-      val[j] = 0u;
+// Rows of the root's words.  A CTA takes a tile of kRowTile symbols, claims its
+// rows with one atomic (rows are sorted next, so their order is free; none is
+// spent on a reference) and looks for files only among those the tile spans.
+constexpr int kRowThreads = 256;
+constexpr int kRowItems = 8;
+constexpr int kRowTile = kRowThreads * kRowItems;
+
+// last file f in [lo, hi] that starts at or before position j of the root
+__device__ __forceinline__ int32_t file_among(const DevGrammar& d, int32_t lo, int32_t hi, int64_t j) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (d.file_off[mid] <= j) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(kRowThreads) root_word_rows_kernel(const DevGrammar d, int kbw,
+                                                                     unsigned long long* __restrict__ n,
+                                                                     uint64_t* __restrict__ key,
+                                                                     uint32_t* __restrict__ val) {
+  __shared__ int32_t s_file[2];
+  __shared__ uint32_t s_warp[kRowThreads / 32];
+  __shared__ unsigned long long s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t j0 = int64_t(blockIdx.x) * kRowTile, j1 = min(d.root_len, j0 + kRowTile);
+  if (threadIdx.x < 2) s_file[threadIdx.x] = file_among(d, 0, d.F - 1, threadIdx.x ? j1 - 1 : j0);
+  int32_t sy[kRowItems];
+  uint32_t c = 0;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    const int64_t j = j0 + k * kRowThreads + threadIdx.x;
+    sy[k] = j < j1 ? d.sym[j] : d.V;
+    c += sy[k] < d.V;
+  }
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kRowThreads / 32; ++w) {
+    before += w < warp ? s_warp[w] : 0u;
+    total += s_warp[w];
+  }
+  if (threadIdx.x == 0) s_base = total ? atomicAdd(n, (unsigned long long)total) : 0ull;
+  __syncthreads();
+  // a warp's rows are written 32 symbols at a time, so that its stores are dense
+  int64_t o = int64_t(s_base) + before;  // the warp's first row
+  const int32_t f_lo = s_file[0], f_hi = s_file[1];
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    const unsigned words = __ballot_sync(0xffffffffu, sy[k] < d.V);
+    if (sy[k] < d.V) {
+      const uint64_t f = uint64_t(file_among(d, f_lo, f_hi, j0 + k * kRowThreads + threadIdx.x));
+      const int64_t at = o + __popc(words & lt);
+      key[at] = (f << kbw) | uint64_t(uint32_t(sy[k]));
+      val[at] = 1u;
     }
+    o += __popc(words);
   }
 }
 
@@ -105,80 +158,71 @@ __global__ void child_word_rows_kernel(const DevGrammar d, int kbw, const int64_
 
 // ---- window rows: key = compact 3-word key, file separately ----
 
-__global__ void root_window_rows_kernel(const DevGrammar d, const int32_t* __restrict__ head,
-                                        const int32_t* __restrict__ tail, int kb, uint64_t pad,
-                                        uint64_t* __restrict__ key, uint64_t* __restrict__ file,
-                                        uint32_t* __restrict__ val) {
-  for (int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; j < d.root_len; j += int64_t(gridDim.x) * blockDim.x) {
-    int32_t r, f;
-    const int64_t end = seq_end(d, j, &r, &f);
-    uint64_t k[2];
-    const int n = windows_at(d, head, tail, j, end, kb, k);
-    for (int i = 0; i < 2; ++i) {
-      key[2 * j + i] = i < n ? k[i] : pad;
-      file[2 * j + i] = uint64_t(uint32_t(f));
-      val[2 * j + i] = i < n ? 1u : 0u;
-    }
+// Rows of the windows the root owns: a tile of kTile symbols per CTA, its rows
+// claimed with one atomic.
+constexpr int kRootWinThreads = kTile / 4;
+
+__global__ void __launch_bounds__(kRootWinThreads) root_window_rows_kernel(const DevGrammar d,
+                                                                           const int32_t* __restrict__ head,
+                                                                           const int32_t* __restrict__ tail, int kb,
+                                                                           FileRows out) {
+  __shared__ uint32_t s_warp[kRootWinThreads / 32];
+  __shared__ unsigned long long s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  TileWin t;
+  int32_t file[4];
+  tile_windows(d, head, tail, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t, file);
+  uint32_t c = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (t.r[i] != 0) t.n[i] = 0;  // rule bodies in the tile that holds the root's end
+    c += t.n[i];
   }
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  uint32_t before = incl - c, total = 0;
+#pragma unroll
+  for (int w = 0; w < kRootWinThreads / 32; ++w) {
+    before += w < warp ? s_warp[w] : 0u;
+    total += s_warp[w];
+  }
+  if (threadIdx.x == 0) s_base = total ? atomicAdd(out.n, (unsigned long long)total) : 0ull;
+  __syncthreads();
+  int64_t o = int64_t(s_base) + before;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (q < t.n[i]) out.put(o++, file[i], t.k[i][q], 1u);
 }
 
+// Rows of every window inside each (file, root child) expansion, from row
+// `first` on (pos: exclusive scan of the windows per edge).
 __global__ void child_window_rows_kernel(const DevGrammar d, int kb, const int64_t* __restrict__ pos,
-                                         uint64_t* __restrict__ key, uint64_t* __restrict__ file,
-                                         uint32_t* __restrict__ val) {
+                                         const unsigned long long* __restrict__ first, FileRows out) {
+  const int64_t base = int64_t(*first);
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < d.ER; e += int64_t(gridDim.x) * blockDim.x) {
-    const uint64_t f = uint64_t(file_of_redge(d, e));
+    const int32_t f = file_of_redge(d, e);
     const uint32_t m = d.redge_mult[e];
-    int64_t o = pos[e];
+    int64_t o = base + pos[e];
     int32_t a = -1, b = -1;
     walk_rule(d, d.redge_child[e], [&](int32_t w) {
-      if (a >= 0) {
-        key[o] = pack_compact(a, b, w, kb);
-        file[o] = f;
-        val[o] = m;
-        ++o;
-      }
+      if (a >= 0) out.put(o++, f, pack_compact(a, b, w, kb), m);
       a = b;
       b = w;
     });
   }
 }
 
-__global__ void reduce_flags_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ val, int64_t n,
-                                    uint64_t pad, int64_t* __restrict__ flag, int64_t* __restrict__ v64) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const bool real = key[i] != pad;
-    flag[i] = real && (i == 0 || key[i] != key[i - 1]);
-    v64[i] = real ? int64_t(val[i]) : 0;
-  }
-}
-
-// One row per distinct (file, word): word, file, summed count.
-__global__ void reduce_write_kernel(const uint64_t* __restrict__ key, int64_t n, const int64_t* __restrict__ flag,
-                                    const int64_t* __restrict__ pos, int kbw, int32_t* __restrict__ word,
-                                    int32_t* __restrict__ file, int64_t* __restrict__ start) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    if (flag[i]) {
-      const int64_t u = pos[i];
-      word[u] = int32_t(key[i] & ((uint64_t(1) << kbw) - 1));
-      file[u] = int32_t(key[i] >> kbw);
-      start[u] = i;
-    }
-}
-
-__global__ void reduce_sum_kernel(const int64_t* __restrict__ start, const int64_t* __restrict__ nr_dev,
-                                  const int64_t* __restrict__ wsum, const int64_t* __restrict__ v64, int64_t n,
-                                  uint64_t* __restrict__ cnt) {
-  const int64_t nr = *nr_dev;
-  for (int64_t u = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; u < nr; u += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t a = start[u], b = u + 1 < nr ? start[u + 1] : n;
-    const int64_t end_sum = b < n ? wsum[b] : wsum[n - 1] + v64[n - 1];
-    cnt[u] = uint64_t(end_sum - wsum[a]);
-  }
-}
-
-__global__ void total_kernel(const int64_t* __restrict__ ex, const int64_t* __restrict__ flag, int64_t n,
-                             int64_t* __restrict__ out) {
-  *out = n > 0 ? ex[n - 1] + flag[n - 1] : 0;
+__global__ void add_rows_kernel(const unsigned long long* __restrict__ first, int64_t more,
+                                unsigned long long* __restrict__ n) {
+  *n = *first + (unsigned long long)more;
 }
 
 // off[f] = first row whose file is >= f (rows sorted by file), f in [0, F].
@@ -199,12 +243,12 @@ __global__ void file_offsets_kernel(const int32_t* __restrict__ file, const int6
 // Inverted index from (file, word) rows: stable sort by word carrying the
 // file, so the files come out ascending inside each word; offsets per word.
 __global__ void word_keys_kernel(const int32_t* __restrict__ word, const int32_t* __restrict__ file,
-                                 const int64_t* __restrict__ n_dev, int64_t bound, int32_t V, uint64_t* __restrict__ k,
+                                 const int64_t* __restrict__ n_dev, uint64_t* __restrict__ k,
                                  uint32_t* __restrict__ f) {
   const int64_t n = *n_dev;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < bound; i += int64_t(gridDim.x) * blockDim.x) {
-    k[i] = i < n ? uint64_t(uint32_t(word[i])) : uint64_t(uint32_t(V));
-    f[i] = i < n ? uint32_t(file[i]) : 0u;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    k[i] = uint64_t(uint32_t(word[i]));
+    f[i] = uint32_t(file[i]);
   }
 }
 
@@ -488,7 +532,7 @@ __global__ void local_pack_kernel(int32_t F, const int64_t* __restrict__ slot_of
 
 // (file, word, count) rows of every file, sorted by (file, word).
 struct WordRows {
-  Buf word, file, cnt, total;
+  Buf word, file, cnt, total, status;  // status: flags raised while the rows were made
   int64_t bound = 0;
 };
 
@@ -530,6 +574,9 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
   const int threads = 256, cap = ctx->num_sms * 16;
   if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
   if (d.N >= (uint64_t(1) << 32)) fail(GT_EOVERFLOW, "per-file analytics need fewer than 2^32 tokens per grammar");
+  out.status = Buf(ctx, 4, s);
+  GT_CUDA(cudaMemsetAsync(out.status.p, 0, 4, s));
+  StatusScope scope(out.status.as<uint32_t>());
   const int kbw = bits_for(d.V);
   const int fb = bits_for(d.F);
   if (g->max_file_len <= kLocalMax && gparam(g, "bu_local", 1)) {
@@ -537,14 +584,15 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
     return;
   }
   if (kbw + fb > 63) fail(GT_EOVERFLOW, "too many files x words for 64-bit (file, word) keys");
-  const uint64_t pad = uint64_t(uint32_t(d.F)) << kbw;
-  const int64_t n = d.root_len + g->bu_words;
+  const int64_t n = g->info.root_words + g->bu_words;
   Phase ph(ctx, "bu_rows", s);
   Buf k0(ctx, size_t(n) * 8, s), v0(ctx, size_t(n) * 4, s), k1(ctx, size_t(n) * 8, s), v1(ctx, size_t(n) * 4, s);
   Buf ecnt(ctx, size_t(d.ER) * 8, s), epos(ctx, size_t(d.ER) * 8, s), sc(ctx, scan_scratch_bytes(d.ER), s);
-  if (d.root_len > 0) {
-    root_word_rows_kernel<<<grid_for(d.root_len, threads, cap), threads, 0, s>>>(d, kbw, pad, k0.as<uint64_t>(),
-                                                                                  v0.as<uint32_t>());
+  Buf claimed(ctx, 8, s);
+  if (g->info.root_words > 0) {
+    GT_CUDA(cudaMemsetAsync(claimed.p, 0, 8, s));
+    root_word_rows_kernel<<<unsigned((d.root_len + kRowTile - 1) / kRowTile), kRowThreads, 0, s>>>(
+        d, kbw, claimed.as<unsigned long long>(), k0.as<uint64_t>(), v0.as<uint32_t>());
     GT_LAUNCH_CHECK();
   }
   if (d.ER > 0) {
@@ -552,8 +600,8 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
     GT_LAUNCH_CHECK();
     exclusive_scan_i64(ecnt.as<int64_t>(), epos.as<int64_t>(), d.ER, sc.p, s);
     child_word_rows_kernel<<<grid_for(d.ER, 128, cap), 128, 0, s>>>(d, kbw, epos.as<int64_t>(),
-                                                                     k0.as<uint64_t>() + d.root_len,
-                                                                     v0.as<uint32_t>() + d.root_len);
+                                                                     k0.as<uint64_t>() + g->info.root_words,
+                                                                     v0.as<uint32_t>() + g->info.root_words);
     GT_LAUNCH_CHECK();
   }
   out.bound = n;
@@ -566,24 +614,16 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
     return;
   }
   Buf rs(ctx, radix_scratch_bytes(n, true, 4), s);
-  radix_sort_u64(k0.as<uint64_t>(), k1.as<uint64_t>(), v0.p, v1.p, 4, n, 0, kbw + fb, rs.p, s);
-  Buf flag(ctx, size_t(n) * 8, s), pos(ctx, size_t(n) * 8, s), v64(ctx, size_t(n) * 8, s), wsum(ctx, size_t(n) * 8, s);
-  Buf sc2(ctx, scan_scratch_bytes(n), s), start(ctx, size_t(n) * 8, s);
-  reduce_flags_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(k1.as<uint64_t>(), v1.as<uint32_t>(), n, pad,
-                                                                     flag.as<int64_t>(), v64.as<int64_t>());
-  GT_LAUNCH_CHECK();
-  exclusive_scan_i64(flag.as<int64_t>(), pos.as<int64_t>(), n, sc2.p, s);
-  exclusive_scan_i64(v64.as<int64_t>(), wsum.as<int64_t>(), n, sc2.p, s);
-  total_kernel<<<1, 1, 0, s>>>(pos.as<int64_t>(), flag.as<int64_t>(), n, out.total.as<int64_t>());
-  GT_LAUNCH_CHECK();
-  reduce_write_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(k1.as<uint64_t>(), n, flag.as<int64_t>(),
-                                                                     pos.as<int64_t>(), kbw, out.word.as<int32_t>(),
-                                                                     out.file.as<int32_t>(), start.as<int64_t>());
-  GT_LAUNCH_CHECK();
-  reduce_sum_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(start.as<int64_t>(), out.total.as<int64_t>(),
-                                                                   wsum.as<int64_t>(), v64.as<int64_t>(), n,
-                                                                   out.cnt.as<uint64_t>());
-  GT_LAUNCH_CHECK();
+  const int kbits = kbw + bits_for(std::max(d.F - 1, 1));
+  const bool b = radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), v0.p, v1.p, 4, n, 0, kbits, kbits, kbits,
+                                     rs.p, s);
+  RunOut o;
+  o.low_bits = kbw;
+  o.word = out.word.as<int32_t>();
+  o.file = out.file.as<int32_t>();
+  o.count = out.cnt.as<uint64_t>();
+  o.rows = out.total.as<int64_t>();
+  reduce_runs(ctx, (b ? k1 : k0).as<uint64_t>(), nullptr, (b ? v1 : v0).as<uint32_t>(), n, nullptr, ~uint64_t(0), o, s);
 }
 
 gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
@@ -591,22 +631,32 @@ gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   const DevGrammar& d = g->d;
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
+  GT_CUDA(cudaMemcpyAsync(rb.status(), wr.status.p, 4, cudaMemcpyDeviceToDevice, s));
+  StatusScope scope(rb.status());
   const int64_t n = wr.bound;
+  const int64_t* nd = wr.total.as<int64_t>();
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(d.V + 1) * 8));
   auto* files = static_cast<int32_t*>(rb.alloc(size_t(n) * 4));
   int64_t* len = rb.new_len_slot();
-  GT_CUDA(cudaMemcpyAsync(len, wr.total.p, 8, cudaMemcpyDeviceToDevice, s));
+  GT_CUDA(cudaMemcpyAsync(len, nd, 8, cudaMemcpyDeviceToDevice, s));
   Buf k0(ctx, size_t(n) * 8, s), k1(ctx, size_t(n) * 8, s), f0(ctx, size_t(n) * 4, s);
   if (n > 0) {
     Buf rs(ctx, radix_scratch_bytes(n, true, 4), s);
-    word_keys_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(wr.word.as<int32_t>(), wr.file.as<int32_t>(),
-                                                                    wr.total.as<int64_t>(), n, d.V, k0.as<uint64_t>(),
-                                                                    f0.as<uint32_t>());
+    const int bits = bits_for(std::max(d.V - 1, 1));
+    // the sorted files have to land in the result: after an even number of
+    // passes that is the buffer the rows start in
+    const bool even = (bits + 7) / 8 % 2 == 0;
+    uint32_t* fa = even ? reinterpret_cast<uint32_t*>(files) : f0.as<uint32_t>();
+    uint32_t* fb = even ? f0.as<uint32_t>() : reinterpret_cast<uint32_t*>(files);
+    word_keys_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(wr.word.as<int32_t>(), wr.file.as<int32_t>(), nd,
+                                                                    k0.as<uint64_t>(), fa);
     GT_LAUNCH_CHECK();
-    radix_sort_u64(k0.as<uint64_t>(), k1.as<uint64_t>(), f0.p, files, 4, n, 0, bits_for(d.V), rs.p, s);
+    if (radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), fa, fb, 4, n, 0, bits, bits, bits, rs.p, s, nd) ==
+        even)
+      fail(GT_EINVAL, "unexpected number of sort passes");
+    if (!even) std::swap(k0, k1);
   }
-  word_offsets_kernel<<<grid_for(int64_t(d.V) + 1, threads, cap), threads, 0, s>>>(k1.as<uint64_t>(),
-                                                                                    wr.total.as<int64_t>(), d.V, off);
+  word_offsets_kernel<<<grid_for(int64_t(d.V) + 1, threads, cap), threads, 0, s>>>(k0.as<uint64_t>(), nd, d.V, off);
   GT_LAUNCH_CHECK();
   rb.field("offsets", off, int64_t(d.V) + 1);
   rb.field_dyn("file", files, len);
@@ -630,7 +680,7 @@ void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** 
     GT_LAUNCH_CHECK();
     for (int i = 0; i < n_tv; ++i)
       tv_out[i] = tv_from_arrays(g->ctx, wr.word.as<int32_t>(), wr.cnt.as<uint64_t>(), toff.as<int64_t>(),
-                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], s, d.V);
+                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], s, wr.status.as<uint32_t>(), d.V);
   }
   if (ii_out) *ii_out = bu_inverted_index(g, wr, s);
 }
@@ -646,12 +696,12 @@ gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s) {
                                                                           rkey.as<uint64_t>());
     GT_LAUNCH_CHECK();
   }
-  return ranked_from_rows(ctx, rkey, wr.file, wr.cnt, wr.total.as<int64_t>(), n, 0, false, uint64_t(g->d.V),
-                          uint64_t(g->max_file_len), s);
+  return ranked_from_rows(ctx, rkey, wr.file, wr.cnt, wr.total.as<int64_t>(), n, 0, false, bits_for(g->d.V),
+                          uint64_t(g->max_file_len), s, wr.status.as<uint32_t>());
 }
 
 // Per-file window rows of small files, built per file in shared memory.
-void bu_local_window_rows(gt_grammar* g, int kb, uint64_t key_pad, cudaStream_t s, Windows& out) {
+void bu_local_window_rows(gt_grammar* g, int kb, cudaStream_t s, Windows& out) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int64_t N = int64_t(d.N);
@@ -686,35 +736,39 @@ void bu_local_window_rows(gt_grammar* g, int kb, uint64_t key_pad, cudaStream_t 
 
 // Per-file window rows: windows owned by the root in each file, plus every
 // window inside each (file, root child) expansion, weighted by multiplicity.
-void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, uint64_t key_pad, cudaStream_t s, Windows& out) {
+void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, cudaStream_t s, Windows& out) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int threads = 256, cap = ctx->num_sms * 16;
   if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
   if (g->max_file_len <= kLocalMax && gparam(g, "bu_local", 1)) {
-    bu_local_window_rows(g, kb, key_pad, s, out);
+    bu_local_window_rows(g, kb, s, out);
     return;
   }
-  const int64_t n = 2 * d.root_len + g->bu_windows;
-  Phase ph(ctx, "bu_rows", s);
-  Buf k0(ctx, size_t(n) * 8, s), f0(ctx, size_t(n) * 8, s), v0(ctx, size_t(n) * 4, s);
-  Buf ecnt(ctx, size_t(d.ER) * 8, s), epos(ctx, size_t(d.ER) * 8, s), sc(ctx, scan_scratch_bytes(d.ER), s);
-  if (d.root_len > 0) {
-    root_window_rows_kernel<<<grid_for(d.root_len, threads, cap), threads, 0, s>>>(
-        d, head.as<int32_t>(), tail.as<int32_t>(), kb, key_pad, k0.as<uint64_t>(), f0.as<uint64_t>(),
-        v0.as<uint32_t>());
-    GT_LAUNCH_CHECK();
+  FileRowBufs rows;
+  {
+    Phase ph(ctx, "bu_rows", s);
+    const FileRows fr = rows.make(ctx, kb, d.F, 2 * d.root_len + g->bu_windows, s);
+    Buf ecnt(ctx, size_t(d.ER) * 8, s), epos(ctx, size_t(d.ER) * 8, s), sc(ctx, scan_scratch_bytes(d.ER), s);
+    Buf first(ctx, 8, s);
+    if (d.root_len > 0) {
+      root_window_rows_kernel<<<unsigned((d.root_len + kTile - 1) / kTile), kRootWinThreads, 0, s>>>(
+          d, head.as<int32_t>(), tail.as<int32_t>(), kb, fr);
+      GT_LAUNCH_CHECK();
+    }
+    if (d.ER > 0) {
+      redge_len_kernel<<<grid_for(d.ER, threads, cap), threads, 0, s>>>(d, true, ecnt.as<int64_t>());
+      GT_LAUNCH_CHECK();
+      exclusive_scan_i64(ecnt.as<int64_t>(), epos.as<int64_t>(), d.ER, sc.p, s);
+      GT_CUDA(cudaMemcpyAsync(first.p, rows.n.p, 8, cudaMemcpyDeviceToDevice, s));
+      child_window_rows_kernel<<<grid_for(d.ER, 128, cap), 128, 0, s>>>(d, kb, epos.as<int64_t>(),
+                                                                       first.as<unsigned long long>(), fr);
+      GT_LAUNCH_CHECK();
+      add_rows_kernel<<<1, 1, 0, s>>>(first.as<unsigned long long>(), g->bu_windows, rows.n.as<unsigned long long>());
+      GT_LAUNCH_CHECK();
+    }
   }
-  if (d.ER > 0) {
-    redge_len_kernel<<<grid_for(d.ER, threads, cap), threads, 0, s>>>(d, true, ecnt.as<int64_t>());
-    GT_LAUNCH_CHECK();
-    exclusive_scan_i64(ecnt.as<int64_t>(), epos.as<int64_t>(), d.ER, sc.p, s);
-    child_window_rows_kernel<<<grid_for(d.ER, 128, cap), 128, 0, s>>>(
-        d, kb, epos.as<int64_t>(), k0.as<uint64_t>() + 2 * d.root_len, f0.as<uint64_t>() + 2 * d.root_len,
-        v0.as<uint32_t>() + 2 * d.root_len);
-    GT_LAUNCH_CHECK();
-  }
-  sort_by_file_key(ctx, k0, f0, v0, n, 3 * kb + 1, bits_for(d.F), s, out);
+  sort_file_rows(ctx, rows, kb, d.F, s, out);
 }
 
 }  // namespace gt

@@ -99,11 +99,13 @@ struct TileWin {
   int n[4];
 };
 
+// file (optional): the file of each symbol of the root.
 __device__ __forceinline__ int tile_windows(const DevGrammar& d, const int32_t* __restrict__ head,
-                                            const int32_t* __restrict__ tail, int kb, int64_t j0, TileWin& t) {
+                                            const int32_t* __restrict__ tail, int kb, int64_t j0, TileWin& t,
+                                            int32_t* file = nullptr) {
   int c = 0;
   int64_t end = -1;  // end of the body sequence holding the previous symbol (rule or root file)
-  int32_t rule = 0, f;
+  int32_t rule = 0, f = -1;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int64_t j = j0 + i;
@@ -114,6 +116,7 @@ __device__ __forceinline__ int tile_windows(const DevGrammar& d, const int32_t* 
       // when the previous one ended (or at a root / rule boundary)
       if (j >= end || j == d.root_len) end = seq_end(d, j, &rule, &f);
       t.r[i] = rule;
+      if (file) file[i] = f;
       t.n[i] = windows_at(d, head, tail, j, end, kb, t.k[i]);
     }
     c += t.n[i];
@@ -154,8 +157,9 @@ __device__ __forceinline__ void publish_aggregate(unsigned long long* flags, int
 // prefix.  Returns the exclusive prefix (to every lane); after kSpinLimit
 // polls of an item that published nothing it sets ST_TIMEOUT in *status,
 // still publishes (so that later items are not held up) and returns -1.
+// publish == false: the item's own word already holds its final value.
 __device__ __forceinline__ int64_t warp_look_back(unsigned long long* flags, int64_t item, uint64_t agg,
-                                                  unsigned* status, int spin_limit = kSpinLimit) {
+                                                  unsigned* status, int spin_limit = kSpinLimit, bool publish = true) {
   const int lane = threadIdx.x & 31;
   if (item == 0) return 0;
   uint64_t excl = 0;
@@ -185,7 +189,7 @@ __device__ __forceinline__ int64_t warp_look_back(unsigned long long* flags, int
   }
   if (lane == 0) {
     if (!ok && status) atomicOr(status, ST_TIMEOUT);
-    atomicExch(&flags[item], kFlagIncl | (excl + agg));
+    if (publish) atomicExch(&flags[item], kFlagIncl | (excl + agg));
   }
   return ok ? int64_t(excl) : -1;
 }

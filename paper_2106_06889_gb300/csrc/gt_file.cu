@@ -945,15 +945,11 @@ __global__ void last_total_kernel(const int64_t* __restrict__ ex, const int64_t*
 // top-k: key = file << 32 | (2^32 - 1 - count), sorted stably over entries that
 // are already in ascending word order inside each file.
 __global__ void topk_keys_kernel(const int32_t* __restrict__ word, const uint64_t* __restrict__ cnt,
-                                 const int64_t* __restrict__ tv_off, int32_t F, int64_t bound,
+                                 const int64_t* __restrict__ tv_off, int32_t F,
                                  uint64_t* __restrict__ keys, uint32_t* __restrict__ idx) {
   const int64_t n = tv_off[F];
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < bound; i += int64_t(gridDim.x) * blockDim.x) {
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     idx[i] = uint32_t(i);
-    if (i >= n) {
-      keys[i] = uint64_t(uint32_t(F)) << 32;  // padding sorts last
-      continue;
-    }
     int32_t lo = 0, hi = F;  // file of entry i: last f with tv_off[f] <= i
     while (hi - lo > 1) {
       const int32_t mid = (lo + hi) >> 1;
@@ -984,7 +980,7 @@ __global__ void topk_gather_kernel(const uint32_t* __restrict__ idx, const int64
 }
 
 struct FileHist {
-  Buf slot_word, slot_cnt, nnz, bits, off, total;
+  Buf slot_word, slot_cnt, nnz, bits, off, total, status;  // status: flags raised while the pieces were made
   int nb = 0;
   int64_t bound = 0;  // bound on term-vector entries (= inverted-index postings)
 };
@@ -1326,6 +1322,9 @@ void file_hist(gt_grammar* g, cudaStream_t s, FileHist& fh) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int32_t F = d.F, V = d.V;
+  fh.status = Buf(ctx, 4, s);
+  GT_CUDA(cudaMemsetAsync(fh.status.p, 0, 4, s));
+  StatusScope scope(fh.status.as<uint32_t>());
   FileWeights fwt;
   {
     Phase ph(ctx, "file_weights", s);
@@ -1390,9 +1389,10 @@ gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t
       GT_LAUNCH_CHECK();
     }
     return tv_from_arrays(ctx, tw.as<int32_t>(), tc.as<uint64_t>(), full_off.as<int64_t>(), fh.total.as<int64_t>(),
-                          nb_, d.F, top_k, s, d.V);
+                          nb_, d.F, top_k, s, fh.status.as<uint32_t>(), d.V);
   }
   ResultBuilder rb(ctx, s);
+  GT_CUDA(cudaMemcpyAsync(rb.status(), fh.status.p, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "tv_out", s);
   auto* tv_off = static_cast<int64_t*>(rb.alloc(size_t(d.F + 1) * 8));
   auto* word = static_cast<int32_t*>(rb.alloc(size_t(nb_) * 4));
@@ -1421,6 +1421,7 @@ gt_result* inverted_index_from(gt_grammar* g, FileHist& fh, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   ResultBuilder rb(ctx, s);
+  GT_CUDA(cudaMemcpyAsync(rb.status(), fh.status.p, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "ii_out", s);
   const int threads = 256, cap = ctx->num_sms * 16;
   const int64_t V = d.V;
@@ -1483,8 +1484,8 @@ gt_result* run_ranked_words(gt_grammar* g, cudaStream_t s) {
                                                                       rkey.as<uint64_t>(), rfile.as<int32_t>());
     GT_LAUNCH_CHECK();
   }
-  return ranked_from_rows(ctx, rkey, rfile, tc, fh.total.as<int64_t>(), bound, 0, false, uint64_t(d.V),
-                          uint64_t(g->max_file_len), s);
+  return ranked_from_rows(ctx, rkey, rfile, tc, fh.total.as<int64_t>(), bound, 0, false, bits_for(d.V),
+                          uint64_t(g->max_file_len), s, fh.status.as<uint32_t>());
 }
 
 __global__ void copy_rows_kernel(const int32_t* __restrict__ w, const uint64_t* __restrict__ c,
@@ -1518,9 +1519,11 @@ __global__ void tfidf_kernel(const int32_t* __restrict__ word, const uint64_t* _
 
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
                           const int64_t* total, int64_t bound, int32_t F, int top_k, cudaStream_t s,
-                          int32_t V) {
+                          const uint32_t* status_in, int32_t V) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
+  GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
+  StatusScope scope(rb.status());
   Phase ph(ctx, "tv_out", s);
   auto* tv_off = static_cast<int64_t*>(rb.alloc(size_t(F + 1) * 8));
   if (top_k <= 0) {
@@ -1554,10 +1557,13 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
     Buf i1(ctx, size_t(bound) * 4, s), rs(ctx, radix_scratch_bytes(bound, true, 4), s);
     Buf kc(ctx, size_t(F) * 8 + 8, s), sc(ctx, scan_scratch_bytes(F + 1), s);
     if (bound > 0) {
-      topk_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, tv_off_in, F, bound,
-                                                                          k0.as<uint64_t>(), i0.as<uint32_t>());
+      topk_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, tv_off_in, F, k0.as<uint64_t>(),
+                                                                          i0.as<uint32_t>());
       GT_LAUNCH_CHECK();
-      radix_sort_u64(k0.as<uint64_t>(), k1.as<uint64_t>(), i0.p, i1.p, 4, bound, 0, 32 + bits_for(F), rs.p, s);
+      const int kbits = 32 + bits_for(std::max(F - 1, 1));
+      if (!radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), i0.p, i1.p, 4, bound, 0, kbits, kbits, kbits, rs.p,
+                               s, total))
+        std::swap(i0, i1);
     }
     topk_count_kernel<<<grid_for(F, 256, cap), 256, 0, s>>>(tv_off_in, F, top_k, kc.as<int64_t>());
     GT_LAUNCH_CHECK();

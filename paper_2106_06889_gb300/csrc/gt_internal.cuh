@@ -45,6 +45,19 @@ extern std::atomic<long long> g_launches;
 // phase timers in primitives that take no context.
 extern thread_local gt_ctx* t_call_ctx;
 
+// The status word that waits inside the primitives (scan, sort, reduction)
+// report to: the one of the enclosing StatusScope on this thread, else the
+// context's (read by gt_sync).
+uint32_t* status_word();
+extern thread_local uint32_t* t_status;
+struct StatusScope {
+  uint32_t* const outer;
+  explicit StatusScope(uint32_t* st) : outer(t_status) { t_status = st; }
+  StatusScope(const StatusScope&) = delete;
+  StatusScope& operator=(const StatusScope&) = delete;
+  ~StatusScope() { t_status = outer; }
+};
+
 // Bits of the device status word.
 enum : uint32_t {
   ST_TABLE_FULL = 1u,
@@ -413,9 +426,12 @@ void run_word_count_multi(gt_grammar* const* gs, uint64_t* const* counts, int n,
 void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s);
 
 // Sorted 3-word window rows: compact keys (kb bits per word, key_pad above
-// every real key), optional file keys, weights; n rows including pads.
+// every real key) and weights; n rows including pads.  Rows that carry files
+// (*n_dev of at most n, no pads) hold them above the key (file_in_key) or, with
+// the weight below, in fkeys (file << 32 | weight).
 struct Windows {
-  Buf keys, fkeys, vals;
+  Buf keys, fkeys, vals, n_dev;
+  bool file_in_key = false;
   int64_t n = 0;
   int kb = 1;
   uint64_t key_pad = 0;
@@ -429,12 +445,34 @@ struct Windows {
 // (expansion of each distinct (file, root child) pair); "file_strategy" 0 = auto
 int file_strategy(const gt_grammar* g);
 
-// gt_seq.cu
-void sort_by_file_key(gt_ctx* ctx, Buf& k0, Buf& f0, Buf& v0, int64_t bound, int key_bits, int file_bits,
-                      cudaStream_t s, Windows& out);
+// gt_seq.cu: per-file window rows under construction, in any order (see
+// sort_file_rows for the two layouts); kernels claim places in *n.
+struct FileRows {
+  uint64_t* key;
+  uint32_t* val;  // file << shift | key, weight here
+  uint64_t* pay;  // or: key, file << 32 | weight here
+  unsigned long long* n;
+  int shift;
+  __device__ __forceinline__ void put(int64_t o, int32_t f, uint64_t k, uint32_t w) const {
+    if (val) {
+      key[o] = (uint64_t(uint32_t(f)) << shift) | k;
+      val[o] = w;
+    } else {
+      key[o] = k;
+      pay[o] = (uint64_t(uint32_t(f)) << 32) | w;
+    }
+  }
+};
+struct FileRowBufs {
+  Buf keys, vals, n;
+  int64_t bound = 0;
+  bool fits = false;
+  FileRows make(gt_ctx* ctx, int kb, int32_t F, int64_t bound, cudaStream_t s);
+};
+void sort_file_rows(gt_ctx* ctx, FileRowBufs& r, int kb, int32_t F, cudaStream_t s, Windows& out);
 
 // gt_bu.cu: bottom-up per-file rows
-void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, uint64_t key_pad, cudaStream_t s, Windows& out);
+void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, cudaStream_t s, Windows& out);
 void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** tv_out, gt_result** ii_out,
                        cudaStream_t s);
 gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s);
@@ -456,7 +494,7 @@ int64_t gparam(const gt_grammar* g, const char* name, int64_t dflt);
 constexpr int kTfIdf = -1;
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
                           const int64_t* total, int64_t bound, int32_t F, int top_k, cudaStream_t s,
-                          int32_t V = 0);
+                          const uint32_t* status_in, int32_t V = 0);
 // Device pointer of a result field and the device slot holding its length
 // (valid on the result's stream before the result completes).
 void result_device_field(gt_result* r, const char* field, void** ptr, const int64_t** d_len);
@@ -467,9 +505,9 @@ gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s);
 gt_result* run_tfidf(gt_grammar* g, cudaStream_t s);
 gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s);
 // gt_seq.cu: rows (key, weight) -> one row per distinct key with the weights
-// summed, ascending key; n rows (host bound), rows past *n_dev hold key_pad
+// summed, ascending key; at most n rows (*n_dev of them, if given), rows of key_pad skipped
 gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int key_bits, uint64_t key_pad,
-                           cudaStream_t s, const uint32_t* status_in = nullptr);
+                           cudaStream_t s, const uint32_t* status_in = nullptr, const int64_t* n_dev = nullptr);
 // gt_seqg.cu: the global count (per_file == 0) by sample-sort buckets
 gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s);
 // owned windows of every tile of kTile symbols, exclusive scan [ntiles + 1]:
@@ -478,9 +516,11 @@ gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s);
 const int64_t* seq_tile_offsets(gt_grammar* g, const int32_t* head, const int32_t* tail, int kb, cudaStream_t s);
 gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s);
 // rows (key, file, count) -> ranked index; keys are compact 3-word keys
-// (windows = true, kb bits per word) or word ids (windows = false)
+// (windows = true, kb bits per word) or word ids (windows = false), all of at
+// most key_bits bits; *status_in: flags raised while the rows were made
 gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
-                            int kb, bool windows, uint64_t key_pad, uint64_t max_count, cudaStream_t s);
+                            int kb, bool windows, int key_bits, uint64_t max_count, cudaStream_t s,
+                            const uint32_t* status_in);
 // gt_file.cu: ranked index over words (rows from the term vector)
 gt_result* run_ranked_words(gt_grammar* g, cudaStream_t s);
 
@@ -508,13 +548,40 @@ bool run_file_batch(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** tv_
                     cudaStream_t s, uint64_t* wc_out = nullptr);
 gt_result* run_inverted_index(gt_grammar* g, cudaStream_t s);
 
+// gt_reduce.cu: runs of equal keys (and equal files, with fkeys) in sorted rows,
+// rows of key_pad at the end skipped; n_dev as for the sort.  vals == nullptr:
+// every row counts 1.  Which arrays are given says what is written per run:
+struct RunOut {
+  int low_bits = 0;           // key = file << low_bits | rest (0: no file in the key)
+  uint64_t* key = nullptr;    // the key (its rest), kb bits per word spread to 21-bit fields (kb 0: as it is)
+  int kb = 0;
+  int32_t* word = nullptr;    // the key's rest as int32
+  int32_t* file = nullptr;    // the run's file: the key's high part, or its fkeys value
+  uint64_t* count = nullptr;  // sum of the values
+  uint32_t* mult = nullptr;   // the same in 32 bits
+  int64_t* off = nullptr;     // the run's first row (vals == nullptr); off[runs] = *off_end, or the rows
+  const int64_t* off_end = nullptr;
+  int64_t* rows = nullptr;    // number of runs (always given)
+  int64_t* rows1 = nullptr;   // number of runs + 1
+};
+void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
+                 const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s);
+
 // gt_sort.cu: device primitives
 size_t scan_scratch_bytes(int64_t n);
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratch, cudaStream_t s);
 size_t radix_scratch_bytes(int64_t n, bool with_values, int value_bytes);
-// Stable LSD radix sort of n uint64 keys on bits [begin_bit, end_bit); values
-// (optional, value_bytes 4 or 8) move with their keys.  Results land in
-// keys_out / vals_out.  keys_in / vals_in are clobbered.
+// Stable LSD radix sort of n uint64 keys on bits [begin_a, end_a) and then
+// [begin_b, end_b); values (optional, value_bytes 4 or 8) move with their keys.
+// The passes alternate between the a and the b buffers: returns true if the
+// sorted rows are in the b buffers, false if they are in the a buffers (an even
+// number of passes).  n_dev (optional): the rows there really are, on the
+// device (at most n).
+bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
+                         int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s,
+                         const int64_t* n_dev = nullptr);
+// The same on bits [begin_bit, end_bit).  Results land in keys_out / vals_out
+// (copied there after an even number of passes).  keys_in / vals_in are clobbered.
 void radix_sort_u64(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* vals_out, int value_bytes,
                     int64_t n, int begin_bit, int end_bit, void* scratch, cudaStream_t s);
 // The same on bits [begin_a, end_a) then [begin_b, end_b) (keys whose other

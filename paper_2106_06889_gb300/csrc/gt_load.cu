@@ -137,31 +137,6 @@ __global__ void __launch_bounds__(kEkThreads) edge_keys_kernel(
   }
 }
 
-__global__ void run_flags_kernel(const uint64_t* __restrict__ k, int64_t n, int64_t* __restrict__ flag) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    flag[i] = (i == 0 || k[i] != k[i - 1]) ? 1 : 0;
-}
-
-__global__ void run_compact_kernel(const uint64_t* __restrict__ k, int64_t n, const int64_t* __restrict__ flag,
-                                   const int64_t* __restrict__ pos, uint64_t* __restrict__ uk,
-                                   int64_t* __restrict__ ustart) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    if (flag[i]) {
-      uk[pos[i]] = k[i];
-      ustart[pos[i]] = i;
-    }
-}
-
-// Split unique (hi << 32 | lo) keys into lo and the run length (multiplicity).
-__global__ void run_split_kernel(const uint64_t* __restrict__ uk, const int64_t* __restrict__ ustart, int64_t nu,
-                                 int64_t n, int32_t* __restrict__ lo_out, uint32_t* __restrict__ mult) {
-  for (int64_t j = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; j < nu; j += int64_t(gridDim.x) * blockDim.x) {
-    lo_out[j] = int32_t(uint32_t(uk[j]));
-    const int64_t next = j + 1 < nu ? ustart[j + 1] : n;
-    mult[j] = uint32_t(next - ustart[j]);
-  }
-}
-
 // off[h] = first index whose high 32 bits are >= h, for h in [0, nh].
 __global__ void csr_offsets_kernel(const uint64_t* __restrict__ keys, int64_t n, int64_t nh, int64_t* __restrict__ off) {
   for (int64_t h = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; h <= nh; h += int64_t(gridDim.x) * blockDim.x)
@@ -554,21 +529,19 @@ int64_t dedup_csr(gt_grammar* g, uint64_t* keys, int64_t n, int hi_bits, int lo_
   Buf sorted(ctx, size_t(n) * 8, s);
   Buf rscratch(ctx, radix_scratch_bytes(n, false, 0), s);
   sort_hi_lo(keys, sorted.as<uint64_t>(), nullptr, nullptr, 0, n, lo_bits, hi_bits, rscratch.p, s);
-  Buf flag(ctx, size_t(n) * 8, s), pos(ctx, size_t(n) * 8, s);
-  Buf sscratch(ctx, scan_scratch_bytes(n), s);
+  // distinct keys and their multiplicities, into scratch (their number is not known yet)
+  Buf du(ctx, size_t(n) * 8, s), dm(ctx, size_t(n) * 4, s), dn(ctx, 8, s);
   int64_t nu = 0;
   if (n > 0) {
-    run_flags_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(sorted.as<uint64_t>(), n, flag.as<int64_t>());
-    GT_LAUNCH_CHECK();
-    exclusive_scan_i64(flag.as<int64_t>(), pos.as<int64_t>(), n, sscratch.p, s);
-    int64_t last_pos = 0, last_flag = 0;
-    GT_CUDA(cudaMemcpyAsync(&last_pos, pos.as<int64_t>() + n - 1, 8, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaMemcpyAsync(&last_flag, flag.as<int64_t>() + n - 1, 8, cudaMemcpyDeviceToHost, s));
+    RunOut o;
+    o.key = du.as<uint64_t>();
+    o.mult = dm.as<uint32_t>();
+    o.rows = dn.as<int64_t>();
+    reduce_runs(ctx, sorted.as<uint64_t>(), nullptr, nullptr, n, nullptr, ~uint64_t(0), o, s);
+    GT_CUDA(cudaMemcpyAsync(&nu, dn.p, 8, cudaMemcpyDeviceToHost, s));
     GT_CUDA(cudaStreamSynchronize(s));
-    nu = last_pos + last_flag;
   }
   uint64_t* uk = dalloc<uint64_t>(g, size_t(prefix + nu), s);
-  Buf ustart(ctx, size_t(nu) * 8, s);
   int32_t* lo = dalloc<int32_t>(g, size_t(prefix + nu), s);
   uint32_t* mult = dalloc<uint32_t>(g, size_t(prefix + nu), s);
   int64_t* off = dalloc<int64_t>(g, size_t(nh) + 1, s);
@@ -579,11 +552,9 @@ int64_t dedup_csr(gt_grammar* g, uint64_t* keys, int64_t n, int hi_bits, int lo_
     GT_CUDA(cudaMemcpyAsync(mult, pre_mult, size_t(prefix) * 4, cudaMemcpyDeviceToDevice, s));
   }
   if (n > 0) {
-    run_compact_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(
-        sorted.as<uint64_t>(), n, flag.as<int64_t>(), pos.as<int64_t>(), uk + prefix, ustart.as<int64_t>());
-    GT_LAUNCH_CHECK();
-    run_split_kernel<<<grid_for(nu, threads, cap), threads, 0, s>>>(uk + prefix, ustart.as<int64_t>(), nu, n,
-                                                                    lo + prefix, mult + prefix);
+    GT_CUDA(cudaMemcpyAsync(uk + prefix, du.p, size_t(nu) * 8, cudaMemcpyDeviceToDevice, s));
+    GT_CUDA(cudaMemcpyAsync(mult + prefix, dm.p, size_t(nu) * 4, cudaMemcpyDeviceToDevice, s));
+    low32_kernel<<<grid_for(nu, threads, cap), threads, 0, s>>>(du.as<uint64_t>(), nu, lo + prefix);
     GT_LAUNCH_CHECK();
   }
   csr_offsets_kernel<<<grid_for(nh + 1, threads, cap), threads, 0, s>>>(uk, prefix + nu, nh, off);
@@ -908,7 +879,9 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     }
     unsigned long long hb[3];
     GT_CUDA(cudaMemcpyAsync(hb, ctr + 12, 24, cudaMemcpyDeviceToHost, s));
+    GT_CUDA(cudaMemcpyAsync(&st, ctx->d_status, 4, cudaMemcpyDeviceToHost, s));
     GT_CUDA(cudaStreamSynchronize(s));
+    if (st & ST_TIMEOUT) fail(GT_ETIMEOUT, "a bounded device wait timed out");
     g->bu_words = int64_t(hb[0]);
     g->bu_windows = int64_t(hb[1]);
     g->max_file_len = int64_t(hb[2]);

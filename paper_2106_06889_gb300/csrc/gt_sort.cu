@@ -3,11 +3,21 @@
 // These back the memory-pool sizing (exclusive scans of per-rule sizes, the
 // "memory pool" of Section IV-B), the edge deduplication at load time and the
 // canonical ordering of every result.
+//
+// Both are single-pass kernels: a CTA takes the next tile by an atomic ticket,
+// publishes the tile's totals and gets what precedes it by a bounded decoupled
+// look-back (see gt_device.cuh); a wait that gives up sets ST_TIMEOUT in the
+// call's status word (status_word()).
 #include <type_traits>
 
 #include "gt_device.cuh"
 
 namespace gt {
+
+thread_local uint32_t* t_status = nullptr;
+
+uint32_t* status_word() { return t_status ? t_status : (t_call_ctx ? t_call_ctx->d_status : nullptr); }
+
 namespace {
 
 constexpr int kScanThreads = 256;
@@ -45,25 +55,26 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
   return r;
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const int64_t* __restrict__ in, int64_t n,
-                                                                   int64_t* __restrict__ bsum) {
-  const int64_t base = int64_t(blockIdx.x) * kScanChunk;
-  int64_t s = 0;
-  for (int i = threadIdx.x; i < kScanChunk; i += kScanThreads) {
-    int64_t idx = base + i;
-    if (idx < n) s += in[idx];
-  }
-  int64_t total;
-  block_excl_scan(s, &total);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int64_t* in, int64_t* out, int64_t n,
-                                                                  const int64_t* __restrict__ boff) {
+// One tile of kScanChunk values per CTA.  With one tile (flags == nullptr) the
+// scan starts at 0; otherwise tiles are taken in ticket order (flags[tiles] is
+// the ticket) and start at the look-back prefix.  Bound by the 16 bytes per
+// value it moves; the former two passes (block sums, then the scan proper, with
+// a recursive scan of the sums between them) read the values twice and took
+// three to five launches.
+__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int64_t* in, int64_t* out, int64_t n,
+                                                            unsigned long long* __restrict__ flags, int64_t tiles,
+                                                            unsigned* __restrict__ status) {
   __shared__ int64_t tile[kScanChunk];
-  const int64_t base = int64_t(blockIdx.x) * kScanChunk;
+  __shared__ int64_t s_item, s_prefix;
+  int64_t item = 0;
+  if (flags) {
+    if (threadIdx.x == 0) s_item = int64_t(atomicAdd(&flags[tiles], 1ull));
+    __syncthreads();
+    item = s_item;
+  }
+  const int64_t base = item * kScanChunk;
   for (int i = threadIdx.x; i < kScanChunk; i += kScanThreads) {
-    int64_t idx = base + i;
+    const int64_t idx = base + i;
     tile[i] = idx < n ? in[idx] : 0;
   }
   __syncthreads();
@@ -74,7 +85,18 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int64_t*
     local[j] = tile[threadIdx.x * kScanItems + j];
     s += local[j];
   }
-  int64_t off = block_excl_scan(s, nullptr) + (boff ? boff[blockIdx.x] : 0);
+  int64_t total;
+  int64_t off = block_excl_scan(s, &total);
+  if (flags) {
+    if (threadIdx.x < 32) {
+      if (threadIdx.x == 0) publish_aggregate(flags, item, uint64_t(total));
+      __syncwarp();
+      const int64_t p = warp_look_back(flags, item, uint64_t(total), status);
+      if (threadIdx.x == 0) s_prefix = p < 0 ? 0 : p;
+    }
+    __syncthreads();
+    off += s_prefix;
+  }
 #pragma unroll
   for (int j = 0; j < kScanItems; ++j) {
     tile[threadIdx.x * kScanItems + j] = off;
@@ -82,142 +104,199 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int64_t*
   }
   __syncthreads();
   for (int i = threadIdx.x; i < kScanChunk; i += kScanThreads) {
-    int64_t idx = base + i;
+    const int64_t idx = base + i;
     if (idx < n) out[idx] = tile[i];
   }
 }
 
 // ---- radix sort -------------------------------------------------------------
+//
+// One histogram kernel reads the keys once and counts the digits of every
+// pass; each pass is then one scatter kernel whose tiles get their digits'
+// first rows by look-back (Adinets & Merrill, "Onesweep: A Faster Least
+// Significant Digit Radix Sort for GPUs", arXiv 2206.01784).
 
 constexpr int kRsThreads = 256;  // one thread per digit value in the per-tile bookkeeping
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsItems = 8;      // keys per thread by default ("radix_items" 16 doubles the tile)
-constexpr int kRsTile = kRsThreads * kRsItems;  // keys per tile (the smallest tile: scratch is sized for it)
+constexpr int kRsBins = 256;
+constexpr int kRsMaxPasses = 8;
+constexpr int kRsSmallItems = 8, kRsLargeItems = 16;  // keys per thread
+// Below this many rows tiles of 2048 keys, above it tiles of 4096.  Measured
+// per pass (60-bit Zipf keys, 4-byte values): 163k rows 8.6 against 10.7 us (few
+// tiles: latency), 4M rows 43 against 38 us (the per-tile bookkeeping over 256
+// digits counts).
+constexpr int64_t kRsLargeRows = int64_t(1) << 20;
 
-// Per-tile digit counts, stored tile-major (hist[tile * 256 + d]) so that
-// each CTA writes one contiguous row.
-template <int ITEMS>
-__global__ void __launch_bounds__(kRsThreads) radix_upsweep_kernel(const uint64_t* __restrict__ keys, int64_t n,
-                                                                   int shift, uint32_t mask,
-                                                                   uint32_t* __restrict__ hist) {
-  constexpr int kRsItems = ITEMS, kRsTile = kRsThreads * ITEMS;
-  __shared__ uint32_t h[kRsWarps][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t wbase = int64_t(blockIdx.x) * kRsTile + int64_t(warp) * 32 * kRsItems;
-  uint64_t key[kRsItems];  // every load issued before the counters are cleared
-#pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t idx = wbase + it * 32 + lane;
-    key[it] = idx < n ? keys[idx] : 0;
-  }
-  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) h[i / 256][i % 256] = 0;
+struct RadixPasses {
+  int shift[kRsMaxPasses];
+  int bits[kRsMaxPasses];
+  int n;
+};
+
+// Digit counts of every pass in one read of the keys: counts[p * 256 + d].
+// Bound by its shared-memory atomics (one per key and pass).
+constexpr int kRhThreads = 512;
+constexpr int kRhItems = 4;
+
+__global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const uint64_t* __restrict__ keys, int64_t n_max,
+                                                                const int64_t* __restrict__ n_dev,
+                                                                const __grid_constant__ RadixPasses ps,
+                                                                unsigned long long* __restrict__ counts) {
+  const int64_t n = n_dev ? min(*n_dev, n_max) : n_max;
+  __shared__ uint32_t h[kRsMaxPasses * kRsBins];
+  for (int i = threadIdx.x; i < ps.n * kRsBins; i += kRhThreads) h[i] = 0;
   __syncthreads();
-  // counting only: one shared atomic per key into the warp's own counters
-  // (measured faster than ballot multisplit, also when all keys share a digit)
+  constexpr int64_t kStep = int64_t(kRhThreads) * kRhItems;
+  for (int64_t b = blockIdx.x * kStep; b < n; b += gridDim.x * kStep) {
+    uint64_t k[kRhItems];
 #pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t idx = wbase + it * 32 + lane;
-    if (idx < n) atomicAdd(&h[warp][uint32_t(key[it] >> shift) & mask], 1u);
+    for (int j = 0; j < kRhItems; ++j) {
+      const int64_t i = b + j * kRhThreads + threadIdx.x;
+      k[j] = i < n ? keys[i] : 0;
+    }
+    for (int p = 0; p < ps.n; ++p) {
+      const uint32_t mask = (1u << ps.bits[p]) - 1u;
+      const int shift = ps.shift[p];
+#pragma unroll
+      for (int j = 0; j < kRhItems; ++j)
+        if (b + j * kRhThreads + threadIdx.x < n) atomicAdd(&h[p * kRsBins + (uint32_t(k[j] >> shift) & mask)], 1u);
+    }
   }
   __syncthreads();
-  const int d = threadIdx.x;
-  uint32_t t = 0;
+  for (int i = threadIdx.x; i < ps.n * kRsBins; i += kRhThreads)
+    if (h[i]) atomicAdd(&counts[i], (unsigned long long)(h[i]));
+}
+
+// Look-back words of a pass: one per (tile, digit), state in the top two bits
+// (1 the tile's own count, 2 the rows of the digit up to and including the
+// tile), value below; 32-bit while the rows fit 30 bits, else 64-bit.
+template <class W>
+struct RsFlag {
+  static constexpr W kAgg = W(1) << (sizeof(W) * 8 - 2), kIncl = W(2) << (sizeof(W) * 8 - 2), kVal = kAgg - 1;
+};
+
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v));
+}
+__device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v));
+}
+
+// Rows of one digit in the tiles before `tile`: words are read four tiles at a
+// time, nearest first, up to the first one that holds a prefix.  Tiles are
+// taken in ticket order, so the ones waited for are running; the wait is
+// bounded anyway (ST_TIMEOUT; the sum so far then keeps every store in range).
+template <class W>
+__device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t tile, int bin, unsigned* status) {
+  W sum = 0;
+  int64_t t = tile - 1;
+  int spins = 0;
+  while (true) {
+    W v[4];
 #pragma unroll
-  for (int w = 0; w < kRsWarps; ++w) t += h[w][d];
-  hist[int64_t(blockIdx.x) * 256 + d] = t;
-}
-
-// Output offsets of every (tile, digit): offs[tile * 256 + d] = (keys of
-// smaller digits) + (keys of digit d in earlier tiles).  Tiles are grouped in
-// chunks of kRsChunk: per-chunk digit sums (digit-major, so one scan orders
-// them by digit, then chunk), then a running sum inside each chunk.
-constexpr int kRsChunk = 64;
-
-__global__ void __launch_bounds__(256) radix_chunk_sum_kernel(const uint32_t* __restrict__ hist, int64_t ntiles,
-                                                               int64_t nchunks, int64_t* __restrict__ csum) {
-  const int64_t c = blockIdx.x;
-  const int d = threadIdx.x;
-  const int64_t t1 = min(ntiles, (c + 1) * kRsChunk);
-  int64_t sum = 0;
-  for (int64_t t = c * kRsChunk; t < t1; ++t) sum += hist[t * 256 + d];
-  csum[int64_t(d) * nchunks + c] = sum;
-}
-
-__global__ void __launch_bounds__(256) radix_chunk_offsets_kernel(const uint32_t* __restrict__ hist,
-                                                                   const int64_t* __restrict__ cpre, int64_t ntiles,
-                                                                   int64_t nchunks, int64_t* __restrict__ offs) {
-  const int64_t c = blockIdx.x;
-  const int d = threadIdx.x;
-  const int64_t t1 = min(ntiles, (c + 1) * kRsChunk);
-  int64_t run = cpre[int64_t(d) * nchunks + c];
-  for (int64_t t = c * kRsChunk; t < t1; ++t) {
-    offs[t * 256 + d] = run;
-    run += hist[t * 256 + d];
+    for (int q = 0; q < 4; ++q) v[q] = t >= q ? ld_relaxed(words + (t - q) * kRsBins + bin) : RsFlag<W>::kIncl;
+    int used = 0;
+    bool more = true;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      more = more && v[q] > RsFlag<W>::kVal;  // published
+      if (more) {
+        sum += v[q] & RsFlag<W>::kVal;
+        ++used;
+        if (v[q] & RsFlag<W>::kIncl) return sum;
+      }
+    }
+    t -= used;
+    if (used == 0) {
+      if (++spins > kSpinLimit) {
+        if (status) atomicOr(status, ST_TIMEOUT);
+        return sum;
+      }
+      __nanosleep(20);
+    }
   }
 }
 
-// Stable scatter of one tile.  Warp w owns the w-th slice of the tile and
-// ranks its keys 32 at a time in lane order; per-digit counts across warps
-// and digits give every key its place in the tile sorted by digit.  The tile
-// is rearranged in shared memory in that order and written out with
-// consecutive threads writing consecutive addresses of each digit's run.
-template <int VB, int ITEMS>
-__global__ void __launch_bounds__(kRsThreads, ITEMS == 8 ? 4 : 2) radix_downsweep_kernel(
-    const uint64_t* __restrict__ kin, uint64_t* __restrict__ kout, const void* __restrict__ vin,
-    void* __restrict__ vout, int64_t n, int shift, uint32_t mask, const int64_t* __restrict__ offs) {
-  constexpr int kRsItems = ITEMS, kRsTile = kRsThreads * ITEMS;
-  __shared__ uint32_t wcnt[kRsWarps][256];
-  __shared__ uint32_t dstart[256];
-  __shared__ uint32_t wsum[kRsWarps];
-  __shared__ int64_t goff[256];
-  extern __shared__ __align__(16) unsigned char rs_smem[];
-  uint64_t* skey = reinterpret_cast<uint64_t*>(rs_smem);
-  unsigned char* sval = rs_smem + kRsTile * 8;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int64_t tbase = int64_t(blockIdx.x) * kRsTile;
-  const int64_t wbase = tbase + int64_t(warp) * 32 * kRsItems;
+// Stable scatter of one tile by one digit.  Warp w owns the w-th slice of the
+// tile.  The slice's digit counts (one shared atomic per key) give, summed over
+// the warps, the tile's counts, published before the keys are ranked; the keys
+// are ranked 32 at a time in lane order (one ballot per digit bit) and staged
+// in shared memory in digit order, then written with consecutive threads on
+// consecutive addresses of each digit's run.
+//
+// Bound by instruction issue and shared-memory bandwidth rather than HBM: a row
+// costs about 25 shared-memory wavefronts per 32 rows (atomic, counter, the
+// scattered 8- and 4-byte staging stores, the read back) against the 34 cycles
+// its 24 bytes take at the measured copy rate.  The look-back is hidden: with
+// every word already published the pass takes 328 instead of 349 us (49M rows).
+template <int VB, int ITEMS, class W>
+__global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 3) radix_downsweep_kernel(
+    const uint64_t* __restrict__ kin, uint64_t* __restrict__ kout, const void* __restrict__ vin_,
+    void* __restrict__ vout_, int64_t n_max, const int64_t* __restrict__ n_dev, int shift, uint32_t mask,
+    const unsigned long long* __restrict__ counts, W* __restrict__ words, unsigned* __restrict__ ticket, unsigned* __restrict__ status) {
+  constexpr int kTileKeys = kRsThreads * ITEMS;
   using VT = typename std::conditional<VB == 8, uint64_t, uint32_t>::type;
-  uint64_t key[kRsItems];
-  uint32_t rank[kRsItems];
-  VT val[kRsItems];
-  // the tile's keys and values and this digit's output offset are all
-  // requested before the first barrier, so one memory round trip starts a tile
-#pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t idx = wbase + it * 32 + lane;
-    const bool valid = idx < n;
-    key[it] = valid ? kin[idx] : 0;
-    val[it] = 0;
-    if (VB != 0 && valid) val[it] = static_cast<const VT*>(vin)[idx];
-  }
-  goff[threadIdx.x] = offs[int64_t(blockIdx.x) * 256 + threadIdx.x];
-  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) wcnt[i / 256][i % 256] = 0;
+  extern __shared__ __align__(16) unsigned char rs_smem[];  // staged keys, then values
+  uint64_t* skey = reinterpret_cast<uint64_t*>(rs_smem);
+  VT* sval = reinterpret_cast<VT*>(rs_smem + size_t(kTileKeys) * 8);
+  __shared__ uint32_t wcnt[kRsWarps][kRsBins];
+  __shared__ W soff[kRsBins];
+  __shared__ W gsum[kRsWarps];
+  __shared__ uint32_t wsum[kRsWarps];
+  __shared__ unsigned s_tile;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  if (tid == 0) s_tile = atomicAdd(ticket, 1u);
+  for (int i = tid; i < kRsWarps * kRsBins; i += kRsThreads) (&wcnt[0][0])[i] = 0;
   __syncthreads();
+  const int64_t tile = s_tile;
+  const int64_t base = tile * kTileKeys;
+  const int64_t n = n_dev ? min(*n_dev, n_max) : n_max;
+  if (base >= n) return;  // fewer rows than the grid was sized for; later tiles have none either
+  const int tn = int(n - base < kTileKeys ? n - base : kTileKeys);
+  const uint64_t* kp = kin + base;
+  const VT* vp = static_cast<const VT*>(vin_) + (VB ? base : 0);
+  const int first = warp * 32 * ITEMS + lane;
+  uint64_t key[ITEMS];
+  VT val[VB ? ITEMS : 1];
+  // keys past the end (last tile) count as the top digit and rank after every
+  // real key: they stay at the end of the staged tile and are not written
+  if (tn == kTileKeys) {
 #pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t idx = wbase + it * 32 + lane;
-    const bool valid = idx < n;
-    const uint32_t d = uint32_t(key[it] >> shift) & mask;
-    const unsigned peers = warp_digit_peers(d, __ballot_sync(0xffffffffu, valid));
-    const uint32_t before = wcnt[warp][d];
-    const uint32_t r = __popc(peers & lt_mask);
-    rank[it] = before + r;
-    __syncwarp();
-    if (valid && r == 0) wcnt[warp][d] = before + __popc(peers);
-    __syncwarp();
+    for (int j = 0; j < ITEMS; ++j) key[j] = kp[first + j * 32];
+    if (VB) {
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) val[j] = vp[first + j * 32];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) key[j] = first + j * 32 < tn ? kp[first + j * 32] : ~uint64_t(0);
+    if (VB) {
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) val[j] = first + j * 32 < tn ? vp[first + j * 32] : VT(0);
+    }
   }
+  uint32_t* wc = wcnt[warp];
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) atomicAdd(&wc[uint32_t(key[j] >> shift) & mask], 1u);
   __syncthreads();
-  // per digit: exclusive prefix over warps, then exclusive prefix over digits
-  const int dd = threadIdx.x;
-  uint32_t run = 0;
+  // thread = digit: the tile's count, published at once
+  uint32_t cnt = 0;
 #pragma unroll
-  for (int w = 0; w < kRsWarps; ++w) {
-    const uint32_t c = wcnt[w][dd];
-    wcnt[w][dd] = run;
-    run += c;
-  }
-  uint32_t incl = run;
+  for (int w = 0; w < kRsWarps; ++w) cnt += wcnt[w][tid];
+  const uint32_t real = cnt - (uint32_t(tid) == mask ? uint32_t(kTileKeys - tn) : 0u);
+  if (tile != 0) st_relaxed(words + tile * kRsBins + tid, RsFlag<W>::kAgg | W(real));
+  uint32_t incl = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -225,237 +304,192 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == 8 ? 4 : 2) radix_downswee
   }
   if (lane == 31) wsum[warp] = incl;
   __syncthreads();
-  uint32_t wpre = 0;
+  uint32_t dstart = incl - cnt;
 #pragma unroll
-  for (int w = 0; w < kRsWarps; ++w) wpre += w < warp ? wsum[w] : 0u;
-  dstart[dd] = wpre + incl - run;
-  __syncthreads();
-#pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t idx = wbase + it * 32 + lane;
-    if (idx < n) {
-      const uint32_t d = uint32_t(key[it] >> shift) & mask;
-      const uint32_t lp = dstart[d] + wcnt[warp][d] + rank[it];
-      skey[lp] = key[it];
-      if (VB != 0) reinterpret_cast<VT*>(sval)[lp] = val[it];
-    }
-  }
-  __syncthreads();
-  const int tn = int(n - tbase < kRsTile ? n - tbase : kRsTile);
-#pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int i = it * kRsThreads + threadIdx.x;
-    if (i < tn) {
-      const uint64_t k = skey[i];
-      const uint32_t d = uint32_t(k >> shift) & mask;
-      const int64_t pos = goff[d] + (i - int64_t(dstart[d]));
-      kout[pos] = k;
-      if (VB != 0) static_cast<VT*>(vout)[pos] = reinterpret_cast<const VT*>(sval)[i];
-    }
-  }
-}
-
-// The same scatter as a persistent kernel (one CTA per tile slot of the
-// SMs) that copies the next full tile's keys and values into shared memory
-// with asynchronous 16-byte copies while it ranks and scatters the current
-// one; the tile it has just ranked is staged in place.  Same results (the
-// ranking order and the offsets are the same).  Needs 16-byte-aligned key and
-// value arrays; the caller checks.
-template <int VB>
-__global__ void __launch_bounds__(kRsThreads, 3) radix_scatter_pf_kernel(
-    const uint64_t* __restrict__ kin, uint64_t* __restrict__ kout, const void* __restrict__ vin,
-    void* __restrict__ vout, int64_t n, int shift, uint32_t mask, const int64_t* __restrict__ offs, int64_t ntiles) {
-  constexpr int kRsItems = 8, kRsTile = kRsThreads * 8;
-  constexpr int kBuf = kRsTile * (8 + VB);  // bytes of one tile (keys, then values)
-  __shared__ uint32_t wcnt[kRsWarps][256];
-  __shared__ uint32_t dstart[256];
-  __shared__ uint32_t wsum[kRsWarps];
-  __shared__ int64_t goff[256];
-  extern __shared__ __align__(16) unsigned char rs_smem[];  // two tile buffers
-  using VT = typename std::conditional<VB == 8, uint64_t, uint32_t>::type;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int64_t nfull = n / kRsTile;  // tiles copied asynchronously; the last partial one is read directly
-  auto prefetch = [&](int64_t t, unsigned char* buf) {
-    if (t >= nfull) return;
-    const unsigned char* gk = reinterpret_cast<const unsigned char*>(kin + t * kRsTile);
-    const unsigned char* gv = static_cast<const unsigned char*>(vin) + t * kRsTile * VB;
-    for (int c = threadIdx.x; c < kBuf / 16; c += kRsThreads) {
-      const unsigned char* src = c < kRsTile * 8 / 16 ? gk + 16 * c : gv + 16 * (c - kRsTile * 8 / 16);
-      const unsigned dst = unsigned(__cvta_generic_to_shared(buf + 16 * c));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-    }
-  };
-  int b = 0;
-  prefetch(blockIdx.x, rs_smem);
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, b ^= 1) {
-    unsigned char* cur = rs_smem + b * kBuf;
-    prefetch(t + gridDim.x, rs_smem + (b ^ 1) * kBuf);  // into the buffer the previous tile staged in
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");  // this tile's copies are done
-    for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) wcnt[i / 256][i % 256] = 0;
-    goff[threadIdx.x] = offs[t * 256 + threadIdx.x];
-    __syncthreads();
-    const int64_t tbase = t * kRsTile;
-    const bool staged = t < nfull;
-    const uint64_t* sk_in = reinterpret_cast<const uint64_t*>(cur);
-    const VT* sv_in = reinterpret_cast<const VT*>(cur + kRsTile * 8);
-    uint64_t key[kRsItems];
-    uint32_t rank[kRsItems];
-    VT val[kRsItems];
-#pragma unroll
-    for (int it = 0; it < kRsItems; ++it) {
-      const int j = warp * 32 * kRsItems + it * 32 + lane;  // the same item order as the one-tile kernel
-      const bool valid = tbase + j < n;
-      key[it] = staged ? sk_in[j] : (valid ? kin[tbase + j] : 0);
-      val[it] = 0;
-      if (VB != 0 && valid) val[it] = staged ? sv_in[j] : static_cast<const VT*>(vin)[tbase + j];
-      const uint32_t d = uint32_t(key[it] >> shift) & mask;
-      const unsigned peers = warp_digit_peers(d, __ballot_sync(0xffffffffu, valid));
-      const uint32_t before = wcnt[warp][d];
-      const uint32_t r = __popc(peers & lt_mask);
-      rank[it] = before + r;
-      __syncwarp();
-      if (valid && r == 0) wcnt[warp][d] = before + __popc(peers);
-      __syncwarp();
-    }
-    __syncthreads();  // also: the tile's buffer is read, it becomes the staging area
-    const int dd = threadIdx.x;
-    uint32_t run = 0;
+  for (int w = 0; w < kRsWarps; ++w) dstart += w < warp ? wsum[w] : 0u;
+  {  // each warp's first place of the digit in the staged tile
+    uint32_t run = dstart;
 #pragma unroll
     for (int w = 0; w < kRsWarps; ++w) {
-      const uint32_t c = wcnt[w][dd];
-      wcnt[w][dd] = run;
+      const uint32_t c = wcnt[w][tid];
+      wcnt[w][tid] = run;
       run += c;
     }
-    uint32_t incl = run;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t d = uint32_t(key[j] >> shift) & mask;
+    const unsigned peers = warp_digit_peers(d, 0xffffffffu);
+    const uint32_t before = wc[d];
+    const uint32_t pos = before + __popc(peers & lt);
+    __syncwarp();
+    if ((peers & lt) == 0) wc[d] = before + __popc(peers);
+    skey[pos] = key[j];
+    if (VB) sval[pos] = val[j];
+    __syncwarp();
+  }
+  // the digit's first row: rows of smaller digits, then of earlier tiles
+  W excl;
+  if (tile == 0) {
+    const W c = W(counts[tid]);
+    W gi = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
+      const W t = __shfl_up_sync(0xffffffffu, gi, o);
+      if (lane >= o) gi += t;
     }
-    if (lane == 31) wsum[warp] = incl;
+    if (lane == 31) gsum[warp] = gi;
     __syncthreads();
-    uint32_t wpre = 0;
+    excl = gi - c;
 #pragma unroll
-    for (int w = 0; w < kRsWarps; ++w) wpre += w < warp ? wsum[w] : 0u;
-    dstart[dd] = wpre + incl - run;
-    __syncthreads();
-    uint64_t* skey = reinterpret_cast<uint64_t*>(cur);
-    VT* sval = reinterpret_cast<VT*>(cur + kRsTile * 8);
-#pragma unroll
-    for (int it = 0; it < kRsItems; ++it) {
-      const int j = warp * 32 * kRsItems + it * 32 + lane;
-      if (tbase + j < n) {
-        const uint32_t d = uint32_t(key[it] >> shift) & mask;
-        const uint32_t lp = dstart[d] + wcnt[warp][d] + rank[it];
-        skey[lp] = key[it];
-        if (VB != 0) sval[lp] = val[it];
-      }
-    }
-    __syncthreads();
-    const int tn = int(n - tbase < kRsTile ? n - tbase : kRsTile);
-    for (int i = threadIdx.x; i < tn; i += kRsThreads) {
-      const uint64_t k = skey[i];
-      const uint32_t d = uint32_t(k >> shift) & mask;
-      const int64_t pos = goff[d] + (i - int64_t(dstart[d]));
-      kout[pos] = k;
-      if (VB != 0) static_cast<VT*>(vout)[pos] = sval[i];
-    }
-    __syncthreads();  // the staging buffer is read before the next prefetch lands in it
+    for (int w = 0; w < kRsWarps; ++w) excl += w < warp ? gsum[w] : W(0);
+  } else {
+    excl = rs_look_back<W>(words, tile, tid, status);
   }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  st_relaxed(words + tile * kRsBins + tid, RsFlag<W>::kIncl | (excl + real));
+  soff[tid] = excl - W(dstart);
+  __syncthreads();
+  VT* __restrict__ vout = static_cast<VT*>(vout_);
+  if (tn == kTileKeys) {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const int i = j * kRsThreads + tid;
+      const uint64_t k = skey[i];
+      const W p = soff[uint32_t(k >> shift) & mask] + W(i);
+      kout[p] = k;
+      if (VB) vout[p] = sval[i];
+    }
+  } else {
+    for (int i = tid; i < tn; i += kRsThreads) {
+      const uint64_t k = skey[i];
+      const W p = soff[uint32_t(k >> shift) & mask] + W(i);
+      kout[p] = k;
+      if (VB) vout[p] = sval[i];
+    }
+  }
 }
 
-template <int VB, int ITEMS>
-void launch_downsweep(const uint64_t* ka, uint64_t* kb, const void* va, void* vb, int64_t n, int shift, uint32_t mask,
-                      int64_t ntiles, const int64_t* offs, cudaStream_t s) {
-  const bool aligned = (reinterpret_cast<uintptr_t>(ka) & 15) == 0 && (reinterpret_cast<uintptr_t>(va) & 15) == 0;
-  if (ITEMS == 8 && aligned && t_call_ctx && t_call_ctx->param("radix_prefetch", 0) != 0) {
-    constexpr size_t smem2 = size_t(2) * kRsTile * (8 + VB);
-    GT_CUDA(cudaFuncSetAttribute(radix_scatter_pf_kernel<VB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(smem2)));
-    const int64_t grid = std::min<int64_t>(ntiles, int64_t(t_call_ctx->num_sms) * 3);
-    Phase ph(t_call_ctx, "radix_pass", s);
-    radix_scatter_pf_kernel<VB><<<unsigned(grid), kRsThreads, smem2, s>>>(ka, kb, va, vb, n, shift, mask, offs,
-                                                                          ntiles);
-    GT_LAUNCH_CHECK();
-    return;
+struct RadixScratch {
+  unsigned long long* counts;  // [passes * 256]
+  unsigned* tickets;           // [passes]
+  char* words;                 // [passes][tiles][256]
+  size_t zero_bytes;
+};
+
+int radix_items(int64_t n) {
+  const int64_t p = t_call_ctx ? t_call_ctx->param("radix_items", kRsSmallItems) : kRsSmallItems;
+  return p == kRsLargeItems || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
+}
+
+bool radix_narrow(int64_t n) { return n < (int64_t(1) << 30); }
+
+size_t radix_layout(int64_t n, int items, int passes, void* scratch, RadixScratch* out) {
+  const int64_t tiles = (n + kRsThreads * items - 1) / (kRsThreads * items);
+  const size_t counts = size_t(passes) * kRsBins * 8, tickets = 16 * sizeof(unsigned);
+  const size_t words = size_t(passes) * size_t(tiles) * kRsBins * (radix_narrow(n) ? 4 : 8);
+  if (out) {
+    out->counts = static_cast<unsigned long long*>(scratch);
+    out->tickets = reinterpret_cast<unsigned*>(static_cast<char*>(scratch) + counts);
+    out->words = static_cast<char*>(scratch) + counts + tickets;
+    out->zero_bytes = counts + tickets + words;
   }
-  constexpr size_t smem = size_t(kRsThreads) * ITEMS * (8 + VB);
-  GT_CUDA(cudaFuncSetAttribute(radix_downsweep_kernel<VB, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return counts + tickets + words;
+}
+
+template <int VB, int ITEMS, class W>
+void launch_scatter(const uint64_t* ka, uint64_t* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
+                    int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
+  constexpr int64_t kTileKeys = int64_t(kRsThreads) * ITEMS;
+  constexpr size_t smem = size_t(kTileKeys) * (8 + VB);
+  const int64_t tiles = (n + kTileKeys - 1) / kTileKeys;
+  GT_CUDA(cudaFuncSetAttribute(radix_downsweep_kernel<VB, ITEMS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(smem)));
   Phase ph(t_call_ctx, "radix_pass", s);  // one span per scatter pass
-  radix_downsweep_kernel<VB, ITEMS><<<unsigned(ntiles), kRsThreads, smem, s>>>(ka, kb, va, vb, n, shift, mask, offs);
+  radix_downsweep_kernel<VB, ITEMS, W><<<unsigned(tiles), kRsThreads, smem, s>>>(
+      ka, kb, va, vb, n, n_dev, shift, mask, rs.counts + size_t(pass) * kRsBins,
+      reinterpret_cast<W*>(rs.words) + size_t(pass) * size_t(tiles) * kRsBins, rs.tickets + pass, status_word());
   GT_LAUNCH_CHECK();
 }
 
-template <int ITEMS>
-void radix_passes(uint64_t* ka, uint64_t* kb, void* va, void* vb, int value_bytes, int64_t n, const int* pass_shift,
-                  const int* pass_bits, int npass, void* scratch, cudaStream_t s, bool& swapped) {
-  constexpr int tile = kRsThreads * ITEMS;
-  const int64_t ntiles = (n + tile - 1) / tile;
-  const int64_t nchunks = (ntiles + kRsChunk - 1) / kRsChunk;
-  const int64_t m = 256 * ntiles, mc = 256 * nchunks;
-  uint32_t* hist = static_cast<uint32_t*>(scratch);
-  int64_t* offs = reinterpret_cast<int64_t*>(static_cast<char*>(scratch) + ((size_t(m) * 4 + 15) / 16 * 16));
-  int64_t* csum = offs + m;
-  int64_t* cpre = csum + mc;
-  void* sscratch = cpre + mc;
-  swapped = false;
-  for (int p = 0; p < npass; ++p) {
-    const int shift = pass_shift[p];
-    const uint32_t mask = (1u << pass_bits[p]) - 1u;
-    radix_upsweep_kernel<ITEMS><<<unsigned(ntiles), kRsThreads, 0, s>>>(ka, n, shift, mask, hist);
-    GT_LAUNCH_CHECK();
-    radix_chunk_sum_kernel<<<unsigned(nchunks), 256, 0, s>>>(hist, ntiles, nchunks, csum);
-    GT_LAUNCH_CHECK();
-    exclusive_scan_i64(csum, cpre, mc, sscratch, s);
-    radix_chunk_offsets_kernel<<<unsigned(nchunks), 256, 0, s>>>(hist, cpre, ntiles, nchunks, offs);
-    GT_LAUNCH_CHECK();
-    if (value_bytes == 4)
-      launch_downsweep<4, ITEMS>(ka, kb, va, vb, n, shift, mask, ntiles, offs, s);
-    else if (value_bytes == 8)
-      launch_downsweep<8, ITEMS>(ka, kb, va, vb, n, shift, mask, ntiles, offs, s);
-    else
-      launch_downsweep<0, ITEMS>(ka, kb, nullptr, nullptr, n, shift, mask, ntiles, offs, s);
-    std::swap(ka, kb);
-    std::swap(va, vb);
-    swapped = !swapped;
+template <int VB>
+void launch_scatter_any(const uint64_t* ka, uint64_t* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
+                        int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
+  if (!radix_narrow(n))
+    launch_scatter<VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+  else if (items == kRsSmallItems)
+    launch_scatter<VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+  else
+    launch_scatter<VB, kRsLargeItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+}
+
+// Digit passes over bits [begin_a, end_a) then [begin_b, end_b), the bits of
+// each range spread evenly over its passes.
+RadixPasses radix_plan(int begin_a, int end_a, int begin_b, int end_b) {
+  RadixPasses ps{};
+  for (int r = 0; r < 2; ++r) {
+    int lo = r ? begin_b : begin_a;
+    const int hi = r ? end_b : end_a;
+    for (int left = (hi - lo + 7) / 8; left > 0; --left) {
+      const int bits = (hi - lo + left - 1) / left;
+      if (ps.n == kRsMaxPasses) fail(GT_EINVAL, "more than 64 bits to sort on");
+      ps.shift[ps.n] = lo;
+      ps.bits[ps.n++] = bits;
+      lo += bits;
+    }
   }
+  return ps;
 }
 
 }  // namespace
 
 size_t scan_scratch_bytes(int64_t n) {
-  int64_t nb = (n + kScanChunk - 1) / kScanChunk;
-  if (nb <= 1) return 0;
-  return size_t(2 * nb) * sizeof(int64_t) + scan_scratch_bytes(nb);
+  const int64_t nb = (n + kScanChunk - 1) / kScanChunk;
+  return nb <= 1 ? 0 : size_t(nb + 1) * sizeof(unsigned long long);
 }
 
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratch, cudaStream_t s) {
   if (n <= 0) return;
-  int64_t nb = (n + kScanChunk - 1) / kScanChunk;
-  if (nb == 1) {
-    scan_apply_kernel<<<1, kScanThreads, 0, s>>>(in, out, n, nullptr);
-    GT_LAUNCH_CHECK();
-    return;
-  }
-  int64_t* bsum = static_cast<int64_t*>(scratch);
-  int64_t* boff = bsum + nb;
-  scan_reduce_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(in, n, bsum);
-  GT_LAUNCH_CHECK();
-  exclusive_scan_i64(bsum, boff, nb, boff + nb, s);
-  scan_apply_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(in, out, n, boff);
+  const int64_t nb = (n + kScanChunk - 1) / kScanChunk;
+  auto* flags = nb > 1 ? static_cast<unsigned long long*>(scratch) : nullptr;
+  if (flags) GT_CUDA(cudaMemsetAsync(flags, 0, scan_scratch_bytes(n), s));
+  scan_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(in, out, n, flags, nb, status_word());
   GT_LAUNCH_CHECK();
 }
 
 size_t radix_scratch_bytes(int64_t n, bool, int) {
-  const int64_t ntiles = (n + kRsTile - 1) / kRsTile;
-  const int64_t nchunks = (ntiles + kRsChunk - 1) / kRsChunk;
-  const int64_t m = 256 * ntiles, mc = 256 * nchunks;
-  return size_t(m) * 4 + size_t(m) * 8 + size_t(2 * mc) * 8 + scan_scratch_bytes(mc) + 256;
+  // for the smaller tile, which "radix_items" may select at any size
+  return radix_layout(n, radix_narrow(n) ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
+}
+
+bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
+                         int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s,
+                         const int64_t* n_dev) {
+  if (n <= 0) return false;
+  const RadixPasses ps = radix_plan(begin_a, end_a, begin_b, end_b);
+  if (ps.n == 0) return false;
+  const int items = radix_narrow(n) ? radix_items(n) : kRsLargeItems;
+  RadixScratch rs;
+  radix_layout(n, items, ps.n, scratch, &rs);
+  GT_CUDA(cudaMemsetAsync(scratch, 0, rs.zero_bytes, s));
+  const int sms = t_call_ctx ? t_call_ctx->num_sms : 152;
+  radix_hist_kernel<<<grid_for(n, kRhThreads * kRhItems, sms * 4), kRhThreads, 0, s>>>(keys_a, n, n_dev, ps,
+                                                                                                 rs.counts);
+  GT_LAUNCH_CHECK();
+  uint64_t *ka = keys_a, *kb = keys_b;
+  void *va = vals_a, *vb = vals_b;
+  for (int p = 0; p < ps.n; ++p) {
+    const uint32_t mask = (1u << ps.bits[p]) - 1u;
+    if (value_bytes == 4)
+      launch_scatter_any<4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+    else if (value_bytes == 8)
+      launch_scatter_any<8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+    else
+      launch_scatter_any<0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+    std::swap(ka, kb);
+    std::swap(va, vb);
+  }
+  return ps.n % 2 == 1;
 }
 
 void radix_sort_u64(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* vals_out, int value_bytes,
@@ -467,32 +501,13 @@ void radix_sort_u64(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* 
 void radix_sort_u64_split(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* vals_out, int value_bytes,
                           int64_t n, int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s) {
   if (n <= 0) return;
-  // digit passes: [begin_a, end_a) then [begin_b, end_b), 8 bits at a time
-  int pass_shift[16], pass_bits[16], npass = 0;
-  for (int r = 0; r < 2; ++r) {
-    const int lo = r ? begin_b : begin_a, hi = r ? end_b : end_a;
-    for (int shift = lo; shift < hi && npass < 16; shift += 8) {
-      pass_shift[npass] = shift;
-      pass_bits[npass++] = hi - shift < 8 ? hi - shift : 8;
-    }
-  }
-  // digit passes over tiles of 2048 keys, or 4096 with "radix_items" 16
-  const int items = t_call_ctx ? int(t_call_ctx->param("radix_items", kRsItems)) : kRsItems;
-  bool swapped = false;
-  if (items == 16)
-    radix_passes<16>(keys_in, keys_out, vals_in, vals_out, value_bytes, n, pass_shift, pass_bits, npass, scratch, s,
-                     swapped);
-  else
-    radix_passes<8>(keys_in, keys_out, vals_in, vals_out, value_bytes, n, pass_shift, pass_bits, npass, scratch, s,
-                    swapped);
-  uint64_t* ka = swapped ? keys_out : keys_in;
-  void* va = swapped ? vals_out : vals_in;
-  // after the loop the sorted data is in ka / va
-  if (ka != keys_out) {
-    GT_CUDA(cudaMemcpyAsync(keys_out, ka, size_t(n) * 8, cudaMemcpyDeviceToDevice, s));
-    if (value_bytes)
-      GT_CUDA(cudaMemcpyAsync(vals_out, va, size_t(n) * value_bytes, cudaMemcpyDeviceToDevice, s));
-  }
+  if (radix_sort_pingpong(keys_in, keys_out, vals_in, vals_out, value_bytes, n, begin_a, end_a, begin_b, end_b,
+                          scratch, s))
+    return;
+  // an even number of passes left the rows in the input buffers
+  GT_CUDA(cudaMemcpyAsync(keys_out, keys_in, size_t(n) * 8, cudaMemcpyDeviceToDevice, s));
+  if (value_bytes)
+    GT_CUDA(cudaMemcpyAsync(vals_out, vals_in, size_t(n) * value_bytes, cudaMemcpyDeviceToDevice, s));
 }
 
 }  // namespace gt

@@ -1,0 +1,105 @@
+"""The one-pass primitives (scan, radix sort, run reduction) through the
+public calls, at the edges of their tiles: 2,048 values per scan and reduction
+tile, 2,048 or 4,096 rows per sort tile, the row count at which the sort
+changes its tile, runs that cover whole tiles, and (file, key) rows that fit
+one 64-bit sort key and that do not.  Whole numbers: equal to the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2106_06889_gb300 import binding as B
+from paper_2106_06889_gb300.corpus import root_only_grammar, sequitur
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = B.gt_create(0)
+    yield c
+    B.gt_destroy(c)
+
+
+def take(r, *fields):
+    out = [B.result_numpy(r, f) for f in fields]
+    B.gt_free_result(r)
+    return out
+
+
+def check(gh, g):
+    for order in (0, 1):
+        for got, want in zip(take(B.gt_sort(gh, order), "word", "count"), oracle.sort_words(g, order)):
+            assert np.array_equal(got, want)
+    for got, want in zip(take(B.gt_sequence_count(gh, 0), "key", "count"), oracle.sequence_count(g, 0)):
+        assert np.array_equal(got, want)
+    for got, want in zip(take(B.gt_sequence_count(gh, 1), "file", "key", "count"), oracle.sequence_count(g, 1)):
+        assert np.array_equal(got, want)
+    for n in (1, 3):
+        for got, want in zip(take(B.gt_ranked_index(gh, n), "offsets", "key", "file", "count"),
+                             oracle.ranked_index(g, n)):
+            assert np.array_equal(got, want)
+    for got, want in zip(take(B.gt_cooccurrence(gh), "key", "count"), oracle.cooccurrence(g)):
+        assert np.array_equal(got, want)
+    for top in (0, 3):
+        for got, want in zip(take(B.gt_term_vector(gh, top), "offsets", "word", "count"), oracle.term_vector(g, top)):
+            assert np.array_equal(got, want)
+    for got, want in zip(take(B.gt_inverted_index(gh), "offsets", "file"), oracle.inverted_index(g)):
+        assert np.array_equal(got, want)
+
+
+# windows = tokens - 2: 2048 and 4096 rows and one more or less, several tiles, one row
+EDGES = [3, 2049, 2050, 2051, 4097, 4098, 4099, 8194, 20_483]
+
+
+@pytest.mark.parametrize("n", EDGES)
+@pytest.mark.parametrize("text", ["one_word", "few", "distinct"])
+def test_tile_edges(ctx, n, text):
+    """One file, no rules: one key whose run covers every tile, a few long runs, all keys distinct."""
+    rng = np.random.default_rng(n)
+    V = {"one_word": 2, "few": 5, "distinct": 30_011}[text]
+    toks = {"one_word": np.ones(n), "few": rng.integers(0, V, n), "distinct": np.arange(n) * 7 % V}[text].astype(np.int32)
+    g = root_only_grammar(toks, [n], V)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        check(gh, g)
+    finally:
+        B.gt_free_grammar(gh)
+
+
+@pytest.mark.parametrize("strategy", [1, 2])
+@pytest.mark.parametrize("V,F", [(2 ** 21, 3), (2 ** 20, 17), (2 ** 20, 15), (70_000, 64)])
+def test_file_keys(ctx, V, F, strategy):
+    """(file, 3-word key) rows of 64 bits and more, of 63 bits and of fewer, top-down and
+    bottom-up (by the global sort), empty files among them."""
+    rng = np.random.default_rng(V + F)
+    toks = (rng.zipf(1.3, 9000) % V).astype(np.int32)
+    toks[1000:2000] = toks[4000:5000]  # a repeated passage: rules
+    toks[-1] = V - 1
+    cuts = np.sort(rng.integers(0, toks.shape[0] + 1, F - 1))
+    cuts[F // 2:F // 2 + 1] = cuts[F // 2 - 1]  # an empty file
+    lens = np.diff(np.concatenate([[0], cuts, [toks.shape[0]]]))
+    g = sequitur(toks, lens, V)
+    B.gt_set_param(ctx, "file_strategy", strategy)
+    B.gt_set_param(ctx, "bu_local", 0)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        check(gh, g)
+    finally:
+        B.gt_free_grammar(gh)
+        B.gt_set_param(ctx, "file_strategy", 0)
+        B.gt_set_param(ctx, "bu_local", 1)
+
+
+@pytest.mark.parametrize("n", [2 ** 20 - 1 + 2, 2 ** 20 + 2, 2 ** 20 + 4099])
+def test_sort_tile_change(ctx, n):
+    """Rows just below and above 2^20, where the sort goes from 2,048- to 4,096-row tiles."""
+    rng = np.random.default_rng(n)
+    toks = (rng.zipf(1.2, n) % 5000).astype(np.int32)
+    g = root_only_grammar(toks, [n // 2, n - n // 2], 5000)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        for per_file, fields in ((0, ("key", "count")), (1, ("file", "key", "count"))):
+            for got, want in zip(take(B.gt_sequence_count(gh, per_file), *fields), oracle.sequence_count(g, per_file)):
+                assert np.array_equal(got, want)
+    finally:
+        B.gt_free_grammar(gh)
