@@ -831,42 +831,6 @@ __device__ __forceinline__ void ii_masks(const uint32_t* __restrict__ bits, int 
   m_hi = lane + 32 < F ? bits[(int64_t(lane + 32) * nb + b) * kTvThreads + t] : 0u;
 }
 
-__global__ void ii_count_kernel(const uint32_t* __restrict__ bits, int nb, int32_t F, int32_t V,
-                                int64_t* __restrict__ cnt) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t w0 = ((blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5) * 32; w0 < V; w0 += nwarps * 32) {
-    uint32_t lo, hi;
-    ii_masks(bits, nb, F, w0, lane, lo, hi);
-    int mine = 0;
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int c = __popc(__ballot_sync(0xffffffffu, (lo >> l) & 1u)) + __popc(__ballot_sync(0xffffffffu, (hi >> l) & 1u));
-      if (lane == l) mine = c;
-    }
-    if (w0 + lane < V) cnt[w0 + lane] = mine;
-  }
-}
-
-__global__ void ii_fill_kernel(const uint32_t* __restrict__ bits, int nb, int32_t F, int32_t V,
-                               const int64_t* __restrict__ off, int32_t* __restrict__ files) {
-  const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t w0 = ((blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5) * 32; w0 < V; w0 += nwarps * 32) {
-    uint32_t lo, hi;
-    ii_masks(bits, nb, F, w0, lane, lo, hi);
-    const int64_t my_off = w0 + lane < V ? off[w0 + lane] : 0;
-    for (int l = 0; l < 32 && w0 + l < V; ++l) {
-      const unsigned a = __ballot_sync(0xffffffffu, (lo >> l) & 1u);
-      const unsigned c = __ballot_sync(0xffffffffu, (hi >> l) & 1u);
-      const int64_t o = __shfl_sync(0xffffffffu, my_off, l);
-      if ((a >> lane) & 1u) files[o + __popc(a & below)] = lane;
-      if ((c >> lane) & 1u) files[o + __popc(a) + __popc(c & below)] = lane + 32;
-    }
-  }
-}
-
 // The inverted index in one pass: CTAs take blocks of kIiWords words in
 // ticket order; each counts the files of its words (one ballot per bit, as
 // above), scans the counts, gets the block's first posting by a bounded
@@ -1369,6 +1333,53 @@ void file_hist(gt_grammar* g, cudaStream_t s, FileHist& fh) {
   GT_LAUNCH_CHECK();
 }
 
+// df[w] += 1 for every term-vector entry of w (the files containing w).
+__global__ void df_kernel(const int32_t* __restrict__ word, const int64_t* __restrict__ total,
+                          uint32_t* __restrict__ df) {
+  const int64_t n = *total;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    atomicAdd(&df[word[i]], 1u);
+}
+
+// idf[d] = ln(F / d) for every possible document frequency d = 1 .. F.
+__global__ void idf_kernel(int32_t F, double* __restrict__ idf) {
+  for (int32_t d = 1 + blockIdx.x * blockDim.x + threadIdx.x; d <= F; d += gridDim.x * blockDim.x)
+    idf[d] = log(double(F) / double(d));
+}
+
+// TF-IDF of every term-vector entry: count * ln(F / df(word)), the logarithm
+// from the table.  A logarithm and a quotient per entry made this bound by the
+// double-precision pipe (91 us for 1.2M entries of 37 files); one product per
+// entry leaves it to the gathers.
+__global__ void tfidf_kernel(const int32_t* __restrict__ word, const uint64_t* __restrict__ cnt,
+                             const int64_t* __restrict__ total, const uint32_t* __restrict__ df,
+                             const double* __restrict__ idf, double* __restrict__ out) {
+  const int64_t n = *total;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    out[i] = double(cnt[i]) * idf[df[word[i]]];
+}
+
+// The "tfidf" field of a term vector under construction: document frequencies
+// counted over its entries, then every entry's value.
+void add_tfidf(gt_ctx* ctx, ResultBuilder& rb, const int32_t* word, const uint64_t* cnt, const int64_t* total,
+               int64_t* len, int64_t bound, int32_t F, int32_t V, cudaStream_t s) {
+  const int threads = 256, cap = ctx->num_sms * 16;
+  if (V <= 0) fail(GT_EINVAL, "TF-IDF needs the vocabulary size");
+  auto* tf = static_cast<double*>(rb.alloc(size_t(bound) * 8));
+  Buf df(ctx, size_t(V) * 4, s), idf(ctx, size_t(F + 1) * 8, s);
+  GT_CUDA(cudaMemsetAsync(df.p, 0, size_t(V) * 4, s));
+  if (bound > 0) {
+    idf_kernel<<<grid_for(F, threads, cap), threads, 0, s>>>(F, idf.as<double>());
+    GT_LAUNCH_CHECK();
+    df_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, total, df.as<uint32_t>());
+    GT_LAUNCH_CHECK();
+    tfidf_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, total, df.as<uint32_t>(),
+                                                                   idf.as<double>(), tf);
+    GT_LAUNCH_CHECK();
+  }
+  rb.field_dyn("tfidf", tf, len);
+}
+
 // With wc (top_k == 0 only), the word counts are written too: the sum over
 // files of the term vectors' counts, added while the pieces are copied.
 gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t s, uint64_t* wc = nullptr) {
@@ -1377,7 +1388,7 @@ gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t
   const int64_t pieces = int64_t(d.F) * fh.nb;
   const int64_t nb_ = fh.bound;
   TvSlots ts{fh.slot_word.as<int32_t>(), fh.slot_cnt.as<uint32_t>(), fh.nnz.as<int64_t>(), fh.bits.as<uint32_t>()};
-  if (top_k != 0) {  // top-k selection or TF-IDF: from the gathered arrays
+  if (top_k > 0) {  // top-k selection: from the gathered arrays
     Buf tw(ctx, size_t(nb_) * 4, s), tc(ctx, size_t(nb_) * 8, s), full_off(ctx, size_t(d.F + 1) * 8, s);
     {
       Phase ph(ctx, "tv_out", s);
@@ -1414,6 +1425,7 @@ gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t
   rb.field("offsets", tv_off, int64_t(d.F) + 1);
   rb.field_dyn("word", word, len);
   rb.field_dyn("count", cnt, len);
+  if (top_k == kTfIdf) add_tfidf(ctx, rb, word, cnt, fh.total.as<int64_t>(), len, nb_, d.F, d.V, s);
   return rb.finish();
 }
 
@@ -1500,23 +1512,6 @@ __global__ void copy_rows_kernel(const int32_t* __restrict__ w, const uint64_t* 
 
 // Term-vector result from (word, count) rows in (file, word) order with file
 // offsets; top_k > 0 keeps each file's top_k counts (count desc, word asc).
-// df[w] += 1 for every term-vector entry of w (the files containing w).
-__global__ void df_kernel(const int32_t* __restrict__ word, const int64_t* __restrict__ total,
-                          uint32_t* __restrict__ df) {
-  const int64_t n = *total;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    atomicAdd(&df[word[i]], 1u);
-}
-
-// TF-IDF of every term-vector entry: count * ln(F / df(word)).
-__global__ void tfidf_kernel(const int32_t* __restrict__ word, const uint64_t* __restrict__ cnt,
-                             const int64_t* __restrict__ total, const uint32_t* __restrict__ df, int32_t F,
-                             double* __restrict__ out) {
-  const int64_t n = *total;
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    out[i] = double(cnt[i]) * log(double(F) / double(df[word[i]]));
-}
-
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
                           const int64_t* total, int64_t bound, int32_t F, int top_k, cudaStream_t s,
                           const uint32_t* status_in, int32_t V) {
@@ -1539,19 +1534,7 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
     rb.field("offsets", tv_off, int64_t(F) + 1);
     rb.field_dyn("word", ow, len);
     rb.field_dyn("count", oc, len);
-    if (top_k == kTfIdf) {
-      if (V <= 0) fail(GT_EINVAL, "TF-IDF needs the vocabulary size");
-      auto* tf = static_cast<double*>(rb.alloc(size_t(bound) * 8));
-      Buf df(ctx, size_t(V) * 4, s);
-      GT_CUDA(cudaMemsetAsync(df.p, 0, size_t(V) * 4, s));
-      if (bound > 0) {
-        df_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(ow, total, df.as<uint32_t>());
-        GT_LAUNCH_CHECK();
-        tfidf_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(ow, oc, total, df.as<uint32_t>(), F, tf);
-        GT_LAUNCH_CHECK();
-      }
-      rb.field_dyn("tfidf", tf, len);
-    }
+    if (top_k == kTfIdf) add_tfidf(ctx, rb, ow, oc, total, len, bound, F, V, s);
   } else {
     Buf k0(ctx, size_t(bound) * 8, s), k1(ctx, size_t(bound) * 8, s), i0(ctx, size_t(bound) * 4, s);
     Buf i1(ctx, size_t(bound) * 4, s), rs(ctx, radix_scratch_bytes(bound, true, 4), s);
