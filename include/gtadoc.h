@@ -344,7 +344,8 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *                   on (that call should happen outside any stream capture);
  *                   not while profiling is enabled.  0: launch kernel by kernel.
  *   "wc_slices"     histogram CTAs per 16k-word bucket in the word count
- *                   (1..64); 0 (default): about 3 x SMs / buckets.
+ *                   (1..64); 0 (default): about 3 x SMs / buckets, at most
+ *                   one per partition CTA.
  *   "bu_local"      1 (default): bottom-up word rows of grammars whose files
  *                   all have at most 8192 tokens are built per file in shared
  *                   memory; 0: always by the global (file, word) sort.

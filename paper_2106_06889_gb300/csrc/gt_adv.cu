@@ -88,7 +88,7 @@ gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s) {
     Buf tail(ctx, size_t(d.R) * 8, s), head(ctx, size_t(d.R) * 8, s);
     {
       Phase ph(ctx, "cooc_rows", s);
-      run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s);
+      run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
       const int threads = 256, cap = ctx->num_sms * 16;
       cooc_rows_kernel<<<grid_for(U, threads, cap), threads, 0, s>>>(
           static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, d.F, keys.as<uint64_t>(), vals.as<uint32_t>(),

@@ -21,6 +21,22 @@ __device__ __forceinline__ unsigned warp_digit_peers(uint32_t d, unsigned active
   return peers;
 }
 
+// ---- chains of small DAG levels in one launch -----------------------------
+// A level pass over a few thousand items is all latency: a launch, dependent
+// loads, and the next level's launch.  The small levels of a grammar (kTailItems
+// items at most, two per thread) run instead inside one thread-block cluster,
+// whose hardware barrier separates the levels (release / acquire at cluster
+// scope orders the global writes too; values written by earlier levels are read
+// through L2).  A level's structure is requested before the barrier that its
+// values wait for.  Larger levels keep a launch of their own: they need more
+// than a cluster's threads.
+constexpr int kTailCtas = 8, kTailThreads = 1024;
+constexpr int64_t kTailItems = 2 * kTailCtas * kTailThreads;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ int64_t upper_bound_dev(const int64_t* a, int64_t n, int64_t x) {
   int64_t lo = 0, hi = n;
   while (lo < hi) {

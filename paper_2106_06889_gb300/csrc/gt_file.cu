@@ -314,6 +314,59 @@ __global__ void __launch_bounds__(256) fweight_level_kernel(WeightRows L, int64_
   }
 }
 
+// The small levels [l0, depth) of the per-file weights in one cluster (see
+// kTailItems): tab holds the first light slot, the first heavy slot and the
+// first heavy piece of every level, depth + 1 of each.
+__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
+    fweight_tail_kernel(WeightRows L, const int64_t* __restrict__ tab, int l0, int depth, uint32_t* w) {
+  const int64_t* const slots = tab;
+  const int64_t* const piece = tab + 2 * (depth + 1);
+  const int lane = threadIdx.x & 31;
+  const int64_t me = int64_t(blockIdx.x) * kTailThreads + threadIdx.x;
+  constexpr int64_t kStride = int64_t(kTailCtas) * kTailThreads;
+  for (int lv = l0; lv < depth; ++lv) {
+    const int64_t a = slots[lv], b = slots[lv + 1];
+    uint2 en[2][kHeavyParents];
+    int n[2];
+    uint32_t to[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int64_t i = a + me + q * kStride;
+      n[q] = 0;
+      to[q] = 0;
+      uint32_t r0 = 0;
+      if (i < b) {
+        r0 = L.row_off[i];
+        n[q] = int(L.row_off[i + 1] - r0);
+        to[q] = L.slot_pair[i];
+      }
+#pragma unroll
+      for (int k = 0; k < kHeavyParents; ++k) en[q][k] = k < n[q] ? L.entries[r0 + k] : make_uint2(0u, 0u);
+    }
+    if (lv > l0) cluster_sync();  // the parents' weights are final
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (n[q] == 0) continue;
+      uint32_t v = __ldcg(&w[to[q]]);
+#pragma unroll
+      for (int k = 0; k < kHeavyParents; ++k) v += k < n[q] ? en[q][k].y * __ldcg(&w[en[q][k].x]) : 0u;
+      w[to[q]] = v;
+    }
+    // heavy pieces: a warp each (their slots are no light slot of the level)
+    for (int64_t h = piece[lv] + me / 32; h < piece[lv + 1]; h += kStride / 32) {
+      const uint4 pc = L.pieces[h];
+      uint32_t v = 0;
+      for (uint32_t e = pc.y + lane; e < pc.z; e += 32) {
+        const uint2 x = L.entries[e];
+        v += x.y * __ldcg(&w[x.x]);
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0 && v) atomicAdd(&w[pc.x], v);
+    }
+  }
+}
+
 // (file << 32 | rule) keys of every (rule, file) slot, rule-major.
 // Pairs of rules without words of their own get file F: sorted after every
 // file's pairs, they stay out of the rule-word chunks.
@@ -1107,7 +1160,20 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
       const int64_t h = g->lvl_heavy[size_t(l)] - NL;  // heavy slots before level l
       if (NH > 0) GT_CUDA(cudaMemcpyAsync(&g->lvl_piece[size_t(l)], ps.as<int64_t>() + h, 8, cudaMemcpyDeviceToHost, s));
     }
+    // the levels' tables on the device, for the launch that runs the small ones
+    auto* tab = static_cast<int64_t*>(grammar_alloc(g, size_t(3 * (d.depth + 1)) * 8, s));
+    const std::vector<int64_t>* host[3] = {&g->lvl_slot, &g->lvl_heavy, &g->lvl_piece};
+    GT_CUDA(cudaStreamSynchronize(s));  // lvl_piece has arrived
+    for (int k = 0; k < 3; ++k)
+      GT_CUDA(cudaMemcpyAsync(tab + k * (d.depth + 1), host[k]->data(), size_t(d.depth + 1) * 8,
+                              cudaMemcpyHostToDevice, s));
     GT_CUDA(cudaStreamSynchronize(s));  // the scratch above is released on return
+    g->lvl_tab = tab;
+    int t = d.depth;
+    while (t > 2 && g->lvl_slot[size_t(t)] - g->lvl_slot[size_t(t) - 1] <= kTailItems &&
+           (g->lvl_piece[size_t(t)] - g->lvl_piece[size_t(t) - 1]) * 32 <= kTailItems)
+      --t;
+    g->fw_tail = d.depth - t >= 2 ? t : d.depth;
   }
   g->fmask = M;
   g->foff = off;
@@ -1269,13 +1335,17 @@ void file_weights(gt_grammar* g, cudaStream_t s, FileWeights& fw) {
   const WeightRows L{g->row_off, g->row_entries, g->row_pieces, g->slot_pair};
   // level by level from the root's children down; level-1 rules have no
   // parent but the root, so their weights are complete already
-  for (int lv = 2; lv < d.depth; ++lv) {
+  for (int lv = 2; lv < g->fw_tail; ++lv) {
     const int64_t a = g->lvl_slot[size_t(lv)], b = g->lvl_slot[size_t(lv) + 1];
     const int64_t ha = g->lvl_piece[size_t(lv)], hb = g->lvl_piece[size_t(lv) + 1];
     if (b <= a && hb <= ha) continue;
     const int lb = b > a ? int(grid_for(b - a, threads, cap)) : 0;
     const int hblk = hb > ha ? int(grid_for((hb - ha) * 32, threads, cap)) : 0;  // a warp per heavy piece
     fweight_level_kernel<<<unsigned(lb + hblk), threads, 0, s>>>(L, a, b, lb, ha, hb, fw.w.as<uint32_t>());
+    GT_LAUNCH_CHECK();
+  }
+  if (g->fw_tail < d.depth) {
+    fweight_tail_kernel<<<kTailCtas, kTailThreads, 0, s>>>(L, g->lvl_tab, g->fw_tail, d.depth, fw.w.as<uint32_t>());
     GT_LAUNCH_CHECK();
   }
 }

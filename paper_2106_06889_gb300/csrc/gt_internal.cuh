@@ -114,6 +114,8 @@ struct DevGrammar {
   int32_t depth;
   const int32_t* level;      // [R]
   const int32_t* lvl_order;  // [R] rules sorted by level
+  const int64_t* lvl_off;   // [depth+1] rules of level l are lvl_order[lvl_off[l] .. lvl_off[l+1])
+  const int64_t* ledge_off; // [depth+1] parent edges of level l's children are ledge_*[ledge_off[l] ..)
   // per-rule facts
   const int32_t* nwords;   // [R] W_r: words in the body
   const int32_t* nrefs;    // [R] S_r: rule references in the body
@@ -222,6 +224,10 @@ struct gt_grammar {
   const uint4* row_pieces = nullptr;
   int64_t row_pieces_n = 0;
   std::vector<int64_t> lvl_piece;
+  // device copies of lvl_slot, lvl_heavy and lvl_piece, and the first of the
+  // deepest levels that are small enough to run in one launch
+  const int64_t* lvl_tab = nullptr;
+  int fw_tail = 0;
   // the rule words (file-major) cut into chunks of at most 4096 words inside
   // each file: chunk c = words [xch_start[c], + xch_len[c]), overlapped by the
   // pairs [xch_p0[c], xch_p1[c]); file f's chunks are [xch_foff[f], xch_foff[f+1])
@@ -423,7 +429,11 @@ void run_word_count(gt_grammar* g, const uint64_t* d_wt, uint64_t* d_counts, cud
 // word counts of up to 64 grammars (one context) in one fused launch sequence
 void run_word_count_multi(gt_grammar* const* gs, uint64_t* const* counts, int n, cudaStream_t s,
                           uint32_t* status = nullptr);
-void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s);
+// children_only: the buffers of rules on level 0, which no rule refers to, are left out
+void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s, bool children_only = false);
+// First level from which on every level has at most kTailItems items (off: the
+// levels' offsets, host), at least `from`; depth when fewer than two such levels.
+int small_levels(const std::vector<int64_t>& off, int from, int depth);
 
 // Sorted 3-word window rows: compact keys (kb bits per word, key_pad above
 // every real key) and weights; n rows including pads.  Rows that carry files

@@ -779,12 +779,12 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     radix_sort_u64(lk.as<uint64_t>(), lks.as<uint64_t>(), nullptr, nullptr, 0, R, 32, 32 + bits_for(lv), rs.p, s);
     low32_kernel<<<grid_for(R, threads, cap), threads, 0, s>>>(lks.as<uint64_t>(), R, order);
     GT_LAUNCH_CHECK();
-    Buf loff(ctx, size_t(lv + 1) * 8, s);
-    csr_offsets_kernel<<<grid_for(lv + 1, threads, cap), threads, 0, s>>>(lks.as<uint64_t>(), R, lv,
-                                                                           loff.as<int64_t>());
+    int64_t* loff = dalloc<int64_t>(g, size_t(lv) + 1, s);
+    csr_offsets_kernel<<<grid_for(lv + 1, threads, cap), threads, 0, s>>>(lks.as<uint64_t>(), R, lv, loff);
     GT_LAUNCH_CHECK();
     g->lvl_off.assign(size_t(lv) + 1, 0);
-    GT_CUDA(cudaMemcpyAsync(g->lvl_off.data(), loff.p, size_t(lv + 1) * 8, cudaMemcpyDeviceToHost, s));
+    GT_CUDA(cudaMemcpyAsync(g->lvl_off.data(), loff, size_t(lv + 1) * 8, cudaMemcpyDeviceToHost, s));
+    d.lvl_off = loff;
     d.level = level;
     d.lvl_order = order;
     // parent edges grouped by the level of their child (for the weight pass)
@@ -793,7 +793,7 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     int32_t* lp = dalloc<int32_t>(g, size_t(E), s);
     uint32_t* lm = dalloc<uint32_t>(g, size_t(E), s);
     Buf ek(ctx, size_t(E) * 8, s), eks(ctx, size_t(E) * 8, s), ers(ctx, radix_scratch_bytes(E, false, 0), s);
-    Buf eoff(ctx, size_t(lv + 1) * 8, s);
+    int64_t* eoff = dalloc<int64_t>(g, size_t(lv) + 1, s);
     if (E > 0) {
       ledge_keys_kernel<<<grid_for(E, threads, cap), threads, 0, s>>>(pedge_child, level, E, ek.as<uint64_t>());
       GT_LAUNCH_CHECK();
@@ -803,11 +803,11 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
                                                                         d.pedge_par, d.pedge_mult, lc, lp, lm);
       GT_LAUNCH_CHECK();
     }
-    csr_offsets_kernel<<<grid_for(lv + 1, threads, cap), threads, 0, s>>>(eks.as<uint64_t>(), E, lv,
-                                                                           eoff.as<int64_t>());
+    csr_offsets_kernel<<<grid_for(lv + 1, threads, cap), threads, 0, s>>>(eks.as<uint64_t>(), E, lv, eoff);
     GT_LAUNCH_CHECK();
     g->ledge_off.assign(size_t(lv) + 1, 0);
-    GT_CUDA(cudaMemcpyAsync(g->ledge_off.data(), eoff.p, size_t(lv + 1) * 8, cudaMemcpyDeviceToHost, s));
+    GT_CUDA(cudaMemcpyAsync(g->ledge_off.data(), eoff, size_t(lv + 1) * 8, cudaMemcpyDeviceToHost, s));
+    d.ledge_off = eoff;
     d.ledge_child = lc;
     d.ledge_par = lp;
     d.ledge_mult = lm;

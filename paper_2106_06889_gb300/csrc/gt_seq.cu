@@ -238,7 +238,7 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
   Buf head(ctx, size_t(d.R) * 8, s), tail(ctx, size_t(d.R) * 8, s);
   {
     Phase ph(ctx, "seq_headtail", s);
-    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s);
+    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
   }
   if (!per_file) {
     // exactly the owned windows (Eq. 1's count, known since load); the pad

@@ -1095,7 +1095,7 @@ gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s) {
   Buf head(ctx, size_t(d.R) * 8, s), tail(ctx, size_t(d.R) * 8, s), wt(ctx, size_t(d.R) * 8, s);
   {
     Phase ph(ctx, "seq_headtail", s);
-    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s);
+    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
     run_rule_weights(g, wt.as<uint64_t>(), s);
   }
   const int nb = int(std::min<int64_t>(kMaxCoarse, std::max<int64_t>(1, (U + kCoarseRows - 1) / kCoarseRows)));

@@ -86,6 +86,72 @@ __global__ void wt_init_kernel(const __grid_constant__ WtRoots<NJ> r) {
   for (int j = threadIdx.x; j < r.n; j += blockDim.x) r.wt[j][0] = 1ull;
 }
 
+// Adds mult * wt[parent] of the edges a warp holds (c = child, ascending, -1
+// none) to the children: summed per child inside the warp, one atomic per
+// child piece.
+__device__ __forceinline__ void add_edges(unsigned long long* wt, int32_t c, unsigned long long v) {
+  const int lane = threadIdx.x & 31;
+  // suffix sums over equal children (children are sorted, so equal ones are adjacent)
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long u = __shfl_down_sync(0xffffffffu, v, o);
+    const int32_t c2 = __shfl_down_sync(0xffffffffu, c, o);
+    if (lane + o < 32 && c2 == c) v += u;
+  }
+  const int32_t cp = __shfl_up_sync(0xffffffffu, c, 1);
+  if (c >= 0 && (lane == 0 || cp != c)) atomicAdd(&wt[c], v);
+}
+
+// The small levels [l0, depth) of a grammar's weight pass in one cluster (see
+// kTailItems).  On a 200k-word corpus (7 levels) the six level launches took
+// 19-21 us one by one and take 13.8 us here: 2.3 us per level, the round trips
+// of the barrier, a weight read through L2 and the atomics.
+struct WtTail {
+  const int32_t* lchild;
+  const int32_t* lpar;
+  const uint32_t* lmult;
+  const int64_t* loff;  // [depth + 1]
+  int l0, depth;
+  unsigned long long* wt;
+};
+
+template <int NJ>
+struct WtTails {
+  WtTail job[NJ];
+  int n;
+};
+
+template <int NJ>
+__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
+    wt_tail_kernel(const __grid_constant__ WtTails<NJ> ts) {
+  const WtTail& t = ts.job[blockIdx.x / kTailCtas];
+  const int lane = threadIdx.x & 31;
+  const int64_t me = int64_t(blockIdx.x % kTailCtas) * kTailThreads + threadIdx.x;
+  constexpr int64_t kStride = int64_t(kTailCtas) * kTailThreads;
+  int64_t a = t.loff[t.l0];
+  for (int lv = t.l0; lv < t.depth; ++lv) {
+    const int64_t b = t.loff[lv + 1];
+    int32_t c[2], p[2];
+    uint32_t m[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {  // two edges per thread: a level has at most kTailItems
+      const int64_t i = a + me + q * kStride;
+      const bool in = i < b;
+      c[q] = in ? t.lchild[i] : -1;
+      p[q] = in ? t.lpar[i] : 0;
+      m[q] = in ? t.lmult[i] : 0u;
+    }
+    if (lv > t.l0) cluster_sync();  // the parents' weights are final
+    unsigned long long v[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) v[q] = c[q] >= 0 ? (unsigned long long)m[q] * __ldcg(&t.wt[p[q]]) : 0ull;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (a + me - lane + q * kStride < b) add_edges(t.wt, c[q], v[q]);
+    a = b;
+  }
+}
+
 // Top-down weights for the children on one level: one thread per parent edge
 // (edges of a level are grouped by child), mult * wt[parent] summed per child
 // inside the warp, one atomic per child piece.  Parents sit on lower,
@@ -106,16 +172,7 @@ __global__ void wt_edges_kernel(const __grid_constant__ WtBatch<NJ> bt) {
   for (int64_t i = jb.a + cta * int64_t(blockDim.x) + threadIdx.x; i - lane < b; i += stride) {
     const bool in = i < b;
     const int32_t c = in ? lchild[i] : -1;
-    unsigned long long v = in ? (unsigned long long)lmult[i] * wt[lpar[i]] : 0ull;
-    // suffix sums over equal children (children are sorted, so equal ones are adjacent)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long u = __shfl_down_sync(0xffffffffu, v, o);
-      const int32_t c2 = __shfl_down_sync(0xffffffffu, c, o);
-      if (lane + o < 32 && c2 == c) v += u;
-    }
-    const int32_t cp = __shfl_up_sync(0xffffffffu, c, 1);
-    if (in && (lane == 0 || cp != c)) atomicAdd(&wt[c], v);
+    add_edges(wt, c, in ? (unsigned long long)lmult[i] * wt[lpar[i]] : 0ull);
   }
 }
 
@@ -385,46 +442,94 @@ __global__ void __launch_bounds__(kReduceThreads) wc_reduce_kernel(const __grid_
 
 // Head/tail buffers (Section IV-C), bottom-up: a rule's first two words come
 // from its first body symbols, taking a child's head when the symbol is a
-// rule (children are on deeper levels, finished earlier).
+// rule (children are on deeper levels, finished earlier).  A rule's own ends:
+// the body's first two and last two symbols (-1 where it has one symbol).
+struct RuleEnds {
+  int64_t lo, hi;
+  int32_t first, second, last, before;
+};
+
+__device__ __forceinline__ RuleEnds rule_ends(const DevGrammar& d, int32_t r) {
+  RuleEnds e;
+  e.lo = d.rule_off[r];
+  e.hi = d.rule_off[r + 1];
+  const bool any = e.hi > e.lo, two = e.hi > e.lo + 1;  // only the root's body may be empty
+  e.first = any ? d.sym[e.lo] : -1;
+  e.second = two ? d.sym[e.lo + 1] : -1;
+  e.last = any ? d.sym[e.hi - 1] : -1;
+  e.before = two ? d.sym[e.hi - 2] : -1;
+  return e;
+}
+
+__device__ __forceinline__ void head_tail_of(const DevGrammar& d, int32_t r, const RuleEnds& e, int32_t* head,
+                                             int32_t* tail) {
+  int2* const heads = reinterpret_cast<int2*>(head);
+  int2* const tails = reinterpret_cast<int2*>(tail);
+  int32_t h[2] = {-1, -1};
+  int n = 0;
+  for (int64_t i = e.lo; i < e.hi && n < 2; ++i) {
+    const int32_t s = i == e.lo ? e.first : (i == e.lo + 1 ? e.second : d.sym[i]);
+    if (s < d.V) {
+      h[n++] = s;
+    } else {
+      const int2 c = __ldcg(&heads[s - d.V]);
+      h[n++] = c.x;
+      if (n < 2 && c.y >= 0) h[n++] = c.y;
+    }
+  }
+  int32_t t[2] = {-1, -1};  // t[1] = last word, t[0] = the one before
+  int m = 0;
+  for (int64_t i = e.hi - 1; i >= e.lo && m < 2; --i) {
+    const int32_t s = i == e.hi - 1 ? e.last : (i == e.hi - 2 ? e.before : d.sym[i]);
+    if (s < d.V) {
+      t[1 - m++] = s;
+    } else {
+      const int2 c = __ldcg(&tails[s - d.V]);
+      t[1 - m++] = c.y;
+      if (m < 2 && c.x >= 0) t[1 - m++] = c.x;
+    }
+  }
+  heads[r] = make_int2(h[0], h[1]);
+  tails[r] = make_int2(t[0], t[1]);
+}
+
 __global__ void head_tail_level_kernel(const int32_t* __restrict__ order, int64_t a, int64_t b, DevGrammar d,
-                                       int32_t* __restrict__ head, int32_t* __restrict__ tail) {
+                                       int32_t* head, int32_t* tail) {
   for (int64_t k = a + blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < b; k += int64_t(gridDim.x) * blockDim.x) {
     const int32_t r = order[k];
-    const int64_t lo = d.rule_off[r], hi = d.rule_off[r + 1];
-    int32_t h[2] = {-1, -1};
-    int n = 0;
-    for (int64_t i = lo; i < hi && n < 2; ++i) {
-      const int32_t s = d.sym[i];
-      if (s < d.V) {
-        h[n++] = s;
-      } else {
-        const int32_t c = s - d.V;
-        const int32_t c0 = head[2 * c], c1 = head[2 * c + 1];
-        h[n++] = c0;
-        if (n < 2 && c1 >= 0) h[n++] = c1;
-      }
+    head_tail_of(d, r, rule_ends(d, r), head, tail);
+  }
+}
+
+// The small levels [l0, d.depth) in one cluster, deepest first (see kTailItems).
+__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
+    head_tail_deep_kernel(DevGrammar d, int l0, int32_t* head, int32_t* tail) {
+  const int64_t me = int64_t(blockIdx.x) * kTailThreads + threadIdx.x;
+  constexpr int64_t kStride = int64_t(kTailCtas) * kTailThreads;
+  for (int lv = d.depth - 1; lv >= l0; --lv) {
+    const int64_t a = d.lvl_off[lv], b = d.lvl_off[lv + 1];
+    int32_t r[2];
+    RuleEnds e[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int64_t k = a + me + q * kStride;
+      r[q] = k < b ? d.lvl_order[k] : -1;
+      if (r[q] >= 0) e[q] = rule_ends(d, r[q]);
     }
-    int32_t t[2] = {-1, -1};  // t[1] = last word, t[0] = the one before
-    int m = 0;
-    for (int64_t i = hi - 1; i >= lo && m < 2; --i) {
-      const int32_t s = d.sym[i];
-      if (s < d.V) {
-        t[1 - m++] = s;
-      } else {
-        const int32_t c = s - d.V;
-        const int32_t c0 = tail[2 * c], c1 = tail[2 * c + 1];
-        t[1 - m++] = c1;
-        if (m < 2 && c0 >= 0) t[1 - m++] = c0;
-      }
-    }
-    head[2 * r] = h[0];
-    head[2 * r + 1] = h[1];
-    tail[2 * r] = t[0];
-    tail[2 * r + 1] = t[1];
+    if (lv < d.depth - 1) cluster_sync();  // the children's buffers are final
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (r[q] >= 0) head_tail_of(d, r[q], e[q], head, tail);
   }
 }
 
 }  // namespace
+
+int small_levels(const std::vector<int64_t>& off, int from, int depth) {
+  int l = depth;
+  while (l > from && off[size_t(l)] - off[size_t(l) - 1] <= kTailItems) --l;
+  return depth - l >= 2 ? l : depth;
+}
 
 namespace {
 
@@ -437,12 +542,18 @@ void weights_batch(gt_grammar* const* gs, uint64_t* const* wts, int n, cudaStrea
   const int threads = 256;
   const int cap = ctx->num_sms * 16;
   WtRoots<NJ> roots{};
+  WtTails<NJ> tails{};
   roots.n = n;
-  int depth = 0;
+  int depth = 0;  // levels with a launch of their own
+  int first[NJ];  // first level of each grammar's tail
   for (int j = 0; j < n; ++j) {
     GT_CUDA(cudaMemsetAsync(wts[j], 0, size_t(gs[j]->d.R) * 8, s));
     roots.wt[j] = reinterpret_cast<unsigned long long*>(wts[j]);
-    depth = std::max(depth, int(gs[j]->d.depth));
+    const DevGrammar& d = gs[j]->d;
+    first[j] = small_levels(gs[j]->ledge_off, 1, d.depth);
+    depth = std::max(depth, first[j]);
+    if (first[j] < d.depth)
+      tails.job[tails.n++] = {d.ledge_child, d.ledge_par, d.ledge_mult, d.ledge_off, first[j], d.depth, roots.wt[j]};
   }
   wt_init_kernel<NJ><<<1, 64, 0, s>>>(roots);
   GT_LAUNCH_CHECK();
@@ -451,7 +562,7 @@ void weights_batch(gt_grammar* const* gs, uint64_t* const* wts, int n, cudaStrea
     int ctas = 0;
     for (int j = 0; j < n; ++j) {
       const gt_grammar* g = gs[j];
-      if (lv >= g->d.depth) continue;
+      if (lv >= first[j]) continue;
       const int64_t a = g->ledge_off[lv], b = g->ledge_off[lv + 1];
       if (b <= a) continue;
       WtJob& jb = bt.job[bt.n];
@@ -462,6 +573,10 @@ void weights_batch(gt_grammar* const* gs, uint64_t* const* wts, int n, cudaStrea
     if (bt.n == 0) continue;
     bt.cta[bt.n] = ctas;
     wt_edges_kernel<NJ><<<ctas, threads, 0, s>>>(bt);
+    GT_LAUNCH_CHECK();
+  }
+  if (tails.n > 0) {
+    wt_tail_kernel<NJ><<<tails.n * kTailCtas, kTailThreads, 0, s>>>(tails);
     GT_LAUNCH_CHECK();
   }
 }
@@ -593,11 +708,26 @@ void run_word_count_multi(gt_grammar* const* gs, uint64_t* const* counts, int n,
   }
 }
 
-void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s) {
+void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s, bool children_only) {
   const DevGrammar& d = g->d;
   const int threads = 256;
   const int cap = g->ctx->num_sms * 8;
-  for (int lv = d.depth - 1; lv >= 0; --lv) {
+  const int top = children_only ? 1 : 0;
+  // pairs are read and written 8 bytes at a time: a caller's buffers may be less aligned
+  const bool aligned = ((reinterpret_cast<uintptr_t>(d_head) | reinterpret_cast<uintptr_t>(d_tail)) & 7) == 0;
+  if (!aligned) {
+    Buf h(g->ctx, size_t(d.R) * 8, s), t(g->ctx, size_t(d.R) * 8, s);
+    run_head_tail(g, h.as<int32_t>(), t.as<int32_t>(), s, children_only);
+    GT_CUDA(cudaMemcpyAsync(d_head, h.p, size_t(d.R) * 8, cudaMemcpyDeviceToDevice, s));
+    GT_CUDA(cudaMemcpyAsync(d_tail, t.p, size_t(d.R) * 8, cudaMemcpyDeviceToDevice, s));
+    return;
+  }
+  const int deep = small_levels(g->lvl_off, top, d.depth);
+  if (deep < d.depth) {
+    head_tail_deep_kernel<<<kTailCtas, kTailThreads, 0, s>>>(d, deep, d_head, d_tail);
+    GT_LAUNCH_CHECK();
+  }
+  for (int lv = deep - 1; lv >= top; --lv) {
     const int64_t a = g->lvl_off[lv], b = g->lvl_off[lv + 1];
     if (b > a) {
       head_tail_level_kernel<<<grid_for(b - a, threads, cap), threads, 0, s>>>(d.lvl_order, a, b, d, d_head, d_tail);
