@@ -884,13 +884,33 @@ __device__ __forceinline__ void ii_masks(const uint32_t* __restrict__ bits, int 
   m_hi = lane + 32 < F ? bits[(int64_t(lane + 32) * nb + b) * kTvThreads + t] : 0u;
 }
 
+// Transpose of the 32 x 32 bit matrix whose row r lane r holds.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+  uint32_t m = 0x0000ffffu;
+#pragma unroll
+  for (int j = 16; j; j >>= 1) {
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+    x = (lane & j) ? (x & ~m) | ((y >> j) & m) : (x & m) | ((y & m) << j);
+    m ^= m << (j >> 1);
+  }
+  return x;
+}
+
 // The inverted index in one pass: CTAs take blocks of kIiWords words in
-// ticket order; each counts the files of its words (one ballot per bit, as
-// above), scans the counts, gets the block's first posting by a bounded
-// decoupled look-back over the preceding blocks, writes the words' offsets
-// and fills their postings.
+// ticket order; each turns the occupancy bits of its words (a lane per file)
+// into the set of files of every word (a lane per word) by a bit transpose,
+// scans their sizes, gets the block's first posting by a bounded decoupled
+// look-back over the preceding blocks, writes the words' offsets and fills
+// their postings: words in few files one per lane, otherwise word by word with
+// a lane per file, so that a word's postings are one dense store.  Bound by
+// instructions: counting by 64 ballots per 32 words and filling every word, the
+// empty ones too, took 52 us for 1M words in 13 files.
 constexpr int kIiThreads = 256;
 constexpr int kIiWords = kIiThreads;  // a warp per 32 words
+// Postings of a word up to which its own lane writes them.  Lane by lane a
+// warp's store touches up to 32 sectors; measured slower than word by word when
+// words have 15 files on average.
+constexpr int kIiLaneFiles = 6;
 
 __global__ void __launch_bounds__(kIiThreads) ii_build_kernel(const uint32_t* __restrict__ bits, int nb, int32_t F,
                                                               int32_t V, unsigned long long* __restrict__ flags,
@@ -906,13 +926,11 @@ __global__ void __launch_bounds__(kIiThreads) ii_build_kernel(const uint32_t* __
   const int64_t w0 = item * kIiWords + warp * 32;
   uint32_t lo = 0, hi = 0;
   if (w0 < V) ii_masks(bits, nb, F, w0, lane, lo, hi);
-  int mine = 0;
-#pragma unroll
-  for (int l = 0; l < 32; ++l) {
-    const int c = __popc(__ballot_sync(0xffffffffu, (lo >> l) & 1u)) + __popc(__ballot_sync(0xffffffffu, (hi >> l) & 1u));
-    if (lane == l) mine = c;
-  }
-  if (w0 + lane >= V) mine = 0;
+  // from here on: the files of word w0 + lane
+  lo = warp_transpose(lo, lane);
+  if (F > 32) hi = warp_transpose(hi, lane);
+  if (w0 + lane >= V) lo = hi = 0;
+  const int mine = __popc(lo) + __popc(hi);
   // exclusive prefix of the counts over the block
   int incl = mine;
 #pragma unroll
@@ -942,13 +960,22 @@ __global__ void __launch_bounds__(kIiThreads) ii_build_kernel(const uint32_t* __
   const int64_t my_off = s_prefix + s_wsum[warp] + incl - mine;
   if (w0 + lane < V) off[w0 + lane] = my_off;
   if (w0 + lane == V - 1) off[V] = my_off + mine;
+  if (__all_sync(0xffffffffu, mine <= kIiLaneFiles)) {
+    int64_t o = my_off;
+    for (unsigned m = lo; m; m &= m - 1) files[o++] = __ffs(m) - 1;
+    for (unsigned m = hi; m; m &= m - 1) files[o++] = __ffs(m) + 31;
+    return;
+  }
   const unsigned below = (1u << lane) - 1u;
-  for (int l = 0; l < 32 && w0 + l < V; ++l) {
-    const unsigned a = __ballot_sync(0xffffffffu, (lo >> l) & 1u);
-    const unsigned c = __ballot_sync(0xffffffffu, (hi >> l) & 1u);
+  for (unsigned todo = __ballot_sync(0xffffffffu, mine > 0); todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const unsigned a = __shfl_sync(0xffffffffu, lo, l);
     const int64_t o = __shfl_sync(0xffffffffu, my_off, l);
     if ((a >> lane) & 1u) files[o + __popc(a & below)] = lane;
-    if ((c >> lane) & 1u) files[o + __popc(a) + __popc(c & below)] = lane + 32;
+    if (F > 32) {
+      const unsigned c = __shfl_sync(0xffffffffu, hi, l);
+      if ((c >> lane) & 1u) files[o + __popc(a) + __popc(c & below)] = lane + 32;
+    }
   }
 }
 

@@ -9,6 +9,7 @@ import pytest
 import oracle
 from paper_2106_06889_gb300 import binding as B
 from paper_2106_06889_gb300.corpus import root_only_grammar, sequitur
+from tests.test_oracle_pins import grammar_from_rules
 
 pytestmark = pytest.mark.gpu
 
@@ -101,5 +102,60 @@ def test_sort_tile_change(ctx, n):
         for per_file, fields in ((0, ("key", "count")), (1, ("file", "key", "count"))):
             for got, want in zip(take(B.gt_sequence_count(gh, per_file), *fields), oracle.sequence_count(g, per_file)):
                 assert np.array_equal(got, want)
+    finally:
+        B.gt_free_grammar(gh)
+
+
+@pytest.mark.parametrize("V", [45, 70_000])
+@pytest.mark.parametrize("F", [1, 31, 32, 33, 64])
+def test_file_sets(ctx, F, V):
+    """Inverted index: words in few files and in most of them, one and two 32-file halves."""
+    rng = np.random.default_rng(F * V)
+    toks = (rng.zipf(1.2, 6000) % V).astype(np.int32)
+    cuts = np.sort(rng.integers(0, toks.shape[0] + 1, F - 1))
+    g = root_only_grammar(toks, np.diff(np.concatenate([[0], cuts, [toks.shape[0]]])), V)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        for got, want in zip(take(B.gt_inverted_index(gh), "offsets", "file"), oracle.inverted_index(g)):
+            assert np.array_equal(got, want)
+        # the same tolerance as the TF-IDF test: one quotient, logarithm (1 ulp) and product in float64
+        for got, want in zip(take(B.gt_tfidf(gh), "offsets", "word", "tfidf"), oracle.tfidf(g)):
+            assert np.allclose(got, want, rtol=1e-15, atol=0)
+    finally:
+        B.gt_free_grammar(gh)
+
+
+def deep_grammar(wide):
+    """A chain of 60 rules (rule r holds a word and rule r + 1), each also used by the root's two
+    files, over ``wide`` rules of two words on one level: with wide = 20,000 that level is too large
+    to share a launch with the small ones."""
+    V, depth = 50, 60
+    rng = np.random.default_rng(wide)
+    chain = [[int(rng.integers(V)), V + r + 1] if r < depth else [3, 4] for r in range(1, depth + 1)]
+    flat = [[int(a), int(b)] for a, b in rng.integers(0, V, (wide, 2))]
+    users = [[V + depth + 1 + i, V + depth + 1 + (i * 7) % wide, int(rng.integers(V))] for i in range(wide)]
+    first = V + depth + 1 + wide
+    root = [V + 1, 5, V + 30, V + 1] + [first + i for i in range(wide)] + [V + r for r in range(1, depth + 1)]
+    return grammar_from_rules(V, [root] + chain + flat + users, [0, 3 + wide // 3, len(root)])
+
+
+@pytest.mark.parametrize("wide", [1, 300, 20_000])
+def test_levels(ctx, wide):
+    """Level passes (weights, per-file weights, head/tail buffers) over many small levels, alone
+    and after a level too large for them; head/tail into buffers that are not 8-byte aligned."""
+    import torch
+    g = deep_grammar(wide)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        w = torch.empty(g.num_rules, dtype=torch.int64, device="cuda")
+        B.gt_rule_weights(gh, w)
+        assert np.array_equal(w.cpu().numpy().astype(np.uint64), oracle.rule_weights(g))
+        raw = [torch.full((2 * g.num_rules + 2,), -7, dtype=torch.int32, device="cuda") for _ in range(2)]
+        for shift in (0, 1):
+            views = [x[shift:shift + 2 * g.num_rules] for x in raw]
+            B.gt_head_tail(gh, *views)
+            for got, want in zip(views, oracle.head_tail(g)):
+                assert np.array_equal(got.cpu().numpy().reshape(-1, 2), np.asarray(want).reshape(-1, 2))
+        check(gh, g)
     finally:
         B.gt_free_grammar(gh)
