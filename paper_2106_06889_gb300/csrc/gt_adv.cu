@@ -20,45 +20,47 @@ namespace gt {
 namespace {
 
 // Rows of the pairs of every 3-gram: (a, b) and (a, c) of key a|b|c with its
-// count, after the files' last pairs (one row per file); *rows counts them all.
+// count, the words kb bits each.  *rows counts them; the files' last pairs follow.
 __global__ void cooc_rows_kernel(const uint64_t* __restrict__ key3, const uint64_t* __restrict__ cnt3,
-                                 const int64_t* __restrict__ n3_dev, int32_t F, uint64_t* __restrict__ keys,
-                                 uint32_t* __restrict__ vals, int64_t* __restrict__ rows) {
+                                 const int64_t* __restrict__ n3_dev, int kb, uint64_t* __restrict__ keys,
+                                 uint32_t* __restrict__ vals, unsigned long long* __restrict__ rows) {
   const int64_t n3 = *n3_dev;
   const uint64_t m = (uint64_t(1) << 21) - 1;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *rows = 2 * n3 + F;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *rows = 2 * (unsigned long long)n3;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n3; i += int64_t(gridDim.x) * blockDim.x) {
     const uint64_t k = key3[i];
     const uint64_t a = k >> 42, b = (k >> 21) & m, cw = k & m;
     const uint32_t c = uint32_t(cnt3[i]);  // below 2^32: fewer than 2^32 tokens
-    keys[F + i] = (a << 21) | b;
-    keys[F + n3 + i] = (a << 21) | cw;
-    vals[F + i] = c;
-    vals[F + n3 + i] = c;
+    keys[i] = (a << kb) | b;
+    keys[n3 + i] = (a << kb) | cw;
+    vals[i] = c;
+    vals[n3 + i] = c;
   }
 }
 
 // Last word of body symbol x (a word, or a rule's last word).
-__device__ __forceinline__ int32_t last_word(const DevGrammar& d, const int32_t* __restrict__ tail, int32_t x) {
-  return x < d.V ? x : tail[2 * (x - d.V) + 1];
+__device__ __forceinline__ int32_t last_word(const DevGrammar& d, const int4* __restrict__ ends, int32_t x) {
+  return x < d.V ? x : ends[x - d.V].w;
 }
 
 // The last pair (second-to-last word, last word) of every file of two or more
-// words, one row each (pad key otherwise).
-__global__ void file_last_pair_kernel(DevGrammar d, const int32_t* __restrict__ tail, uint64_t key_pad,
-                                      uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+// words, one row each, claimed in *rows (rows are sorted next).
+__global__ void file_last_pair_kernel(DevGrammar d, const int4* __restrict__ ends, int kb,
+                                      unsigned long long* __restrict__ rows, uint64_t* __restrict__ keys,
+                                      uint32_t* __restrict__ vals) {
   for (int32_t f = blockIdx.x * blockDim.x + threadIdx.x; f < d.F; f += gridDim.x * blockDim.x) {
     const int64_t fo = d.file_off[f], fe = d.file_off[f + 1];
     int32_t last = -1, prev = -1;
     if (fe > fo) {
       const int32_t x = d.sym[fe - 1];
-      last = last_word(d, tail, x);
-      if (x >= d.V) prev = tail[2 * (x - d.V)];  // -1 for a rule of one word
-      if (prev < 0 && fe - 2 >= fo) prev = last_word(d, tail, d.sym[fe - 2]);
+      last = last_word(d, ends, x);
+      if (x >= d.V) prev = ends[x - d.V].z;  // -1 for a rule of one word
+      if (prev < 0 && fe - 2 >= fo) prev = last_word(d, ends, d.sym[fe - 2]);
     }
-    const bool ok = last >= 0 && prev >= 0;
-    keys[f] = ok ? (uint64_t(uint32_t(prev)) << 21) | uint64_t(uint32_t(last)) : key_pad;
-    vals[f] = ok ? 1u : 0u;
+    if (last < 0 || prev < 0) continue;
+    const unsigned long long o = atomicAdd(rows, 1ull);
+    keys[o] = (uint64_t(uint32_t(prev)) << kb) | uint64_t(uint32_t(last));
+    vals[o] = 1u;
   }
 }
 
@@ -75,7 +77,8 @@ gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   if (d.V > (1 << 21)) fail(GT_EOVERFLOW, "pair keys need num_words <= 2^21");
-  gt_result* seq = run_sequence_count(g, 0, s);
+  Buf ends;
+  gt_result* seq = run_sequence_count(g, 0, s, &ends);
   try {
     void *k3 = nullptr, *c3 = nullptr;
     const int64_t* n3 = nullptr;
@@ -83,22 +86,25 @@ gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s) {
     result_device_field(seq, "count", &c3, &n3);
     const int64_t U = g->info.owned_windows;  // distinct 3-grams at most
     const int64_t n = 2 * U + d.F;
-    const uint64_t key_pad = uint64_t(1) << 42;  // above every pair key
+    int kb = 1;  // bits per word id
+    while ((int64_t(1) << kb) < d.V) ++kb;
     Buf keys(ctx, size_t(n) * 8, s), vals(ctx, size_t(n) * 4, s), rows(ctx, 8, s);
-    Buf tail(ctx, size_t(d.R) * 8, s), head(ctx, size_t(d.R) * 8, s);
     {
       Phase ph(ctx, "cooc_rows", s);
-      run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
+      if (!ends.p) {
+        ends = Buf(ctx, size_t(d.R) * 16, s);
+        run_rule_ends(g, ends.as<int4>(), s, true);
+      }
       const int threads = 256, cap = ctx->num_sms * 16;
       cooc_rows_kernel<<<grid_for(U, threads, cap), threads, 0, s>>>(
-          static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, d.F, keys.as<uint64_t>(), vals.as<uint32_t>(),
-          rows.as<int64_t>());
+          static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, kb, keys.as<uint64_t>(), vals.as<uint32_t>(),
+          rows.as<unsigned long long>());
       GT_LAUNCH_CHECK();
       file_last_pair_kernel<<<grid_for(d.F, threads, cap), threads, 0, s>>>(
-          d, tail.as<int32_t>(), key_pad, keys.as<uint64_t>(), vals.as<uint32_t>());
+          d, ends.as<int4>(), kb, rows.as<unsigned long long>(), keys.as<uint64_t>(), vals.as<uint32_t>());
       GT_LAUNCH_CHECK();
     }
-    gt_result* out = reduce_key_rows(ctx, keys, vals, n, 43, key_pad, s, reinterpret_cast<uint32_t*>(seq->d_lens),
+    gt_result* out = reduce_key_rows(ctx, keys, vals, n, kb, 2 * kb, s, reinterpret_cast<uint32_t*>(seq->d_lens),
                                      rows.as<int64_t>());
     out->deps.push_back(seq);  // the 3-gram result's buffers live until this result is freed
     return out;

@@ -163,15 +163,14 @@ __global__ void child_word_rows_kernel(const DevGrammar d, int kbw, const int64_
 constexpr int kRootWinThreads = kTile / 4;
 
 __global__ void __launch_bounds__(kRootWinThreads) root_window_rows_kernel(const DevGrammar d,
-                                                                           const int32_t* __restrict__ head,
-                                                                           const int32_t* __restrict__ tail, int kb,
+                                                                           const int4* __restrict__ ends, int kb,
                                                                            FileRows out) {
   __shared__ uint32_t s_warp[kRootWinThreads / 32];
   __shared__ unsigned long long s_base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   TileWin t;
   int32_t file[4];
-  tile_windows(d, head, tail, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t, file);
+  tile_windows(d, ends, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t, file);
   uint32_t c = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -680,7 +679,8 @@ void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** 
     GT_LAUNCH_CHECK();
     for (int i = 0; i < n_tv; ++i)
       tv_out[i] = tv_from_arrays(g->ctx, wr.word.as<int32_t>(), wr.cnt.as<uint64_t>(), toff.as<int64_t>(),
-                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], s, wr.status.as<uint32_t>(), d.V);
+                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], uint64_t(g->max_file_len), s,
+                                 wr.status.as<uint32_t>(), d.V);
   }
   if (ii_out) *ii_out = bu_inverted_index(g, wr, s);
 }
@@ -736,7 +736,7 @@ void bu_local_window_rows(gt_grammar* g, int kb, cudaStream_t s, Windows& out) {
 
 // Per-file window rows: windows owned by the root in each file, plus every
 // window inside each (file, root child) expansion, weighted by multiplicity.
-void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, cudaStream_t s, Windows& out) {
+void bu_window_rows(gt_grammar* g, Buf& ends, int kb, cudaStream_t s, Windows& out) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int threads = 256, cap = ctx->num_sms * 16;
@@ -753,7 +753,7 @@ void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, cudaStream_t s,
     Buf first(ctx, 8, s);
     if (d.root_len > 0) {
       root_window_rows_kernel<<<unsigned((d.root_len + kTile - 1) / kTile), kRootWinThreads, 0, s>>>(
-          d, head.as<int32_t>(), tail.as<int32_t>(), kb, fr);
+          d, ends.as<int4>(), kb, fr);
       GT_LAUNCH_CHECK();
     }
     if (d.ER > 0) {

@@ -53,18 +53,15 @@ struct Sym3 {
   int32_t first, second, second_last, last;  // -1 where the expansion is too short
 };
 
-__device__ __forceinline__ Sym3 sym_words(const DevGrammar& d, const int32_t* __restrict__ head,
-                                          const int32_t* __restrict__ tail, int32_t x) {
+__device__ __forceinline__ Sym3 sym_words(const DevGrammar& d, const int4* __restrict__ ends, int32_t x) {
   Sym3 r;
   if (x < d.V) {
     r.first = r.last = x;
     r.second = r.second_last = -1;
   } else {
     const int32_t c = x - d.V;
-    r.first = head[2 * c];
-    r.second = head[2 * c + 1];
-    r.second_last = tail[2 * c];
-    r.last = tail[2 * c + 1];
+    const int4 e = ends[c];
+    r = {e.x, e.y, e.z, e.w};
   }
   return r;
 }
@@ -89,15 +86,14 @@ __device__ __forceinline__ int64_t seq_end(const DevGrammar& d, int64_t j, int32
 }
 
 // The (at most two) owned windows starting in body symbol j; returns how many.
-__device__ __forceinline__ int windows_at(const DevGrammar& d, const int32_t* __restrict__ head,
-                                          const int32_t* __restrict__ tail, int64_t j, int64_t end, int kb,
+__device__ __forceinline__ int windows_at(const DevGrammar& d, const int4* __restrict__ ends, int64_t j, int64_t end, int kb,
                                           uint64_t* k) {
   if (j + 1 >= end) return 0;
-  const Sym3 a = sym_words(d, head, tail, d.sym[j]);
-  const Sym3 b = sym_words(d, head, tail, d.sym[j + 1]);
+  const Sym3 a = sym_words(d, ends, d.sym[j]);
+  const Sym3 b = sym_words(d, ends, d.sym[j + 1]);
   const int32_t n1 = b.first;
   int32_t n2 = b.second;
-  if (n2 < 0) n2 = j + 2 < end ? sym_words(d, head, tail, d.sym[j + 2]).first : -1;
+  if (n2 < 0) n2 = j + 2 < end ? sym_words(d, ends, d.sym[j + 2]).first : -1;
   // k[0], k[1] are always written (fixed indices keep them in registers)
   const bool w0 = a.second_last >= 0;  // child with >= 2 words
   const uint64_t x0 = w0 ? pack_compact(a.second_last, a.last, n1, kb) : 0;
@@ -116,8 +112,7 @@ struct TileWin {
 };
 
 // file (optional): the file of each symbol of the root.
-__device__ __forceinline__ int tile_windows(const DevGrammar& d, const int32_t* __restrict__ head,
-                                            const int32_t* __restrict__ tail, int kb, int64_t j0, TileWin& t,
+__device__ __forceinline__ int tile_windows(const DevGrammar& d, const int4* __restrict__ ends, int kb, int64_t j0, TileWin& t,
                                             int32_t* file = nullptr) {
   int c = 0;
   int64_t end = -1;  // end of the body sequence holding the previous symbol (rule or root file)
@@ -133,11 +128,74 @@ __device__ __forceinline__ int tile_windows(const DevGrammar& d, const int32_t* 
       if (j >= end || j == d.root_len) end = seq_end(d, j, &rule, &f);
       t.r[i] = rule;
       if (file) file[i] = f;
-      t.n[i] = windows_at(d, head, tail, j, end, kb, t.k[i]);
+      t.n[i] = windows_at(d, ends, j, end, kb, t.k[i]);
     }
     c += t.n[i];
   }
   return c;
+}
+
+// ---- windows of a tile from shared memory -----------------------------------
+// The words at both ends of every symbol of a tile (and of the two after it),
+// looked up once per symbol, and a bit per symbol that ends its body sequence
+// (file or rule).  A symbol's windows then need only its neighbours' entries:
+// enumerating them from global memory looked up each symbol's ends three times,
+// in dependent loads (2.6 times as long per window).
+constexpr int kWinThreads = kTile / 4;
+
+struct TileEnds {
+  int4 words[kTile + 2];  // first, second, second to last, last (-1 where there is none)
+  uint32_t last[kTile / 32 + 1];
+};
+
+// By the whole CTA (kWinThreads threads).
+__device__ __forceinline__ void load_tile_ends(const DevGrammar& d, const int4* __restrict__ ends, int64_t t0, TileEnds& e) {
+  const int tid = threadIdx.x;
+  if (tid <= kTile / 32) e.last[tid] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    const int i = q * kWinThreads + tid;
+    if (i >= kTile + 2) break;
+    const int64_t j = t0 + i;
+    int4 w = make_int4(-1, -1, -1, -1);
+    if (j < d.G) {
+      const int32_t s = d.sym[j];
+      if (s < d.V) {
+        w.x = w.w = s;
+      } else {
+        w = ends[s - d.V];
+      }
+      if (j >= d.root_len && i <= kTile) {
+        const int32_t* sr = d.sym_rule + (j - d.first_rule_tile * kTile);
+        if (j + 1 == d.G || sr[0] != sr[1]) atomicOr(&e.last[i >> 5], 1u << (i & 31));
+      }
+    }
+    e.words[i] = w;
+  }
+  if (t0 < d.root_len) {  // files that end in the tile (an empty one marks the end before it again)
+    const int64_t t1 = t0 + kTile + 1;
+    const int64_t f0 = upper_bound_dev(d.file_off, int64_t(d.F) + 1, t0);  // first f with file_off[f] > t0
+    for (int64_t f = f0 + tid; f <= d.F; f += kWinThreads) {
+      const int64_t i = d.file_off[f] - 1 - t0;
+      if (d.file_off[f] > t1) break;
+      atomicOr(&e.last[i >> 5], 1u << (i & 31));
+    }
+  }
+  __syncthreads();
+}
+
+// The windows starting in symbol i of the tile, in text order: bit 0 of the
+// result says that k[0] is one (a child of two or more words), bit 1 that k[1] is.
+__device__ __forceinline__ int windows_in(const TileEnds& e, int i, int kb, uint64_t* k) {
+  if ((e.last[i >> 5] >> (i & 31)) & 1u) return 0;
+  const int4 a = e.words[i], b = e.words[i + 1];
+  int32_t n2 = b.y;
+  if (n2 < 0 && !((e.last[(i + 1) >> 5] >> ((i + 1) & 31)) & 1u)) n2 = e.words[i + 2].x;
+  const bool w0 = a.z >= 0, w1 = n2 >= 0;
+  k[0] = w0 ? pack_compact(a.z, a.w, b.x, kb) : 0;
+  k[1] = w1 ? pack_compact(a.w, b.x, n2, kb) : 0;
+  return int(w0) | int(w1) << 1;
 }
 
 // compact key (kb bits per word) -> w1 << 42 | w2 << 21 | w3; kb == 0 keeps it

@@ -986,10 +986,11 @@ __global__ void last_total_kernel(const int64_t* __restrict__ ex, const int64_t*
   if (out2) *out2 = t;
 }
 
-// top-k: key = file << 32 | (2^32 - 1 - count), sorted stably over entries that
-// are already in ascending word order inside each file.
+// top-k: key = file << cbits | (max_count - count), sorted stably over entries that
+// are already in ascending word order inside each file (no count exceeds
+// max_count, the longest file's length).
 __global__ void topk_keys_kernel(const int32_t* __restrict__ word, const uint64_t* __restrict__ cnt,
-                                 const int64_t* __restrict__ tv_off, int32_t F,
+                                 const int64_t* __restrict__ tv_off, int32_t F, uint64_t max_count, int cbits,
                                  uint64_t* __restrict__ keys, uint32_t* __restrict__ idx) {
   const int64_t n = tv_off[F];
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
@@ -1000,7 +1001,7 @@ __global__ void topk_keys_kernel(const int32_t* __restrict__ word, const uint64_
       if (tv_off[mid] <= i) lo = mid;
       else hi = mid;
     }
-    keys[i] = (uint64_t(lo) << 32) | uint64_t(0xffffffffu - uint32_t(cnt[i]));
+    keys[i] = (uint64_t(lo) << cbits) | (max_count - cnt[i]);
   }
 }
 
@@ -1497,7 +1498,7 @@ gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t
       GT_LAUNCH_CHECK();
     }
     return tv_from_arrays(ctx, tw.as<int32_t>(), tc.as<uint64_t>(), full_off.as<int64_t>(), fh.total.as<int64_t>(),
-                          nb_, d.F, top_k, s, fh.status.as<uint32_t>(), d.V);
+                          nb_, d.F, top_k, uint64_t(g->max_file_len), s, fh.status.as<uint32_t>(), d.V);
   }
   ResultBuilder rb(ctx, s);
   GT_CUDA(cudaMemcpyAsync(rb.status(), fh.status.p, 4, cudaMemcpyDeviceToDevice, s));
@@ -1610,7 +1611,7 @@ __global__ void copy_rows_kernel(const int32_t* __restrict__ w, const uint64_t* 
 // Term-vector result from (word, count) rows in (file, word) order with file
 // offsets; top_k > 0 keeps each file's top_k counts (count desc, word asc).
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
-                          const int64_t* total, int64_t bound, int32_t F, int top_k, cudaStream_t s,
+                          const int64_t* total, int64_t bound, int32_t F, int top_k, uint64_t max_count, cudaStream_t s,
                           const uint32_t* status_in, int32_t V) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
@@ -1637,10 +1638,10 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
     Buf i1(ctx, size_t(bound) * 4, s), rs(ctx, radix_scratch_bytes(bound, true, 4), s);
     Buf kc(ctx, size_t(F) * 8 + 8, s), sc(ctx, scan_scratch_bytes(F + 1), s);
     if (bound > 0) {
-      topk_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, tv_off_in, F, k0.as<uint64_t>(),
-                                                                          i0.as<uint32_t>());
+      const int cbits = bits_for(int64_t(max_count)), kbits = cbits + bits_for(std::max(F - 1, 1));
+      topk_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, tv_off_in, F, max_count, cbits,
+                                                                          k0.as<uint64_t>(), i0.as<uint32_t>());
       GT_LAUNCH_CHECK();
-      const int kbits = 32 + bits_for(std::max(F - 1, 1));
       if (!radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), i0.p, i1.p, 4, bound, 0, kbits, kbits, kbits, rs.p,
                                s, total))
         std::swap(i0, i1);

@@ -429,8 +429,10 @@ void run_word_count(gt_grammar* g, const uint64_t* d_wt, uint64_t* d_counts, cud
 // word counts of up to 64 grammars (one context) in one fused launch sequence
 void run_word_count_multi(gt_grammar* const* gs, uint64_t* const* counts, int n, cudaStream_t s,
                           uint32_t* status = nullptr);
-// children_only: the buffers of rules on level 0, which no rule refers to, are left out
-void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s, bool children_only = false);
+void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s);
+// Head and tail side by side, per rule: first, second, second to last and last
+// word.  children_only: rules on level 0, which no rule refers to, are left out.
+void run_rule_ends(gt_grammar* g, int4* ends, cudaStream_t s, bool children_only);
 // First level from which on every level has at most kTailItems items (off: the
 // levels' offsets, host), at least `from`; depth when fewer than two such levels.
 int small_levels(const std::vector<int64_t>& off, int from, int depth);
@@ -482,7 +484,7 @@ struct FileRowBufs {
 void sort_file_rows(gt_ctx* ctx, FileRowBufs& r, int kb, int32_t F, cudaStream_t s, Windows& out);
 
 // gt_bu.cu: bottom-up per-file rows
-void bu_window_rows(gt_grammar* g, Buf& head, Buf& tail, int kb, cudaStream_t s, Windows& out);
+void bu_window_rows(gt_grammar* g, Buf& ends, int kb, cudaStream_t s, Windows& out);
 void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** tv_out, gt_result** ii_out,
                        cudaStream_t s);
 gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s);
@@ -503,27 +505,29 @@ int64_t gparam(const gt_grammar* g, const char* name, int64_t dflt);
 // top_k == kTfIdf: the term vector with a "tfidf" field (float64) instead of top-k selection
 constexpr int kTfIdf = -1;
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
-                          const int64_t* total, int64_t bound, int32_t F, int top_k, cudaStream_t s,
+                          const int64_t* total, int64_t bound, int32_t F, int top_k, uint64_t max_count, cudaStream_t s,
                           const uint32_t* status_in, int32_t V = 0);
 // Device pointer of a result field and the device slot holding its length
 // (valid on the result's stream before the result completes).
 void result_device_field(gt_result* r, const char* field, void** ptr, const int64_t** d_len);
 
 // gt_seq.cu: sequence count (l = 3) and ranked inverted index
-gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s);
+// keep_ends (optional): receives the rules' first and last words it built (left empty on "seq_path" 2)
+gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s, Buf* keep_ends = nullptr);
 // gt_adv.cu: TF-IDF (term vector with idf weights) and word co-occurrence
 gt_result* run_tfidf(gt_grammar* g, cudaStream_t s);
 gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s);
-// gt_seq.cu: rows (key, weight) -> one row per distinct key with the weights
-// summed, ascending key; at most n rows (*n_dev of them, if given), rows of key_pad skipped
-gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int key_bits, uint64_t key_pad,
-                           cudaStream_t s, const uint32_t* status_in = nullptr, const int64_t* n_dev = nullptr);
+// gt_seq.cu: rows (key of key_bits bits, kb per word; weight) -> one row per distinct
+// key with the weights summed, ascending key, 21 bits per word; at most n rows (*n_dev
+// of them, if given)
+gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int kb, int key_bits, cudaStream_t s,
+                           const uint32_t* status_in = nullptr, const int64_t* n_dev = nullptr);
 // gt_seqg.cu: the global count (per_file == 0) by sample-sort buckets
 gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s);
 // owned windows of every tile of kTile symbols, exclusive scan [ntiles + 1]:
 // structure, built by the first call and kept with the grammar (outside
 // stream capture; GT_EINVAL if the first call is captured)
-const int64_t* seq_tile_offsets(gt_grammar* g, const int32_t* head, const int32_t* tail, int kb, cudaStream_t s);
+const int64_t* seq_tile_offsets(gt_grammar* g, const int4* ends, int kb, cudaStream_t s);
 gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s);
 // rows (key, file, count) -> ranked index; keys are compact 3-word keys
 // (windows = true, kb bits per word) or word ids (windows = false), all of at

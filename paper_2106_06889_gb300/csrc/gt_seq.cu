@@ -30,8 +30,6 @@ namespace {
 // tile's first row comes from the per-grammar tile offsets (the windows of
 // every tile counted and scanned once, seq_tile_offsets), and the emit pass
 // ranks the windows inside the tile.
-constexpr int kWinThreads = kTile / 4;
-
 // Exclusive prefix of v over the CTA (kWinThreads threads); *total gets the sum.
 __device__ __forceinline__ int cta_excl_scan(int v, int* total) {
   __shared__ int warp_tot[kWinThreads / 32];
@@ -57,41 +55,72 @@ __device__ __forceinline__ int cta_excl_scan(int v, int* total) {
 }
 
 // Rows of rules nothing references (weight 0) get the pad key.  Rows past
-// `bound` are not written; the status word records it.
-__global__ void __launch_bounds__(kWinThreads) win_emit_kernel(DevGrammar d, const int32_t* __restrict__ head,
-                                                               const int32_t* __restrict__ tail,
-                                                               const uint64_t* __restrict__ wt, int kb,
-                                                               uint64_t key_pad, const int64_t* __restrict__ tile_off,
-                                                               int64_t bound, uint64_t* __restrict__ keys,
-                                                               uint32_t* __restrict__ vals,
-                                                               unsigned* __restrict__ status) {
-  TileWin t;
-  const int c = tile_windows(d, head, tail, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t);
-  // the tile's first row and the owners' weights are requested before the
-  // scan's barriers, so they arrive while the CTA ranks its windows
+// `bound` are not written; the status word records it.  A warp takes 128
+// consecutive symbols, 32 at a time, so that two ballots give the rows' order;
+// rows are staged in shared memory and written in one dense run per tile.
+struct WinStage {
+  uint64_t key[2 * kTile];
+  uint32_t val[2 * kTile];
+};
+
+__global__ void __launch_bounds__(kWinThreads, 3) win_emit_kernel(DevGrammar d, const int4* __restrict__ ends,
+                                                                  const uint64_t* __restrict__ wt, int kb,
+                                                                  uint64_t key_pad,
+                                                                  const int64_t* __restrict__ tile_off, int64_t bound,
+                                                                  uint64_t* __restrict__ keys,
+                                                                  uint32_t* __restrict__ vals,
+                                                                  unsigned* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char win_smem[];
+  TileEnds& te = *reinterpret_cast<TileEnds*>(win_smem);
+  WinStage& stage = *reinterpret_cast<WinStage*>(win_smem);  // takes the ends' room once they are read
+  __shared__ int warp_tot[kWinThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t t0 = int64_t(blockIdx.x) * kTile;
   const int64_t first = tile_off[blockIdx.x];
-  uint32_t wv[4];
+  load_tile_ends(d, ends, t0, te);
+  uint64_t k[4][2];
+  uint32_t w[4];
+  int at[4], n = 0;  // at: the symbol's first row in the warp
+  unsigned has = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) wv[i] = t.n[i] ? uint32_t(wt[t.r[i]]) : 0u;
-  int total;
-  int64_t pos = first + cta_excl_scan(c, &total);
-  bool over = false;
+  for (int q = 0; q < 4; ++q) {
+    const int i = warp * 128 + q * 32 + lane;
+    const int64_t j = t0 + i;
+    const int h = j < d.G ? windows_in(te, i, kb, k[q]) : 0;
+    const unsigned b0 = __ballot_sync(0xffffffffu, h & 1), b1 = __ballot_sync(0xffffffffu, h & 2);
+    has |= unsigned(h) << (2 * q);
+    at[q] = n + __popc(b0 & lt) + __popc(b1 & lt);
+    n += __popc(b0) + __popc(b1);
+    w[q] = 0;
+    if (h) w[q] = j < d.root_len ? uint32_t(wt[0]) : uint32_t(wt[d.sym_rule[j - d.first_rule_tile * kTile]]);
+  }
+  if (lane == 0) warp_tot[warp] = n;
+  __syncthreads();  // also: the ends are read, the stage takes their room
+  int before = 0, total = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t w = wv[i];
+  for (int x = 0; x < kWinThreads / 32; ++x) {
+    before += x < warp ? warp_tot[x] : 0;
+    total += warp_tot[x];
+  }
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
-      if (q < t.n[i]) {
-        if (pos < bound) {
-          keys[pos] = w ? t.k[i][q] : key_pad;
-          vals[pos] = w;
-        } else {
-          over = true;
-        }
-        ++pos;
+  for (int q = 0; q < 4; ++q) {
+    int o = before + at[q];
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+      if ((has >> (2 * q + z)) & 1u) {
+        stage.key[o] = w[q] ? k[q][z] : key_pad;
+        stage.val[o] = w[q];
+        ++o;
       }
   }
-  if (over) atomicOr(status, ST_OVERFLOW);
+  __syncthreads();
+  for (int i = threadIdx.x; i < total; i += kWinThreads)
+    if (first + i < bound) {
+      keys[first + i] = stage.key[i];
+      vals[first + i] = stage.val[i];
+    }
+  if (threadIdx.x == 0 && first + total > bound) atomicOr(status, ST_OVERFLOW);
 }
 
 // Per-file rows, top-down: every window once per file of its rule (the root's
@@ -101,14 +130,14 @@ __global__ void __launch_bounds__(kWinThreads) win_emit_kernel(DevGrammar d, con
 // over all symbols, a scan of the counts and a second enumeration (61 + 40 + 79
 // us on 7.1M symbols).
 __global__ void __launch_bounds__(kWinThreads) win_emit_file_kernel(
-    DevGrammar d, const int32_t* __restrict__ head, const int32_t* __restrict__ tail,
+    DevGrammar d, const int4* __restrict__ ends,
     const unsigned long long* __restrict__ mask, const int64_t* __restrict__ woff,
     const uint32_t* __restrict__ slot_pair, const uint32_t* __restrict__ fw, int kb, FileRows out) {
   __shared__ unsigned long long s_base;
   TileWin t;
   int32_t file[4];
   const int64_t j0 = int64_t(blockIdx.x) * kTile + threadIdx.x * 4;
-  tile_windows(d, head, tail, kb, j0, t, file);
+  tile_windows(d, ends, kb, j0, t, file);
   unsigned long long m[4];
   int c = 0;
 #pragma unroll
@@ -225,7 +254,8 @@ void sort_file_rows(gt_ctx* ctx, FileRowBufs& r, int kb, int32_t F, cudaStream_t
 namespace {
 
 // Device-detected failures go to *status (the result's own status word).
-void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, uint32_t* status) {
+void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, uint32_t* status,
+                    Buf* keep_ends = nullptr) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int threads = 256, cap = ctx->num_sms * 16;
@@ -233,12 +263,15 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
   if (d.N >= (uint64_t(1) << 32)) fail(GT_EOVERFLOW, "sequence count needs fewer than 2^32 tokens per grammar");
   const int kb = bits_for(d.V > 1 ? d.V - 1 : 1);  // bits per word id
   out.kb = kb;
-  out.key_pad = uint64_t(1) << (3 * kb);  // above every real key: unused rows sort last
-  const int key_bits = 3 * kb + 1;
-  Buf head(ctx, size_t(d.R) * 8, s), tail(ctx, size_t(d.R) * 8, s);
+  // the pad sorts after every real key: all ones where that is none (word IDs below
+  // 2^kb - 1 and so no bit of its own to sort on), else the next power of two
+  const bool ones = d.V < (int64_t(1) << kb);
+  out.key_pad = (uint64_t(1) << (3 * kb)) - (ones ? 1 : 0);
+  const int key_bits = 3 * kb + (ones ? 0 : 1);
+  Buf ends(ctx, size_t(d.R) * 16, s);
   {
     Phase ph(ctx, "seq_headtail", s);
-    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
+    run_rule_ends(g, ends.as<int4>(), s, true);
   }
   if (!per_file) {
     // exactly the owned windows (Eq. 1's count, known since load); the pad
@@ -253,8 +286,10 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
       run_rule_weights(g, wt.as<uint64_t>(), s);
       const int64_t nt = d.ntiles;
       // each tile's first row: structure of the grammar, counted once and kept
-      const int64_t* toff = seq_tile_offsets(g, head.as<int32_t>(), tail.as<int32_t>(), kb, s);
-      win_emit_kernel<<<unsigned(nt), kWinThreads, 0, s>>>(d, head.as<int32_t>(), tail.as<int32_t>(),
+      const int64_t* toff = seq_tile_offsets(g, ends.as<int4>(), kb, s);
+      constexpr size_t smem = std::max(sizeof(TileEnds), sizeof(WinStage));
+      GT_CUDA(cudaFuncSetAttribute(win_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+      win_emit_kernel<<<unsigned(nt), kWinThreads, smem, s>>>(d, ends.as<int4>(),
                                                             wt.as<uint64_t>(), kb, out.key_pad, toff, n,
                                                             k0.as<uint64_t>(), v0.as<uint32_t>(), status);
       GT_LAUNCH_CHECK();
@@ -268,10 +303,11 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
                                        key_bits, rs.p, s);
     out.keys = std::move(b ? k1 : k0);
     out.vals = std::move(b ? v1 : v0);
+    if (keep_ends) *keep_ends = std::move(ends);
     return;
   }
   if (file_strategy(g) == 2) {
-    bu_window_rows(g, head, tail, kb, s, out);
+    bu_window_rows(g, ends, kb, s, out);
     return;
   }
   // ---- per file, top-down: windows x files of the rule ----
@@ -282,7 +318,7 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
     file_weights(g, s, fw);
     const FileRows fr = rows.make(ctx, kb, d.F, 2 * d.root_len + 2 * g->fsym_bound, s);
     if (rows.bound > 0 && d.ntiles > 0) {
-      win_emit_file_kernel<<<unsigned(d.ntiles), kWinThreads, 0, s>>>(d, head.as<int32_t>(), tail.as<int32_t>(),
+      win_emit_file_kernel<<<unsigned(d.ntiles), kWinThreads, 0, s>>>(d, ends.as<int4>(),
                                                                      fw.mask, fw.off, fw.slot_pair,
                                                                      fw.w.as<uint32_t>(), kb, fr);
       GT_LAUNCH_CHECK();
@@ -395,8 +431,8 @@ gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const
   return rb.finish();
 }
 
-gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int key_bits, uint64_t key_pad,
-                           cudaStream_t s, const uint32_t* status_in, const int64_t* n_dev) {
+gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int kb, int key_bits, cudaStream_t s,
+                           const uint32_t* status_in, const int64_t* n_dev) {
   ResultBuilder rb(ctx, s);
   if (status_in) GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
   StatusScope scope(rb.status());
@@ -410,9 +446,11 @@ gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int key
                                        key_bits, rs.p, s, n_dev);
     RunOut o;
     o.key = key;
+    o.kb = kb;
     o.count = count;
     o.rows = len;
-    reduce_runs(ctx, (b ? k1 : keys).as<uint64_t>(), nullptr, (b ? v1 : vals).as<uint32_t>(), n, n_dev, key_pad, o, s);
+    reduce_runs(ctx, (b ? k1 : keys).as<uint64_t>(), nullptr, (b ? v1 : vals).as<uint32_t>(), n, n_dev, ~uint64_t(0), o,
+                s);
   } else {
     GT_CUDA(cudaMemsetAsync(len, 0, 8, s));
   }
@@ -439,7 +477,7 @@ gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s) {
                           uint64_t(g->max_file_len), s, st.as<uint32_t>());
 }
 
-gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s) {
+gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s, Buf* keep_ends) {
   // global count: the one-row-per-window radix sort (default, measured faster
   // on the 500M-token corpus) or the sample-sort buckets (seq_path = 2)
   if (!per_file && gparam(g, "seq_path", 1) == 2) return run_sequence_count_global(g, s);
@@ -447,7 +485,7 @@ gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s) {
   ResultBuilder rb(ctx, s);
   StatusScope scope(rb.status());
   Windows w;
-  sorted_windows(g, per_file != 0, s, w, rb.status());
+  sorted_windows(g, per_file != 0, s, w, rb.status(), keep_ends);
   Phase ph(ctx, "seq_reduce", s);
   auto* key = static_cast<uint64_t*>(rb.alloc(size_t(w.n) * 8));
   auto* count = static_cast<uint64_t*>(rb.alloc(size_t(w.n) * 8));

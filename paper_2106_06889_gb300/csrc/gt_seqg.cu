@@ -124,8 +124,7 @@ __device__ __forceinline__ uint32_t scan_counts(const uint32_t* h, uint32_t* st,
 // Arguments of the passes over the grammar and over its rows.
 struct SgArgs {
   DevGrammar d;
-  const int32_t* head;
-  const int32_t* tail;
+  const int4* ends;
   const uint64_t* wt;        // rule weights (Algorithm 1)
   const uint64_t* spl;       // coarse bounds, nspl of them
   const uint16_t* lut;       // [2^lut_bits + 1]: first bucket of each key prefix
@@ -165,7 +164,7 @@ __global__ void __launch_bounds__(1024) sg_bounds_kernel(const __grid_constant__
     int32_t r, f;
     const int64_t end = seq_end(a.d, j, &r, &f);
     uint64_t k[2];
-    int n = windows_at(a.d, a.head, a.tail, j, end, a.kb, k);
+    int n = windows_at(a.d, a.ends, j, end, a.kb, k);
     if (a.wt[r] == 0) n = 0;  // rules nothing references own no rows
     s_keys[2 * i] = n > 0 ? k[0] : kEmpty;
     s_keys[2 * i + 1] = n > 1 ? k[1] : kEmpty;
@@ -201,12 +200,11 @@ __device__ __forceinline__ void cta_tiles(int64_t ntiles, int64_t* t0, int64_t* 
 }
 
 // Windows of every tile (structure only: independent of the weights).
-__global__ void __launch_bounds__(kSgThreads) sg_tile_count_kernel(DevGrammar d, const int32_t* __restrict__ head,
-                                                                   const int32_t* __restrict__ tail, int kb,
+__global__ void __launch_bounds__(kSgThreads) sg_tile_count_kernel(DevGrammar d, const int4* __restrict__ ends, int kb,
                                                                    int64_t* __restrict__ tcnt) {
   TileWin t;
   uint32_t total;
-  block_scan_u32<kSgThreads>(tile_windows(d, head, tail, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t),
+  block_scan_u32<kSgThreads>(tile_windows(d, ends, kb, int64_t(blockIdx.x) * kTile + threadIdx.x * 4, t),
                              &total);
   if (threadIdx.x == 0) tcnt[blockIdx.x] = total;
 }
@@ -231,7 +229,7 @@ __global__ void __launch_bounds__(kSgThreads) sg_emit_kernel(const __grid_consta
   for (int64_t tl = t0; tl < t1; ++tl) {
     TileWin t;
     uint32_t total;
-    const uint32_t mine = tile_windows(a.d, a.head, a.tail, a.kb, tl * kTile + threadIdx.x * 4, t);
+    const uint32_t mine = tile_windows(a.d, a.ends, a.kb, tl * kTile + threadIdx.x * 4, t);
     // first row and weights requested before the scan's barriers
     const int64_t first = a.tile_off[tl];
     uint64_t wv[4];
@@ -1048,7 +1046,7 @@ __global__ void __launch_bounds__(kRdThreads, 2) sg_reduce_kernel(const __grid_c
 
 // Row offsets of every tile (the tile's first owned window in position
 // order), built once per grammar; later calls on other streams wait for it.
-const int64_t* seq_tile_offsets(gt_grammar* g, const int32_t* head, const int32_t* tail, int kb, cudaStream_t s) {
+const int64_t* seq_tile_offsets(gt_grammar* g, const int4* ends, int kb, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g->seq_mu);
   if (g->seq_tile_off) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1064,7 +1062,7 @@ const int64_t* seq_tile_offsets(gt_grammar* g, const int32_t* head, const int32_
   auto* off = static_cast<int64_t*>(grammar_alloc(g, size_t(nt + 1) * 8, s));
   Buf cnt(g->ctx, size_t(nt + 1) * 8, s), sc(g->ctx, scan_scratch_bytes(nt + 1), s);
   GT_CUDA(cudaMemsetAsync(cnt.as<int64_t>() + nt, 0, 8, s));
-  sg_tile_count_kernel<<<unsigned(nt), kSgThreads, 0, s>>>(g->d, head, tail, kb, cnt.as<int64_t>());
+  sg_tile_count_kernel<<<unsigned(nt), kSgThreads, 0, s>>>(g->d, ends, kb, cnt.as<int64_t>());
   GT_LAUNCH_CHECK();
   exclusive_scan_i64(cnt.as<int64_t>(), off, nt + 1, sc.p, s);
   cudaEvent_t ev;
@@ -1092,10 +1090,10 @@ gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s) {
   rb.field_dyn("count", ocnt, len);
   if (U == 0 || d.G == 0) return rb.finish();
 
-  Buf head(ctx, size_t(d.R) * 8, s), tail(ctx, size_t(d.R) * 8, s), wt(ctx, size_t(d.R) * 8, s);
+  Buf ends(ctx, size_t(d.R) * 16, s), wt(ctx, size_t(d.R) * 8, s);
   {
     Phase ph(ctx, "seq_headtail", s);
-    run_head_tail(g, head.as<int32_t>(), tail.as<int32_t>(), s, true);
+    run_rule_ends(g, ends.as<int4>(), s, true);
     run_rule_weights(g, wt.as<uint64_t>(), s);
   }
   const int nb = int(std::min<int64_t>(kMaxCoarse, std::max<int64_t>(1, (U + kCoarseRows - 1) / kCoarseRows)));
@@ -1119,11 +1117,11 @@ gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s) {
   auto* ticket = flags + fmax;
   auto* ftot = reinterpret_cast<int64_t*>(flags + fmax + 1);
   GT_CUDA(cudaMemsetAsync(lb.p, 0, size_t(fmax + 2) * 8, s));
-  SgArgs a{d, head.as<int32_t>(), tail.as<int32_t>(), wt.as<uint64_t>(), spl.as<uint64_t>(), lut.as<uint16_t>(),
+  SgArgs a{d, ends.as<int4>(), wt.as<uint64_t>(), spl.as<uint64_t>(), lut.as<uint16_t>(),
            nullptr, kb, nb - 1, lut_bits, 3 * kb - lut_bits};
   {
     Phase ph(ctx, "seq_part", s);
-    a.tile_off = seq_tile_offsets(g, head.as<int32_t>(), tail.as<int32_t>(), kb, s);
+    a.tile_off = seq_tile_offsets(g, ends.as<int4>(), kb, s);
     if (nb > 1) {
       const int smem = kSampKeys * 8;
       GT_CUDA(cudaFuncSetAttribute(sg_bounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

@@ -461,10 +461,10 @@ __device__ __forceinline__ RuleEnds rule_ends(const DevGrammar& d, int32_t r) {
   return e;
 }
 
-__device__ __forceinline__ void head_tail_of(const DevGrammar& d, int32_t r, const RuleEnds& e, int32_t* head,
-                                             int32_t* tail) {
-  int2* const heads = reinterpret_cast<int2*>(head);
-  int2* const tails = reinterpret_cast<int2*>(tail);
+// ends[r] = first two and last two words of rule r's expansion (-1 pads one
+// word): the head and the tail buffer side by side, so that a reference costs
+// one 16-byte lookup instead of two of 8.
+__device__ __forceinline__ void ends_of(const DevGrammar& d, int32_t r, const RuleEnds& e, int4* ends) {
   int32_t h[2] = {-1, -1};
   int n = 0;
   for (int64_t i = e.lo; i < e.hi && n < 2; ++i) {
@@ -472,7 +472,7 @@ __device__ __forceinline__ void head_tail_of(const DevGrammar& d, int32_t r, con
     if (s < d.V) {
       h[n++] = s;
     } else {
-      const int2 c = __ldcg(&heads[s - d.V]);
+      const int4 c = __ldcg(&ends[s - d.V]);
       h[n++] = c.x;
       if (n < 2 && c.y >= 0) h[n++] = c.y;
     }
@@ -484,26 +484,25 @@ __device__ __forceinline__ void head_tail_of(const DevGrammar& d, int32_t r, con
     if (s < d.V) {
       t[1 - m++] = s;
     } else {
-      const int2 c = __ldcg(&tails[s - d.V]);
-      t[1 - m++] = c.y;
-      if (m < 2 && c.x >= 0) t[1 - m++] = c.x;
+      const int4 c = __ldcg(&ends[s - d.V]);
+      t[1 - m++] = c.w;
+      if (m < 2 && c.z >= 0) t[1 - m++] = c.z;
     }
   }
-  heads[r] = make_int2(h[0], h[1]);
-  tails[r] = make_int2(t[0], t[1]);
+  ends[r] = make_int4(h[0], h[1], t[0], t[1]);
 }
 
 __global__ void head_tail_level_kernel(const int32_t* __restrict__ order, int64_t a, int64_t b, DevGrammar d,
-                                       int32_t* head, int32_t* tail) {
+                                       int4* ends) {
   for (int64_t k = a + blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < b; k += int64_t(gridDim.x) * blockDim.x) {
     const int32_t r = order[k];
-    head_tail_of(d, r, rule_ends(d, r), head, tail);
+    ends_of(d, r, rule_ends(d, r), ends);
   }
 }
 
 // The small levels [l0, d.depth) in one cluster, deepest first (see kTailItems).
 __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
-    head_tail_deep_kernel(DevGrammar d, int l0, int32_t* head, int32_t* tail) {
+    head_tail_deep_kernel(DevGrammar d, int l0, int4* ends) {
   const int64_t me = int64_t(blockIdx.x) * kTailThreads + threadIdx.x;
   constexpr int64_t kStride = int64_t(kTailCtas) * kTailThreads;
   for (int lv = d.depth - 1; lv >= l0; --lv) {
@@ -519,7 +518,18 @@ __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads
     if (lv < d.depth - 1) cluster_sync();  // the children's buffers are final
 #pragma unroll
     for (int q = 0; q < 2; ++q)
-      if (r[q] >= 0) head_tail_of(d, r[q], e[q], head, tail);
+      if (r[q] >= 0) ends_of(d, r[q], e[q], ends);
+  }
+}
+
+__global__ void split_ends_kernel(const int4* __restrict__ ends, int32_t R, int32_t* __restrict__ head,
+                                  int32_t* __restrict__ tail) {
+  for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < R; r += int64_t(gridDim.x) * blockDim.x) {
+    const int4 e = ends[r];
+    head[2 * r] = e.x;
+    head[2 * r + 1] = e.y;
+    tail[2 * r] = e.z;
+    tail[2 * r + 1] = e.w;
   }
 }
 
@@ -708,32 +718,31 @@ void run_word_count_multi(gt_grammar* const* gs, uint64_t* const* counts, int n,
   }
 }
 
-void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s, bool children_only) {
+void run_rule_ends(gt_grammar* g, int4* ends, cudaStream_t s, bool children_only) {
   const DevGrammar& d = g->d;
   const int threads = 256;
   const int cap = g->ctx->num_sms * 8;
   const int top = children_only ? 1 : 0;
-  // pairs are read and written 8 bytes at a time: a caller's buffers may be less aligned
-  const bool aligned = ((reinterpret_cast<uintptr_t>(d_head) | reinterpret_cast<uintptr_t>(d_tail)) & 7) == 0;
-  if (!aligned) {
-    Buf h(g->ctx, size_t(d.R) * 8, s), t(g->ctx, size_t(d.R) * 8, s);
-    run_head_tail(g, h.as<int32_t>(), t.as<int32_t>(), s, children_only);
-    GT_CUDA(cudaMemcpyAsync(d_head, h.p, size_t(d.R) * 8, cudaMemcpyDeviceToDevice, s));
-    GT_CUDA(cudaMemcpyAsync(d_tail, t.p, size_t(d.R) * 8, cudaMemcpyDeviceToDevice, s));
-    return;
-  }
   const int deep = small_levels(g->lvl_off, top, d.depth);
   if (deep < d.depth) {
-    head_tail_deep_kernel<<<kTailCtas, kTailThreads, 0, s>>>(d, deep, d_head, d_tail);
+    head_tail_deep_kernel<<<kTailCtas, kTailThreads, 0, s>>>(d, deep, ends);
     GT_LAUNCH_CHECK();
   }
   for (int lv = deep - 1; lv >= top; --lv) {
     const int64_t a = g->lvl_off[lv], b = g->lvl_off[lv + 1];
     if (b > a) {
-      head_tail_level_kernel<<<grid_for(b - a, threads, cap), threads, 0, s>>>(d.lvl_order, a, b, d, d_head, d_tail);
+      head_tail_level_kernel<<<grid_for(b - a, threads, cap), threads, 0, s>>>(d.lvl_order, a, b, d, ends);
       GT_LAUNCH_CHECK();
     }
   }
+}
+
+void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t s) {
+  const int32_t R = g->d.R;
+  Buf ends(g->ctx, size_t(R) * 16, s);
+  run_rule_ends(g, ends.as<int4>(), s, false);
+  split_ends_kernel<<<grid_for(R, 256, g->ctx->num_sms * 8), 256, 0, s>>>(ends.as<int4>(), R, d_head, d_tail);
+  GT_LAUNCH_CHECK();
 }
 
 }  // namespace gt

@@ -159,3 +159,4 @@ def test_levels(ctx, wide):
         check(gh, g)
     finally:
         B.gt_free_grammar(gh)
+
