@@ -737,38 +737,321 @@ void bu_local_window_rows(gt_grammar* g, int kb, cudaStream_t s, Windows& out) {
 // Per-file window rows: windows owned by the root in each file, plus every
 // window inside each (file, root child) expansion, weighted by multiplicity.
 void bu_window_rows(gt_grammar* g, Buf& ends, int kb, cudaStream_t s, Windows& out) {
-  gt_ctx* ctx = g->ctx;
-  const DevGrammar& d = g->d;
-  const int threads = 256, cap = ctx->num_sms * 16;
-  if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
+  if (g->d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
   if (g->max_file_len <= kLocalMax && gparam(g, "bu_local", 1)) {
     bu_local_window_rows(g, kb, s, out);
     return;
   }
   FileRowBufs rows;
-  {
-    Phase ph(ctx, "bu_rows", s);
-    const FileRows fr = rows.make(ctx, kb, d.F, 2 * d.root_len + g->bu_windows, s);
-    Buf ecnt(ctx, size_t(d.ER) * 8, s), epos(ctx, size_t(d.ER) * 8, s), sc(ctx, scan_scratch_bytes(d.ER), s);
-    Buf first(ctx, 8, s);
-    if (d.root_len > 0) {
-      root_window_rows_kernel<<<unsigned((d.root_len + kTile - 1) / kTile), kRootWinThreads, 0, s>>>(
-          d, ends.as<int4>(), kb, fr);
+  const FileRows fr = rows.make(g->ctx, kb, g->d.F, bu_row_bound(g), s);
+  bu_emit_windows(g, ends, kb, fr, s);
+  sort_file_rows(g->ctx, rows, kb, g->d.F, s, out);
+}
+
+int64_t bu_row_bound(const gt_grammar* g) { return 2 * g->d.root_len + g->bu_windows; }
+
+void bu_emit_windows(gt_grammar* g, Buf& ends, int kb, const FileRows& fr, cudaStream_t s) {
+  gt_ctx* ctx = g->ctx;
+  const DevGrammar& d = g->d;
+  const int threads = 256, cap = ctx->num_sms * 16;
+  if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
+  Phase ph(ctx, "bu_rows", s);
+  Buf ecnt(ctx, size_t(d.ER) * 8, s), epos(ctx, size_t(d.ER) * 8, s), sc(ctx, scan_scratch_bytes(d.ER), s);
+  Buf first(ctx, 8, s);
+  if (d.root_len > 0) {
+    root_window_rows_kernel<<<unsigned((d.root_len + kTile - 1) / kTile), kRootWinThreads, 0, s>>>(d, ends.as<int4>(),
+                                                                                                  kb, fr);
+    GT_LAUNCH_CHECK();
+  }
+  if (d.ER > 0) {
+    redge_len_kernel<<<grid_for(d.ER, threads, cap), threads, 0, s>>>(d, true, ecnt.as<int64_t>());
+    GT_LAUNCH_CHECK();
+    exclusive_scan_i64(ecnt.as<int64_t>(), epos.as<int64_t>(), d.ER, sc.p, s);
+    GT_CUDA(cudaMemcpyAsync(first.p, fr.n, 8, cudaMemcpyDeviceToDevice, s));
+    child_window_rows_kernel<<<grid_for(d.ER, 128, cap), 128, 0, s>>>(d, kb, epos.as<int64_t>(),
+                                                                     first.as<unsigned long long>(), fr);
+    GT_LAUNCH_CHECK();
+    add_rows_kernel<<<1, 1, 0, s>>>(first.as<unsigned long long>(), g->bu_windows, fr.n);
+    GT_LAUNCH_CHECK();
+  }
+}
+
+namespace {
+
+// ---- the files' words, expanded --------------------------------------------------
+
+// words[0, N): the expansion of the root, files back to back.  A tile of kRowTile
+// root symbols per CTA in ticket order, kRowItems consecutive ones per thread; a
+// tile's first word comes from a bounded look-back over the tiles' lengths.
+__global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGrammar d, int64_t tiles,
+                                                                  unsigned long long* __restrict__ look,
+                                                                  int32_t* __restrict__ words,
+                                                                  unsigned* __restrict__ status) {
+  __shared__ int64_t s_warp[kRowThreads / 32];
+  __shared__ int64_t s_item, s_prefix;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_item = int64_t(atomicAdd(look + tiles, 1ull));
+  __syncthreads();
+  const int64_t item = s_item, j0 = item * kRowTile + tid * kRowItems;
+  int32_t sy[kRowItems];
+  int64_t len = 0, ln[kRowItems];
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) sy[k] = j0 + k < d.root_len ? d.sym[j0 + k] : -1;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    ln[k] = sy[k] < 0 ? 0 : (sy[k] < d.V ? 1 : int64_t(d.exp_len[sy[k] - d.V]));
+    len += ln[k];
+  }
+  int64_t incl = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  int64_t before = incl - len, total = 0;
+#pragma unroll
+  for (int w = 0; w < kRowThreads / 32; ++w) {
+    before += w < warp ? s_warp[w] : 0;
+    total += s_warp[w];
+  }
+  if (warp == 0) {
+    if (lane == 0) publish_aggregate(look, item, uint64_t(total));
+    __syncwarp();
+    const int64_t p = warp_look_back(look, item, uint64_t(total), status);
+    if (lane == 0) s_prefix = p < 0 ? 0 : p;
+  }
+  __syncthreads();
+  int64_t o = s_prefix + before;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    if (sy[k] < 0) continue;
+    if (sy[k] < d.V) {
+      words[o] = sy[k];
+    } else {
+      int64_t q = o;
+      walk_rule(d, sy[k] - d.V, [&](int32_t w) { words[q++] = w; });
+    }
+    o += ln[k];
+  }
+}
+
+// cnt[f] = windows of file f, len[f] = its words (0 for f = F)
+__global__ void file_windows_kernel(const uint64_t* __restrict__ file_len, int32_t F, int64_t* __restrict__ len,
+                                    int64_t* __restrict__ cnt) {
+  for (int32_t f = blockIdx.x * blockDim.x + threadIdx.x; f <= F; f += gridDim.x * blockDim.x) {
+    const int64_t l = f < F ? int64_t(file_len[f]) : 0;
+    len[f] = l;
+    cnt[f] = l > 2 ? l - 2 : 0;
+  }
+}
+
+// One row per window, in text order: key and file.
+__global__ void __launch_bounds__(kRowThreads) token_windows_kernel(const int32_t* __restrict__ words, int64_t N,
+                                                                    const int64_t* __restrict__ first, int32_t F,
+                                                                    const int64_t* __restrict__ row, int kb,
+                                                                    uint64_t* __restrict__ keys,
+                                                                    uint32_t* __restrict__ files) {
+  __shared__ int32_t s_file[2];
+  const int64_t p0 = int64_t(blockIdx.x) * kRowTile, p1 = min(N, p0 + kRowTile);
+  if (threadIdx.x < 2) s_file[threadIdx.x] = int32_t(upper_bound_dev(first, int64_t(F) + 1, threadIdx.x ? p1 - 1 : p0) - 1);
+  __syncthreads();
+  const int32_t f_lo = s_file[0], f_hi = s_file[1];
+#pragma unroll 4
+  for (int k = 0; k < kRowItems; ++k) {
+    const int64_t p = p0 + k * kRowThreads + threadIdx.x;
+    if (p >= p1) continue;
+    int32_t lo = f_lo, hi = f_hi;  // last file that starts at or before p
+    while (lo < hi) {
+      const int32_t mid = (lo + hi + 1) >> 1;
+      if (first[mid] <= p) lo = mid;
+      else hi = mid - 1;
+    }
+    if (p + 2 >= first[lo + 1]) continue;
+    const int64_t o = row[lo] + (p - first[lo]);
+    keys[o] = pack_compact(words[p], words[p + 1], words[p + 2], kb);
+    files[o] = uint32_t(lo);
+  }
+}
+
+// ---- rank order inside the runs of a key --------------------------------------------
+
+constexpr int kRankThread = 8;    // rows of a run put in order by one thread
+constexpr int kRankWarp = 256;    // by one warp; longer runs by a CTA
+
+// Files of a key: count descending, file ascending.  Most keys have one file.
+__global__ void rank_short_kernel(const int64_t* __restrict__ off, const int64_t* __restrict__ nkeys,
+                                  const int32_t* __restrict__ file, const uint64_t* __restrict__ cnt,
+                                  int32_t* __restrict__ ofile, uint64_t* __restrict__ ocnt,
+                                  unsigned long long* __restrict__ nlist, int64_t* __restrict__ mid,
+                                  int64_t* __restrict__ lng) {
+  const int64_t n = *nkeys;
+  for (int64_t u = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; u < n; u += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t s = off[u], len = off[u + 1] - s;
+    if (len == 1) {
+      ofile[s] = file[s];
+      ocnt[s] = cnt[s];
+    } else if (len <= kRankThread) {
+      for (int a = 0; a < int(len); ++a) {
+        const uint64_t c = cnt[s + a];
+        int r = 0;
+        for (int b = 0; b < int(len); ++b) {
+          const uint64_t x = cnt[s + b];
+          r += x > c || (x == c && b < a);
+        }
+        ofile[s + r] = file[s + a];
+        ocnt[s + r] = c;
+      }
+    } else if (len <= kRankWarp) {
+      mid[atomicAdd(&nlist[0], 1ull)] = u;
+    } else {
+      lng[atomicAdd(&nlist[1], 1ull)] = u;
+    }
+  }
+}
+
+__global__ void rank_mid_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ file,
+                                const uint64_t* __restrict__ cnt, int32_t* __restrict__ ofile,
+                                uint64_t* __restrict__ ocnt, const unsigned long long* __restrict__ nlist,
+                                const int64_t* __restrict__ mid) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = int64_t(nlist[0]), warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+  for (int64_t q = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; q < n; q += warps) {
+    const int64_t s = off[mid[q]];
+    const int len = int(off[mid[q] + 1] - s);
+    for (int a = lane; a < len; a += 32) {
+      const uint64_t c = cnt[s + a];
+      int r = 0;
+      for (int b = 0; b < len; ++b) {  // one address per step: a broadcast
+        const uint64_t x = cnt[s + b];
+        r += x > c || (x == c && b < a);
+      }
+      ofile[s + r] = file[s + a];
+      ocnt[s + r] = c;
+    }
+  }
+}
+
+// Runs of up to kMaxRankFiles rows: a stable sort in shared memory by max_count -
+// count, the row's place above it.
+__global__ void __launch_bounds__(kLocalThreads) rank_long_kernel(
+    const int64_t* __restrict__ off, const int32_t* __restrict__ file, const uint64_t* __restrict__ cnt,
+    uint64_t max_count, int cbits, int cap, int32_t* __restrict__ ofile, uint64_t* __restrict__ ocnt,
+    const unsigned long long* __restrict__ nlist, const int64_t* __restrict__ lng) {
+  extern __shared__ __align__(16) uint32_t lsm[];
+  uint64_t* ka = reinterpret_cast<uint64_t*>(lsm);
+  uint64_t* kz = ka + cap;
+  __shared__ uint32_t wcnt[kLocalWarps][256];
+  __shared__ uint32_t dstart[256];
+  __shared__ uint32_t dtot[kLocalWarps];
+  const int64_t n = int64_t(nlist[1]);
+  for (int64_t q = blockIdx.x; q < n; q += gridDim.x) {
+    const int64_t s = off[lng[q]];
+    const int len = int(off[lng[q] + 1] - s);
+    for (int i = threadIdx.x; i < len; i += kLocalThreads)
+      ka[i] = (uint64_t(i) << cbits) | (max_count - cnt[s + i]);
+    __syncthreads();
+    const uint64_t* r = local_sort(ka, kz, len, cbits, wcnt, dstart, dtot);
+    for (int i = threadIdx.x; i < len; i += kLocalThreads) {
+      ofile[s + i] = file[s + int64_t(r[i] >> cbits)];
+      ocnt[s + i] = max_count - (r[i] & ((uint64_t(1) << cbits) - 1));
+    }
+    __syncthreads();
+  }
+}
+
+}  // namespace
+
+void bu_token_windows(gt_grammar* g, int kb, Buf& keys, Buf& files, Buf& n, cudaStream_t s) {
+  gt_ctx* ctx = g->ctx;
+  const DevGrammar& d = g->d;
+  if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
+  Phase ph(ctx, "bu_rows", s);
+  const int64_t N = int64_t(d.N), tiles = (d.root_len + kRowTile - 1) / kRowTile;
+  keys = Buf(ctx, size_t(N) * 8, s);
+  files = Buf(ctx, size_t(N) * 4, s);
+  n = Buf(ctx, 8, s);
+  Buf words(ctx, size_t(N) * 4, s), look(ctx, size_t(tiles + 1) * 8, s);
+  Buf len(ctx, size_t(d.F + 1) * 8, s), cnt(ctx, size_t(d.F + 1) * 8, s), first(ctx, size_t(d.F + 1) * 8, s);
+  Buf row(ctx, size_t(d.F + 1) * 8, s), sc(ctx, scan_scratch_bytes(d.F + 1), s);
+  file_windows_kernel<<<grid_for(int64_t(d.F) + 1, 256, ctx->num_sms * 8), 256, 0, s>>>(d.file_len, d.F,
+                                                                                     len.as<int64_t>(),
+                                                                                     cnt.as<int64_t>());
+  GT_LAUNCH_CHECK();
+  exclusive_scan_i64(len.as<int64_t>(), first.as<int64_t>(), d.F + 1, sc.p, s);
+  exclusive_scan_i64(cnt.as<int64_t>(), row.as<int64_t>(), d.F + 1, sc.p, s);
+  GT_CUDA(cudaMemcpyAsync(n.p, row.as<int64_t>() + d.F, 8, cudaMemcpyDeviceToDevice, s));
+  if (tiles == 0) return;
+  GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(tiles + 1) * 8, s));
+  expand_root_kernel<<<unsigned(tiles), kRowThreads, 0, s>>>(d, tiles, look.as<unsigned long long>(),
+                                                             words.as<int32_t>(), status_word());
+  GT_LAUNCH_CHECK();
+  token_windows_kernel<<<unsigned((N + kRowTile - 1) / kRowTile), kRowThreads, 0, s>>>(
+      words.as<int32_t>(), N, first.as<int64_t>(), d.F, row.as<int64_t>(), kb, keys.as<uint64_t>(),
+      files.as<uint32_t>());
+  GT_LAUNCH_CHECK();
+}
+
+gt_result* ranked_from_key_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
+                                int kb, int32_t F, uint64_t max_count, cudaStream_t s, const uint32_t* status_in) {
+  const int threads = 256, cap = ctx->num_sms * 16;
+  ResultBuilder rb(ctx, s);
+  GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
+  StatusScope scope(rb.status());
+  Phase ph(ctx, "ranked", s);
+  auto* off = static_cast<int64_t*>(rb.alloc(size_t(bound + 1) * 8));
+  auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));
+  auto* ofile = static_cast<int32_t*>(rb.alloc(size_t(bound) * 4));
+  auto* ocnt = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));
+  int64_t* len_off = rb.new_len_slot();
+  int64_t* len_key = rb.new_len_slot();
+  int64_t* len_row = rb.new_len_slot();
+  if (bound == 0) {
+    GT_CUDA(cudaMemsetAsync(off, 0, 8, s));
+    const int64_t one = 1;
+    GT_CUDA(cudaMemcpyAsync(len_off, &one, 8, cudaMemcpyHostToDevice, s));
+  } else {
+    if (max_count >= (uint64_t(1) << 31)) fail(GT_EOVERFLOW, "ranked index counts need files below 2^31 tokens");
+    GT_CUDA(cudaMemcpyAsync(len_row, n_dev, 8, cudaMemcpyDeviceToDevice, s));
+    RunOut o;
+    o.key = okey;
+    o.kb = kb;
+    o.off = off;
+    o.off_end = n_dev;
+    o.rows = len_key;
+    o.rows1 = len_off;
+    reduce_runs(ctx, rkey.as<uint64_t>(), nullptr, nullptr, bound, n_dev, ~uint64_t(0), o, s);
+    const int64_t nm = bound / (kRankThread + 1) + 1, nl = bound / (kRankWarp + 1) + 1;
+    Buf nlist(ctx, 16, s), mid(ctx, size_t(nm) * 8, s), lng(ctx, size_t(nl) * 8, s);
+    GT_CUDA(cudaMemsetAsync(nlist.p, 0, 16, s));
+    rank_short_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(
+        off, len_key, rfile.as<int32_t>(), rcnt.as<uint64_t>(), ofile, ocnt, nlist.as<unsigned long long>(),
+        mid.as<int64_t>(), lng.as<int64_t>());
+    GT_LAUNCH_CHECK();
+    if (F > kRankThread) {
+      rank_mid_kernel<<<grid_for(nm * 32, threads, ctx->num_sms * 8), threads, 0, s>>>(
+          off, rfile.as<int32_t>(), rcnt.as<uint64_t>(), ofile, ocnt, nlist.as<unsigned long long>(),
+          mid.as<int64_t>());
       GT_LAUNCH_CHECK();
     }
-    if (d.ER > 0) {
-      redge_len_kernel<<<grid_for(d.ER, threads, cap), threads, 0, s>>>(d, true, ecnt.as<int64_t>());
-      GT_LAUNCH_CHECK();
-      exclusive_scan_i64(ecnt.as<int64_t>(), epos.as<int64_t>(), d.ER, sc.p, s);
-      GT_CUDA(cudaMemcpyAsync(first.p, rows.n.p, 8, cudaMemcpyDeviceToDevice, s));
-      child_window_rows_kernel<<<grid_for(d.ER, 128, cap), 128, 0, s>>>(d, kb, epos.as<int64_t>(),
-                                                                       first.as<unsigned long long>(), fr);
-      GT_LAUNCH_CHECK();
-      add_rows_kernel<<<1, 1, 0, s>>>(first.as<unsigned long long>(), g->bu_windows, rows.n.as<unsigned long long>());
+    if (F > kRankWarp) {
+      int cbits = 1;
+      while ((uint64_t(1) << cbits) <= max_count) ++cbits;
+      const int room = (F + 255) / 256 * 256;  // a key's files
+      const size_t smem = size_t(room) * 16;
+      GT_CUDA(cudaFuncSetAttribute(rank_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+      rank_long_kernel<<<unsigned(std::min<int64_t>(nl, 2 * ctx->num_sms)), kLocalThreads, smem, s>>>(
+          off, rfile.as<int32_t>(), rcnt.as<uint64_t>(), max_count, cbits, room, ofile, ocnt,
+          nlist.as<unsigned long long>(), lng.as<int64_t>());
       GT_LAUNCH_CHECK();
     }
   }
-  sort_file_rows(ctx, rows, kb, d.F, s, out);
+  rb.field_dyn("offsets", off, len_off);
+  rb.field_dyn("key", okey, len_key);
+  rb.field_dyn("file", ofile, len_row);
+  rb.field_dyn("count", ocnt, len_row);
+  return rb.finish();
 }
 
 }  // namespace gt

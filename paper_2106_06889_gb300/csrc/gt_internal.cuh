@@ -461,13 +461,14 @@ int file_strategy(const gt_grammar* g);
 // sort_file_rows for the two layouts); kernels claim places in *n.
 struct FileRows {
   uint64_t* key;
-  uint32_t* val;  // file << shift | key, weight here
+  uint32_t* val;  // file << shift | key << key_shift, weight here
   uint64_t* pay;  // or: key, file << 32 | weight here
   unsigned long long* n;
   int shift;
+  int key_shift = 0;
   __device__ __forceinline__ void put(int64_t o, int32_t f, uint64_t k, uint32_t w) const {
     if (val) {
-      key[o] = (uint64_t(uint32_t(f)) << shift) | k;
+      key[o] = (uint64_t(uint32_t(f)) << shift) | (k << key_shift);
       val[o] = w;
     } else {
       key[o] = k;
@@ -482,6 +483,16 @@ struct FileRowBufs {
   FileRows make(gt_ctx* ctx, int kb, int32_t F, int64_t bound, cudaStream_t s);
 };
 void sort_file_rows(gt_ctx* ctx, FileRowBufs& r, int kb, int32_t F, cudaStream_t s, Windows& out);
+// gt_bu.cu: the per-file window rows, bottom-up, in any order; and one row (key,
+// file) per window of the expanded files, in file order, *n of them
+int64_t bu_row_bound(const gt_grammar* g);
+void bu_emit_windows(gt_grammar* g, Buf& ends, int kb, const FileRows& fr, cudaStream_t s);
+void bu_token_windows(gt_grammar* g, int kb, Buf& keys, Buf& files, Buf& n, cudaStream_t s);
+// Ranked index from rows (key, file, count) in (key, file) order: only the files
+// of each key still have to be put in rank order.  For at most kMaxRankFiles files.
+constexpr int32_t kMaxRankFiles = 8192;
+gt_result* ranked_from_key_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
+                                int kb, int32_t F, uint64_t max_count, cudaStream_t s, const uint32_t* status_in);
 
 // gt_bu.cu: bottom-up per-file rows
 void bu_window_rows(gt_grammar* g, Buf& ends, int kb, cudaStream_t s, Windows& out);
@@ -568,6 +579,7 @@ gt_result* run_inverted_index(gt_grammar* g, cudaStream_t s);
 struct RunOut {
   int low_bits = 0;           // key = file << low_bits | rest (0: no file in the key)
   uint64_t* key = nullptr;    // the key (its rest), kb bits per word spread to 21-bit fields (kb 0: as it is)
+  uint64_t* hi = nullptr;     // the key above low_bits
   int kb = 0;
   int32_t* word = nullptr;    // the key's rest as int32
   int32_t* file = nullptr;    // the run's file: the key's high part, or its fkeys value
@@ -580,6 +592,9 @@ struct RunOut {
 };
 void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
                  const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s);
+// rows (key, file), every one counting 1: runs of equal (key, file)
+void reduce_file_runs(gt_ctx* ctx, const uint64_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,
+                      const RunOut& out, cudaStream_t s);
 
 // gt_sort.cu: device primitives
 size_t scan_scratch_bytes(int64_t n);

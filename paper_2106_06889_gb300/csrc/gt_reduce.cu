@@ -11,7 +11,7 @@
 // publishes that second word as final at once, so the look-back normally ends
 // at the preceding tile, whatever the length of a run.
 //
-// fkeys holds (file << 32 | value) per row: rows are equal if key and file are.
+// fkeys holds (file << 32 | value) per row, or vals the file: rows are equal if key and file are.
 //
 // Bound by HBM: 12 bytes read per row and 16 written per run.  The former form
 // (count heads, scan, write; each head's sum by walking its run) read the rows
@@ -31,11 +31,15 @@ __device__ __forceinline__ bool run_head(uint64_t k, uint64_t prev, uint32_t f, 
   return k != prev || (kFile && f != prev_f);
 }
 
-template <bool kFile, bool kVals>
+// What a row carries beside its key.
+enum RunRows { kKeyVal, kKeyOnly, kKeyFileVal, kKeyFile };
+
+template <RunRows kRows>
 __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     const uint64_t* __restrict__ keys, const uint64_t* __restrict__ fkeys, const uint32_t* __restrict__ vals,
     int64_t n_max, const int64_t* __restrict__ n_dev, uint64_t key_pad, const __grid_constant__ RunOut out,
     unsigned long long* __restrict__ look, int64_t tiles_max, unsigned* __restrict__ status) {
+  constexpr bool kFile = kRows == kKeyFileVal || kRows == kKeyFile, kVals = kRows == kKeyVal;
   __shared__ uint64_t s_key[kRunTile];
   __shared__ uint64_t s_before[kRunTile];  // values of the tile before each head
   __shared__ uint32_t s_file[kFile ? kRunTile : 1];
@@ -70,7 +74,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
       k[2 * j] = x.x;
       k[2 * j + 1] = x.y;
     }
-    if (kVals && !kFile) {
+    if (kVals) {
       const uint4* vp = reinterpret_cast<const uint4*>(vals + i0);
 #pragma unroll
       for (int j = 0; j < kRunItems / 4; ++j) {
@@ -81,7 +85,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
         v[4 * j + 3] = x.w;
       }
     }
-    if (kFile) {
+    if (kRows == kKeyFileVal) {
 #pragma unroll
       for (int j = 0; j < kRunItems; ++j) {
         const uint64_t x = fkeys[i0 + j];
@@ -89,17 +93,22 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
         v[j] = uint32_t(x);
       }
     }
+    if (kRows == kKeyFile) {
+#pragma unroll
+      for (int j = 0; j < kRunItems; ++j) f[j] = vals[i0 + j];
+    }
   } else {
 #pragma unroll
     for (int j = 0; j < kRunItems; ++j) {
       const bool in = i0 + j < n;
       k[j] = in ? keys[i0 + j] : key_pad;
-      if (kVals && !kFile) v[j] = in ? vals[i0 + j] : 0u;
-      if (kFile) {
+      if (kVals) v[j] = in ? vals[i0 + j] : 0u;
+      if (kRows == kKeyFileVal) {
         const uint64_t x = in ? fkeys[i0 + j] : 0;
         f[j] = uint32_t(x >> 32);
         v[j] = uint32_t(x);
       }
+      if (kRows == kKeyFile) f[j] = in ? vals[i0 + j] : 0u;
     }
   }
   // the row before this thread's first one
@@ -107,7 +116,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
   uint32_t prev_f = kFile ? __shfl_up_sync(0xffffffffu, f[kFile ? kRunItems - 1 : 0], 1) : 0u;
   if (lane == 0 && i0 > 0 && i0 <= n) {
     prev = keys[i0 - 1];
-    if (kFile) prev_f = uint32_t(fkeys[i0 - 1] >> 32);
+    if (kFile) prev_f = kRows == kKeyFileVal ? uint32_t(fkeys[i0 - 1] >> 32) : vals[i0 - 1];
   }
   uint32_t heads = 0;  // bit j: row j starts a run
   uint64_t sum = 0;
@@ -116,7 +125,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     const bool real = k[j] != key_pad;
     const bool h = real && ((j == 0 && i0 == 0) || run_head<kFile>(k[j], prev, kFile ? f[kFile ? j : 0] : 0u, prev_f));
     heads |= uint32_t(h) << j;
-    if (!kVals) v[j] = 1u;
+    if (kRows == kKeyOnly || kRows == kKeyFile) v[j] = 1u;
     if (!real) v[j] = 0u;
     sum += v[j];
     prev = k[j];
@@ -186,6 +195,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     const uint64_t key = s_key[r];
     const int64_t o = o0 + r;
     if (out.key) out.key[o] = to_output_key(out.low_bits ? key & ((uint64_t(1) << out.low_bits) - 1) : key, out.kb);
+    if (out.hi) out.hi[o] = key >> out.low_bits;
     if (out.file) out.file[o] = kFile ? int32_t(s_file[r]) : int32_t(key >> out.low_bits);
     if (out.word) out.word[o] = int32_t(key & ((uint64_t(1) << out.low_bits) - 1));
     if (out.off) out.off[o] = item * kRunTile + int64_t(s_before[r]);
@@ -207,25 +217,33 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
 
 }  // namespace
 
-void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
+namespace {
+
+template <RunRows kRows>
+void launch_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
                  const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s) {
   const int64_t tiles = n > 0 ? (n + kRunTile - 1) / kRunTile : 1;
   if ((reinterpret_cast<uintptr_t>(keys) & 15) || (reinterpret_cast<uintptr_t>(vals) & 15))
     fail(GT_EINVAL, "rows to reduce must be 16-byte aligned");
   Buf look(ctx, size_t(2 * tiles + 1) * 8, s);
   GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(2 * tiles + 1) * 8, s));
-  auto* lk = look.as<unsigned long long>();
-  const unsigned grid = unsigned(tiles);
-  if (fkeys)
-    reduce_runs_kernel<true, true><<<grid, kRunThreads, 0, s>>>(keys, fkeys, vals, n, n_dev, key_pad, out, lk, tiles,
-                                                                status_word());
-  else if (vals)
-    reduce_runs_kernel<false, true><<<grid, kRunThreads, 0, s>>>(keys, nullptr, vals, n, n_dev, key_pad, out, lk,
-                                                                 tiles, status_word());
-  else
-    reduce_runs_kernel<false, false><<<grid, kRunThreads, 0, s>>>(keys, nullptr, nullptr, n, n_dev, key_pad, out, lk,
-                                                                  tiles, status_word());
+  reduce_runs_kernel<kRows><<<unsigned(tiles), kRunThreads, 0, s>>>(
+      keys, fkeys, vals, n, n_dev, key_pad, out, look.as<unsigned long long>(), tiles, status_word());
   GT_LAUNCH_CHECK();
+}
+
+}  // namespace
+
+void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
+                 const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s) {
+  if (fkeys) launch_runs<kKeyFileVal>(ctx, keys, fkeys, nullptr, n, n_dev, key_pad, out, s);
+  else if (vals) launch_runs<kKeyVal>(ctx, keys, nullptr, vals, n, n_dev, key_pad, out, s);
+  else launch_runs<kKeyOnly>(ctx, keys, nullptr, nullptr, n, n_dev, key_pad, out, s);
+}
+
+void reduce_file_runs(gt_ctx* ctx, const uint64_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,
+                      const RunOut& out, cudaStream_t s) {
+  launch_runs<kKeyFile>(ctx, keys, nullptr, files, n, n_dev, ~uint64_t(0), out, s);
 }
 
 }  // namespace gt

@@ -253,6 +253,20 @@ void sort_file_rows(gt_ctx* ctx, FileRowBufs& r, int kb, int32_t F, cudaStream_t
 
 namespace {
 
+// Per-file window rows, top-down: windows x files of the rule.
+int64_t td_row_bound(const gt_grammar* g) { return 2 * g->d.root_len + 2 * g->fsym_bound; }
+
+void td_emit_windows(gt_grammar* g, Buf& ends, int kb, const FileRows& fr, cudaStream_t s) {
+  const DevGrammar& d = g->d;
+  Phase ph(g->ctx, "seq_emit", s);
+  FileWeights fw;
+  file_weights(g, s, fw);
+  if (d.ntiles == 0) return;
+  win_emit_file_kernel<<<unsigned(d.ntiles), kWinThreads, 0, s>>>(d, ends.as<int4>(), fw.mask, fw.off, fw.slot_pair,
+                                                                 fw.w.as<uint32_t>(), kb, fr);
+  GT_LAUNCH_CHECK();
+}
+
 // Device-detected failures go to *status (the result's own status word).
 void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, uint32_t* status,
                     Buf* keep_ends = nullptr) {
@@ -310,20 +324,9 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
     bu_window_rows(g, ends, kb, s, out);
     return;
   }
-  // ---- per file, top-down: windows x files of the rule ----
   FileRowBufs rows;
-  {
-    Phase ph(ctx, "seq_emit", s);
-    FileWeights fw;
-    file_weights(g, s, fw);
-    const FileRows fr = rows.make(ctx, kb, d.F, 2 * d.root_len + 2 * g->fsym_bound, s);
-    if (rows.bound > 0 && d.ntiles > 0) {
-      win_emit_file_kernel<<<unsigned(d.ntiles), kWinThreads, 0, s>>>(d, ends.as<int4>(),
-                                                                     fw.mask, fw.off, fw.slot_pair,
-                                                                     fw.w.as<uint32_t>(), kb, fr);
-      GT_LAUNCH_CHECK();
-    }
-  }
+  const FileRows fr = rows.make(ctx, kb, d.F, td_row_bound(g), s);
+  td_emit_windows(g, ends, kb, fr, s);
   sort_file_rows(ctx, rows, kb, d.F, s, out);
 }
 
@@ -355,6 +358,27 @@ __global__ void rank_keys_kernel(const uint64_t* __restrict__ cnt, const int32_t
   const int64_t n = *n_dev;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     k[i] = ((max_count - cnt[i]) << 32) | uint32_t(file[i]);
+}
+
+// rkey[i] = key << cbits | (max_count - count), in place
+__global__ void rank_key_count_kernel(const uint64_t* __restrict__ cnt, const int64_t* __restrict__ n_dev,
+                                      uint64_t max_count, int cbits, uint64_t* __restrict__ rkey) {
+  const int64_t n = *n_dev;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    rkey[i] = (rkey[i] << cbits) | (max_count - cnt[i]);
+}
+
+// back to the key (in place), the count and the file
+__global__ void rank_split_kernel(uint64_t* __restrict__ rkey, const int32_t* __restrict__ rfile,
+                                  const int64_t* __restrict__ n_dev, uint64_t max_count, int cbits,
+                                  int32_t* __restrict__ file, uint64_t* __restrict__ cnt) {
+  const int64_t n = *n_dev;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    const uint64_t x = rkey[i];
+    cnt[i] = max_count - (x & ((uint64_t(1) << cbits) - 1));
+    rkey[i] = x >> cbits;
+    file[i] = rfile[i];
+  }
 }
 
 __global__ void rank_unpack_kernel(const uint64_t* __restrict__ pay, const int64_t* __restrict__ n_dev,
@@ -394,27 +418,45 @@ gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const
     GT_CUDA(cudaMemcpyAsync(len_off, &one, 8, cudaMemcpyHostToDevice, s));
   } else {
     if (max_count >= (uint64_t(1) << 31)) fail(GT_EOVERFLOW, "ranked index counts need files below 2^31 tokens");
-    // sort 1: stable by count descending, key ((max_count - count) << 32 |
-    // file), payload the row key; sort 2: stable by row key, payload sort 1's key
-    Buf k0(ctx, size_t(bound) * 8, s), k1(ctx, size_t(bound) * 8, s), v1(ctx, size_t(bound) * 8, s);
-    Buf rs(ctx, radix_scratch_bytes(bound, true, 8), s);
-    rank_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(rcnt.as<uint64_t>(), rfile.as<int32_t>(), n_dev,
-                                                                        max_count, k0.as<uint64_t>());
-    GT_LAUNCH_CHECK();
     const int cbits = bits_for(int64_t(max_count));  // max_count < 2^31
-    if (radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), rkey.p, v1.p, 8, bound, 32, 32 + cbits, 32 + cbits,
-                            32 + cbits, rs.p, s, n_dev)) {
-      std::swap(k0, k1);
-      std::swap(rkey, v1);
+    Buf k1(ctx, size_t(bound) * 8, s), rs(ctx, radix_scratch_bytes(bound, true, 8), s);
+    if (key_bits + cbits < 64) {
+      // one sort by (key, max_count - count) carrying the file: stable, so the
+      // files of equal counts stay ascending
+      Buf f1(ctx, size_t(bound) * 4, s);
+      rank_key_count_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(rcnt.as<uint64_t>(), n_dev, max_count,
+                                                                              cbits, rkey.as<uint64_t>());
+      GT_LAUNCH_CHECK();
+      const int bits = key_bits + cbits;
+      if (radix_sort_pingpong(rkey.as<uint64_t>(), k1.as<uint64_t>(), rfile.p, f1.p, 4, bound, 0, bits, bits, bits, rs.p,
+                              s, n_dev)) {
+        std::swap(rkey, k1);
+        std::swap(rfile, f1);
+      }
+      rank_split_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(rkey.as<uint64_t>(), rfile.as<int32_t>(), n_dev,
+                                                                          max_count, cbits, ofile, ocnt);
+      GT_LAUNCH_CHECK();
+    } else {
+      // sort 1: stable by count descending, key ((max_count - count) << 32 |
+      // file), payload the row key; sort 2: stable by row key, payload sort 1's key
+      Buf k0(ctx, size_t(bound) * 8, s), v1(ctx, size_t(bound) * 8, s);
+      rank_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(rcnt.as<uint64_t>(), rfile.as<int32_t>(), n_dev,
+                                                                          max_count, k0.as<uint64_t>());
+      GT_LAUNCH_CHECK();
+      if (radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), rkey.p, v1.p, 8, bound, 32, 32 + cbits, 32 + cbits,
+                              32 + cbits, rs.p, s, n_dev)) {
+        std::swap(k0, k1);
+        std::swap(rkey, v1);
+      }
+      if (radix_sort_pingpong(rkey.as<uint64_t>(), v1.as<uint64_t>(), k0.p, k1.p, 8, bound, 0, key_bits, key_bits,
+                              key_bits, rs.p, s, n_dev)) {
+        std::swap(k0, k1);
+        std::swap(rkey, v1);
+      }
+      rank_unpack_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(k0.as<uint64_t>(), n_dev, max_count, ofile,
+                                                                            ocnt);
+      GT_LAUNCH_CHECK();
     }
-    if (radix_sort_pingpong(rkey.as<uint64_t>(), v1.as<uint64_t>(), k0.p, k1.p, 8, bound, 0, key_bits, key_bits,
-                            key_bits, rs.p, s, n_dev)) {
-      std::swap(k0, k1);
-      std::swap(rkey, v1);
-    }
-    rank_unpack_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(k0.as<uint64_t>(), n_dev, max_count, ofile,
-                                                                          ocnt);
-    GT_LAUNCH_CHECK();
     RunOut o;
     o.key = okey;
     o.kb = windows ? kb : 0;
@@ -461,10 +503,65 @@ gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int kb,
 
 gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
+  const DevGrammar& d = g->d;
   Windows w;
   Buf st(ctx, 4, s);
   GT_CUDA(cudaMemsetAsync(st.p, 0, 4, s));
   StatusScope scope(st.as<uint32_t>());
+  // Rows sorted straight into (key, file) order, when a key has few enough files
+  // to put in rank order afterwards: as one word (key << file bits | file), or,
+  // if that is too wide, from the expanded files, whose windows come in file
+  // order (not if the expansion is far larger than the rows of the root and its
+  // children).  Sorting each file's windows first and then all rows by count and
+  // by key takes two more sorts (8,000 short files: 1.9 against 1.1 ms of kernels).
+  const int fb = bits_for(std::max(d.F - 1, 1)), kb = bits_for(std::max(d.V - 1, 1));
+  const bool bottom_up = file_strategy(g) == 2, one_word = 3 * kb + fb < 64;
+  if (d.F <= kMaxRankFiles && d.V <= (1 << 21) && d.N < (uint64_t(1) << 32) && (bottom_up || one_word) &&
+      (one_word || int64_t(d.N) <= 2 * bu_row_bound(g))) {
+    const int64_t bound = one_word ? (bottom_up ? bu_row_bound(g) : td_row_bound(g)) : int64_t(d.N);
+    Buf rkey(ctx, size_t(bound) * 8, s), rfile(ctx, size_t(bound) * 4, s), rcnt(ctx, size_t(bound) * 8, s);
+    Buf nd(ctx, 8, s);
+    RunOut o;
+    o.count = rcnt.as<uint64_t>();
+    o.rows = nd.as<int64_t>();
+    if (one_word) {
+      Buf ends(ctx, size_t(d.R) * 16, s);
+      {
+        Phase ph(ctx, "seq_headtail", s);
+        run_rule_ends(g, ends.as<int4>(), s, true);
+      }
+      FileRowBufs rows;
+      FileRows fr = rows.make(ctx, kb, d.F, bound, s);
+      fr.shift = 0;
+      fr.key_shift = fb;
+      if (bottom_up) bu_emit_windows(g, ends, kb, fr, s);
+      else td_emit_windows(g, ends, kb, fr, s);
+      if (bound > 0) {
+        Buf k1(ctx, size_t(bound) * 8, s), v1(ctx, size_t(bound) * 4, s), rs(ctx, radix_scratch_bytes(bound, true, 4), s);
+        const bool b = radix_sort_pingpong(rows.keys.as<uint64_t>(), k1.as<uint64_t>(), rows.vals.p, v1.p, 4, bound, 0,
+                                           3 * kb + fb, 3 * kb + fb, 3 * kb + fb, rs.p, s, rows.n.as<int64_t>());
+        o.low_bits = fb;
+        o.hi = rkey.as<uint64_t>();
+        o.word = rfile.as<int32_t>();
+        reduce_runs(ctx, (b ? k1 : rows.keys).as<uint64_t>(), nullptr, (b ? v1 : rows.vals).as<uint32_t>(), bound,
+                    rows.n.as<int64_t>(), ~uint64_t(0), o, s);
+      }
+    } else {
+      Buf keys, files, n;
+      bu_token_windows(g, kb, keys, files, n, s);
+      if (bound > 0) {
+        Buf k1(ctx, size_t(bound) * 8, s), f1(ctx, size_t(bound) * 4, s), rs(ctx, radix_scratch_bytes(bound, true, 4), s);
+        const bool b = radix_sort_pingpong(keys.as<uint64_t>(), k1.as<uint64_t>(), files.p, f1.p, 4, bound, 0, 3 * kb,
+                                           3 * kb, 3 * kb, rs.p, s, n.as<int64_t>());
+        o.key = rkey.as<uint64_t>();
+        o.file = rfile.as<int32_t>();
+        reduce_file_runs(ctx, (b ? k1 : keys).as<uint64_t>(), (b ? f1 : files).as<uint32_t>(), bound, n.as<int64_t>(), o,
+                         s);
+      }
+    }
+    return ranked_from_key_rows(ctx, rkey, rfile, rcnt, nd.as<int64_t>(), bound, kb, d.F, uint64_t(g->max_file_len), s,
+                                st.as<uint32_t>());
+  }
   sorted_windows(g, true, s, w, st.as<uint32_t>());
   if (w.reduced)
     return ranked_from_rows(ctx, w.keys, w.rfile, w.rcnt, w.total.as<int64_t>(), w.n, w.kb, true, 3 * w.kb,

@@ -160,3 +160,24 @@ def test_levels(ctx, wide):
     finally:
         B.gt_free_grammar(gh)
 
+
+@pytest.mark.parametrize("V", [6, 70_000, 200_000])
+@pytest.mark.parametrize("F", [65, 300, 700])
+def test_ranked_runs(ctx, F, V):
+    """Ranked index of many files, keys in 1 to all of them (put in order by a thread, a warp or a
+    CTA): (key, file) in one word for the two smaller vocabularies, by the expanded files otherwise;
+    files of 0 to 2 words among them, repeated passages (rules) in some."""
+    rng = np.random.default_rng(F + V)
+    lens = rng.integers(0, 60, F)
+    lens[:4] = [0, 1, 2, 3]
+    n = int(lens.sum())
+    toks = np.where(rng.random(n) < 0.9, rng.integers(0, 3, n), rng.integers(0, V, n)).astype(np.int32)
+    g = sequitur(toks, lens, V)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        for k in (1, 3):
+            for got, want in zip(take(B.gt_ranked_index(gh, k), "offsets", "key", "file", "count"),
+                                 oracle.ranked_index(g, k)):
+                assert np.array_equal(got, want)
+    finally:
+        B.gt_free_grammar(gh)
