@@ -80,16 +80,16 @@ __global__ void compact_words_kernel(const uint64_t* __restrict__ c, int64_t n, 
 }
 
 // key = N - count: ascending key order is descending count; words with count
-// zero get key N and sort last.
-__global__ void count_keys_kernel(const uint64_t* __restrict__ c, int64_t n, uint64_t N, uint64_t* __restrict__ keys,
+// zero get key N and sort last (N < 2^32: the word count checks it).
+__global__ void count_keys_kernel(const uint64_t* __restrict__ c, int64_t n, uint64_t N, uint32_t* __restrict__ keys,
                                   uint32_t* __restrict__ vals) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    keys[i] = N - c[i];
+    keys[i] = uint32_t(N - c[i]);
     vals[i] = uint32_t(i);
   }
 }
 
-__global__ void count_unkey_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t n,
+__global__ void count_unkey_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t n,
                                    uint64_t N, int32_t* __restrict__ words, uint64_t* __restrict__ counts,
                                    int64_t* __restrict__ total) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
@@ -463,18 +463,16 @@ gt_result* sort_from_counts(gt_grammar* g, const uint64_t* wc, int order, cudaSt
     GT_LAUNCH_CHECK();
   } else {
     const uint64_t N = g->d.N;
-    Buf k0(ctx, size_t(V) * 8, s), k1(ctx, size_t(V) * 8, s), v0(ctx, size_t(V) * 4, s), v1(ctx, size_t(V) * 4, s);
+    Buf k0(ctx, size_t(V) * 4, s), k1(ctx, size_t(V) * 4, s), v0(ctx, size_t(V) * 4, s), v1(ctx, size_t(V) * 4, s);
     Buf rs(ctx, gt::radix_scratch_bytes(V, true, 4), s);
-    count_keys_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(wc, V, N, k0.as<uint64_t>(),
+    count_keys_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(wc, V, N, k0.as<uint32_t>(),
                                                                         v0.as<uint32_t>());
     GT_LAUNCH_CHECK();
-    const int kbits = bits_for(N);
-    if (!gt::radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), v0.p, v1.p, 4, V, 0, kbits, kbits, kbits, rs.p,
-                                 s)) {
+    if (!gt::radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), v0.p, v1.p, 4, V, bits_for(N), rs.p, s)) {
       std::swap(k0, k1);
       std::swap(v0, v1);
     }
-    count_unkey_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(k1.as<uint64_t>(), v1.as<uint32_t>(), V, N,
+    count_unkey_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(k1.as<uint32_t>(), v1.as<uint32_t>(), V, N,
                                                                          words, counts, nlen);
     GT_LAUNCH_CHECK();
   }

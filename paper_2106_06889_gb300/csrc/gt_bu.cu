@@ -529,9 +529,120 @@ __global__ void local_pack_kernel(int32_t F, const int64_t* __restrict__ slot_of
   }
 }
 
-// (file, word, count) rows of every file, sorted by (file, word).
+// ---- the files' words, expanded --------------------------------------------------
+
+// words[0, N): the expansion of the root, files back to back.  A tile of kRowTile
+// root symbols per CTA in ticket order, kRowItems consecutive ones per thread; a
+// tile's first word comes from a bounded look-back over the tiles' lengths.
+__global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGrammar d, int64_t tiles,
+                                                                  unsigned long long* __restrict__ look,
+                                                                  int32_t* __restrict__ words,
+                                                                  unsigned* __restrict__ status) {
+  __shared__ int64_t s_warp[kRowThreads / 32];
+  __shared__ int64_t s_item, s_prefix;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_item = int64_t(atomicAdd(look + tiles, 1ull));
+  __syncthreads();
+  const int64_t item = s_item, j0 = item * kRowTile + tid * kRowItems;
+  int32_t sy[kRowItems];
+  int64_t len = 0, ln[kRowItems];
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) sy[k] = j0 + k < d.root_len ? d.sym[j0 + k] : -1;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    ln[k] = sy[k] < 0 ? 0 : (sy[k] < d.V ? 1 : int64_t(d.exp_len[sy[k] - d.V]));
+    len += ln[k];
+  }
+  int64_t incl = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  int64_t before = incl - len, total = 0;
+#pragma unroll
+  for (int w = 0; w < kRowThreads / 32; ++w) {
+    before += w < warp ? s_warp[w] : 0;
+    total += s_warp[w];
+  }
+  if (warp == 0) {
+    if (lane == 0) publish_aggregate(look, item, uint64_t(total));
+    __syncwarp();
+    const int64_t p = warp_look_back(look, item, uint64_t(total), status);
+    if (lane == 0) s_prefix = p < 0 ? 0 : p;
+  }
+  __syncthreads();
+  int64_t o = s_prefix + before;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    if (sy[k] < 0) continue;
+    if (sy[k] < d.V) {
+      words[o] = sy[k];
+    } else {
+      int64_t q = o;
+      walk_rule(d, sy[k] - d.V, [&](int32_t w) { words[q++] = w; });
+    }
+    o += ln[k];
+  }
+}
+
+// last file f in [lo, hi] whose first word is at or before position p
+__device__ __forceinline__ int32_t file_from(const int64_t* __restrict__ first, int32_t lo, int32_t hi, int64_t p) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (first[mid] <= p) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// cnt[f] = windows of file f (0 for f = F)
+__global__ void file_windows_kernel(const uint64_t* __restrict__ file_len, int32_t F, int64_t* __restrict__ cnt) {
+  for (int32_t f = blockIdx.x * blockDim.x + threadIdx.x; f <= F; f += gridDim.x * blockDim.x)
+    cnt[f] = f < F && file_len[f] > 2 ? int64_t(file_len[f]) - 2 : 0;
+}
+
+// The file of every word.
+__global__ void __launch_bounds__(kRowThreads) token_files_kernel(int64_t N, const int64_t* __restrict__ first, int32_t F,
+                                                                  uint32_t* __restrict__ files) {
+  __shared__ int32_t s_file[2];
+  const int64_t p0 = int64_t(blockIdx.x) * kRowTile, p1 = min(N, p0 + kRowTile);
+  if (threadIdx.x < 2) s_file[threadIdx.x] = int32_t(upper_bound_dev(first, int64_t(F) + 1, threadIdx.x ? p1 - 1 : p0) - 1);
+  __syncthreads();
+  for (int k = 0; k < kRowItems; ++k) {
+    const int64_t p = p0 + k * kRowThreads + threadIdx.x;
+    if (p < p1) files[p] = uint32_t(file_from(first, s_file[0], s_file[1], p));
+  }
+}
+
+// Words of every file back to back, and each file's first word (F + 1 offsets).
+void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s) {
+  gt_ctx* ctx = g->ctx;
+  const DevGrammar& d = g->d;
+  const int64_t tiles = (d.root_len + kRowTile - 1) / kRowTile;
+  words = Buf(ctx, size_t(d.N) * 4, s);
+  first = Buf(ctx, size_t(d.F + 1) * 8, s);
+  Buf look(ctx, size_t(tiles + 1) * 8, s), len(ctx, size_t(d.F + 1) * 8, s), sc(ctx, scan_scratch_bytes(d.F + 1), s);
+  file_len_i64_kernel<<<grid_for(int64_t(d.F) + 1, 256, ctx->num_sms * 8), 256, 0, s>>>(d.file_len, d.F,
+                                                                                     len.as<int64_t>());
+  GT_LAUNCH_CHECK();
+  exclusive_scan_i64(len.as<int64_t>(), first.as<int64_t>(), d.F + 1, sc.p, s);
+  if (tiles == 0) return;
+  GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(tiles + 1) * 8, s));
+  expand_root_kernel<<<unsigned(tiles), kRowThreads, 0, s>>>(d, tiles, look.as<unsigned long long>(),
+                                                             words.as<int32_t>(), status_word());
+  GT_LAUNCH_CHECK();
+}
+
+// One row (file, word, count) per distinct word of every file, *total of them: in
+// (file, word) order, or in (word, file) order (by_word; the counts beside the
+// words in pay, word << 32 | count).
 struct WordRows {
   Buf word, file, cnt, total, status;  // status: flags raised while the rows were made
+  Buf pay;
+  bool by_word = false;
   int64_t bound = 0;
 };
 
@@ -583,6 +694,41 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
     return;
   }
   if (kbw + fb > 63) fail(GT_EOVERFLOW, "too many files x words for 64-bit (file, word) keys");
+  // The expanded files come in file order, so a stable sort by word alone puts
+  // their words in (word, file) order - the inverted index's - on 32-bit keys;
+  // the distinct rows, about a third, then take two short passes to file order.
+  // Rows of (file, word) keys take four passes, and the distinct ones three more
+  // for the index.  Not if the expansion is far larger than the rows of the root
+  // and its children.
+  if (int64_t(d.N) <= 2 * (g->info.root_words + g->bu_words) && d.N < (uint64_t(1) << 30)) {
+    Phase ph(ctx, "bu_rows", s);
+    const int64_t N = int64_t(d.N);
+    out.by_word = true;
+    out.bound = N;
+    out.word = Buf(ctx, size_t(N) * 4, s);
+    out.file = Buf(ctx, size_t(N) * 4, s);
+    out.pay = Buf(ctx, size_t(N) * 8, s);
+    out.total = Buf(ctx, 8, s);
+    if (N == 0) {
+      GT_CUDA(cudaMemsetAsync(out.total.p, 0, 8, s));
+      return;
+    }
+    Buf words, first, files(ctx, size_t(N) * 4, s), w1(ctx, size_t(N) * 4, s), f1(ctx, size_t(N) * 4, s);
+    expand_files(g, words, first, s);
+    token_files_kernel<<<unsigned((N + kRowTile - 1) / kRowTile), kRowThreads, 0, s>>>(N, first.as<int64_t>(), d.F,
+                                                                                      files.as<uint32_t>());
+    GT_LAUNCH_CHECK();
+    Buf rs(ctx, radix_scratch_bytes(N, true, 4), s);
+    const bool b = radix_sort_pingpong32(words.as<uint32_t>(), w1.as<uint32_t>(), files.p, f1.p, 4, N,
+                                         bits_for(std::max(d.V - 1, 1)), rs.p, s);
+    RunOut o;
+    o.word = out.word.as<int32_t>();
+    o.file = out.file.as<int32_t>();
+    o.pay = out.pay.as<uint64_t>();
+    o.rows = out.total.as<int64_t>();
+    reduce_file_runs(ctx, (b ? w1 : words).as<uint32_t>(), (b ? f1 : files).as<uint32_t>(), N, nullptr, o, s);
+    return;
+  }
   const int64_t n = g->info.root_words + g->bu_words;
   Phase ph(ctx, "bu_rows", s);
   Buf k0(ctx, size_t(n) * 8, s), v0(ctx, size_t(n) * 4, s), k1(ctx, size_t(n) * 8, s), v1(ctx, size_t(n) * 4, s);
@@ -625,6 +771,59 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
   reduce_runs(ctx, (b ? k1 : k0).as<uint64_t>(), nullptr, (b ? v1 : v0).as<uint32_t>(), n, nullptr, ~uint64_t(0), o, s);
 }
 
+__global__ void unpack_pay_kernel(const uint64_t* __restrict__ pay, const int64_t* __restrict__ n_dev,
+                                  int32_t* __restrict__ word, uint64_t* __restrict__ cnt) {
+  const int64_t n = *n_dev;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    const uint64_t x = pay[i];
+    if (word) word[i] = int32_t(x >> 32);
+    cnt[i] = x & 0xffffffffu;
+  }
+}
+
+// Rows in (word, file) order to (file, word) order: stable by file.
+void rows_by_file(gt_grammar* g, WordRows& wr, cudaStream_t s) {
+  if (!wr.by_word) return;
+  gt_ctx* ctx = g->ctx;
+  StatusScope scope(wr.status.as<uint32_t>());
+  const int64_t n = wr.bound;
+  const int64_t* nd = wr.total.as<int64_t>();
+  wr.by_word = false;
+  wr.cnt = Buf(ctx, size_t(n) * 8, s);
+  if (n == 0) return;
+  Buf f1(ctx, size_t(n) * 4, s), p1(ctx, size_t(n) * 8, s), rs(ctx, radix_scratch_bytes(n, true, 8), s);
+  if (radix_sort_pingpong32(wr.file.as<uint32_t>(), f1.as<uint32_t>(), wr.pay.p, p1.p, 8, n,
+                            bits_for(std::max(g->d.F - 1, 1)), rs.p, s, nd)) {
+    std::swap(wr.file, f1);
+    std::swap(wr.pay, p1);
+  }
+  unpack_pay_kernel<<<grid_for(n, 256, ctx->num_sms * 16), 256, 0, s>>>(wr.pay.as<uint64_t>(), nd,
+                                                                       wr.word.as<int32_t>(), wr.cnt.as<uint64_t>());
+  GT_LAUNCH_CHECK();
+}
+
+__global__ void copy_files_kernel(const int32_t* __restrict__ file, const int64_t* __restrict__ n_dev,
+                                  int32_t* __restrict__ out) {
+  const int64_t n = *n_dev;
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    out[i] = file[i];
+}
+
+// off[w] = first row whose word is >= w
+__global__ void word_starts_kernel(const int32_t* __restrict__ word, const int64_t* __restrict__ n_dev, int32_t V,
+                                   int64_t* __restrict__ off) {
+  const int64_t n = *n_dev;
+  for (int64_t w = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; w <= V; w += int64_t(gridDim.x) * blockDim.x) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (word[mid] < w) lo = mid + 1;
+      else hi = mid;
+    }
+    off[w] = lo;
+  }
+}
+
 gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
@@ -638,6 +837,15 @@ gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   auto* files = static_cast<int32_t*>(rb.alloc(size_t(n) * 4));
   int64_t* len = rb.new_len_slot();
   GT_CUDA(cudaMemcpyAsync(len, nd, 8, cudaMemcpyDeviceToDevice, s));
+  if (wr.by_word) {  // the rows are the postings
+    word_starts_kernel<<<grid_for(int64_t(d.V) + 1, threads, cap), threads, 0, s>>>(wr.word.as<int32_t>(), nd, d.V, off);
+    GT_LAUNCH_CHECK();
+    copy_files_kernel<<<grid_for(n, threads, cap), threads, 0, s>>>(wr.file.as<int32_t>(), nd, files);
+    GT_LAUNCH_CHECK();
+    rb.field("offsets", off, int64_t(d.V) + 1);
+    rb.field_dyn("file", files, len);
+    return rb.finish();
+  }
   Buf k0(ctx, size_t(n) * 8, s), k1(ctx, size_t(n) * 8, s), f0(ctx, size_t(n) * 4, s);
   if (n > 0) {
     Buf rs(ctx, radix_scratch_bytes(n, true, 4), s);
@@ -671,7 +879,13 @@ void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** 
   WordRows wr;
   bu_word_rows(g, s, wr);
   const DevGrammar& d = g->d;
+  // rows in word order: the index first, the term vectors re-order them
+  if (ii_out && wr.by_word) {
+    *ii_out = bu_inverted_index(g, wr, s);
+    ii_out = nullptr;
+  }
   if (n_tv > 0) {
+    rows_by_file(g, wr, s);
     Buf toff(g->ctx, size_t(d.F + 1) * 8, s);
     file_offsets_kernel<<<grid_for(int64_t(d.F) + 1, 256, 4096), 256, 0, s>>>(wr.file.as<int32_t>(),
                                                                               wr.total.as<int64_t>(), d.F,
@@ -691,6 +905,20 @@ gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s) {
   const int64_t n = wr.bound;
   gt_ctx* ctx = g->ctx;
   Buf rkey(ctx, size_t(n) * 8, s);
+  if (wr.by_word && g->d.F <= kMaxRankFiles) {  // rows in (key, file) order already
+    wr.cnt = Buf(ctx, size_t(n) * 8, s);
+    if (n > 0) {
+      widen_i32_kernel<<<grid_for(n, 256, ctx->num_sms * 16), 256, 0, s>>>(
+          wr.word.as<int32_t>(), wr.total.as<int64_t>(), rkey.as<uint64_t>());
+      GT_LAUNCH_CHECK();
+      unpack_pay_kernel<<<grid_for(n, 256, ctx->num_sms * 16), 256, 0, s>>>(
+          wr.pay.as<uint64_t>(), wr.total.as<int64_t>(), nullptr, wr.cnt.as<uint64_t>());
+      GT_LAUNCH_CHECK();
+    }
+    return ranked_from_key_rows(ctx, rkey, wr.file, wr.cnt, wr.total.as<int64_t>(), n, 0, g->d.F,
+                                uint64_t(g->max_file_len), s, wr.status.as<uint32_t>());
+  }
+  rows_by_file(g, wr, s);
   if (n > 0) {
     widen_i32_kernel<<<grid_for(n, 256, ctx->num_sms * 16), 256, 0, s>>>(wr.word.as<int32_t>(), wr.total.as<int64_t>(),
                                                                           rkey.as<uint64_t>());
@@ -778,75 +1006,6 @@ void bu_emit_windows(gt_grammar* g, Buf& ends, int kb, const FileRows& fr, cudaS
 
 namespace {
 
-// ---- the files' words, expanded --------------------------------------------------
-
-// words[0, N): the expansion of the root, files back to back.  A tile of kRowTile
-// root symbols per CTA in ticket order, kRowItems consecutive ones per thread; a
-// tile's first word comes from a bounded look-back over the tiles' lengths.
-__global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGrammar d, int64_t tiles,
-                                                                  unsigned long long* __restrict__ look,
-                                                                  int32_t* __restrict__ words,
-                                                                  unsigned* __restrict__ status) {
-  __shared__ int64_t s_warp[kRowThreads / 32];
-  __shared__ int64_t s_item, s_prefix;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_item = int64_t(atomicAdd(look + tiles, 1ull));
-  __syncthreads();
-  const int64_t item = s_item, j0 = item * kRowTile + tid * kRowItems;
-  int32_t sy[kRowItems];
-  int64_t len = 0, ln[kRowItems];
-#pragma unroll
-  for (int k = 0; k < kRowItems; ++k) sy[k] = j0 + k < d.root_len ? d.sym[j0 + k] : -1;
-#pragma unroll
-  for (int k = 0; k < kRowItems; ++k) {
-    ln[k] = sy[k] < 0 ? 0 : (sy[k] < d.V ? 1 : int64_t(d.exp_len[sy[k] - d.V]));
-    len += ln[k];
-  }
-  int64_t incl = len;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int64_t u = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += u;
-  }
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  int64_t before = incl - len, total = 0;
-#pragma unroll
-  for (int w = 0; w < kRowThreads / 32; ++w) {
-    before += w < warp ? s_warp[w] : 0;
-    total += s_warp[w];
-  }
-  if (warp == 0) {
-    if (lane == 0) publish_aggregate(look, item, uint64_t(total));
-    __syncwarp();
-    const int64_t p = warp_look_back(look, item, uint64_t(total), status);
-    if (lane == 0) s_prefix = p < 0 ? 0 : p;
-  }
-  __syncthreads();
-  int64_t o = s_prefix + before;
-#pragma unroll
-  for (int k = 0; k < kRowItems; ++k) {
-    if (sy[k] < 0) continue;
-    if (sy[k] < d.V) {
-      words[o] = sy[k];
-    } else {
-      int64_t q = o;
-      walk_rule(d, sy[k] - d.V, [&](int32_t w) { words[q++] = w; });
-    }
-    o += ln[k];
-  }
-}
-
-// cnt[f] = windows of file f, len[f] = its words (0 for f = F)
-__global__ void file_windows_kernel(const uint64_t* __restrict__ file_len, int32_t F, int64_t* __restrict__ len,
-                                    int64_t* __restrict__ cnt) {
-  for (int32_t f = blockIdx.x * blockDim.x + threadIdx.x; f <= F; f += gridDim.x * blockDim.x) {
-    const int64_t l = f < F ? int64_t(file_len[f]) : 0;
-    len[f] = l;
-    cnt[f] = l > 2 ? l - 2 : 0;
-  }
-}
-
 // One row per window, in text order: key and file.
 __global__ void __launch_bounds__(kRowThreads) token_windows_kernel(const int32_t* __restrict__ words, int64_t N,
                                                                     const int64_t* __restrict__ first, int32_t F,
@@ -862,12 +1021,7 @@ __global__ void __launch_bounds__(kRowThreads) token_windows_kernel(const int32_
   for (int k = 0; k < kRowItems; ++k) {
     const int64_t p = p0 + k * kRowThreads + threadIdx.x;
     if (p >= p1) continue;
-    int32_t lo = f_lo, hi = f_hi;  // last file that starts at or before p
-    while (lo < hi) {
-      const int32_t mid = (lo + hi + 1) >> 1;
-      if (first[mid] <= p) lo = mid;
-      else hi = mid - 1;
-    }
+    const int32_t lo = file_from(first, f_lo, f_hi, p);
     if (p + 2 >= first[lo + 1]) continue;
     const int64_t o = row[lo] + (p - first[lo]);
     keys[o] = pack_compact(words[p], words[p + 1], words[p + 2], kb);
@@ -968,25 +1122,19 @@ void bu_token_windows(gt_grammar* g, int kb, Buf& keys, Buf& files, Buf& n, cuda
   const DevGrammar& d = g->d;
   if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
   Phase ph(ctx, "bu_rows", s);
-  const int64_t N = int64_t(d.N), tiles = (d.root_len + kRowTile - 1) / kRowTile;
+  const int64_t N = int64_t(d.N);
   keys = Buf(ctx, size_t(N) * 8, s);
   files = Buf(ctx, size_t(N) * 4, s);
   n = Buf(ctx, 8, s);
-  Buf words(ctx, size_t(N) * 4, s), look(ctx, size_t(tiles + 1) * 8, s);
-  Buf len(ctx, size_t(d.F + 1) * 8, s), cnt(ctx, size_t(d.F + 1) * 8, s), first(ctx, size_t(d.F + 1) * 8, s);
-  Buf row(ctx, size_t(d.F + 1) * 8, s), sc(ctx, scan_scratch_bytes(d.F + 1), s);
+  Buf words, first, cnt(ctx, size_t(d.F + 1) * 8, s), row(ctx, size_t(d.F + 1) * 8, s);
+  Buf sc(ctx, scan_scratch_bytes(d.F + 1), s);
+  expand_files(g, words, first, s);
   file_windows_kernel<<<grid_for(int64_t(d.F) + 1, 256, ctx->num_sms * 8), 256, 0, s>>>(d.file_len, d.F,
-                                                                                     len.as<int64_t>(),
                                                                                      cnt.as<int64_t>());
   GT_LAUNCH_CHECK();
-  exclusive_scan_i64(len.as<int64_t>(), first.as<int64_t>(), d.F + 1, sc.p, s);
   exclusive_scan_i64(cnt.as<int64_t>(), row.as<int64_t>(), d.F + 1, sc.p, s);
   GT_CUDA(cudaMemcpyAsync(n.p, row.as<int64_t>() + d.F, 8, cudaMemcpyDeviceToDevice, s));
-  if (tiles == 0) return;
-  GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(tiles + 1) * 8, s));
-  expand_root_kernel<<<unsigned(tiles), kRowThreads, 0, s>>>(d, tiles, look.as<unsigned long long>(),
-                                                             words.as<int32_t>(), status_word());
-  GT_LAUNCH_CHECK();
+  if (N == 0) return;
   token_windows_kernel<<<unsigned((N + kRowTile - 1) / kRowTile), kRowThreads, 0, s>>>(
       words.as<int32_t>(), N, first.as<int64_t>(), d.F, row.as<int64_t>(), kb, keys.as<uint64_t>(),
       files.as<uint32_t>());

@@ -989,9 +989,10 @@ __global__ void last_total_kernel(const int64_t* __restrict__ ex, const int64_t*
 // top-k: key = file << cbits | (max_count - count), sorted stably over entries that
 // are already in ascending word order inside each file (no count exceeds
 // max_count, the longest file's length).
+template <class K>
 __global__ void topk_keys_kernel(const int32_t* __restrict__ word, const uint64_t* __restrict__ cnt,
                                  const int64_t* __restrict__ tv_off, int32_t F, uint64_t max_count, int cbits,
-                                 uint64_t* __restrict__ keys, uint32_t* __restrict__ idx) {
+                                 K* __restrict__ keys, uint32_t* __restrict__ idx) {
   const int64_t n = tv_off[F];
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     idx[i] = uint32_t(i);
@@ -1001,7 +1002,7 @@ __global__ void topk_keys_kernel(const int32_t* __restrict__ word, const uint64_
       if (tv_off[mid] <= i) lo = mid;
       else hi = mid;
     }
-    keys[i] = (uint64_t(lo) << cbits) | (max_count - cnt[i]);
+    keys[i] = K((uint64_t(lo) << cbits) | (max_count - cnt[i]));
   }
 }
 
@@ -1639,12 +1640,20 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
     Buf kc(ctx, size_t(F) * 8 + 8, s), sc(ctx, scan_scratch_bytes(F + 1), s);
     if (bound > 0) {
       const int cbits = bits_for(int64_t(max_count)), kbits = cbits + bits_for(std::max(F - 1, 1));
-      topk_keys_kernel<<<grid_for(bound, threads, cap), threads, 0, s>>>(word, cnt, tv_off_in, F, max_count, cbits,
-                                                                          k0.as<uint64_t>(), i0.as<uint32_t>());
-      GT_LAUNCH_CHECK();
-      if (!radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), i0.p, i1.p, 4, bound, 0, kbits, kbits, kbits, rs.p,
-                               s, total))
-        std::swap(i0, i1);
+      bool b;
+      if (kbits <= 32) {
+        topk_keys_kernel<uint32_t><<<grid_for(bound, threads, cap), threads, 0, s>>>(
+            word, cnt, tv_off_in, F, max_count, cbits, k0.as<uint32_t>(), i0.as<uint32_t>());
+        GT_LAUNCH_CHECK();
+        b = radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), i0.p, i1.p, 4, bound, kbits, rs.p, s, total);
+      } else {
+        topk_keys_kernel<uint64_t><<<grid_for(bound, threads, cap), threads, 0, s>>>(
+            word, cnt, tv_off_in, F, max_count, cbits, k0.as<uint64_t>(), i0.as<uint32_t>());
+        GT_LAUNCH_CHECK();
+        b = radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), i0.p, i1.p, 4, bound, 0, kbits, kbits, kbits,
+                                rs.p, s, total);
+      }
+      if (!b) std::swap(i0, i1);
     }
     topk_count_kernel<<<grid_for(F, 256, cap), 256, 0, s>>>(tv_off_in, F, top_k, kc.as<int64_t>());
     GT_LAUNCH_CHECK();

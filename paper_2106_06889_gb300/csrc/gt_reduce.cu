@@ -26,21 +26,21 @@ constexpr int kRunItems = 8;  // consecutive rows per thread
 constexpr int kRunTile = kRunThreads * kRunItems;
 constexpr int kRunWarps = kRunThreads / 32;
 
-template <bool kFile>
-__device__ __forceinline__ bool run_head(uint64_t k, uint64_t prev, uint32_t f, uint32_t prev_f) {
+template <bool kFile, class K>
+__device__ __forceinline__ bool run_head(K k, K prev, uint32_t f, uint32_t prev_f) {
   return k != prev || (kFile && f != prev_f);
 }
 
 // What a row carries beside its key.
 enum RunRows { kKeyVal, kKeyOnly, kKeyFileVal, kKeyFile };
 
-template <RunRows kRows>
+template <class K, RunRows kRows>
 __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
-    const uint64_t* __restrict__ keys, const uint64_t* __restrict__ fkeys, const uint32_t* __restrict__ vals,
-    int64_t n_max, const int64_t* __restrict__ n_dev, uint64_t key_pad, const __grid_constant__ RunOut out,
+    const K* __restrict__ keys, const uint64_t* __restrict__ fkeys, const uint32_t* __restrict__ vals,
+    int64_t n_max, const int64_t* __restrict__ n_dev, K key_pad, const __grid_constant__ RunOut out,
     unsigned long long* __restrict__ look, int64_t tiles_max, unsigned* __restrict__ status) {
   constexpr bool kFile = kRows == kKeyFileVal || kRows == kKeyFile, kVals = kRows == kKeyVal;
-  __shared__ uint64_t s_key[kRunTile];
+  __shared__ K s_key[kRunTile];
   __shared__ uint64_t s_before[kRunTile];  // values of the tile before each head
   __shared__ uint32_t s_file[kFile ? kRunTile : 1];
   __shared__ uint64_t w_sum[kRunWarps];
@@ -63,16 +63,28 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     return;
   }
   const int64_t i0 = item * kRunTile + tid * kRunItems;
-  uint64_t k[kRunItems];
+  K k[kRunItems];
   uint32_t v[kRunItems];
   uint32_t f[kFile ? kRunItems : 1];
   if (i0 + kRunItems <= n) {  // rows are 16-byte aligned (checked by the caller)
-    const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(keys + i0);
+    if (sizeof(K) == 8) {
+      const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(keys + i0);
 #pragma unroll
-    for (int j = 0; j < kRunItems / 2; ++j) {
-      const ulonglong2 x = kp[j];
-      k[2 * j] = x.x;
-      k[2 * j + 1] = x.y;
+      for (int j = 0; j < kRunItems / 2; ++j) {
+        const ulonglong2 x = kp[j];
+        k[2 * j] = K(x.x);
+        k[2 * j + 1] = K(x.y);
+      }
+    } else {
+      const uint4* kp = reinterpret_cast<const uint4*>(keys + i0);
+#pragma unroll
+      for (int j = 0; j < kRunItems / 4; ++j) {
+        const uint4 x = kp[j];
+        k[4 * j] = K(x.x);
+        k[4 * j + 1] = K(x.y);
+        k[4 * j + 2] = K(x.z);
+        k[4 * j + 3] = K(x.w);
+      }
     }
     if (kVals) {
       const uint4* vp = reinterpret_cast<const uint4*>(vals + i0);
@@ -112,7 +124,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     }
   }
   // the row before this thread's first one
-  uint64_t prev = __shfl_up_sync(0xffffffffu, k[kRunItems - 1], 1);
+  K prev = __shfl_up_sync(0xffffffffu, k[kRunItems - 1], 1);
   uint32_t prev_f = kFile ? __shfl_up_sync(0xffffffffu, f[kFile ? kRunItems - 1 : 0], 1) : 0u;
   if (lane == 0 && i0 > 0 && i0 <= n) {
     prev = keys[i0 - 1];
@@ -190,14 +202,16 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
   auto put_sum = [&](int64_t o, uint64_t x) {
     if (out.count) out.count[o] = x;
     if (out.mult) out.mult[o] = uint32_t(x);
+    if (out.pay) reinterpret_cast<uint32_t*>(out.pay)[2 * o] = uint32_t(x);
   };
   for (uint32_t r = tid; r < h_total; r += kRunThreads) {
     const uint64_t key = s_key[r];
     const int64_t o = o0 + r;
     if (out.key) out.key[o] = to_output_key(out.low_bits ? key & ((uint64_t(1) << out.low_bits) - 1) : key, out.kb);
+    if (out.pay) reinterpret_cast<uint32_t*>(out.pay)[2 * o + 1] = uint32_t(key);
     if (out.hi) out.hi[o] = key >> out.low_bits;
     if (out.file) out.file[o] = kFile ? int32_t(s_file[r]) : int32_t(key >> out.low_bits);
-    if (out.word) out.word[o] = int32_t(key & ((uint64_t(1) << out.low_bits) - 1));
+    if (out.word) out.word[o] = int32_t(out.low_bits ? key & ((uint64_t(1) << out.low_bits) - 1) : key);
     if (out.off) out.off[o] = item * kRunTile + int64_t(s_before[r]);
     if (r + 1 < h_total) put_sum(o, s_before[r + 1] - s_before[r]);
   }
@@ -219,15 +233,15 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
 
 namespace {
 
-template <RunRows kRows>
-void launch_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
-                 const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s) {
+template <RunRows kRows, class K>
+void launch_runs(gt_ctx* ctx, const K* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
+                 const int64_t* n_dev, K key_pad, const RunOut& out, cudaStream_t s) {
   const int64_t tiles = n > 0 ? (n + kRunTile - 1) / kRunTile : 1;
   if ((reinterpret_cast<uintptr_t>(keys) & 15) || (reinterpret_cast<uintptr_t>(vals) & 15))
     fail(GT_EINVAL, "rows to reduce must be 16-byte aligned");
   Buf look(ctx, size_t(2 * tiles + 1) * 8, s);
   GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(2 * tiles + 1) * 8, s));
-  reduce_runs_kernel<kRows><<<unsigned(tiles), kRunThreads, 0, s>>>(
+  reduce_runs_kernel<K, kRows><<<unsigned(tiles), kRunThreads, 0, s>>>(
       keys, fkeys, vals, n, n_dev, key_pad, out, look.as<unsigned long long>(), tiles, status_word());
   GT_LAUNCH_CHECK();
 }
@@ -244,6 +258,11 @@ void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const
 void reduce_file_runs(gt_ctx* ctx, const uint64_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,
                       const RunOut& out, cudaStream_t s) {
   launch_runs<kKeyFile>(ctx, keys, nullptr, files, n, n_dev, ~uint64_t(0), out, s);
+}
+
+void reduce_file_runs(gt_ctx* ctx, const uint32_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,
+                      const RunOut& out, cudaStream_t s) {
+  launch_runs<kKeyFile>(ctx, keys, nullptr, files, n, n_dev, ~uint32_t(0), out, s);
 }
 
 }  // namespace gt

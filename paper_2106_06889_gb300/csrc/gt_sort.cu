@@ -138,7 +138,8 @@ struct RadixPasses {
 constexpr int kRhThreads = 512;
 constexpr int kRhItems = 4;
 
-__global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const uint64_t* __restrict__ keys, int64_t n_max,
+template <class K>
+__global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const K* __restrict__ keys, int64_t n_max,
                                                                 const int64_t* __restrict__ n_dev,
                                                                 const __grid_constant__ RadixPasses ps,
                                                                 unsigned long long* __restrict__ counts) {
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const uint64_t* 
   __syncthreads();
   constexpr int64_t kStep = int64_t(kRhThreads) * kRhItems;
   for (int64_t b = blockIdx.x * kStep; b < n; b += gridDim.x * kStep) {
-    uint64_t k[kRhItems];
+    K k[kRhItems];
 #pragma unroll
     for (int j = 0; j < kRhItems; ++j) {
       const int64_t i = b + j * kRhThreads + threadIdx.x;
@@ -239,16 +240,17 @@ __device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t t
 // scattered 8- and 4-byte staging stores, the read back) against the 34 cycles
 // its 24 bytes take at the measured copy rate.  The look-back is hidden: with
 // every word already published the pass takes 328 instead of 349 us (49M rows).
-template <int VB, int ITEMS, class W>
-__global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 3) radix_downsweep_kernel(
-    const uint64_t* __restrict__ kin, uint64_t* __restrict__ kout, const void* __restrict__ vin_,
+template <class K, int VB, int ITEMS, class W>
+__global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems || sizeof(K) + VB == 8 ? 4 : 3)
+    radix_downsweep_kernel(
+    const K* __restrict__ kin, K* __restrict__ kout, const void* __restrict__ vin_,
     void* __restrict__ vout_, int64_t n_max, const int64_t* __restrict__ n_dev, int shift, uint32_t mask,
     const unsigned long long* __restrict__ counts, W* __restrict__ words, unsigned* __restrict__ ticket, unsigned* __restrict__ status) {
   constexpr int kTileKeys = kRsThreads * ITEMS;
   using VT = typename std::conditional<VB == 8, uint64_t, uint32_t>::type;
   extern __shared__ __align__(16) unsigned char rs_smem[];  // staged keys, then values
-  uint64_t* skey = reinterpret_cast<uint64_t*>(rs_smem);
-  VT* sval = reinterpret_cast<VT*>(rs_smem + size_t(kTileKeys) * 8);
+  K* skey = reinterpret_cast<K*>(rs_smem);
+  VT* sval = reinterpret_cast<VT*>(rs_smem + size_t(kTileKeys) * sizeof(K));
   __shared__ uint32_t wcnt[kRsWarps][kRsBins];
   __shared__ W soff[kRsBins];
   __shared__ W gsum[kRsWarps];
@@ -264,10 +266,10 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 3) ra
   const int64_t n = n_dev ? min(*n_dev, n_max) : n_max;
   if (base >= n) return;  // fewer rows than the grid was sized for; later tiles have none either
   const int tn = int(n - base < kTileKeys ? n - base : kTileKeys);
-  const uint64_t* kp = kin + base;
+  const K* kp = kin + base;
   const VT* vp = static_cast<const VT*>(vin_) + (VB ? base : 0);
   const int first = warp * 32 * ITEMS + lane;
-  uint64_t key[ITEMS];
+  K key[ITEMS];
   VT val[VB ? ITEMS : 1];
   // keys past the end (last tile) count as the top digit and rank after every
   // real key: they stay at the end of the staged tile and are not written
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 3) ra
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) key[j] = first + j * 32 < tn ? kp[first + j * 32] : ~uint64_t(0);
+    for (int j = 0; j < ITEMS; ++j) key[j] = first + j * 32 < tn ? kp[first + j * 32] : K(~K(0));
     if (VB) {
 #pragma unroll
       for (int j = 0; j < ITEMS; ++j) val[j] = first + j * 32 < tn ? vp[first + j * 32] : VT(0);
@@ -355,14 +357,14 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 3) ra
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
       const int i = j * kRsThreads + tid;
-      const uint64_t k = skey[i];
+      const K k = skey[i];
       const W p = soff[uint32_t(k >> shift) & mask] + W(i);
       kout[p] = k;
       if (VB) vout[p] = sval[i];
     }
   } else {
     for (int i = tid; i < tn; i += kRsThreads) {
-      const uint64_t k = skey[i];
+      const K k = skey[i];
       const W p = soff[uint32_t(k >> shift) & mask] + W(i);
       kout[p] = k;
       if (VB) vout[p] = sval[i];
@@ -397,30 +399,30 @@ size_t radix_layout(int64_t n, int items, int passes, void* scratch, RadixScratc
   return counts + tickets + words;
 }
 
-template <int VB, int ITEMS, class W>
-void launch_scatter(const uint64_t* ka, uint64_t* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
+template <class K, int VB, int ITEMS, class W>
+void launch_scatter(const K* ka, K* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
                     int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
   constexpr int64_t kTileKeys = int64_t(kRsThreads) * ITEMS;
-  constexpr size_t smem = size_t(kTileKeys) * (8 + VB);
+  constexpr size_t smem = size_t(kTileKeys) * (sizeof(K) + VB);
   const int64_t tiles = (n + kTileKeys - 1) / kTileKeys;
-  GT_CUDA(cudaFuncSetAttribute(radix_downsweep_kernel<VB, ITEMS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  GT_CUDA(cudaFuncSetAttribute(radix_downsweep_kernel<K, VB, ITEMS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(smem)));
   Phase ph(t_call_ctx, "radix_pass", s);  // one span per scatter pass
-  radix_downsweep_kernel<VB, ITEMS, W><<<unsigned(tiles), kRsThreads, smem, s>>>(
+  radix_downsweep_kernel<K, VB, ITEMS, W><<<unsigned(tiles), kRsThreads, smem, s>>>(
       ka, kb, va, vb, n, n_dev, shift, mask, rs.counts + size_t(pass) * kRsBins,
       reinterpret_cast<W*>(rs.words) + size_t(pass) * size_t(tiles) * kRsBins, rs.tickets + pass, status_word());
   GT_LAUNCH_CHECK();
 }
 
-template <int VB>
-void launch_scatter_any(const uint64_t* ka, uint64_t* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
+template <class K, int VB>
+void launch_scatter_any(const K* ka, K* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
                         int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
   if (!radix_narrow(n))
-    launch_scatter<VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
   else if (items == kRsSmallItems)
-    launch_scatter<VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
   else
-    launch_scatter<VB, kRsLargeItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsLargeItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
 }
 
 // Digit passes over bits [begin_a, end_a) then [begin_b, end_b), the bits of
@@ -462,9 +464,11 @@ size_t radix_scratch_bytes(int64_t n, bool, int) {
   return radix_layout(n, radix_narrow(n) ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
 }
 
-bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
-                         int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s,
-                         const int64_t* n_dev) {
+namespace {
+
+template <class K>
+bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n, int begin_a,
+                    int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s, const int64_t* n_dev) {
   if (n <= 0) return false;
   const RadixPasses ps = radix_plan(begin_a, end_a, begin_b, end_b);
   if (ps.n == 0) return false;
@@ -473,23 +477,38 @@ bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void*
   radix_layout(n, items, ps.n, scratch, &rs);
   GT_CUDA(cudaMemsetAsync(scratch, 0, rs.zero_bytes, s));
   const int sms = t_call_ctx ? t_call_ctx->num_sms : 152;
-  radix_hist_kernel<<<grid_for(n, kRhThreads * kRhItems, sms * 4), kRhThreads, 0, s>>>(keys_a, n, n_dev, ps,
+  radix_hist_kernel<K><<<grid_for(n, kRhThreads * kRhItems, sms * 4), kRhThreads, 0, s>>>(keys_a, n, n_dev, ps,
                                                                                                  rs.counts);
   GT_LAUNCH_CHECK();
-  uint64_t *ka = keys_a, *kb = keys_b;
+  K *ka = keys_a, *kb = keys_b;
   void *va = vals_a, *vb = vals_b;
   for (int p = 0; p < ps.n; ++p) {
     const uint32_t mask = (1u << ps.bits[p]) - 1u;
     if (value_bytes == 4)
-      launch_scatter_any<4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
     else if (value_bytes == 8)
-      launch_scatter_any<8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
     else
-      launch_scatter_any<0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, s);
     std::swap(ka, kb);
     std::swap(va, vb);
   }
   return ps.n % 2 == 1;
+}
+
+}  // namespace
+
+bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
+                         int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s,
+                         const int64_t* n_dev) {
+  return radix_sort_any<uint64_t>(keys_a, keys_b, vals_a, vals_b, value_bytes, n, begin_a, end_a, begin_b, end_b,
+                                  scratch, s, n_dev);
+}
+
+bool radix_sort_pingpong32(uint32_t* keys_a, uint32_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
+                           int bits, void* scratch, cudaStream_t s, const int64_t* n_dev) {
+  return radix_sort_any<uint32_t>(keys_a, keys_b, vals_a, vals_b, value_bytes, n, 0, bits, bits, bits, scratch, s,
+                                  n_dev);
 }
 
 void radix_sort_u64(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* vals_out, int value_bytes,
