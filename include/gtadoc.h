@@ -358,7 +358,7 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *                   sorted in global memory.
  *   "radix_items"   keys per thread of the LSD radix sort's scatter passes:
  *                   8 (default): tiles of 2048 keys below 2^20 rows and of
- *                   4096 keys from there on; 16: always tiles of 4096.
+ *                   6144 keys from there on; 16: always tiles of 6144.
  *                   GT_EINVAL otherwise.  Same results.
  *   "radix_prefetch" accepted, without effect: it selected a persistent
  *                   scatter that was slower than one CTA per tile.

@@ -120,11 +120,14 @@ constexpr int kRsThreads = 256;  // one thread per digit value in the per-tile b
 constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsBins = 256;
 constexpr int kRsMaxPasses = 8;
-constexpr int kRsSmallItems = 8, kRsLargeItems = 16;  // keys per thread
-// Below this many rows tiles of 2048 keys, above it tiles of 4096.  Measured
-// per pass (60-bit Zipf keys, 4-byte values): 163k rows 8.6 against 10.7 us (few
-// tiles: latency), 4M rows 43 against 38 us (the per-tile bookkeeping over 256
-// digits counts).
+constexpr int kRsSmallItems = 8, kRsLargeItems = 24;  // keys per thread
+// Below this many rows tiles of 2048 keys, from there on tiles of 6144: small
+// sorts are latency (few tiles), large ones the per-tile bookkeeping over 256
+// digits.  Measured for a whole sort (60-bit Zipf keys, 4-byte values), small
+// against large tile: 163k rows 77 against 93 us, 700k 111 against 108, 1.4M 157
+// against 134, 3.7M 312 against 243, 49M 3379 against 2607.  Tiles of 4096 rows
+// take 261 us at 3.7M and 2909 at 49M, of 8192 rows (one CTA less per SM) 9% and
+// 14% more than of 6144.
 constexpr int64_t kRsLargeRows = int64_t(1) << 20;
 
 struct RadixPasses {
@@ -239,9 +242,10 @@ __device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t t
 // costs about 25 shared-memory wavefronts per 32 rows (atomic, counter, the
 // scattered 8- and 4-byte staging stores, the read back) against the 34 cycles
 // its 24 bytes take at the measured copy rate.  The look-back is hidden: with
-// every word already published the pass takes 328 instead of 349 us (49M rows).
+// every word already published a pass over 49M rows is 6% shorter.  One such pass
+// takes 326 us, 173 at the copy rate (32-bit keys, 25M rows: 142 and 59).
 template <class K, int VB, int ITEMS, class W>
-__global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems || sizeof(K) + VB == 8 ? 4 : 3)
+__global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 2)
     radix_downsweep_kernel(
     const K* __restrict__ kin, K* __restrict__ kout, const void* __restrict__ vin_,
     void* __restrict__ vout_, int64_t n_max, const int64_t* __restrict__ n_dev, int shift, uint32_t mask,
@@ -381,7 +385,7 @@ struct RadixScratch {
 
 int radix_items(int64_t n) {
   const int64_t p = t_call_ctx ? t_call_ctx->param("radix_items", kRsSmallItems) : kRsSmallItems;
-  return p == kRsLargeItems || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
+  return p == 16 || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
 }
 
 bool radix_narrow(int64_t n) { return n < (int64_t(1) << 30); }
@@ -460,7 +464,7 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
 }
 
 size_t radix_scratch_bytes(int64_t n, bool, int) {
-  // for the smaller tile, which "radix_items" may select at any size
+  // for the smaller tile: the most look-back words of the two
   return radix_layout(n, radix_narrow(n) ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
 }
 

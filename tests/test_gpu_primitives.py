@@ -1,6 +1,6 @@
 """The one-pass primitives (scan, radix sort, run reduction) through the
 public calls, at the edges of their tiles: 2,048 values per scan and reduction
-tile, 2,048 or 4,096 rows per sort tile, the row count at which the sort
+tile, 2,048 or 6,144 rows per sort tile, the row count at which the sort
 changes its tile, runs that cover whole tiles, and (file, key) rows that fit
 one 64-bit sort key and that do not.  Whole numbers: equal to the oracle's."""
 import numpy as np
@@ -91,9 +91,10 @@ def test_file_keys(ctx, V, F, strategy):
         B.gt_set_param(ctx, "bu_local", 1)
 
 
-@pytest.mark.parametrize("n", [2 ** 20 - 1 + 2, 2 ** 20 + 2, 2 ** 20 + 4099])
+@pytest.mark.parametrize("n", [2 ** 20 - 1 + 2, 2 ** 20 + 2, 171 * 6144 + 2, 171 * 6144 + 3])
 def test_sort_tile_change(ctx, n):
-    """Rows just below and above 2^20, where the sort goes from 2,048- to 4,096-row tiles."""
+    """Rows just below and above 2^20, where the sort goes from 2,048- to 6,144-row tiles, and at
+    the edge of a large tile."""
     rng = np.random.default_rng(n)
     toks = (rng.zipf(1.2, n) % 5000).astype(np.int32)
     g = root_only_grammar(toks, [n // 2, n - n // 2], 5000)
