@@ -157,6 +157,14 @@ __global__ void level_slot_off_kernel(const int64_t* __restrict__ lvl_off, int32
   }
 }
 
+// lvl_piece[l] = first piece of level l's heavy slots (scan: pieces before each
+// heavy slot; index depth holds the end).
+__global__ void level_piece_kernel(const int64_t* __restrict__ lvl_heavy, int32_t depth, int64_t n_light,
+                                   int64_t n_heavy, const int64_t* __restrict__ scan,
+                                   int64_t* __restrict__ lvl_piece) {
+  for (int l = threadIdx.x; l <= depth; l += blockDim.x) lvl_piece[l] = n_heavy ? scan[lvl_heavy[l] - n_light] : 0;
+}
+
 // Rows, edge-parallel over the non-root parent edges p -> c: every file f
 // of p gets an entry (p's slot for f, mult) in the row of c's slot for f.
 // With fill == false only the row lengths are counted; with fill == true the
@@ -255,8 +263,9 @@ __global__ void pair_gather_kernel(const uint32_t* __restrict__ by_slot, const u
     by_pair[q] = by_slot[pair_slot[q]];
 }
 
-__global__ void rows_to_pairs_kernel(uint2* __restrict__ entries, int64_t ne, uint4* __restrict__ pieces, int64_t np,
-                                     const uint32_t* __restrict__ slot_pair) {
+__global__ void rows_to_pairs_kernel(uint2* __restrict__ entries, int64_t ne, uint4* __restrict__ pieces,
+                                     const int64_t* __restrict__ n_pieces, const uint32_t* __restrict__ slot_pair) {
+  const int64_t np = *n_pieces;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < ne + np; i += int64_t(gridDim.x) * blockDim.x) {
     if (i < ne) entries[i].x = slot_pair[entries[i].x];
     else pieces[i - ne].x = slot_pair[pieces[i - ne].x];
@@ -1102,10 +1111,12 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
   if (EB >= (int64_t(1) << 32)) fail(GT_EOVERFLOW, "2^32 or more (rule, file) pairs");
   g->light_slots = hn[0];
   GT_CUDA(cudaMemcpyAsync(nnz, &EB, 8, cudaMemcpyHostToDevice, s));
-  // owners of the slots and each level's first light and heavy slot
-  void* po = grammar_alloc(g, size_t(2 * (d.depth + 1)) * 8 + 64, s);
+  // owners of the slots; each level's first light slot, heavy slot and heavy piece
+  void* po = grammar_alloc(g, size_t(3 * (d.depth + 1)) * 8 + 64, s);
   auto* lslot = static_cast<int64_t*>(po);
   auto* lheavy = lslot + d.depth + 1;
+  auto* lpiece = lheavy + d.depth + 1;
+  g->lvl_tab = lslot;
   owners = Buf(ctx, size_t(EB) * 5 + 64, s);
   auto* srule = owners.as<int32_t>();
   auto* sfile = reinterpret_cast<uint8_t*>(srule + EB);
@@ -1113,16 +1124,9 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
                                                                      nl, M, d.pedge_off, d.R, off, srule, sfile);
   GT_LAUNCH_CHECK();
   {
-    Buf loff(ctx, size_t(d.depth + 1) * 8, s);
-    GT_CUDA(cudaMemcpyAsync(loff.p, g->lvl_off.data(), size_t(d.depth + 1) * 8, cudaMemcpyHostToDevice, s));
-    level_slot_off_kernel<<<1, 128, 0, s>>>(loff.as<int64_t>(), d.depth, sl.as<int64_t>(), sh.as<int64_t>(), nl, d.R,
-                                            lslot, lheavy);
+    level_slot_off_kernel<<<1, 128, 0, s>>>(d.lvl_off, d.depth, sl.as<int64_t>(), sh.as<int64_t>(), nl, d.R, lslot,
+                                            lheavy);
     GT_LAUNCH_CHECK();
-    g->lvl_slot.assign(size_t(d.depth + 1), 0);
-    g->lvl_heavy.assign(size_t(d.depth + 1), 0);
-    GT_CUDA(cudaMemcpyAsync(g->lvl_slot.data(), lslot, size_t(d.depth + 1) * 8, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaMemcpyAsync(g->lvl_heavy.data(), lheavy, size_t(d.depth + 1) * 8, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaStreamSynchronize(s));  // loff, EB and lvl_off's host copy are read by now
   }
   // the root's references in slot layout (every weight's starting value)
   {
@@ -1162,10 +1166,13 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
     g->row_off = roff;
     g->row_entries = ent;
     g->row_entries_n = nent;
-    // the heavy slots' rows in pieces, and each level's first piece
+    // the heavy slots' rows in pieces, and each level's first piece; the pieces
+    // are at most one per slot and one per kPieceEntries entries (their number
+    // stays on the device: nothing here waits for it)
     const int64_t NL = hn[0], NH = EB - NL;
     Buf pc(ctx, size_t(NH) * 8 + 16, s), ps(ctx, size_t(NH + 1) * 8, s), sc6(ctx, scan_scratch_bytes(NH), s);
-    int64_t npieces = 0;
+    const int64_t npieces = NH > 0 ? NH + nent / kPieceEntries : 0;
+    auto* pieces = static_cast<uint4*>(grammar_alloc(g, size_t(npieces) * 16 + 16, s));
     if (NH > 0) {
       row_pieces_kernel<false><<<grid_for(NH, threads, cap), threads, 0, s>>>(roff, NL, EB, pc.as<int64_t>(),
                                                                                nullptr, nullptr);
@@ -1173,36 +1180,13 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
       exclusive_scan_i64(pc.as<int64_t>(), ps.as<int64_t>(), NH, sc6.p, s);
       last_total_kernel<<<1, 1, 0, s>>>(ps.as<int64_t>(), pc.as<int64_t>(), NH, ps.as<int64_t>() + NH, nullptr);
       GT_LAUNCH_CHECK();
-      GT_CUDA(cudaMemcpyAsync(&npieces, ps.as<int64_t>() + NH, 8, cudaMemcpyDeviceToHost, s));
-      GT_CUDA(cudaStreamSynchronize(s));
-    }
-    auto* pieces = static_cast<uint4*>(grammar_alloc(g, size_t(npieces) * 16 + 16, s));
-    if (npieces > 0) {
       row_pieces_kernel<true><<<grid_for(NH, threads, cap), threads, 0, s>>>(roff, NL, EB, nullptr,
                                                                               ps.as<int64_t>(), pieces);
       GT_LAUNCH_CHECK();
     }
+    level_piece_kernel<<<1, 128, 0, s>>>(lheavy, d.depth, NL, NH, ps.as<int64_t>(), lpiece);
+    GT_LAUNCH_CHECK();
     g->row_pieces = pieces;
-    g->row_pieces_n = npieces;
-    g->lvl_piece.assign(size_t(d.depth + 1), 0);
-    for (int l = 0; l <= d.depth; ++l) {
-      const int64_t h = g->lvl_heavy[size_t(l)] - NL;  // heavy slots before level l
-      if (NH > 0) GT_CUDA(cudaMemcpyAsync(&g->lvl_piece[size_t(l)], ps.as<int64_t>() + h, 8, cudaMemcpyDeviceToHost, s));
-    }
-    // the levels' tables on the device, for the launch that runs the small ones
-    auto* tab = static_cast<int64_t*>(grammar_alloc(g, size_t(3 * (d.depth + 1)) * 8, s));
-    const std::vector<int64_t>* host[3] = {&g->lvl_slot, &g->lvl_heavy, &g->lvl_piece};
-    GT_CUDA(cudaStreamSynchronize(s));  // lvl_piece has arrived
-    for (int k = 0; k < 3; ++k)
-      GT_CUDA(cudaMemcpyAsync(tab + k * (d.depth + 1), host[k]->data(), size_t(d.depth + 1) * 8,
-                              cudaMemcpyHostToDevice, s));
-    GT_CUDA(cudaStreamSynchronize(s));  // the scratch above is released on return
-    g->lvl_tab = tab;
-    int t = d.depth;
-    while (t > 2 && g->lvl_slot[size_t(t)] - g->lvl_slot[size_t(t) - 1] <= kTailItems &&
-           (g->lvl_piece[size_t(t)] - g->lvl_piece[size_t(t) - 1]) * 32 <= kTailItems)
-      --t;
-    g->fw_tail = d.depth - t >= 2 ? t : d.depth;
   }
   g->fmask = M;
   g->foff = off;
@@ -1245,12 +1229,10 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
       pair_gather_kernel<<<grid_for(EB, threads, cap), threads, 0, s>>>(w0b.as<uint32_t>(), fslot, EB, r0);
       GT_LAUNCH_CHECK();
     }
-    const int64_t ne = g->row_entries_n, np = g->row_pieces_n;
-    if (ne + np > 0) {
-      rows_to_pairs_kernel<<<grid_for(ne + np, threads, cap), threads, 0, s>>>(
-          const_cast<uint2*>(g->row_entries), ne, const_cast<uint4*>(g->row_pieces), np, sp);
-      GT_LAUNCH_CHECK();
-    }
+    const int64_t ne = g->row_entries_n;
+    rows_to_pairs_kernel<<<grid_for(ne + EB, threads, cap), threads, 0, s>>>(
+        const_cast<uint2*>(g->row_entries), ne, const_cast<uint4*>(g->row_pieces), lpiece + d.depth, sp);
+    GT_LAUNCH_CHECK();
     g->slot_pair = sp;
     g->root_pairs = r0;
   }
@@ -1268,7 +1250,6 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
   GT_LAUNCH_CHECK();
   chunk_pairs_kernel<<<grid_for(nxc, threads, cap), threads, 0, s>>>(xcs, xcl, xcn, fpos, EB, xp0, xp1);
   GT_LAUNCH_CHECK();
-  GT_CUDA(cudaMemcpyAsync(&g->rule_chunks, xcn, 8, cudaMemcpyDeviceToHost, s));
   // the rules' own words, for the chunks' expansion
   {
     Buf wc(ctx, size_t(d.R) * 8, s), wo(ctx, size_t(d.R) * 8 + 8, s), sc4(ctx, scan_scratch_bytes(d.R), s);
@@ -1277,10 +1258,7 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
     exclusive_scan_i64(wc.as<int64_t>(), wo.as<int64_t>(), d.R, sc4.p, s);
     last_total_kernel<<<1, 1, 0, s>>>(wo.as<int64_t>(), wc.as<int64_t>(), d.R, wo.as<int64_t>() + d.R, nullptr);
     GT_LAUNCH_CHECK();
-    int64_t nw = 0;
-    GT_CUDA(cudaMemcpyAsync(&nw, wo.as<int64_t>() + d.R, 8, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaStreamSynchronize(s));
-    words = Buf(ctx, size_t(d.R) * 4 + size_t(nw) * 4 + 64, s);
+    words = Buf(ctx, size_t(d.R) * 4 + size_t(d.G - d.root_len) * 4 + 64, s);  // at most every symbol past the root
     auto* woff = words.as<uint32_t>();
     auto* rw = reinterpret_cast<int32_t*>(woff + d.R + (d.R & 3 ? 4 - (d.R & 3) : 0));
     rule_words_kernel<<<grid_for(d.R, threads, cap), threads, 0, s>>>(d, wo.as<int64_t>(), woff, rw);
@@ -1292,7 +1270,6 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
     rule_words = rw;
     fe_wbeg = rec;
     fe_pos32 = rec + EB;
-    GT_CUDA(cudaStreamSynchronize(s));  // the scratch above is released on return
   }
   g->xch_start = xcs;
   g->xch_len = xcl;
@@ -1300,30 +1277,27 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
   g->xch_count = xcn;
   g->xch_p0 = xp0;
   g->xch_p1 = xp1;
-  GT_CUDA(cudaStreamSynchronize(s));
   // the rule words of every file sorted by 16k-word bucket, each entry its
   // (file, rule) pair relative to the chunk's first pair above its 14-bit
   // index, in 32 bits (structure: a query gathers its weights by pair)
   {
     const int nb = int((d.V + kFBucket - 1) / kFBucket);
-    const int64_t nxc2 = g->rule_chunks;
-    void* px = grammar_alloc(g, size_t(g->fword_bound) * 4 + 16 + size_t(nxc2) * nb * 12 + 64, s);
+    void* px = grammar_alloc(g, size_t(g->fword_bound) * 4 + 16 + size_t(nxc) * nb * 12 + 64, s);
     auto* xrs = static_cast<int64_t*>(px);
-    auto* xrl = reinterpret_cast<int32_t*>(xrs + nxc2 * nb);
-    auto* xent = reinterpret_cast<uint32_t*>(xrl + nxc2 * nb + 4);
-    if (nxc2 > 0) {
+    auto* xrl = reinterpret_cast<int32_t*>(xrs + nxc * nb);
+    auto* xent = reinterpret_cast<uint32_t*>(xrl + nxc * nb + 4);
+    if (nxc > 0) {
       Buf ident(ctx, size_t(EB) * 4 + 16, s), wide(ctx, size_t(g->fword_bound) * 8 + 16, s);
       iota_u32_kernel<<<grid_for(EB, threads, cap), threads, 0, s>>>(ident.as<uint32_t>(), EB);
       GT_LAUNCH_CHECK();
       Chunks xc{xcs, xcl, xcf, xcn, xp0, xp1};
       // "weight" of pair q = ident[ident[q]] = q: every entry carries its pair
       const PairWords pw{fe_wbeg, ident.as<uint32_t>(), fe_pos32, ident.as<uint32_t>(), rule_words};
-      launch_chunk_sort<true>(unsigned(std::min<int64_t>(nxc2, 65535)), s, xc, nullptr, pw, nb, d.V, wide.p, xrs,
+      launch_chunk_sort<true>(unsigned(std::min<int64_t>(nxc, 65535)), s, xc, nullptr, pw, nb, d.V, wide.p, xrs,
                               xrl);
-      narrow_entries_kernel<<<unsigned(std::min<int64_t>(nxc2, 65535)), 256, 0, s>>>(
+      narrow_entries_kernel<<<unsigned(std::min<int64_t>(nxc, 65535)), 256, 0, s>>>(
           wide.as<uint64_t>(), xcs, xcl, xcn, xp0, xent);
       GT_LAUNCH_CHECK();
-      GT_CUDA(cudaStreamSynchronize(s));  // ident and wide are released on return
     }
     g->xent = xent;
     g->xrun_start = xrs;
@@ -1331,10 +1305,20 @@ void file_sizes(gt_grammar* g, cudaStream_t s) {
   }
   // files by length, longest first (launch order of per-file work)
   std::vector<uint64_t> hl(size_t(d.F));
-  if (d.F > 0) {
-    GT_CUDA(cudaMemcpyAsync(hl.data(), d.file_len, size_t(d.F) * 8, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaStreamSynchronize(s));
-  }
+  GT_CUDA(cudaMemcpyAsync(hl.data(), d.file_len, size_t(d.F) * 8, cudaMemcpyDeviceToHost, s));
+  // ... and what the host keeps of the levels
+  const size_t nlv = size_t(d.depth) + 1;
+  std::vector<int64_t> tab(3 * nlv);
+  GT_CUDA(cudaMemcpyAsync(tab.data(), g->lvl_tab, 3 * nlv * 8, cudaMemcpyDeviceToHost, s));
+  GT_CUDA(cudaStreamSynchronize(s));
+  g->lvl_slot.assign(tab.begin(), tab.begin() + long(nlv));
+  g->lvl_heavy.assign(tab.begin() + long(nlv), tab.begin() + long(2 * nlv));
+  g->lvl_piece.assign(tab.begin() + long(2 * nlv), tab.end());
+  int t = d.depth;
+  while (t > 2 && g->lvl_slot[size_t(t)] - g->lvl_slot[size_t(t) - 1] <= kTailItems &&
+         (g->lvl_piece[size_t(t)] - g->lvl_piece[size_t(t) - 1]) * 32 <= kTailItems)
+    --t;
+  g->fw_tail = d.depth - t >= 2 ? t : d.depth;
   std::vector<int32_t> ord(size_t(d.F));
   for (int32_t f = 0; f < d.F; ++f) ord[size_t(f)] = f;
   std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return hl[size_t(a)] > hl[size_t(b)]; });

@@ -222,7 +222,6 @@ struct gt_grammar {
   const uint2* row_entries = nullptr;
   int64_t row_entries_n = 0;
   const uint4* row_pieces = nullptr;
-  int64_t row_pieces_n = 0;
   std::vector<int64_t> lvl_piece;
   // device copies of lvl_slot, lvl_heavy and lvl_piece, and the first of the
   // deepest levels that are small enough to run in one launch
@@ -231,7 +230,6 @@ struct gt_grammar {
   // the rule words (file-major) cut into chunks of at most 4096 words inside
   // each file: chunk c = words [xch_start[c], + xch_len[c]), overlapped by the
   // pairs [xch_p0[c], xch_p1[c]); file f's chunks are [xch_foff[f], xch_foff[f+1])
-  int64_t rule_chunks = 0;  // host copy of *xch_count
   // the rule words of each file sorted by 16k-word bucket per rule-word chunk:
   // entry = (pair - chunk's first pair) << 14 | index in bucket, runs per (chunk, bucket)
   const uint32_t* xent = nullptr;
