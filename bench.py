@@ -141,7 +141,9 @@ def kernel_bytes(workload: str, info: dict, out: dict) -> dict:
     (8 B key + 4 B weight) stand in for the per-window table updates of the
     paper's sequence support (Section IV-D): radix_downsweep_kernel<4> and sg_scatter_kernel read and write
     every row once per launch (24 B), sg_reduce_kernel reads them (12 B) and
-    writes the distinct 3-grams (16 B each)."""
+    writes the distinct 3-grams (16 B each).  Where the sort's rows hold their
+    weight in the key's word (num_words up to 2^20 and at most three tokens per
+    window), radix_downsweep_kernel<0> moves 16 B per row."""
     G, V = info["num_syms"], info["num_words"]
     root_len = out["root_len"]
     if workload == "multi64_50m":
@@ -150,7 +152,8 @@ def kernel_bytes(workload: str, info: dict, out: dict) -> dict:
                 "chunk_sort_rules": ("chunk_sort_kernel<1>", 4 * info["file_pairs"] + 4 * (G - root_len)),
                 "wc_partition": ("wc_partition_kernel", 4 * G)}
     U = info["owned_windows"]
-    return {"radix_pass": ("radix_downsweep_kernel<4>", 24 * U),
+    coded = V <= 1 << 20 and 0 < info.get("num_tokens", 0) <= 3 * U
+    return {"radix_pass": ("radix_downsweep_kernel<0>", 16 * U) if coded else ("radix_downsweep_kernel<4>", 24 * U),
             "seq_scatter": ("sg_scatter_kernel", 24 * U),
             "seq_reduce": ("sg_reduce_kernel", 12 * U + 16 * out["distinct_3grams"]),
             "wc_partition": ("wc_partition_kernel", 4 * G)}

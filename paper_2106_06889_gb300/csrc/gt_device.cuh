@@ -8,6 +8,34 @@
 
 namespace gt {
 
+// ---- rows of one word: key << kCodeBits | code of a weight -----------------------
+// A code stands for m x 4^s (m 1 to 3 in its low bits, s above), or for 2^8, 2^12,
+// 2^16, 2^20 (m 0).  A weight takes one row per component: 1 to 3 take one, and a
+// weight w at most 1 + (w - 1) / 4.
+constexpr int kCodeBits = 4;
+
+__device__ __forceinline__ uint32_t code_weight(uint32_t code) {
+  const uint32_t m = code & 3u, s = (code >> 2) & 3u;
+  return m ? m << (2 * s) : 256u << (4 * s);
+}
+
+// rows that a weight takes
+__device__ __forceinline__ uint32_t weight_rows(uint32_t w) {
+  return uint32_t(__popc((w | (w >> 1)) & 0x55u)) + ((w >> 8) & 15u) + ((w >> 12) & 15u) + ((w >> 16) & 15u) + (w >> 20);
+}
+
+// code of a component of w > 0, and what is left of w without it
+__device__ __forceinline__ uint32_t take_code(uint32_t& w) {
+  if (w & 0xffu) {
+    const uint32_t s = uint32_t(__ffs(int(w & 0xffu)) - 1) >> 1, m = (w >> (2 * s)) & 3u;
+    w &= ~(3u << (2 * s));
+    return s << 2 | m;
+  }
+  const uint32_t s = (w & 0xf00u) ? 0u : (w & 0xf000u) ? 1u : (w & 0xf0000u) ? 2u : 3u;
+  w -= 256u << (4 * s);
+  return s << 2;
+}
+
 // Lanes of the warp holding the same 8-bit digit as this lane (among `active`),
 // from one ballot per digit bit.  Every lane of the warp must call it.  Bound by
 // instruction issue in the sort that ranks 32 rows per call: written so that the

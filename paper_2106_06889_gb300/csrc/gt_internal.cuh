@@ -443,6 +443,8 @@ struct Windows {
   Buf keys, fkeys, vals, n_dev;
   bool file_in_key = false;
   int64_t n = 0;
+  int64_t max_runs = 0;  // distinct keys at most
+  bool coded = false;    // keys hold their weights' codes (no vals), *n_dev rows
   int kb = 1;
   uint64_t key_pad = 0;
   // already one row per distinct (file, key): keys[0, *total) with rfile
@@ -591,6 +593,9 @@ struct RunOut {
 };
 void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
                  const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s);
+// rows (key << kCodeBits | code of a weight): runs of equal keys
+void reduce_coded_runs(gt_ctx* ctx, const uint64_t* keys, int64_t n, const int64_t* n_dev, const RunOut& out,
+                       cudaStream_t s);
 // rows (key, file), every one counting 1: runs of equal (key, file)
 void reduce_file_runs(gt_ctx* ctx, const uint64_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,
                       const RunOut& out, cudaStream_t s);

@@ -32,7 +32,7 @@ __device__ __forceinline__ bool run_head(K k, K prev, uint32_t f, uint32_t prev_
 }
 
 // What a row carries beside its key.
-enum RunRows { kKeyVal, kKeyOnly, kKeyFileVal, kKeyFile };
+enum RunRows { kKeyVal, kKeyOnly, kKeyFileVal, kKeyFile, kKeyCode };
 
 template <class K, RunRows kRows>
 __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     int64_t n_max, const int64_t* __restrict__ n_dev, K key_pad, const __grid_constant__ RunOut out,
     unsigned long long* __restrict__ look, int64_t tiles_max, unsigned* __restrict__ status) {
   constexpr bool kFile = kRows == kKeyFileVal || kRows == kKeyFile, kVals = kRows == kKeyVal;
+  constexpr int kShift = kRows == kKeyCode ? kCodeBits : 0;
   __shared__ K s_key[kRunTile];
   __shared__ uint64_t s_before[kRunTile];  // values of the tile before each head
   __shared__ uint32_t s_file[kFile ? kRunTile : 1];
@@ -109,6 +110,13 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
 #pragma unroll
       for (int j = 0; j < kRunItems; ++j) f[j] = vals[i0 + j];
     }
+    if (kRows == kKeyCode) {
+#pragma unroll
+      for (int j = 0; j < kRunItems; ++j) {
+        v[j] = code_weight(uint32_t(k[j]));
+        k[j] >>= kShift;
+      }
+    }
   } else {
 #pragma unroll
     for (int j = 0; j < kRunItems; ++j) {
@@ -121,13 +129,17 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
         v[j] = uint32_t(x);
       }
       if (kRows == kKeyFile) f[j] = in ? vals[i0 + j] : 0u;
+      if (kRows == kKeyCode) {
+        v[j] = in ? code_weight(uint32_t(k[j])) : 0u;
+        if (in) k[j] >>= kShift;
+      }
     }
   }
   // the row before this thread's first one
   K prev = __shfl_up_sync(0xffffffffu, k[kRunItems - 1], 1);
   uint32_t prev_f = kFile ? __shfl_up_sync(0xffffffffu, f[kFile ? kRunItems - 1 : 0], 1) : 0u;
   if (lane == 0 && i0 > 0 && i0 <= n) {
-    prev = keys[i0 - 1];
+    prev = keys[i0 - 1] >> kShift;
     if (kFile) prev_f = kRows == kKeyFileVal ? uint32_t(fkeys[i0 - 1] >> 32) : vals[i0 - 1];
   }
   uint32_t heads = 0;  // bit j: row j starts a run
@@ -253,6 +265,11 @@ void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const
   if (fkeys) launch_runs<kKeyFileVal>(ctx, keys, fkeys, nullptr, n, n_dev, key_pad, out, s);
   else if (vals) launch_runs<kKeyVal>(ctx, keys, nullptr, vals, n, n_dev, key_pad, out, s);
   else launch_runs<kKeyOnly>(ctx, keys, nullptr, nullptr, n, n_dev, key_pad, out, s);
+}
+
+void reduce_coded_runs(gt_ctx* ctx, const uint64_t* keys, int64_t n, const int64_t* n_dev, const RunOut& out,
+                       cudaStream_t s) {
+  launch_runs<kKeyCode>(ctx, keys, nullptr, nullptr, n, n_dev, ~uint64_t(0), out, s);
 }
 
 void reduce_file_runs(gt_ctx* ctx, const uint64_t* keys, const uint32_t* files, int64_t n, const int64_t* n_dev,

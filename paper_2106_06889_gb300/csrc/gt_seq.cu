@@ -123,6 +123,93 @@ __global__ void __launch_bounds__(kWinThreads, 3) win_emit_kernel(DevGrammar d, 
   if (threadIdx.x == 0 && first + total > bound) atomicOr(status, ST_OVERFLOW);
 }
 
+// The same windows as rows of one word (key << kCodeBits | code): a window of
+// weight 1 to 3 is one row, a heavier one a row per component of its weight.  The
+// rows are sorted next, so their order is free: a tile claims its rows with one
+// atomic; every window's first row goes through the stage, the others (none in the
+// root's tiles) are written by their threads.  425 us for 41M symbols and 49M
+// windows, like the (key, weight) form: bound by the latency of its phases, not by
+// the 8 bytes per row it writes.
+__global__ void __launch_bounds__(kWinThreads, 3) win_emit_coded_kernel(DevGrammar d, const int4* __restrict__ ends,
+                                                                        const uint64_t* __restrict__ wt, int kb,
+                                                                        unsigned long long* __restrict__ n_rows,
+                                                                        int64_t bound, uint64_t* __restrict__ keys,
+                                                                        unsigned* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char win_smem[];
+  TileEnds& te = *reinterpret_cast<TileEnds*>(win_smem);
+  uint64_t* const stage = reinterpret_cast<uint64_t*>(win_smem);  // takes the ends' room once they are read
+  __shared__ int warp_tot[kWinThreads / 32];
+  __shared__ unsigned long long s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t t0 = int64_t(blockIdx.x) * kTile;
+  load_tile_ends(d, ends, t0, te);
+  uint64_t k[4][2];
+  uint32_t w[4];  // weight, then what the first row leaves of it
+  int at[4], n = 0, more = 0;
+  unsigned has = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = warp * 128 + q * 32 + lane;
+    const int64_t j = t0 + i;
+    const int h = j < d.G ? windows_in(te, i, kb, k[q]) : 0;
+    w[q] = 0;
+    if (h) w[q] = j < d.root_len ? uint32_t(wt[0]) : uint32_t(wt[d.sym_rule[j - d.first_rule_tile * kTile]]);
+    if (w[q]) has |= unsigned(h) << (2 * q);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const unsigned h = (has >> (2 * q)) & 3u;
+    const unsigned b0 = __ballot_sync(0xffffffffu, h & 1u), b1 = __ballot_sync(0xffffffffu, h & 2u);
+    at[q] = n + __popc(b0 & lt) + __popc(b1 & lt);
+    n += __popc(b0) + __popc(b1);
+    if (h) {
+      const uint32_t code = take_code(w[q]);
+      k[q][0] = k[q][0] << kCodeBits | code;
+      k[q][1] = k[q][1] << kCodeBits | code;
+      more += __popc(h) * int(weight_rows(w[q]));
+    }
+  }
+  if (lane == 0) warp_tot[warp] = n;
+  const int any_more = __syncthreads_or(more);  // also: the ends are read, the stage takes their room
+  int before = 0, total = 0;
+#pragma unroll
+  for (int x = 0; x < kWinThreads / 32; ++x) {
+    before += x < warp ? warp_tot[x] : 0;
+    total += warp_tot[x];
+  }
+  int all_more = 0;
+  int64_t my_more = any_more ? cta_excl_scan(more, &all_more) : 0;
+  if (threadIdx.x == 0) s_base = total ? atomicAdd(n_rows, (unsigned long long)(total + all_more)) : 0ull;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    int o = before + at[q];
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+      if ((has >> (2 * q + z)) & 1u) stage[o++] = k[q][z];
+  }
+  __syncthreads();
+  const int64_t first = int64_t(s_base);
+  if (first + total + all_more > bound) {  // cannot be: the bound holds for all weights
+    if (threadIdx.x == 0) atomicOr(status, ST_OVERFLOW);
+    return;
+  }
+  for (int i = threadIdx.x; i < total; i += kWinThreads) keys[first + i] = stage[i];
+  if (more == 0) return;
+  uint64_t* o = keys + first + total + my_more;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const unsigned h = (has >> (2 * q)) & 3u;
+    if (!h) continue;
+    while (w[q]) {
+      const uint32_t code = take_code(w[q]);
+#pragma unroll
+      for (int z = 0; z < 2; ++z)
+        if ((h >> z) & 1u) *o++ = (k[q][z] & ~uint64_t((1 << kCodeBits) - 1)) | code;
+    }
+  }
+}
+
 // Per-file rows, top-down: every window once per file of its rule (the root's
 // once, in its own file), weighted by the rule's per-file weight.  A CTA counts
 // the rows of its tile, claims their places with one atomic (the rows are
@@ -287,6 +374,40 @@ void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, 
     Phase ph(ctx, "seq_headtail", s);
     run_rule_ends(g, ends.as<int4>(), s, true);
   }
+  const int64_t windows = g->info.owned_windows, tokens = int64_t(d.N);
+  if (!per_file && windows > 0 && 3 * kb + kCodeBits <= 64 && tokens <= 3 * windows) {
+    // Rows of one word, weight code and all: a pass moves 16 bytes per row instead
+    // of 24.  The weights of the windows add up to the windows of all files, so a
+    // row per component is at most windows + (tokens - windows) / 4 rows; three
+    // tokens per window is where those rows take no more room than (key, weight)
+    // rows.  100M nested words, 49M windows: the count and the word sort
+    // take 3581 us so and 4131 us with (key, weight) rows.
+    const int64_t bound = windows + std::max<int64_t>(tokens - windows, 0) / 4 + 1;
+    Buf k0(ctx, size_t(bound) * 8, s), k1(ctx, size_t(bound) * 8, s);
+    out.n_dev = Buf(ctx, 8, s);
+    out.n = bound;
+    out.max_runs = windows;
+    out.coded = true;
+    GT_CUDA(cudaMemsetAsync(out.n_dev.p, 0, 8, s));
+    {
+      Phase ph(ctx, "seq_emit", s);
+      Buf wt(ctx, size_t(d.R) * 8, s);
+      run_rule_weights(g, wt.as<uint64_t>(), s);
+      constexpr size_t smem = std::max(sizeof(TileEnds), size_t(2 * kTile) * 8);
+      GT_CUDA(cudaFuncSetAttribute(win_emit_coded_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+      win_emit_coded_kernel<<<unsigned(d.ntiles), kWinThreads, smem, s>>>(
+          d, ends.as<int4>(), wt.as<uint64_t>(), kb, out.n_dev.as<unsigned long long>(), bound, k0.as<uint64_t>(), status);
+      GT_LAUNCH_CHECK();
+    }
+    Phase ph(ctx, "seq_sort", s);
+    Buf rs(ctx, radix_scratch_bytes(bound, false, 0), s);
+    const int hi = kCodeBits + 3 * kb;
+    const bool b = radix_sort_pingpong(k0.as<uint64_t>(), k1.as<uint64_t>(), nullptr, nullptr, 0, bound, kCodeBits, hi,
+                                       hi, hi, rs.p, s, out.n_dev.as<int64_t>());
+    out.keys = std::move(b ? k1 : k0);
+    if (keep_ends) *keep_ends = std::move(ends);
+    return;
+  }
   if (!per_file) {
     // exactly the owned windows (Eq. 1's count, known since load); the pad
     // key fills any rows the emit pass leaves
@@ -343,6 +464,10 @@ void reduce_windows(gt_ctx* ctx, Windows& w, bool per_file, bool output_keys, ui
   if (per_file && w.file_in_key) o.low_bits = 3 * w.kb;
   if (w.n == 0) {
     GT_CUDA(cudaMemsetAsync(rows, 0, 8, s));
+    return;
+  }
+  if (w.coded) {
+    reduce_coded_runs(ctx, w.keys.as<uint64_t>(), w.n, w.n_dev.as<int64_t>(), o, s);
     return;
   }
   // rows that carry files end at *n_dev and hold no pads
@@ -584,8 +709,9 @@ gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s, Buf* 
   Windows w;
   sorted_windows(g, per_file != 0, s, w, rb.status(), keep_ends);
   Phase ph(ctx, "seq_reduce", s);
-  auto* key = static_cast<uint64_t*>(rb.alloc(size_t(w.n) * 8));
-  auto* count = static_cast<uint64_t*>(rb.alloc(size_t(w.n) * 8));
+  const int64_t runs = w.coded ? w.max_runs : w.n;
+  auto* key = static_cast<uint64_t*>(rb.alloc(size_t(runs) * 8));
+  auto* count = static_cast<uint64_t*>(rb.alloc(size_t(runs) * 8));
   int32_t* file = per_file ? static_cast<int32_t*>(rb.alloc(size_t(w.n) * 4)) : nullptr;
   int64_t* len = rb.new_len_slot();
   if (w.reduced) {

@@ -129,6 +129,10 @@ constexpr int kRsSmallItems = 8, kRsLargeItems = 24;  // keys per thread
 // take 261 us at 3.7M and 2909 at 49M, of 8192 rows (one CTA less per SM) 9% and
 // 14% more than of 6144.
 constexpr int64_t kRsLargeRows = int64_t(1) << 20;
+// 64-bit keys without values: tiles of 8192 rows from here on (1.4M rows 124 us
+// against 117 with tiles of 6144, 7.9M 370 against 391, 49M 1941 against 2128).
+constexpr int kRsKeyItems = 32;
+constexpr int64_t kRsKeyRows = int64_t(1) << 22;
 
 struct RadixPasses {
   int shift[kRsMaxPasses];
@@ -383,7 +387,8 @@ struct RadixScratch {
   size_t zero_bytes;
 };
 
-int radix_items(int64_t n) {
+int radix_items(int64_t n, bool keys64) {
+  if (keys64 && n >= kRsKeyRows) return kRsKeyItems;
   const int64_t p = t_call_ctx ? t_call_ctx->param("radix_items", kRsSmallItems) : kRsSmallItems;
   return p == 16 || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
 }
@@ -423,6 +428,9 @@ void launch_scatter_any(const K* ka, K* kb, const void* va, void* vb, int64_t n,
                         int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
   if (!radix_narrow(n))
     launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+  else if (sizeof(K) == 8 && VB == 0 && items == kRsKeyItems)
+    launch_scatter<K, VB, sizeof(K) == 8 && VB == 0 ? kRsKeyItems : kRsLargeItems, uint32_t>(
+        ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
   else if (items == kRsSmallItems)
     launch_scatter<K, VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
   else
@@ -464,8 +472,8 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
 }
 
 size_t radix_scratch_bytes(int64_t n, bool, int) {
-  // for the smaller tile: the most look-back words of the two
-  return radix_layout(n, radix_narrow(n) ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
+  // for the smallest tile that a sort of n rows may take
+  return radix_layout(n, n < kRsLargeRows ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
 }
 
 namespace {
@@ -476,7 +484,7 @@ bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_
   if (n <= 0) return false;
   const RadixPasses ps = radix_plan(begin_a, end_a, begin_b, end_b);
   if (ps.n == 0) return false;
-  const int items = radix_narrow(n) ? radix_items(n) : kRsLargeItems;
+  const int items = radix_narrow(n) ? radix_items(n, sizeof(K) == 8 && value_bytes == 0) : kRsLargeItems;
   RadixScratch rs;
   radix_layout(n, items, ps.n, scratch, &rs);
   GT_CUDA(cudaMemsetAsync(scratch, 0, rs.zero_bytes, s));

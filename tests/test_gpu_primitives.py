@@ -182,3 +182,27 @@ def test_ranked_runs(ctx, F, V):
                 assert np.array_equal(got, want)
     finally:
         B.gt_free_grammar(gh)
+
+
+@pytest.mark.parametrize("V", [50, 2 ** 20, 2 ** 20 + 1])
+@pytest.mark.parametrize("w", [1, 3, 4, 192, 255, 256, 0xfff3, (1 << 20) + 0xabcde])
+@pytest.mark.parametrize("long_root", [True, False])
+def test_weight_components(ctx, w, V, long_root):
+    """3-word rows whose weight is part of the key's word (vocabularies up to 2^20, at most three
+    tokens per window: the long root) and beside it: a rule x x x of weight w, used by doubling rules,
+    x the largest word, so that all bits of the key are set where V is a power of two."""
+    x, top = V - 1, w.bit_length() - 1
+    rules = [[x, x, x]] + [[V + k, V + k] for k in range(1, top + 1)]  # rule k + 1 = 2^k times x x x
+    uses = [V + 1 + k for k in range(top + 1) if (w >> k) & 1]
+    rng = np.random.default_rng(w)
+    n = 100 + (2 * w if long_root else 0)
+    root = rng.integers(0, V, n).tolist()
+    for i, u in enumerate(uses):
+        root.insert(3 * i + 1, u)
+    g = grammar_from_rules(V, [root] + rules, [0, 40, len(root)])
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        for got, want in zip(take(B.gt_sequence_count(gh, 0), "key", "count"), oracle.sequence_count(g, 0)):
+            assert np.array_equal(got, want)
+    finally:
+        B.gt_free_grammar(gh)
