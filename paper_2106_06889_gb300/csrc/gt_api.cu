@@ -468,7 +468,7 @@ gt_result* sort_from_counts(gt_grammar* g, const uint64_t* wc, int order, cudaSt
     count_keys_kernel<<<gt::grid_for(V, threads, cap), threads, 0, s>>>(wc, V, N, k0.as<uint32_t>(),
                                                                         v0.as<uint32_t>());
     GT_LAUNCH_CHECK();
-    if (!gt::radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), v0.p, v1.p, 4, V, bits_for(N), rs.p, s)) {
+    if (!gt::radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), v0.p, v1.p, 4, V, 0, bits_for(N), rs.p, s)) {
       std::swap(k0, k1);
       std::swap(v0, v1);
     }

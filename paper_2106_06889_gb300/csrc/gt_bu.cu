@@ -531,17 +531,48 @@ __global__ void local_pack_kernel(int32_t F, const int64_t* __restrict__ slot_of
 
 // ---- the files' words, expanded --------------------------------------------------
 
+// last file f in [lo, hi] whose first word is at or before position p
+__device__ __forceinline__ int32_t file_from(const int64_t* __restrict__ first, int32_t lo, int32_t hi, int64_t p) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (first[mid] <= p) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 // words[0, N): the expansion of the root, files back to back.  A tile of kRowTile
 // root symbols per CTA in ticket order, kRowItems consecutive ones per thread; a
-// tile's first word comes from a bounded look-back over the tiles' lengths.
+// tile's first word comes from a bounded look-back over the tiles' lengths.  The
+// first kExpandWords words of a tile pass through shared memory, so that they are
+// written dense (a thread's words are consecutive: direct stores touch a sector
+// per lane); a tile that expands further writes the rest from its threads.
+// The references that fit are listed first and walked by all threads in turn, each
+// at its place in the stage, which holds the rule till then: bound by the latency of
+// the walks (dependent loads of short rule bodies), and a thread's own references
+// one after the other made the longest chain.
+//
+// file_bits >= 0: words[p] is word << file_bits | file instead.
+constexpr int kExpandWords = 6 * 1024;
+
+template <bool kFiles>
 __global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGrammar d, int64_t tiles,
                                                                   unsigned long long* __restrict__ look,
+                                                                  const int64_t* __restrict__ first, int file_bits,
                                                                   int32_t* __restrict__ words,
                                                                   unsigned* __restrict__ status) {
   __shared__ int64_t s_warp[kRowThreads / 32];
   __shared__ int64_t s_item, s_prefix;
+  __shared__ int32_t s_file[2];
+  __shared__ int32_t s_words[kExpandWords];
+  __shared__ uint16_t s_list[kRowTile];  // first words of the listed references
+  __shared__ int s_staged, s_refs;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_item = int64_t(atomicAdd(look + tiles, 1ull));
+  if (tid == 0) {
+    s_item = int64_t(atomicAdd(look + tiles, 1ull));
+    s_staged = kExpandWords;
+    s_refs = 0;
+  }
   __syncthreads();
   const int64_t item = s_item, j0 = item * kRowTile + tid * kRowItems;
   int32_t sy[kRowItems];
@@ -567,35 +598,63 @@ __global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGramm
     before += w < warp ? s_warp[w] : 0;
     total += s_warp[w];
   }
+  if (tid == 0) publish_aggregate(look, item, uint64_t(total));
+  int64_t o = before;
+#pragma unroll
+  for (int k = 0; k < kRowItems; ++k) {
+    const bool fits = sy[k] >= 0 && ln[k] > 0 && o + ln[k] <= kExpandWords, ref = fits && sy[k] >= d.V;
+    if (fits) s_words[o] = sy[k];
+    const unsigned m = __ballot_sync(0xffffffffu, ref);
+    int at = 0;
+    if (lane == 0 && m) at = atomicAdd(&s_refs, __popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (ref) s_list[at + __popc(m & ((1u << lane) - 1u))] = uint16_t(o);
+    o += ln[k];
+  }
+  __syncthreads();
+  for (int i = tid; i < s_refs; i += kRowThreads) {
+    int q = s_list[i];
+    walk_rule(d, s_words[q] - d.V, [&](int32_t w) { s_words[q++] = w; });
+  }
   if (warp == 0) {
-    if (lane == 0) publish_aggregate(look, item, uint64_t(total));
     __syncwarp();
     const int64_t p = warp_look_back(look, item, uint64_t(total), status);
     if (lane == 0) s_prefix = p < 0 ? 0 : p;
   }
   __syncthreads();
-  int64_t o = s_prefix + before;
+  const int64_t base = s_prefix;
+  if (kFiles) {
+    if (tid < 2 && total > 0)
+      s_file[tid] = int32_t(upper_bound_dev(first, int64_t(d.F) + 1, tid ? base + total - 1 : base) - 1);
+    __syncthreads();
+  }
+  if (total > kExpandWords) {  // the symbols from the first one on that does not fit
+    o = before;
 #pragma unroll
-  for (int k = 0; k < kRowItems; ++k) {
-    if (sy[k] < 0) continue;
-    if (sy[k] < d.V) {
-      words[o] = sy[k];
-    } else {
-      int64_t q = o;
-      walk_rule(d, sy[k] - d.V, [&](int32_t w) { words[q++] = w; });
+    for (int k = 0; k < kRowItems; ++k) {
+      if (sy[k] >= 0 && o + ln[k] > kExpandWords) {
+        if (o <= kExpandWords) s_staged = int(o);
+        // a symbol's words are in one file
+        const int32_t f = kFiles && ln[k] > 0 ? file_from(first, s_file[0], s_file[1], base + o) : 0;
+        if (sy[k] < d.V) {
+          words[base + o] = kFiles ? int32_t(uint32_t(sy[k]) << file_bits | uint32_t(f)) : sy[k];
+        } else {
+          int64_t q = base + o;
+          walk_rule(d, sy[k] - d.V, [&](int32_t w) {
+            words[q++] = kFiles ? int32_t(uint32_t(w) << file_bits | uint32_t(f)) : w;
+          });
+        }
+      }
+      o += ln[k];
     }
-    o += ln[k];
+    __syncthreads();
   }
-}
-
-// last file f in [lo, hi] whose first word is at or before position p
-__device__ __forceinline__ int32_t file_from(const int64_t* __restrict__ first, int32_t lo, int32_t hi, int64_t p) {
-  while (lo < hi) {
-    const int32_t mid = (lo + hi + 1) >> 1;
-    if (first[mid] <= p) lo = mid;
-    else hi = mid - 1;
+  const int staged = int(total < s_staged ? total : int64_t(s_staged));
+  for (int i = tid; i < staged; i += kRowThreads) {
+    const int32_t w = s_words[i];
+    words[base + i] =
+        kFiles ? int32_t(uint32_t(w) << file_bits | uint32_t(file_from(first, s_file[0], s_file[1], base + i))) : w;
   }
-  return lo;
 }
 
 // cnt[f] = windows of file f (0 for f = F)
@@ -617,8 +676,9 @@ __global__ void __launch_bounds__(kRowThreads) token_files_kernel(int64_t N, con
   }
 }
 
-// Words of every file back to back, and each file's first word (F + 1 offsets).
-void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s) {
+// Words of every file back to back (word << file_bits | file where that is not
+// negative), and each file's first word (F + 1 offsets).
+void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s, int file_bits = -1) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int64_t tiles = (d.root_len + kRowTile - 1) / kRowTile;
@@ -631,8 +691,8 @@ void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s) {
   exclusive_scan_i64(len.as<int64_t>(), first.as<int64_t>(), d.F + 1, sc.p, s);
   if (tiles == 0) return;
   GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(tiles + 1) * 8, s));
-  expand_root_kernel<<<unsigned(tiles), kRowThreads, 0, s>>>(d, tiles, look.as<unsigned long long>(),
-                                                             words.as<int32_t>(), status_word());
+  (file_bits >= 0 ? expand_root_kernel<true> : expand_root_kernel<false>)<<<unsigned(tiles), kRowThreads, 0, s>>>(
+      d, tiles, look.as<unsigned long long>(), first.as<int64_t>(), file_bits, words.as<int32_t>(), status_word());
   GT_LAUNCH_CHECK();
 }
 
@@ -713,19 +773,32 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
       GT_CUDA(cudaMemsetAsync(out.total.p, 0, 8, s));
       return;
     }
-    Buf words, first, files(ctx, size_t(N) * 4, s), w1(ctx, size_t(N) * 4, s), f1(ctx, size_t(N) * 4, s);
+    Buf words, first, w1(ctx, size_t(N) * 4, s), rs(ctx, radix_scratch_bytes(N, true, 4), s);
+    const int vbits = bits_for(std::max(d.V - 1, 1)), fbits = bits_for(std::max(d.F - 1, 1));
+    RunOut o;
+    o.pay = out.pay.as<uint64_t>();
+    o.rows = out.total.as<int64_t>();
+    if (vbits + fbits < 32) {
+      // a row is one 32-bit word, sorted on its word bits: 8 bytes per row and pass
+      // instead of 16 (2,000 files, 25M words: 1305 -> 1168 us)
+      expand_files(g, words, first, s, fbits);
+      const bool b = radix_sort_pingpong32(words.as<uint32_t>(), w1.as<uint32_t>(), nullptr, nullptr, 0, N, fbits,
+                                           fbits + vbits, rs.p, s);
+      o.low_bits = fbits;
+      o.file = out.word.as<int32_t>();  // the high bits
+      o.word = out.file.as<int32_t>();  // the low bits
+      reduce_runs32(ctx, (b ? w1 : words).as<uint32_t>(), N, o, s);
+      return;
+    }
+    Buf files(ctx, size_t(N) * 4, s), f1(ctx, size_t(N) * 4, s);
     expand_files(g, words, first, s);
     token_files_kernel<<<unsigned((N + kRowTile - 1) / kRowTile), kRowThreads, 0, s>>>(N, first.as<int64_t>(), d.F,
                                                                                       files.as<uint32_t>());
     GT_LAUNCH_CHECK();
-    Buf rs(ctx, radix_scratch_bytes(N, true, 4), s);
-    const bool b = radix_sort_pingpong32(words.as<uint32_t>(), w1.as<uint32_t>(), files.p, f1.p, 4, N,
-                                         bits_for(std::max(d.V - 1, 1)), rs.p, s);
-    RunOut o;
+    const bool b =
+        radix_sort_pingpong32(words.as<uint32_t>(), w1.as<uint32_t>(), files.p, f1.p, 4, N, 0, vbits, rs.p, s);
     o.word = out.word.as<int32_t>();
     o.file = out.file.as<int32_t>();
-    o.pay = out.pay.as<uint64_t>();
-    o.rows = out.total.as<int64_t>();
     reduce_file_runs(ctx, (b ? w1 : words).as<uint32_t>(), (b ? f1 : files).as<uint32_t>(), N, nullptr, o, s);
     return;
   }
@@ -792,7 +865,7 @@ void rows_by_file(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   wr.cnt = Buf(ctx, size_t(n) * 8, s);
   if (n == 0) return;
   Buf f1(ctx, size_t(n) * 4, s), p1(ctx, size_t(n) * 8, s), rs(ctx, radix_scratch_bytes(n, true, 8), s);
-  if (radix_sort_pingpong32(wr.file.as<uint32_t>(), f1.as<uint32_t>(), wr.pay.p, p1.p, 8, n,
+  if (radix_sort_pingpong32(wr.file.as<uint32_t>(), f1.as<uint32_t>(), wr.pay.p, p1.p, 8, n, 0,
                             bits_for(std::max(g->d.F - 1, 1)), rs.p, s, nd)) {
     std::swap(wr.file, f1);
     std::swap(wr.pay, p1);

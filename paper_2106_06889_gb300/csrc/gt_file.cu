@@ -1629,7 +1629,7 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
         topk_keys_kernel<uint32_t><<<grid_for(bound, threads, cap), threads, 0, s>>>(
             word, cnt, tv_off_in, F, max_count, cbits, k0.as<uint32_t>(), i0.as<uint32_t>());
         GT_LAUNCH_CHECK();
-        b = radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), i0.p, i1.p, 4, bound, kbits, rs.p, s, total);
+        b = radix_sort_pingpong32(k0.as<uint32_t>(), k1.as<uint32_t>(), i0.p, i1.p, 4, bound, 0, kbits, rs.p, s, total);
       } else {
         topk_keys_kernel<uint64_t><<<grid_for(bound, threads, cap), threads, 0, s>>>(
             word, cnt, tv_off_in, F, max_count, cbits, k0.as<uint64_t>(), i0.as<uint32_t>());

@@ -585,7 +585,7 @@ struct RunOut {
   int32_t* file = nullptr;    // the run's file: the key's high part, or its fkeys value
   uint64_t* count = nullptr;  // sum of the values
   uint32_t* mult = nullptr;   // the same in 32 bits
-  uint64_t* pay = nullptr;    // rest << 32 | sum (both of at most 32 bits)
+  uint64_t* pay = nullptr;    // (key above low_bits) << 32 | sum (both of at most 32 bits)
   int64_t* off = nullptr;     // the run's first row (vals == nullptr); off[runs] = *off_end, or the rows
   const int64_t* off_end = nullptr;
   int64_t* rows = nullptr;    // number of runs (always given)
@@ -593,6 +593,8 @@ struct RunOut {
 };
 void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const uint32_t* vals, int64_t n,
                  const int64_t* n_dev, uint64_t key_pad, const RunOut& out, cudaStream_t s);
+// rows that are their 32-bit keys
+void reduce_runs32(gt_ctx* ctx, const uint32_t* keys, int64_t n, const RunOut& out, cudaStream_t s);
 // rows (key << kCodeBits | code of a weight): runs of equal keys
 void reduce_coded_runs(gt_ctx* ctx, const uint64_t* keys, int64_t n, const int64_t* n_dev, const RunOut& out,
                        cudaStream_t s);
@@ -615,10 +617,10 @@ size_t radix_scratch_bytes(int64_t n, bool with_values, int value_bytes);
 bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
                          int begin_a, int end_a, int begin_b, int end_b, void* scratch, cudaStream_t s,
                          const int64_t* n_dev = nullptr);
-// 32-bit keys on bits [0, bits): two thirds of the bytes per row, and of the
+// 32-bit keys on bits [begin, end): two thirds of the bytes per row, and of the
 // shared-memory traffic that bounds a pass.
 bool radix_sort_pingpong32(uint32_t* keys_a, uint32_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
-                           int bits, void* scratch, cudaStream_t s, const int64_t* n_dev = nullptr);
+                           int begin, int end, void* scratch, cudaStream_t s, const int64_t* n_dev = nullptr);
 // The same on bits [begin_bit, end_bit) of 64-bit keys.  Results land in keys_out / vals_out
 // (copied there after an even number of passes).  keys_in / vals_in are clobbered.
 void radix_sort_u64(uint64_t* keys_in, uint64_t* keys_out, void* vals_in, void* vals_out, int value_bytes,

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     const uint64_t key = s_key[r];
     const int64_t o = o0 + r;
     if (out.key) out.key[o] = to_output_key(out.low_bits ? key & ((uint64_t(1) << out.low_bits) - 1) : key, out.kb);
-    if (out.pay) reinterpret_cast<uint32_t*>(out.pay)[2 * o + 1] = uint32_t(key);
+    if (out.pay) reinterpret_cast<uint32_t*>(out.pay)[2 * o + 1] = uint32_t(key >> out.low_bits);
     if (out.hi) out.hi[o] = key >> out.low_bits;
     if (out.file) out.file[o] = kFile ? int32_t(s_file[r]) : int32_t(key >> out.low_bits);
     if (out.word) out.word[o] = int32_t(out.low_bits ? key & ((uint64_t(1) << out.low_bits) - 1) : key);
@@ -265,6 +265,10 @@ void reduce_runs(gt_ctx* ctx, const uint64_t* keys, const uint64_t* fkeys, const
   if (fkeys) launch_runs<kKeyFileVal>(ctx, keys, fkeys, nullptr, n, n_dev, key_pad, out, s);
   else if (vals) launch_runs<kKeyVal>(ctx, keys, nullptr, vals, n, n_dev, key_pad, out, s);
   else launch_runs<kKeyOnly>(ctx, keys, nullptr, nullptr, n, n_dev, key_pad, out, s);
+}
+
+void reduce_runs32(gt_ctx* ctx, const uint32_t* keys, int64_t n, const RunOut& out, cudaStream_t s) {
+  launch_runs<kKeyOnly>(ctx, keys, nullptr, nullptr, n, nullptr, ~uint32_t(0), out, s);
 }
 
 void reduce_coded_runs(gt_ctx* ctx, const uint64_t* keys, int64_t n, const int64_t* n_dev, const RunOut& out,

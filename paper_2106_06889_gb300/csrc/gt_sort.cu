@@ -129,7 +129,7 @@ constexpr int kRsSmallItems = 8, kRsLargeItems = 24;  // keys per thread
 // take 261 us at 3.7M and 2909 at 49M, of 8192 rows (one CTA less per SM) 9% and
 // 14% more than of 6144.
 constexpr int64_t kRsLargeRows = int64_t(1) << 20;
-// 64-bit keys without values: tiles of 8192 rows from here on (1.4M rows 124 us
+// Keys without values: tiles of 8192 rows from here on (64 bits: 1.4M rows 124 us
 // against 117 with tiles of 6144, 7.9M 370 against 391, 49M 1941 against 2128).
 constexpr int kRsKeyItems = 32;
 constexpr int64_t kRsKeyRows = int64_t(1) << 22;
@@ -387,8 +387,8 @@ struct RadixScratch {
   size_t zero_bytes;
 };
 
-int radix_items(int64_t n, bool keys64) {
-  if (keys64 && n >= kRsKeyRows) return kRsKeyItems;
+int radix_items(int64_t n, bool keys_only) {
+  if (keys_only && n >= kRsKeyRows) return kRsKeyItems;
   const int64_t p = t_call_ctx ? t_call_ctx->param("radix_items", kRsSmallItems) : kRsSmallItems;
   return p == 16 || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
 }
@@ -428,8 +428,8 @@ void launch_scatter_any(const K* ka, K* kb, const void* va, void* vb, int64_t n,
                         int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
   if (!radix_narrow(n))
     launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
-  else if (sizeof(K) == 8 && VB == 0 && items == kRsKeyItems)
-    launch_scatter<K, VB, sizeof(K) == 8 && VB == 0 ? kRsKeyItems : kRsLargeItems, uint32_t>(
+  else if (VB == 0 && items == kRsKeyItems)
+    launch_scatter<K, VB, VB == 0 ? kRsKeyItems : kRsLargeItems, uint32_t>(
         ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
   else if (items == kRsSmallItems)
     launch_scatter<K, VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
@@ -484,7 +484,7 @@ bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_
   if (n <= 0) return false;
   const RadixPasses ps = radix_plan(begin_a, end_a, begin_b, end_b);
   if (ps.n == 0) return false;
-  const int items = radix_narrow(n) ? radix_items(n, sizeof(K) == 8 && value_bytes == 0) : kRsLargeItems;
+  const int items = radix_narrow(n) ? radix_items(n, value_bytes == 0) : kRsLargeItems;
   RadixScratch rs;
   radix_layout(n, items, ps.n, scratch, &rs);
   GT_CUDA(cudaMemsetAsync(scratch, 0, rs.zero_bytes, s));
@@ -518,8 +518,8 @@ bool radix_sort_pingpong(uint64_t* keys_a, uint64_t* keys_b, void* vals_a, void*
 }
 
 bool radix_sort_pingpong32(uint32_t* keys_a, uint32_t* keys_b, void* vals_a, void* vals_b, int value_bytes, int64_t n,
-                           int bits, void* scratch, cudaStream_t s, const int64_t* n_dev) {
-  return radix_sort_any<uint32_t>(keys_a, keys_b, vals_a, vals_b, value_bytes, n, 0, bits, bits, bits, scratch, s,
+                           int begin, int end, void* scratch, cudaStream_t s, const int64_t* n_dev) {
+  return radix_sort_any<uint32_t>(keys_a, keys_b, vals_a, vals_b, value_bytes, n, begin, end, end, end, scratch, s,
                                   n_dev);
 }
 

@@ -206,3 +206,29 @@ def test_weight_components(ctx, w, V, long_root):
             assert np.array_equal(got, want)
     finally:
         B.gt_free_grammar(gh)
+
+
+@pytest.mark.parametrize("F,V", [(65, 6), (300, 70_000), (2_000, 200_000), (2_100, 2_000_000)])
+def test_word_rows(ctx, F, V):
+    """Term vectors and inverted index of more than 64 files from the expanded files: a row of a word
+    and its file in 32 bits, or (the last) in two words; one file that expands past a tile's stage
+    from few symbols, files of 0 and 1 words."""
+    rng = np.random.default_rng(F + V)
+    lens = rng.integers(0, 50, F)
+    lens[:3] = [0, 1, 9000]
+    n = int(lens.sum())
+    toks = np.where(rng.random(n) < 0.7, rng.integers(0, 5, n), rng.integers(0, V, n)).astype(np.int32)
+    toks[1:9001] = np.tile(toks[1:10], 1000)
+    toks[-1] = V - 1
+    g = sequitur(toks, lens, V)
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        tv, ii = B.gt_run_batch(ctx, [(gh, B.GT_Q_TERM_VECTOR, 0, None), (gh, B.GT_Q_INVERTED_INDEX, 0, None)])
+        for got, want in zip(take(tv, "offsets", "word", "count"), oracle.term_vector(g, 0)):
+            assert np.array_equal(got, want)
+        for got, want in zip(take(ii, "offsets", "file"), oracle.inverted_index(g)):
+            assert np.array_equal(got, want)
+        for got, want in zip(take(B.gt_term_vector(gh, 2), "offsets", "word", "count"), oracle.term_vector(g, 2)):
+            assert np.array_equal(got, want)
+    finally:
+        B.gt_free_grammar(gh)
