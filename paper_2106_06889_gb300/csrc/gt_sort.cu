@@ -141,9 +141,12 @@ struct RadixPasses {
 };
 
 // Digit counts of every pass in one read of the keys: counts[p * 256 + d].
-// Bound by its shared-memory atomics (one per key and pass).
+// Bound by its shared-memory atomics (one per key and pass), and by frequent digits,
+// whose atomics in a warp go one after the other: kRhSplit counters per digit, by
+// lane, shorten those chains (49M 60-bit keys: 175 -> 152 us).
 constexpr int kRhThreads = 512;
 constexpr int kRhItems = 4;
+constexpr int kRhSplit = 4;
 
 template <class K>
 __global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const K* __restrict__ keys, int64_t n_max,
@@ -151,8 +154,9 @@ __global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const K* __restr
                                                                 const __grid_constant__ RadixPasses ps,
                                                                 unsigned long long* __restrict__ counts) {
   const int64_t n = n_dev ? min(*n_dev, n_max) : n_max;
-  __shared__ uint32_t h[kRsMaxPasses * kRsBins];
-  for (int i = threadIdx.x; i < ps.n * kRsBins; i += kRhThreads) h[i] = 0;
+  __shared__ __align__(16) uint32_t h[kRsMaxPasses * kRsBins * kRhSplit];
+  for (int i = threadIdx.x; i < ps.n * kRsBins * kRhSplit; i += kRhThreads) h[i] = 0;
+  const uint32_t part = threadIdx.x & (kRhSplit - 1);
   __syncthreads();
   constexpr int64_t kStep = int64_t(kRhThreads) * kRhItems;
   for (int64_t b = blockIdx.x * kStep; b < n; b += gridDim.x * kStep) {
@@ -167,12 +171,17 @@ __global__ void __launch_bounds__(kRhThreads) radix_hist_kernel(const K* __restr
       const int shift = ps.shift[p];
 #pragma unroll
       for (int j = 0; j < kRhItems; ++j)
-        if (b + j * kRhThreads + threadIdx.x < n) atomicAdd(&h[p * kRsBins + (uint32_t(k[j] >> shift) & mask)], 1u);
+        if (b + j * kRhThreads + threadIdx.x < n) 
+          atomicAdd(&h[(p * kRsBins + (uint32_t(k[j] >> shift) & mask)) * kRhSplit + part], 1u);
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < ps.n * kRsBins; i += kRhThreads)
-    if (h[i]) atomicAdd(&counts[i], (unsigned long long)(h[i]));
+  for (int i = threadIdx.x; i < ps.n * kRsBins; i += kRhThreads) {
+    uint32_t c = 0;
+#pragma unroll
+    for (int q = 0; q < kRhSplit; ++q) c += h[i * kRhSplit + q];
+    if (c) atomicAdd(&counts[i], (unsigned long long)(c));
+  }
 }
 
 // Look-back words of a pass: one per (tile, digit), state in the top two bits
