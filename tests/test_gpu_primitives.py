@@ -208,13 +208,15 @@ def test_weight_components(ctx, w, V, long_root):
         B.gt_free_grammar(gh)
 
 
-@pytest.mark.parametrize("F,V", [(65, 6), (300, 70_000), (2_000, 200_000), (2_100, 2_000_000)])
-def test_word_rows(ctx, F, V):
+@pytest.mark.parametrize("F,V,per_file", [(65, 6, 50), (300, 70_000, 50), (2_000, 200_000, 50), (2_100, 2_000_000, 50),
+                                          (300, 70_000, 16_000), (70, 2 ** 25, 60_000)])
+def test_word_rows(ctx, F, V, per_file):
     """Term vectors and inverted index of more than 64 files from the expanded files: a row of a word
     and its file in 32 bits, or (the last) in two words; one file that expands past a tile's stage
-    from few symbols, files of 0 and 1 words."""
+    from few symbols, files of 0 and 1 words; the two largest have a root of more than 2^20 symbols,
+    whose references to short rules are expanded from the rules' ends."""
     rng = np.random.default_rng(F + V)
-    lens = rng.integers(0, 50, F)
+    lens = rng.integers(0, per_file, F)
     lens[:3] = [0, 1, 9000]
     n = int(lens.sum())
     toks = np.where(rng.random(n) < 0.7, rng.integers(0, 5, n), rng.integers(0, V, n)).astype(np.int32)
