@@ -41,22 +41,30 @@ __device__ __forceinline__ uint32_t take_code(uint32_t& w) {
 // instruction issue in the sort that ranks 32 rows per call: written so that the
 // bit's predicate both votes and complements (a select of the ballot or its
 // complement in C++ takes 4 to 8% more of a scatter pass).
-__device__ __forceinline__ unsigned warp_digit_peers(uint32_t d, unsigned active) {
+__device__ __forceinline__ unsigned digit_bit_peers(uint32_t d, int b, unsigned peers) {
+  asm volatile(
+      "{\n\t"
+      ".reg .pred p;\n\t"
+      ".reg .b32 t;\n\t"
+      "and.b32 t, %1, %2;\n\t"
+      "setp.ne.u32 p, t, 0;\n\t"
+      "vote.sync.ballot.b32 t, p, 0xffffffff;\n\t"
+      "@!p not.b32 t, t;\n\t"
+      "and.b32 %0, %0, t;\n\t"
+      "}"
+      : "+r"(peers)
+      : "r"(d), "r"(1 << b));
+  return peers;
+}
+
+// mask (uniform): the digit's bits; the ballots of bits 6 and 7 are skipped where it has none.
+__device__ __forceinline__ unsigned warp_digit_peers(uint32_t d, unsigned active, uint32_t mask = 0xffu) {
   unsigned peers = active;
 #pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    asm volatile(
-        "{\n\t"
-        ".reg .pred p;\n\t"
-        ".reg .b32 t;\n\t"
-        "and.b32 t, %1, %2;\n\t"
-        "setp.ne.u32 p, t, 0;\n\t"
-        "vote.sync.ballot.b32 t, p, 0xffffffff;\n\t"
-        "@!p not.b32 t, t;\n\t"
-        "and.b32 %0, %0, t;\n\t"
-        "}"
-        : "+r"(peers)
-        : "r"(d), "r"(1 << b));
+  for (int b = 0; b < 6; ++b) peers = digit_bit_peers(d, b, peers);
+  if (mask & 0xc0u) {
+    peers = digit_bit_peers(d, 6, peers);
+    if (mask & 0x80u) peers = digit_bit_peers(d, 7, peers);
   }
   return peers;
 }
