@@ -658,13 +658,13 @@ def many_files(B, ctx, reps=3):
 
 def sequence_paths(B, ctx, g, stream, reps=3):
     """The global 3-word count by the one-row-per-window LSD radix sort (the
-    default, with scatter tiles chosen by the rows and of 4096 keys) and by the
+    default, with scatter tiles chosen by the rows and large at any size) and by the
     sample-sort buckets, on the same grammar."""
     import torch
     gh = B.gt_load_grammar(ctx, g, stream)
     out = {}
     with torch.cuda.stream(stream):
-        for name, path, items in (("bucketed", 2, 8), ("radix_sort_tile4096", 1, 16), ("radix_sort", 1, 8)):
+        for name, path, items in (("bucketed", 2, 8), ("radix_sort_large_tiles", 1, 16), ("radix_sort", 1, 8)):
             B.gt_set_param(ctx, "seq_path", path)
             B.gt_set_param(ctx, "radix_items", items)
             B.gt_free_result(B.gt_sequence_count(gh, 0, stream))

@@ -357,8 +357,9 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *                   bucket path (2..3072, default 3072); fuller buckets are
  *                   sorted in global memory.
  *   "radix_items"   keys per thread of the LSD radix sort's scatter passes:
- *                   8 (default): tiles of 2048 keys below 2^20 rows and of
- *                   6144 keys from there on; 16: always tiles of 6144.
+ *                   8 (default): tiles of 2048 keys below 2^20 rows, of 6144
+ *                   from there on (of 8192 for keys without values from 2^22
+ *                   on); 16: no tiles of 2048.
  *                   GT_EINVAL otherwise.  Same results.
  *   "radix_prefetch" accepted, without effect: it selected a persistent
  *                   scatter that was slower than one CTA per tile.
