@@ -143,7 +143,8 @@ def kernel_bytes(workload: str, info: dict, out: dict) -> dict:
     every row once per launch (24 B), sg_reduce_kernel reads them (12 B) and
     writes the distinct 3-grams (16 B each).  Where the sort's rows hold their
     weight in the key's word (num_words up to 2^20 and at most three tokens per
-    window), radix_downsweep_kernel<0> moves 16 B per row."""
+    window), radix_downsweep_kernel<0> moves 16 B per row and reduce_runs_kernel
+    reads 8 B per row."""
     G, V = info["num_syms"], info["num_words"]
     root_len = out["root_len"]
     if workload == "multi64_50m":
@@ -153,9 +154,10 @@ def kernel_bytes(workload: str, info: dict, out: dict) -> dict:
                 "wc_partition": ("wc_partition_kernel", 4 * G)}
     U = info["owned_windows"]
     coded = V <= 1 << 20 and 0 < info.get("num_tokens", 0) <= 3 * U
+    out_bytes = 16 * out["distinct_3grams"]
     return {"radix_pass": ("radix_downsweep_kernel<0>", 16 * U) if coded else ("radix_downsweep_kernel<4>", 24 * U),
             "seq_scatter": ("sg_scatter_kernel", 24 * U),
-            "seq_reduce": ("sg_reduce_kernel", 12 * U + 16 * out["distinct_3grams"]),
+            "seq_reduce": ("reduce_runs_kernel", 8 * U + out_bytes) if coded else ("sg_reduce_kernel", 12 * U + out_bytes),
             "wc_partition": ("wc_partition_kernel", 4 * G)}
 
 
