@@ -28,10 +28,11 @@
  *     list, a row count past its bound, an invalid symbol) are recorded in a
  *     device status word and reported by gt_sync / gt_result_view.  The
  *     only waits inside kernels are decoupled look-backs (scans, the radix
- *     sort, the reduction of equal keys, the global sequence count's bucket
- *     path and the inverted index: a CTA polls the published totals of the
- *     items taken before its own); each gives up after a bounded number of
- *     polls with GT_ETIMEOUT.
+ *     sort, the reduction of equal keys, the root expansion, the global
+ *     sequence count's bucket path and the inverted index: a CTA polls the
+ *     published totals of the items taken before its own), each bounded.  When
+ *     one of the first four runs out the CTA works the missing total out itself
+ *     and the result is right; the other two give up with GT_ETIMEOUT.
  *   - There is no CPU fallback: if no usable sm_103a device is present,
  *     gt_create fails with GT_ECUDA.
  */
@@ -363,6 +364,10 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *                   GT_EINVAL otherwise.  Same results.
  *   "radix_prefetch" accepted, without effect: it selected a persistent
  *                   scatter that was slower than one CTA per tile.
+ *   "look_back_polls" polls of an unpublished total before a scan, sort,
+ *                   reduction or root expansion works it out itself: 0 to 2^22
+ *                   (default; at least 0.25 s).  GT_EINVAL otherwise.  Same
+ *                   results.
  *   "file_strategy" per-file analytics (term vector, inverted index, per-file
  *                   sequence count, ranked index): 0 (default) picks top-down
  *                   for at most 64 files and bottom-up otherwise (the paper's

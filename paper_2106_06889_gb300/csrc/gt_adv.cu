@@ -22,9 +22,9 @@ namespace {
 // Rows of the pairs of every 3-gram: (a, b) and (a, c) of key a|b|c with its
 // count, the words kb bits each.  *rows counts them; the files' last pairs follow.
 __global__ void cooc_rows_kernel(const uint64_t* __restrict__ key3, const uint64_t* __restrict__ cnt3,
-                                 const int64_t* __restrict__ n3_dev, int kb, uint64_t* __restrict__ keys,
+                                 const int64_t* __restrict__ n3_dev, int64_t n3_max, int kb, uint64_t* __restrict__ keys,
                                  uint32_t* __restrict__ vals, unsigned long long* __restrict__ rows) {
-  const int64_t n3 = *n3_dev;
+  const int64_t n3 = min(*n3_dev, n3_max);  // the bucket path may give up
   const uint64_t m = (uint64_t(1) << 21) - 1;
   if (blockIdx.x == 0 && threadIdx.x == 0) *rows = 2 * (unsigned long long)n3;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n3; i += int64_t(gridDim.x) * blockDim.x) {
@@ -97,7 +97,7 @@ gt_result* run_cooccurrence(gt_grammar* g, cudaStream_t s) {
       }
       const int threads = 256, cap = ctx->num_sms * 16;
       cooc_rows_kernel<<<grid_for(U, threads, cap), threads, 0, s>>>(
-          static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, kb, keys.as<uint64_t>(), vals.as<uint32_t>(),
+          static_cast<uint64_t*>(k3), static_cast<uint64_t*>(c3), n3, U, kb, keys.as<uint64_t>(), vals.as<uint32_t>(),
           rows.as<unsigned long long>());
       GT_LAUNCH_CHECK();
       file_last_pair_kernel<<<grid_for(d.F, threads, cap), threads, 0, s>>>(

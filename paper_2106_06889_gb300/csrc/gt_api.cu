@@ -451,7 +451,6 @@ gt_result* sort_from_counts(gt_grammar* g, const uint64_t* wc, int order, cudaSt
   auto* counts = static_cast<uint64_t*>(rb.alloc(size_t(V) * 8));
   int64_t* nlen = rb.new_len_slot();
   GT_CUDA(cudaMemcpyAsync(rb.status(), wc_status, 4, cudaMemcpyDeviceToDevice, s));
-  gt::StatusScope scope(rb.status());
   gt::Phase ph(ctx, "sort_canon", s);
   if (order == 0) {
     Buf flag(ctx, size_t(V) * 8, s), pos(ctx, size_t(V) * 8, s), sc(ctx, gt::scan_scratch_bytes(V), s);
@@ -817,9 +816,13 @@ GT_API gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, 
 GT_API gt_status gt_set_param(gt_ctx* ctx, const char* name, int64_t value) {
   if (!ctx || !name) return GT_EINVAL;
   static const char* known[] = {"wc_aggregate", "use_graphs", "file_strategy", "wc_slices", "bu_local", "seq_path",
-                                "seq_table_cap", "radix_items", "radix_prefetch"};
+                                "seq_table_cap", "radix_items", "radix_prefetch", "look_back_polls"};
   if (std::strcmp(name, "radix_items") == 0 && value != 8 && value != 16) {
     ctx->last_error = "radix_items must be 8 or 16";
+    return GT_EINVAL;
+  }
+  if (std::strcmp(name, "look_back_polls") == 0 && (value < 0 || value > gt::kSpinLimit)) {
+    ctx->last_error = "look_back_polls must be 0 to 2^22";
     return GT_EINVAL;
   }
   for (const char* k : known)

@@ -562,13 +562,26 @@ constexpr int kExpandWords = 6 * 1024;
 // over 1M rules: 253 -> 188 us, and 36 us for the ends).
 constexpr int64_t kExpandEnds = int64_t(1) << 20;
 
+// The flag word of a whole tile, from its symbols (by one warp).
+__device__ __forceinline__ uint64_t expand_tile_flag(const int32_t* __restrict__ sym, const uint64_t* __restrict__ exp_len,
+                                                  int32_t V, int64_t tile) {
+  int64_t len = 0;
+#pragma unroll 1
+  for (int i = threadIdx.x & 31; i < kRowTile; i += 32) {
+    const int32_t sy = sym[tile * kRowTile + i];
+    len += sy < V ? 1 : int64_t(exp_len[sy - V]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) len += __shfl_xor_sync(0xffffffffu, len, o);
+  return (tile == 0 ? kFlagIncl : kFlagAgg) | uint64_t(len);
+}
+
 template <bool kFiles>
 __global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGrammar d, int64_t tiles,
                                                                   unsigned long long* __restrict__ look,
                                                                   const int4* __restrict__ ends,
                                                                   const int64_t* __restrict__ first, int file_bits,
-                                                                  int32_t* __restrict__ words,
-                                                                  unsigned* __restrict__ status) {
+                                                                  int32_t* __restrict__ words, int polls) {
   __shared__ int64_t s_warp[kRowThreads / 32];
   __shared__ int64_t s_item, s_prefix;
   __shared__ int32_t s_file[2];
@@ -641,8 +654,9 @@ __global__ void __launch_bounds__(kRowThreads) expand_root_kernel(const DevGramm
   }
   if (warp == 0) {
     __syncwarp();
-    const int64_t p = warp_look_back(look, item, uint64_t(total), status);
-    if (lane == 0) s_prefix = p < 0 ? 0 : p;
+    const int64_t p = warp_look_back(look, item, uint64_t(total), nullptr, polls, true,
+                                     [&](int64_t t) { return expand_tile_flag(d.sym, d.exp_len, d.V, t); });
+    if (lane == 0) s_prefix = p;
   }
   __syncthreads();
   const int64_t base = s_prefix;
@@ -718,7 +732,8 @@ void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s, int fil
   if (tiles == 0) return;
   GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(tiles + 1) * 8, s));
   (file_bits >= 0 ? expand_root_kernel<true> : expand_root_kernel<false>)<<<unsigned(tiles), kRowThreads, 0, s>>>(
-      d, tiles, look.as<unsigned long long>(), by_ends ? ends.as<int4>() : nullptr, first.as<int64_t>(), file_bits, words.as<int32_t>(), status_word());
+      d, tiles, look.as<unsigned long long>(), by_ends ? ends.as<int4>() : nullptr, first.as<int64_t>(), file_bits,
+      words.as<int32_t>(), look_back_polls());
   GT_LAUNCH_CHECK();
 }
 
@@ -772,7 +787,6 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
   if (d.N >= (uint64_t(1) << 32)) fail(GT_EOVERFLOW, "per-file analytics need fewer than 2^32 tokens per grammar");
   out.status = Buf(ctx, 4, s);
   GT_CUDA(cudaMemsetAsync(out.status.p, 0, 4, s));
-  StatusScope scope(out.status.as<uint32_t>());
   const int kbw = bits_for(d.V);
   const int fb = bits_for(d.F);
   if (g->max_file_len <= kLocalMax && gparam(g, "bu_local", 1)) {
@@ -884,7 +898,6 @@ __global__ void unpack_pay_kernel(const uint64_t* __restrict__ pay, const int64_
 void rows_by_file(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   if (!wr.by_word) return;
   gt_ctx* ctx = g->ctx;
-  StatusScope scope(wr.status.as<uint32_t>());
   const int64_t n = wr.bound;
   const int64_t* nd = wr.total.as<int64_t>();
   wr.by_word = false;
@@ -929,7 +942,6 @@ gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
   GT_CUDA(cudaMemcpyAsync(rb.status(), wr.status.p, 4, cudaMemcpyDeviceToDevice, s));
-  StatusScope scope(rb.status());
   const int64_t n = wr.bound;
   const int64_t* nd = wr.total.as<int64_t>();
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(d.V + 1) * 8));
@@ -1245,7 +1257,6 @@ gt_result* ranked_from_key_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, c
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
   GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
-  StatusScope scope(rb.status());
   Phase ph(ctx, "ranked", s);
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(bound + 1) * 8));
   auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));

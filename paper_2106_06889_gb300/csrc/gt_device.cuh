@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "gt_internal.cuh"
 
@@ -257,7 +258,13 @@ __device__ __forceinline__ uint64_t to_output_key(uint64_t k, int kb) {
 // Flag word per item: state in the top two bits (0 nothing published, 1 the
 // item's own total, 2 the inclusive prefix through the item), value below.
 // An item only waits on items with smaller tickets, i.e. ones already
-// running, so every wait ends; each is bounded anyway.
+// running, so every wait ends; each is bounded anyway.  What follows a wait
+// that ran out depends on the caller: the primitives (scan, radix sort, run
+// reduction, root expansion) work the missing item's value out of its input
+// themselves and go on - a later kernel takes their output for indices, and the
+// grammar keeps some of it, so it has to be right whatever happened - and the
+// inverted index and the bucket path, whose output goes to the caller only,
+// record ST_TIMEOUT.
 constexpr uint64_t kFlagAgg = 1ull << 62, kFlagIncl = 2ull << 62, kFlagVal = (1ull << 62) - 1;
 constexpr int kSpinLimit = 1 << 22;  // look-back polls before giving up (>= 0.25 s)
 
@@ -273,15 +280,20 @@ __device__ __forceinline__ void publish_aggregate(unsigned long long* flags, int
   atomicExch(&flags[item], (item == 0 ? kFlagIncl : kFlagAgg) | agg);
 }
 
+struct NoRedo {};
+
 // By one warp: reads the flags of the 32 preceding items at once, adds their
 // values up to the nearest one with a published prefix, and moves 32 items
 // further back while there is none; then publishes the item's inclusive
-// prefix.  Returns the exclusive prefix (to every lane); after kSpinLimit
-// polls of an item that published nothing it sets ST_TIMEOUT in *status,
-// still publishes (so that later items are not held up) and returns -1.
-// publish == false: the item's own word already holds its final value.
+// prefix.  Returns the exclusive prefix (to every lane).  After spin_limit polls
+// in which an item published nothing, redo(item) (called by the whole warp)
+// gives the flag word it would have published; without redo it sets ST_TIMEOUT
+// in *status, still publishes (so that later items are not held up) and returns
+// -1.  publish == false: the item's own word already holds its final value.
+template <class Redo = NoRedo>
 __device__ __forceinline__ int64_t warp_look_back(unsigned long long* flags, int64_t item, uint64_t agg,
-                                                  unsigned* status, int spin_limit = kSpinLimit, bool publish = true) {
+                                                  unsigned* status, int spin_limit = kSpinLimit, bool publish = true,
+                                                  Redo redo = Redo()) {
   const int lane = threadIdx.x & 31;
   if (item == 0) return 0;
   uint64_t excl = 0;
@@ -290,15 +302,30 @@ __device__ __forceinline__ int64_t warp_look_back(unsigned long long* flags, int
   bool ok = true;
   while (true) {
     const int64_t j = top - lane;
-    const unsigned long long v = j >= 0 ? ld_acquire_u64(&flags[j]) : kFlagIncl;
-    const uint64_t st = v & ~kFlagVal;
+    unsigned long long v = j >= 0 ? ld_acquire_u64(&flags[j]) : kFlagIncl;
+    uint64_t st = v & ~kFlagVal;
     if (__any_sync(0xffffffffu, st == 0)) {
-      if (++spins > spin_limit) {
+      if (++spins <= spin_limit) {
+        __nanosleep(32);
+        continue;
+      }
+      if constexpr (std::is_same<Redo, NoRedo>::value) {
         ok = false;
         break;
+      } else {  // the missing items before the nearest prefix, one after the other
+#pragma unroll 1
+        for (int l = 0; l < 32; ++l) {
+          const uint64_t seen = __shfl_sync(0xffffffffu, st, l);
+          if (seen == kFlagIncl) break;
+          if (seen) continue;
+          const uint64_t x = redo(top - l);
+          if (lane == l) {
+            v = x;
+            st = x & ~kFlagVal;
+          }
+          if ((x & ~kFlagVal) == kFlagIncl) break;
+        }
       }
-      __nanosleep(32);
-      continue;
     }
     const unsigned incl = __ballot_sync(0xffffffffu, st == kFlagIncl);
     const int stop = incl ? __ffs(incl) - 1 : 31;  // nearest item with a prefix, else the whole window

@@ -1371,7 +1371,6 @@ void file_hist(gt_grammar* g, cudaStream_t s, FileHist& fh) {
   const int32_t F = d.F, V = d.V;
   fh.status = Buf(ctx, 4, s);
   GT_CUDA(cudaMemsetAsync(fh.status.p, 0, 4, s));
-  StatusScope scope(fh.status.as<uint32_t>());
   FileWeights fwt;
   {
     Phase ph(ctx, "file_weights", s);
@@ -1601,7 +1600,6 @@ gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt,
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
   GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
-  StatusScope scope(rb.status());
   Phase ph(ctx, "tv_out", s);
   auto* tv_off = static_cast<int64_t*>(rb.alloc(size_t(F + 1) * 8));
   if (top_k <= 0) {

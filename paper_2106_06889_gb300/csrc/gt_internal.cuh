@@ -45,18 +45,9 @@ extern std::atomic<long long> g_launches;
 // phase timers in primitives that take no context.
 extern thread_local gt_ctx* t_call_ctx;
 
-// The status word that waits inside the primitives (scan, sort, reduction)
-// report to: the one of the enclosing StatusScope on this thread, else the
-// context's (read by gt_sync).
-uint32_t* status_word();
-extern thread_local uint32_t* t_status;
-struct StatusScope {
-  uint32_t* const outer;
-  explicit StatusScope(uint32_t* st) : outer(t_status) { t_status = st; }
-  StatusScope(const StatusScope&) = delete;
-  StatusScope& operator=(const StatusScope&) = delete;
-  ~StatusScope() { t_status = outer; }
-};
+// Polls of a tile that published nothing before a look-back of the primitives
+// works the tile's totals out itself ("look_back_polls").
+int look_back_polls();
 
 // Bits of the device status word.
 enum : uint32_t {
@@ -606,6 +597,7 @@ void reduce_file_runs(gt_ctx* ctx, const uint32_t* keys, const uint32_t* files, 
 
 // gt_sort.cu: device primitives
 size_t scan_scratch_bytes(int64_t n);
+// in and out do not overlap: a look-back may read its tiles of `in` again
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratch, cudaStream_t s);
 size_t radix_scratch_bytes(int64_t n, bool with_values, int value_bytes);
 // Stable LSD radix sort of n uint64 keys on bits [begin_a, end_a) and then

@@ -34,11 +34,55 @@ __device__ __forceinline__ bool run_head(K k, K prev, uint32_t f, uint32_t prev_
 // What a row carries beside its key.
 enum RunRows { kKeyVal, kKeyOnly, kKeyFileVal, kKeyFile, kKeyCode };
 
+// The two flag words of a whole tile, from its rows (by one warp): the number of
+// its heads, and the part of the run open at its end that lies in it.
+struct TileFlags {
+  uint64_t heads, open;
+};
+
+template <class K, RunRows kRows>
+__device__ __forceinline__ TileFlags run_tile_flags(const K* __restrict__ keys, const uint64_t* __restrict__ fkeys,
+                                                 const uint32_t* __restrict__ vals, K key_pad, int64_t tile) {
+  constexpr bool kFile = kRows == kKeyFileVal || kRows == kKeyFile;
+  constexpr int kShift = kRows == kKeyCode ? kCodeBits : 0;
+  const int lane = threadIdx.x & 31;
+  uint64_t heads = 0, open = 0;
+#pragma unroll 1
+  for (int64_t i0 = tile * kRunTile; i0 < (tile + 1) * kRunTile; i0 += 32) {
+    const int64_t i = i0 + lane;
+    const K k = keys[i] >> kShift, prev = i > 0 ? keys[i - 1] >> kShift : K(0);
+    uint32_t f = 0, prev_f = 0, v = 1;
+    if (kRows == kKeyVal) v = vals[i];
+    if (kRows == kKeyCode) v = code_weight(uint32_t(keys[i]));
+    if (kRows == kKeyFileVal) {
+      f = uint32_t(fkeys[i] >> 32);
+      v = uint32_t(fkeys[i]);
+      prev_f = i > 0 ? uint32_t(fkeys[i - 1] >> 32) : 0u;
+    }
+    if (kRows == kKeyFile) {
+      f = vals[i];
+      prev_f = i > 0 ? vals[i - 1] : 0u;
+    }
+    const bool real = k != key_pad;
+    const unsigned h = __ballot_sync(0xffffffffu, real && (i == 0 || run_head<kFile>(k, prev, f, prev_f)));
+    if (!real) v = 0;
+    if (h) {
+      heads += unsigned(__popc(h));
+      open = lane >= 31 - __clz(h) ? v : 0u;
+    } else {
+      open += v;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) open += __shfl_xor_sync(0xffffffffu, open, o);
+  return {(tile == 0 ? kFlagIncl : kFlagAgg) | heads, (tile == 0 || heads ? kFlagIncl : kFlagAgg) | open};
+}
+
 template <class K, RunRows kRows>
 __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
     const K* __restrict__ keys, const uint64_t* __restrict__ fkeys, const uint32_t* __restrict__ vals,
     int64_t n_max, const int64_t* __restrict__ n_dev, K key_pad, const __grid_constant__ RunOut out,
-    unsigned long long* __restrict__ look, int64_t tiles_max, unsigned* __restrict__ status) {
+    unsigned long long* __restrict__ look, int64_t tiles_max, int polls) {
   constexpr bool kFile = kRows == kKeyFileVal || kRows == kKeyFile, kVals = kRows == kKeyVal;
   constexpr int kShift = kRows == kKeyCode ? kCodeBits : 0;
   __shared__ K s_key[kRunTile];
@@ -196,8 +240,10 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
   }
   __syncthreads();
   if (warp == 0) {
-    const int64_t p = warp_look_back(head_flags, item, h_total, status);
-    if (lane == 0) s_prefix = p < 0 ? 0 : p;
+    const int64_t p = warp_look_back(head_flags, item, h_total, nullptr, polls, true, [&](int64_t t) {
+      return run_tile_flags<K, kRows>(keys, fkeys, vals, key_pad, t).heads;
+    });
+    if (lane == 0) s_prefix = p;
   } else if (warp == 1) {
     // values of the open run in earlier tiles; a tile with a head ends the look-back there
     const uint64_t open = h_total ? s_total - s_before[h_total - 1] : s_total;
@@ -206,8 +252,10 @@ __global__ void __launch_bounds__(kRunThreads) reduce_runs_kernel(
       else publish_aggregate(open_flags, item, open);
     }
     __syncwarp();
-    const int64_t c = warp_look_back(open_flags, item, open, status, kSpinLimit, h_total == 0);
-    if (lane == 0) s_carry = c < 0 ? 0 : c;
+    const int64_t c = warp_look_back(open_flags, item, open, nullptr, polls, h_total == 0, [&](int64_t t) {
+      return run_tile_flags<K, kRows>(keys, fkeys, vals, key_pad, t).open;
+    });
+    if (lane == 0) s_carry = c;
   }
   __syncthreads();
   const int64_t o0 = s_prefix;
@@ -254,7 +302,7 @@ void launch_runs(gt_ctx* ctx, const K* keys, const uint64_t* fkeys, const uint32
   Buf look(ctx, size_t(2 * tiles + 1) * 8, s);
   GT_CUDA(cudaMemsetAsync(look.p, 0, size_t(2 * tiles + 1) * 8, s));
   reduce_runs_kernel<K, kRows><<<unsigned(tiles), kRunThreads, 0, s>>>(
-      keys, fkeys, vals, n, n_dev, key_pad, out, look.as<unsigned long long>(), tiles, status_word());
+      keys, fkeys, vals, n, n_dev, key_pad, out, look.as<unsigned long long>(), tiles, look_back_polls());
   GT_LAUNCH_CHECK();
 }
 

@@ -526,7 +526,6 @@ gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
   GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
-  StatusScope scope(rb.status());
   Phase ph(ctx, "ranked", s);
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(bound + 1) * 8));
   auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));
@@ -602,7 +601,6 @@ gt_result* reduce_key_rows(gt_ctx* ctx, Buf& keys, Buf& vals, int64_t n, int kb,
                            const uint32_t* status_in, const int64_t* n_dev) {
   ResultBuilder rb(ctx, s);
   if (status_in) GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
-  StatusScope scope(rb.status());
   auto* key = static_cast<uint64_t*>(rb.alloc(size_t(n) * 8));
   auto* count = static_cast<uint64_t*>(rb.alloc(size_t(n) * 8));
   int64_t* len = rb.new_len_slot();
@@ -632,7 +630,6 @@ gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s) {
   Windows w;
   Buf st(ctx, 4, s);
   GT_CUDA(cudaMemsetAsync(st.p, 0, 4, s));
-  StatusScope scope(st.as<uint32_t>());
   // Rows sorted straight into (key, file) order, when a key has few enough files
   // to put in rank order afterwards: as one word (key << file bits | file), or,
   // if that is too wide, from the expanded files, whose windows come in file
@@ -705,7 +702,6 @@ gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s, Buf* 
   if (!per_file && gparam(g, "seq_path", 1) == 2) return run_sequence_count_global(g, s);
   gt_ctx* ctx = g->ctx;
   ResultBuilder rb(ctx, s);
-  StatusScope scope(rb.status());
   Windows w;
   sorted_windows(g, per_file != 0, s, w, rb.status(), keep_ends);
   Phase ph(ctx, "seq_reduce", s);

@@ -1081,7 +1081,6 @@ gt_result* run_sequence_count_global(gt_grammar* g, cudaStream_t s) {
   int kb = 1;  // bits per word id
   while ((int64_t(1) << kb) <= std::max<int64_t>(d.V - 1, 1)) ++kb;
   ResultBuilder rb(ctx, s);
-  StatusScope scope(rb.status());
   const int64_t U = g->info.owned_windows;  // rows at most (rules of weight 0 own none)
   auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(U) * 8));
   auto* ocnt = static_cast<uint64_t*>(rb.alloc(size_t(U) * 8));

@@ -6,17 +6,17 @@
 //
 // Both are single-pass kernels: a CTA takes the next tile by an atomic ticket,
 // publishes the tile's totals and gets what precedes it by a bounded decoupled
-// look-back (see gt_device.cuh); a wait that gives up sets ST_TIMEOUT in the
-// call's status word (status_word()).
+// look-back (see gt_device.cuh); a wait that runs out counts the tile waited for
+// from its input instead, so the results are right whatever happened.
 #include <type_traits>
 
 #include "gt_device.cuh"
 
 namespace gt {
 
-thread_local uint32_t* t_status = nullptr;
-
-uint32_t* status_word() { return t_status ? t_status : (t_call_ctx ? t_call_ctx->d_status : nullptr); }
+int look_back_polls() {
+  return t_call_ctx ? int(t_call_ctx->param("look_back_polls", kSpinLimit)) : kSpinLimit;
+}
 
 namespace {
 
@@ -55,6 +55,16 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
   return r;
 }
 
+// The flag word of a whole tile, from its values (by one warp).
+__device__ __forceinline__ uint64_t scan_tile_flag(const int64_t* __restrict__ in, int64_t tile) {
+  int64_t sum = 0;
+#pragma unroll 1
+  for (int i = threadIdx.x & 31; i < kScanChunk; i += 32) sum += in[tile * kScanChunk + i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return (tile == 0 ? kFlagIncl : kFlagAgg) | uint64_t(sum);
+}
+
 // One tile of kScanChunk values per CTA.  With one tile (flags == nullptr) the
 // scan starts at 0; otherwise tiles are taken in ticket order (flags[tiles] is
 // the ticket) and start at the look-back prefix.  Bound by the 16 bytes per
@@ -63,7 +73,7 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
 // three to five launches.
 __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int64_t* in, int64_t* out, int64_t n,
                                                             unsigned long long* __restrict__ flags, int64_t tiles,
-                                                            unsigned* __restrict__ status) {
+                                                            int polls) {
   __shared__ int64_t tile[kScanChunk];
   __shared__ int64_t s_item, s_prefix;
   int64_t item = 0;
@@ -91,8 +101,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int64_t* in, i
     if (threadIdx.x < 32) {
       if (threadIdx.x == 0) publish_aggregate(flags, item, uint64_t(total));
       __syncwarp();
-      const int64_t p = warp_look_back(flags, item, uint64_t(total), status);
-      if (threadIdx.x == 0) s_prefix = p < 0 ? 0 : p;
+      const int64_t p = warp_look_back(flags, item, uint64_t(total), nullptr, polls, true,
+                                       [&](int64_t t) { return scan_tile_flag(in, t); });
+      if (threadIdx.x == 0) s_prefix = p;
     }
     __syncthreads();
     off += s_prefix;
@@ -212,9 +223,10 @@ __device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v) {
 // Rows of one digit in the tiles before `tile`: words are read four tiles at a
 // time, nearest first, up to the first one that holds a prefix.  Tiles are
 // taken in ticket order, so the ones waited for are running; the wait is
-// bounded anyway (ST_TIMEOUT; the sum so far then keeps every store in range).
-template <class W>
-__device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t tile, int bin, unsigned* status) {
+// bounded anyway: after `polls` polls redo(t) gives the word that tile t would
+// have published.
+template <class W, class Redo>
+__device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t tile, int bin, int polls, Redo redo) {
   W sum = 0;
   int64_t t = tile - 1;
   int spins = 0;
@@ -235,13 +247,31 @@ __device__ __forceinline__ W rs_look_back(const W* __restrict__ words, int64_t t
     }
     t -= used;
     if (used == 0) {
-      if (++spins > kSpinLimit) {
-        if (status) atomicOr(status, ST_TIMEOUT);
-        return sum;
+      if (++spins <= polls) {
+        __nanosleep(20);
+        continue;
       }
-      __nanosleep(20);
+      const W x = redo(t);
+      sum += x & RsFlag<W>::kVal;
+      if (x & RsFlag<W>::kIncl) return sum;
+      --t;
     }
   }
+}
+
+// The word of digit `bin` of a whole tile, from its keys (by one thread; tile 0's
+// holds the rows of all smaller digits too).
+template <class W, class K>
+__device__ __forceinline__ W rs_tile_word(const K* __restrict__ kin, int64_t tile, int tile_keys, int shift, uint32_t mask,
+                                       uint32_t bin, const unsigned long long* __restrict__ counts) {
+  const K* k = kin + tile * tile_keys;
+  W c = 0;
+#pragma unroll 1
+  for (int i = 0; i < tile_keys; ++i) c += (uint32_t(k[i] >> shift) & mask) == bin;
+  if (tile != 0) return RsFlag<W>::kAgg | c;
+#pragma unroll 1
+  for (uint32_t b = 0; b < bin; ++b) c += W(counts[b]);
+  return RsFlag<W>::kIncl | c;
 }
 
 // Stable scatter of one tile by one digit.  Warp w owns the w-th slice of the
@@ -263,7 +293,8 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 2)
     radix_downsweep_kernel(
     const K* __restrict__ kin, K* __restrict__ kout, const void* __restrict__ vin_,
     void* __restrict__ vout_, int64_t n_max, const int64_t* __restrict__ n_dev, int shift, uint32_t mask,
-    const unsigned long long* __restrict__ counts, W* __restrict__ words, unsigned* __restrict__ ticket, unsigned* __restrict__ status) {
+    const unsigned long long* __restrict__ counts, W* __restrict__ words, unsigned* __restrict__ ticket,
+    int polls) {
   constexpr int kTileKeys = kRsThreads * ITEMS;
   using VT = typename std::conditional<VB == 8, uint64_t, uint32_t>::type;
   extern __shared__ __align__(16) unsigned char rs_smem[];  // staged keys, then values
@@ -367,7 +398,9 @@ __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 2)
 #pragma unroll
     for (int w = 0; w < kRsWarps; ++w) excl += w < warp ? gsum[w] : W(0);
   } else {
-    excl = rs_look_back<W>(words, tile, tid, status);
+    excl = rs_look_back<W>(words, tile, tid, polls, [&](int64_t t) {
+      return rs_tile_word<W, K>(kin, t, kTileKeys, shift, mask, uint32_t(tid), counts);
+    });
   }
   st_relaxed(words + tile * kRsBins + tid, RsFlag<W>::kIncl | (excl + real));
   soff[tid] = excl - W(dstart);
@@ -422,7 +455,7 @@ size_t radix_layout(int64_t n, int items, int passes, void* scratch, RadixScratc
 
 template <class K, int VB, int ITEMS, class W>
 void launch_scatter(const K* ka, K* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
-                    int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
+                    int shift, uint32_t mask, const RadixScratch& rs, int pass, int polls, cudaStream_t s) {
   constexpr int64_t kTileKeys = int64_t(kRsThreads) * ITEMS;
   constexpr size_t smem = size_t(kTileKeys) * (sizeof(K) + VB);
   const int64_t tiles = (n + kTileKeys - 1) / kTileKeys;
@@ -431,22 +464,22 @@ void launch_scatter(const K* ka, K* kb, const void* va, void* vb, int64_t n, con
   Phase ph(t_call_ctx, "radix_pass", s);  // one span per scatter pass
   radix_downsweep_kernel<K, VB, ITEMS, W><<<unsigned(tiles), kRsThreads, smem, s>>>(
       ka, kb, va, vb, n, n_dev, shift, mask, rs.counts + size_t(pass) * kRsBins,
-      reinterpret_cast<W*>(rs.words) + size_t(pass) * size_t(tiles) * kRsBins, rs.tickets + pass, status_word());
+      reinterpret_cast<W*>(rs.words) + size_t(pass) * size_t(tiles) * kRsBins, rs.tickets + pass, polls);
   GT_LAUNCH_CHECK();
 }
 
 template <class K, int VB>
 void launch_scatter_any(const K* ka, K* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
-                        int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, cudaStream_t s) {
+                        int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, int polls, cudaStream_t s) {
   if (!radix_narrow(n))
-    launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, polls, s);
   else if (VB == 0 && items == kRsKeyItems)
     launch_scatter<K, VB, VB == 0 ? kRsKeyItems : kRsLargeItems, uint32_t>(
-        ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+        ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, polls, s);
   else if (items == kRsSmallItems)
-    launch_scatter<K, VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsSmallItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, polls, s);
   else
-    launch_scatter<K, VB, kRsLargeItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, s);
+    launch_scatter<K, VB, kRsLargeItems, uint32_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, polls, s);
 }
 
 // Digit passes over bits [begin_a, end_a) then [begin_b, end_b), the bits of
@@ -479,7 +512,7 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
   const int64_t nb = (n + kScanChunk - 1) / kScanChunk;
   auto* flags = nb > 1 ? static_cast<unsigned long long*>(scratch) : nullptr;
   if (flags) GT_CUDA(cudaMemsetAsync(flags, 0, scan_scratch_bytes(n), s));
-  scan_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(in, out, n, flags, nb, status_word());
+  scan_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(in, out, n, flags, nb, look_back_polls());
   GT_LAUNCH_CHECK();
 }
 
@@ -504,16 +537,17 @@ bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_
   radix_hist_kernel<K><<<grid_for(n, kRhThreads * kRhItems, sms * 4), kRhThreads, 0, s>>>(keys_a, n, n_dev, ps,
                                                                                                  rs.counts);
   GT_LAUNCH_CHECK();
+  const int polls = look_back_polls();
   K *ka = keys_a, *kb = keys_b;
   void *va = vals_a, *vb = vals_b;
   for (int p = 0; p < ps.n; ++p) {
     const uint32_t mask = (1u << ps.bits[p]) - 1u;
     if (value_bytes == 4)
-      launch_scatter_any<K, 4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
     else if (value_bytes == 8)
-      launch_scatter_any<K, 8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
     else
-      launch_scatter_any<K, 0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, s);
+      launch_scatter_any<K, 0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
     std::swap(ka, kb);
     std::swap(va, vb);
   }
