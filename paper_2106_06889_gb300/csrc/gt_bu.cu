@@ -741,7 +741,7 @@ void expand_files(gt_grammar* g, Buf& words, Buf& first, cudaStream_t s, int fil
 // (file, word) order, or in (word, file) order (by_word; the counts beside the
 // words in pay, word << 32 | count).
 struct WordRows {
-  Buf word, file, cnt, total, status;  // status: flags raised while the rows were made
+  Buf word, file, cnt, total;
   Buf pay;
   bool by_word = false;
   int64_t bound = 0;
@@ -785,8 +785,6 @@ void bu_word_rows(gt_grammar* g, cudaStream_t s, WordRows& out) {
   const int threads = 256, cap = ctx->num_sms * 16;
   if (d.depth > kMaxStack) fail(GT_EOVERFLOW, "bottom-up expansion supports DAG depth <= 64");
   if (d.N >= (uint64_t(1) << 32)) fail(GT_EOVERFLOW, "per-file analytics need fewer than 2^32 tokens per grammar");
-  out.status = Buf(ctx, 4, s);
-  GT_CUDA(cudaMemsetAsync(out.status.p, 0, 4, s));
   const int kbw = bits_for(d.V);
   const int fb = bits_for(d.F);
   if (g->max_file_len <= kLocalMax && gparam(g, "bu_local", 1)) {
@@ -941,7 +939,6 @@ gt_result* bu_inverted_index(gt_grammar* g, WordRows& wr, cudaStream_t s) {
   const DevGrammar& d = g->d;
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), wr.status.p, 4, cudaMemcpyDeviceToDevice, s));
   const int64_t n = wr.bound;
   const int64_t* nd = wr.total.as<int64_t>();
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(d.V + 1) * 8));
@@ -1004,8 +1001,7 @@ void run_file_batch_bu(gt_grammar* g, const int* tv_topk, int n_tv, gt_result** 
     GT_LAUNCH_CHECK();
     for (int i = 0; i < n_tv; ++i)
       tv_out[i] = tv_from_arrays(g->ctx, wr.word.as<int32_t>(), wr.cnt.as<uint64_t>(), toff.as<int64_t>(),
-                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], uint64_t(g->max_file_len), s,
-                                 wr.status.as<uint32_t>(), d.V);
+                                 wr.total.as<int64_t>(), wr.bound, d.F, tv_topk[i], uint64_t(g->max_file_len), s, d.V);
   }
   if (ii_out) *ii_out = bu_inverted_index(g, wr, s);
 }
@@ -1027,7 +1023,7 @@ gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s) {
       GT_LAUNCH_CHECK();
     }
     return ranked_from_key_rows(ctx, rkey, wr.file, wr.cnt, wr.total.as<int64_t>(), n, 0, g->d.F,
-                                uint64_t(g->max_file_len), s, wr.status.as<uint32_t>());
+                                uint64_t(g->max_file_len), s);
   }
   rows_by_file(g, wr, s);
   if (n > 0) {
@@ -1036,7 +1032,7 @@ gt_result* run_ranked_words_bu(gt_grammar* g, cudaStream_t s) {
     GT_LAUNCH_CHECK();
   }
   return ranked_from_rows(ctx, rkey, wr.file, wr.cnt, wr.total.as<int64_t>(), n, 0, false, bits_for(g->d.V),
-                          uint64_t(g->max_file_len), s, wr.status.as<uint32_t>());
+                          uint64_t(g->max_file_len), s);
 }
 
 // Per-file window rows of small files, built per file in shared memory.
@@ -1253,10 +1249,9 @@ void bu_token_windows(gt_grammar* g, int kb, Buf& keys, Buf& files, Buf& n, cuda
 }
 
 gt_result* ranked_from_key_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
-                                int kb, int32_t F, uint64_t max_count, cudaStream_t s, const uint32_t* status_in) {
+                                int kb, int32_t F, uint64_t max_count, cudaStream_t s) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "ranked", s);
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(bound + 1) * 8));
   auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));

@@ -1035,7 +1035,7 @@ __global__ void topk_gather_kernel(const uint32_t* __restrict__ idx, const int64
 }
 
 struct FileHist {
-  Buf slot_word, slot_cnt, nnz, bits, off, total, status;  // status: flags raised while the pieces were made
+  Buf slot_word, slot_cnt, nnz, bits, off, total;
   int nb = 0;
   int64_t bound = 0;  // bound on term-vector entries (= inverted-index postings)
 };
@@ -1369,8 +1369,6 @@ void file_hist(gt_grammar* g, cudaStream_t s, FileHist& fh) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   const int32_t F = d.F, V = d.V;
-  fh.status = Buf(ctx, 4, s);
-  GT_CUDA(cudaMemsetAsync(fh.status.p, 0, 4, s));
   FileWeights fwt;
   {
     Phase ph(ctx, "file_weights", s);
@@ -1482,10 +1480,9 @@ gt_result* term_vector_from(gt_grammar* g, FileHist& fh, int top_k, cudaStream_t
       GT_LAUNCH_CHECK();
     }
     return tv_from_arrays(ctx, tw.as<int32_t>(), tc.as<uint64_t>(), full_off.as<int64_t>(), fh.total.as<int64_t>(),
-                          nb_, d.F, top_k, uint64_t(g->max_file_len), s, fh.status.as<uint32_t>(), d.V);
+                          nb_, d.F, top_k, uint64_t(g->max_file_len), s, d.V);
   }
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), fh.status.p, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "tv_out", s);
   auto* tv_off = static_cast<int64_t*>(rb.alloc(size_t(d.F + 1) * 8));
   auto* word = static_cast<int32_t*>(rb.alloc(size_t(nb_) * 4));
@@ -1515,7 +1512,6 @@ gt_result* inverted_index_from(gt_grammar* g, FileHist& fh, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), fh.status.p, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "ii_out", s);
   const int threads = 256, cap = ctx->num_sms * 16;
   const int64_t V = d.V;
@@ -1579,7 +1575,7 @@ gt_result* run_ranked_words(gt_grammar* g, cudaStream_t s) {
     GT_LAUNCH_CHECK();
   }
   return ranked_from_rows(ctx, rkey, rfile, tc, fh.total.as<int64_t>(), bound, 0, false, bits_for(d.V),
-                          uint64_t(g->max_file_len), s, fh.status.as<uint32_t>());
+                          uint64_t(g->max_file_len), s);
 }
 
 __global__ void copy_rows_kernel(const int32_t* __restrict__ w, const uint64_t* __restrict__ c,
@@ -1596,10 +1592,9 @@ __global__ void copy_rows_kernel(const int32_t* __restrict__ w, const uint64_t* 
 // offsets; top_k > 0 keeps each file's top_k counts (count desc, word asc).
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
                           const int64_t* total, int64_t bound, int32_t F, int top_k, uint64_t max_count, cudaStream_t s,
-                          const uint32_t* status_in, int32_t V) {
+                          int32_t V) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "tv_out", s);
   auto* tv_off = static_cast<int64_t*>(rb.alloc(size_t(F + 1) * 8));
   if (top_k <= 0) {

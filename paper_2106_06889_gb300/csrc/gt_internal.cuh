@@ -483,7 +483,7 @@ void bu_token_windows(gt_grammar* g, int kb, Buf& keys, Buf& files, Buf& n, cuda
 // of each key still have to be put in rank order.  For at most kMaxRankFiles files.
 constexpr int32_t kMaxRankFiles = 8192;
 gt_result* ranked_from_key_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
-                                int kb, int32_t F, uint64_t max_count, cudaStream_t s, const uint32_t* status_in);
+                                int kb, int32_t F, uint64_t max_count, cudaStream_t s);
 
 // gt_bu.cu: bottom-up per-file rows
 void bu_window_rows(gt_grammar* g, Buf& ends, int kb, cudaStream_t s, Windows& out);
@@ -508,7 +508,7 @@ int64_t gparam(const gt_grammar* g, const char* name, int64_t dflt);
 constexpr int kTfIdf = -1;
 gt_result* tv_from_arrays(gt_ctx* ctx, const int32_t* word, const uint64_t* cnt, const int64_t* tv_off_in,
                           const int64_t* total, int64_t bound, int32_t F, int top_k, uint64_t max_count, cudaStream_t s,
-                          const uint32_t* status_in, int32_t V = 0);
+                          int32_t V = 0);
 // Device pointer of a result field and the device slot holding its length
 // (valid on the result's stream before the result completes).
 void result_device_field(gt_result* r, const char* field, void** ptr, const int64_t** d_len);
@@ -533,10 +533,9 @@ const int64_t* seq_tile_offsets(gt_grammar* g, const int4* ends, int kb, cudaStr
 gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s);
 // rows (key, file, count) -> ranked index; keys are compact 3-word keys
 // (windows = true, kb bits per word) or word ids (windows = false), all of at
-// most key_bits bits; *status_in: flags raised while the rows were made
+// most key_bits bits
 gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
-                            int kb, bool windows, int key_bits, uint64_t max_count, cudaStream_t s,
-                            const uint32_t* status_in);
+                            int kb, bool windows, int key_bits, uint64_t max_count, cudaStream_t s);
 // gt_file.cu: ranked index over words (rows from the term vector)
 gt_result* run_ranked_words(gt_grammar* g, cudaStream_t s);
 

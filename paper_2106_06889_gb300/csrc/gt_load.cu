@@ -956,9 +956,7 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     // one wait for every total (and for the level offsets copied above)
     unsigned long long hv[9];
     GT_CUDA(cudaMemcpyAsync(hv, ctr + 6, 72, cudaMemcpyDeviceToHost, s));
-    GT_CUDA(cudaMemcpyAsync(&st, ctx->d_status, 4, cudaMemcpyDeviceToHost, s));
     GT_CUDA(cudaStreamSynchronize(s));
-    if (st & ST_TIMEOUT) fail(GT_ETIMEOUT, "a bounded device wait timed out");
     d.N = hv[4];
     g->info.num_tokens = int64_t(hv[4]);
     g->info.root_words = int64_t(hv[2]);

@@ -354,7 +354,7 @@ void td_emit_windows(gt_grammar* g, Buf& ends, int kb, const FileRows& fr, cudaS
   GT_LAUNCH_CHECK();
 }
 
-// Device-detected failures go to *status (the result's own status word).
+// Device-detected failures of the global rows go to *status (the result's own status word).
 void sorted_windows(gt_grammar* g, bool per_file, cudaStream_t s, Windows& out, uint32_t* status,
                     Buf* keep_ends = nullptr) {
   gt_ctx* ctx = g->ctx;
@@ -521,11 +521,9 @@ __global__ void rank_unpack_kernel(const uint64_t* __restrict__ pay, const int64
 // Rows (key, file, count), n_dev of them (bound allocated) -> ranked index:
 // keys ascending; inside a key, count descending then file ascending.
 gt_result* ranked_from_rows(gt_ctx* ctx, Buf& rkey, Buf& rfile, Buf& rcnt, const int64_t* n_dev, int64_t bound,
-                            int kb, bool windows, int key_bits, uint64_t max_count, cudaStream_t s,
-                            const uint32_t* status_in) {
+                            int kb, bool windows, int key_bits, uint64_t max_count, cudaStream_t s) {
   const int threads = 256, cap = ctx->num_sms * 16;
   ResultBuilder rb(ctx, s);
-  GT_CUDA(cudaMemcpyAsync(rb.status(), status_in, 4, cudaMemcpyDeviceToDevice, s));
   Phase ph(ctx, "ranked", s);
   auto* off = static_cast<int64_t*>(rb.alloc(size_t(bound + 1) * 8));
   auto* okey = static_cast<uint64_t*>(rb.alloc(size_t(bound) * 8));
@@ -628,8 +626,6 @@ gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s) {
   gt_ctx* ctx = g->ctx;
   const DevGrammar& d = g->d;
   Windows w;
-  Buf st(ctx, 4, s);
-  GT_CUDA(cudaMemsetAsync(st.p, 0, 4, s));
   // Rows sorted straight into (key, file) order, when a key has few enough files
   // to put in rank order afterwards: as one word (key << file bits | file), or,
   // if that is too wide, from the expanded files, whose windows come in file
@@ -681,19 +677,18 @@ gt_result* run_ranked_windows(gt_grammar* g, cudaStream_t s) {
                          s);
       }
     }
-    return ranked_from_key_rows(ctx, rkey, rfile, rcnt, nd.as<int64_t>(), bound, kb, d.F, uint64_t(g->max_file_len), s,
-                                st.as<uint32_t>());
+    return ranked_from_key_rows(ctx, rkey, rfile, rcnt, nd.as<int64_t>(), bound, kb, d.F, uint64_t(g->max_file_len), s);
   }
-  sorted_windows(g, true, s, w, st.as<uint32_t>());
+  sorted_windows(g, true, s, w, nullptr);
   if (w.reduced)
     return ranked_from_rows(ctx, w.keys, w.rfile, w.rcnt, w.total.as<int64_t>(), w.n, w.kb, true, 3 * w.kb,
-                            uint64_t(g->max_file_len), s, st.as<uint32_t>());
+                            uint64_t(g->max_file_len), s);
   // per-file 3-gram rows (file, key, count) in (file, key) order
   Buf rkey(ctx, size_t(w.n) * 8, s), rfile(ctx, size_t(w.n) * 4, s), rcnt(ctx, size_t(w.n) * 8, s), nd(ctx, 8, s);
   reduce_windows(ctx, w, true, false, rkey.as<uint64_t>(), rfile.as<int32_t>(), rcnt.as<uint64_t>(), nd.as<int64_t>(),
                  s);
   return ranked_from_rows(ctx, rkey, rfile, rcnt, nd.as<int64_t>(), w.n, w.kb, true, 3 * w.kb,
-                          uint64_t(g->max_file_len), s, st.as<uint32_t>());
+                          uint64_t(g->max_file_len), s);
 }
 
 gt_result* run_sequence_count(gt_grammar* g, int per_file, cudaStream_t s, Buf* keep_ends) {
