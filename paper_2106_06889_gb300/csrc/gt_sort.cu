@@ -8,6 +8,7 @@
 // publishes the tile's totals and gets what precedes it by a bounded decoupled
 // look-back (see gt_device.cuh); a wait that runs out counts the tile waited for
 // from its input instead, so the results are right whatever happened.
+#include <algorithm>
 #include <type_traits>
 
 #include "gt_device.cuh"
@@ -517,8 +518,10 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
 }
 
 size_t radix_scratch_bytes(int64_t n, bool, int) {
-  // for the smallest tile that a sort of n rows may take
-  return radix_layout(n, n < kRsLargeRows ? kRsSmallItems : kRsLargeItems, kRsMaxPasses, nullptr, nullptr);
+  // enough for a sort of any number of rows up to n: below kRsLargeRows the tiles
+  // are smaller and have more words
+  const size_t small = radix_layout(std::min(n, kRsLargeRows - 1), kRsSmallItems, kRsMaxPasses, nullptr, nullptr);
+  return n < kRsLargeRows ? small : std::max(small, radix_layout(n, kRsLargeItems, kRsMaxPasses, nullptr, nullptr));
 }
 
 namespace {
