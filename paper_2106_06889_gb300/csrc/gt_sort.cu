@@ -72,7 +72,7 @@ __device__ __forceinline__ uint64_t scan_tile_flag(const int64_t* __restrict__ i
 // value it moves; the former two passes (block sums, then the scan proper, with
 // a recursive scan of the sums between them) read the values twice and took
 // three to five launches.
-__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int64_t* in, int64_t* out, int64_t n,
+__global__ void __launch_bounds__(kScanThreads, 6) scan_kernel(const int64_t* in, int64_t* out, int64_t n,
                                                             unsigned long long* __restrict__ flags, int64_t tiles,
                                                             int polls) {
   __shared__ int64_t tile[kScanChunk];
