@@ -1348,7 +1348,8 @@ void file_weights(gt_grammar* g, cudaStream_t s, FileWeights& fw) {
   const WeightRows L{g->row_off, g->row_entries, g->row_pieces, g->slot_pair};
   // level by level from the root's children down; level-1 rules have no
   // parent but the root, so their weights are complete already
-  for (int lv = 2; lv < g->fw_tail; ++lv) {
+  const int tail = capturing(s) ? d.depth : g->fw_tail;
+  for (int lv = 2; lv < tail; ++lv) {
     const int64_t a = g->lvl_slot[size_t(lv)], b = g->lvl_slot[size_t(lv) + 1];
     const int64_t ha = g->lvl_piece[size_t(lv)], hb = g->lvl_piece[size_t(lv) + 1];
     if (b <= a && hb <= ha) continue;
@@ -1357,8 +1358,8 @@ void file_weights(gt_grammar* g, cudaStream_t s, FileWeights& fw) {
     fweight_level_kernel<<<unsigned(lb + hblk), threads, 0, s>>>(L, a, b, lb, ha, hb, fw.w.as<uint32_t>());
     GT_LAUNCH_CHECK();
   }
-  if (g->fw_tail < d.depth) {
-    fweight_tail_kernel<<<kTailCtas, kTailThreads, 0, s>>>(L, g->lvl_tab, g->fw_tail, d.depth, fw.w.as<uint32_t>());
+  if (tail < d.depth) {
+    fweight_tail_kernel<<<kTailCtas, kTailThreads, 0, s>>>(L, g->lvl_tab, tail, d.depth, fw.w.as<uint32_t>());
     GT_LAUNCH_CHECK();
   }
 }

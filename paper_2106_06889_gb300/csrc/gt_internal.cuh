@@ -423,8 +423,10 @@ void run_head_tail(gt_grammar* g, int32_t* d_head, int32_t* d_tail, cudaStream_t
 // word.  children_only: rules on level 0, which no rule refers to, are left out.
 void run_rule_ends(gt_grammar* g, int4* ends, cudaStream_t s, bool children_only);
 // First level from which on every level has at most kTailItems items (off: the
-// levels' offsets, host), at least `from`; depth when fewer than two such levels.
-int small_levels(const std::vector<int64_t>& off, int from, int depth);
+// levels' offsets, host), at least `from`; depth when fewer than two such levels, or
+// when s is being captured.
+int small_levels(const std::vector<int64_t>& off, int from, int depth, cudaStream_t s);
+bool capturing(cudaStream_t s);
 
 // Sorted 3-word window rows: compact keys (kb bits per word, key_pad above
 // every real key) and weights; n rows including pads.  Rows that carry files

@@ -103,9 +103,8 @@ __device__ __forceinline__ void add_edges(unsigned long long* wt, int32_t c, uns
 }
 
 // The small levels [l0, depth) of a grammar's weight pass in one cluster (see
-// kTailItems).  On a 200k-word corpus (7 levels) the six level launches took
-// 19-21 us one by one and take 13.8 us here: 2.3 us per level, the round trips
-// of the barrier, a weight read through L2 and the atomics.
+// kTailItems): 2.3 us per level, the round trips of the barrier, a weight read
+// through L2 and the atomics.
 struct WtTail {
   const int32_t* lchild;
   const int32_t* lpar;
@@ -535,7 +534,14 @@ __global__ void split_ends_kernel(const int4* __restrict__ ends, int32_t R, int3
 
 }  // namespace
 
-int small_levels(const std::vector<int64_t>& off, int from, int depth) {
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  GT_CUDA(cudaStreamIsCapturing(s, &c));
+  return c != cudaStreamCaptureStatusNone;
+}
+
+int small_levels(const std::vector<int64_t>& off, int from, int depth, cudaStream_t s) {
+  if (capturing(s)) return depth;
   int l = depth;
   while (l > from && off[size_t(l)] - off[size_t(l) - 1] <= kTailItems) --l;
   return depth - l >= 2 ? l : depth;
@@ -560,7 +566,7 @@ void weights_batch(gt_grammar* const* gs, uint64_t* const* wts, int n, cudaStrea
     GT_CUDA(cudaMemsetAsync(wts[j], 0, size_t(gs[j]->d.R) * 8, s));
     roots.wt[j] = reinterpret_cast<unsigned long long*>(wts[j]);
     const DevGrammar& d = gs[j]->d;
-    first[j] = small_levels(gs[j]->ledge_off, 1, d.depth);
+    first[j] = small_levels(gs[j]->ledge_off, 1, d.depth, s);
     depth = std::max(depth, first[j]);
     if (first[j] < d.depth)
       tails.job[tails.n++] = {d.ledge_child, d.ledge_par, d.ledge_mult, d.ledge_off, first[j], d.depth, roots.wt[j]};
@@ -723,7 +729,7 @@ void run_rule_ends(gt_grammar* g, int4* ends, cudaStream_t s, bool children_only
   const int threads = 256;
   const int cap = g->ctx->num_sms * 8;
   const int top = children_only ? 1 : 0;
-  const int deep = small_levels(g->lvl_off, top, d.depth);
+  const int deep = small_levels(g->lvl_off, top, d.depth, s);
   if (deep < d.depth) {
     head_tail_deep_kernel<<<kTailCtas, kTailThreads, 0, s>>>(d, deep, ends);
     GT_LAUNCH_CHECK();
