@@ -813,10 +813,12 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     Buf fcnt(ctx, size_t(R) * 8, s), foff(ctx, size_t(R) * 8, s), fsc(ctx, scan_scratch_bytes(R), s);
     while (b > a) {
       const int64_t n = b - a;
-      // rules of a few children on average (up to 8): longer ones want more warps.
-      // (With one wait for all totals: load, file preparation and first index of 8M
-      // words in 13 files 2449 -> 2391 us.)
-      if (lv > 0 && n <= kTailItems && d.E <= 8 * int64_t(R)) {
+      // rules of no more children on average than a thread takes itself: longer ones
+      // want more warps.  Load of 8 levels of 2,000 rules, us, a launch per level
+      // against the cluster, by references per rule: 2: 1230 / 1143, 4: 1232 / 1155,
+      // 5: 1249 / 1390, 8: 1264 / 1346, 32: 1189 / 1205; 8,000 rules 4: 1417 / 1282, 5:
+      // 1440 / 1488.
+      if (lv > 0 && n <= kTailItems && d.E <= kFrontierOwn * int64_t(R)) {
         frontier_tail_kernel<<<kTailCtas, kTailThreads, 0, s>>>(a, b, lv, d.cedge_off, d.cedge_child, rem.as<int32_t>(),
                                                                 level, korder.as<int32_t>(), tail, ctr + 4);
         GT_LAUNCH_CHECK();

@@ -1,11 +1,13 @@
 """Passes over the DAG's levels: launched one by one or, for small levels, in one
-cluster; a captured plan always launches them one by one."""
+cluster; a captured plan always launches them one by one.  And the load's
+frontiers of rules with few references (one cluster) and with more (launches)."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2106_06889_gb300 import binding as B
-from tests.test_gpu_primitives import deep_grammar
+from tests.test_gpu_primitives import check, deep_grammar
+from tests.test_oracle_pins import grammar_from_rules
 
 pytestmark = pytest.mark.gpu
 
@@ -38,4 +40,26 @@ def test_captured_levels(ctx, wide):
             assert np.array_equal(counts.cpu().numpy().astype(np.uint64), oracle.word_count(g).astype(np.uint64))
     finally:
         B.gt_plan_destroy(p)
+        B.gt_free_grammar(gh)
+
+
+@pytest.mark.parametrize("n", [1, 40, 300])
+@pytest.mark.parametrize("refs", [3, 4, 5, 8])
+def test_frontiers(ctx, refs, n):
+    """Layers of n rules with refs references to the next layer: on either side of four distinct references per rule."""
+    V, depth = 40, 4
+    rng = np.random.default_rng(refs * n)
+    rules = []
+    for l in range(depth):
+        for i in range(n):
+            nxt = V + 1 + (l + 1) * n
+            rules.append([int(rng.integers(V))] + [nxt + (i + k * 3) % n if l + 1 < depth else int(rng.integers(V))
+                                                   for k in range(refs)])
+    root = [V + 1 + i for i in range(n)] + [1, 2, V + 1]
+    g = grammar_from_rules(V, [root] + rules, [0, n // 2, len(root)])
+    gh = B.gt_load_grammar(ctx, g)
+    try:
+        assert B.gt_grammar_info_get(gh)["depth"] == depth + 1
+        check(gh, g)
+    finally:
         B.gt_free_grammar(gh)
