@@ -558,9 +558,12 @@ __device__ __forceinline__ int32_t file_from(const int64_t* __restrict__ first, 
 // file_bits >= 0: words[p] is word << file_bits | file instead.
 constexpr int kExpandWords = 6 * 1024;
 
-// From this many root symbols on the ends are worked out first (16M root symbols
-// over 1M rules: 253 -> 188 us, and 36 us for the ends).
-constexpr int64_t kExpandEnds = int64_t(1) << 20;
+// From this many root symbols on the ends are worked out first: they take a pass
+// over all rules and its launches.  Term vector and index of many files, us, by
+// walking every reference / with the ends: 0.7M root symbols 399 / 414, 2.5M 504 /
+// 515, 5.6M 600 / 614, 8.2M 733 / 738, 10.8M 862 / 861, 13.4M 998 / 988, 16.6M
+// 1170 / 1135 (the expansion itself 253 / 188, the ends 36).
+constexpr int64_t kExpandEnds = int64_t(12) << 20;
 
 // The flag word of a whole tile, from its symbols (by one warp).
 __device__ __forceinline__ uint64_t expand_tile_flag(const int32_t* __restrict__ sym, const uint64_t* __restrict__ exp_len,
