@@ -39,19 +39,19 @@ __device__ __forceinline__ uint32_t take_code(uint32_t& w) {
 
 // Lanes of the warp holding the same 8-bit digit as this lane (among `active`),
 // from one ballot per digit bit.  Every lane of the warp must call it.  Bound by
-// instruction issue in the sort that ranks 32 rows per call: written so that the
-// bit's predicate both votes and complements (a select of the ballot or its
-// complement in C++ takes 4 to 8% more of a scatter pass).
+// instruction issue in the sort that ranks 32 rows per call: the bit's predicate
+// both votes and selects a mask, ready with the ballot, that turns the ballot into
+// the lanes that agree with this one.
 __device__ __forceinline__ unsigned digit_bit_peers(uint32_t d, int b, unsigned peers) {
   asm volatile(
       "{\n\t"
-      ".reg .pred p;\n\t"
-      ".reg .b32 t;\n\t"
-      "and.b32 t, %1, %2;\n\t"
-      "setp.ne.u32 p, t, 0;\n\t"
-      "vote.sync.ballot.b32 t, p, 0xffffffff;\n\t"
-      "@!p not.b32 t, t;\n\t"
-      "and.b32 %0, %0, t;\n\t"
+      ".reg .pred has;\n\t"
+      ".reg .b32 flip, votes;\n\t"
+      "and.b32 flip, %1, %2;\n\t"
+      "setp.ne.b32 has, flip, 0;\n\t"
+      "selp.b32 flip, 0, -1, has;\n\t"
+      "vote.sync.ballot.b32 votes, has, 0xffffffff;\n\t"
+      "lop3.b32 %0, %0, votes, flip, 0x60;\n\t"  // peers and (votes xor flip)
       "}"
       : "+r"(peers)
       : "r"(d), "r"(1 << b));
