@@ -439,12 +439,16 @@ int radix_items(int64_t n, bool keys_only) {
   return p == 16 || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
 }
 
-bool radix_narrow(int64_t n) { return n < (int64_t(1) << 30); }
+// 32-bit look-back words hold the rows; "radix_wide" takes 64-bit ones at any size,
+// which otherwise start at 2^30 rows
+bool radix_narrow(int64_t n) {
+  return n < (int64_t(1) << 30) && !(t_call_ctx && t_call_ctx->param("radix_wide", 0));
+}
 
-size_t radix_layout(int64_t n, int items, int passes, void* scratch, RadixScratch* out) {
+size_t radix_layout(int64_t n, int items, int passes, bool narrow, void* scratch, RadixScratch* out) {
   const int64_t tiles = (n + kRsThreads * items - 1) / (kRsThreads * items);
   const size_t counts = size_t(passes) * kRsBins * 8, tickets = 16 * sizeof(unsigned);
-  const size_t words = size_t(passes) * size_t(tiles) * kRsBins * (radix_narrow(n) ? 4 : 8);
+  const size_t words = size_t(passes) * size_t(tiles) * kRsBins * (narrow ? 4 : 8);
   if (out) {
     out->counts = static_cast<unsigned long long*>(scratch);
     out->tickets = reinterpret_cast<unsigned*>(static_cast<char*>(scratch) + counts);
@@ -471,8 +475,9 @@ void launch_scatter(const K* ka, K* kb, const void* va, void* vb, int64_t n, con
 
 template <class K, int VB>
 void launch_scatter_any(const K* ka, K* kb, const void* va, void* vb, int64_t n, const int64_t* n_dev,
-                        int items, int shift, uint32_t mask, const RadixScratch& rs, int pass, int polls, cudaStream_t s) {
-  if (!radix_narrow(n))
+                        int items, bool narrow, int shift, uint32_t mask, const RadixScratch& rs, int pass, int polls,
+                        cudaStream_t s) {
+  if (!narrow)
     launch_scatter<K, VB, kRsLargeItems, uint64_t>(ka, kb, va, vb, n, n_dev, shift, mask, rs, pass, polls, s);
   else if (VB == 0 && items == kRsKeyItems)
     launch_scatter<K, VB, VB == 0 ? kRsKeyItems : kRsLargeItems, uint32_t>(
@@ -520,8 +525,10 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
 size_t radix_scratch_bytes(int64_t n, bool, int) {
   // enough for a sort of any number of rows up to n: below kRsLargeRows the tiles
   // are smaller and have more words
-  const size_t small = radix_layout(std::min(n, kRsLargeRows - 1), kRsSmallItems, kRsMaxPasses, nullptr, nullptr);
-  return n < kRsLargeRows ? small : std::max(small, radix_layout(n, kRsLargeItems, kRsMaxPasses, nullptr, nullptr));
+  const bool narrow = radix_narrow(n);
+  auto bytes = [&](int64_t rows, int items) { return radix_layout(rows, items, kRsMaxPasses, narrow, nullptr, nullptr); };
+  const size_t small = bytes(std::min(n, kRsLargeRows - 1), kRsSmallItems);
+  return n < kRsLargeRows ? small : std::max(small, bytes(n, kRsLargeItems));
 }
 
 namespace {
@@ -532,9 +539,10 @@ bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_
   if (n <= 0) return false;
   const RadixPasses ps = radix_plan(begin_a, end_a, begin_b, end_b);
   if (ps.n == 0) return false;
-  const int items = radix_narrow(n) ? radix_items(n, value_bytes == 0) : kRsLargeItems;
+  const bool narrow = radix_narrow(n);
+  const int items = narrow ? radix_items(n, value_bytes == 0) : kRsLargeItems;
   RadixScratch rs;
-  radix_layout(n, items, ps.n, scratch, &rs);
+  radix_layout(n, items, ps.n, narrow, scratch, &rs);
   GT_CUDA(cudaMemsetAsync(scratch, 0, rs.zero_bytes, s));
   const int sms = t_call_ctx ? t_call_ctx->num_sms : 152;
   radix_hist_kernel<K><<<grid_for(n, kRhThreads * kRhItems, sms * 4), kRhThreads, 0, s>>>(keys_a, n, n_dev, ps,
@@ -546,11 +554,11 @@ bool radix_sort_any(K* keys_a, K* keys_b, void* vals_a, void* vals_b, int value_
   for (int p = 0; p < ps.n; ++p) {
     const uint32_t mask = (1u << ps.bits[p]) - 1u;
     if (value_bytes == 4)
-      launch_scatter_any<K, 4>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
+      launch_scatter_any<K, 4>(ka, kb, va, vb, n, n_dev, items, narrow, ps.shift[p], mask, rs, p, polls, s);
     else if (value_bytes == 8)
-      launch_scatter_any<K, 8>(ka, kb, va, vb, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
+      launch_scatter_any<K, 8>(ka, kb, va, vb, n, n_dev, items, narrow, ps.shift[p], mask, rs, p, polls, s);
     else
-      launch_scatter_any<K, 0>(ka, kb, nullptr, nullptr, n, n_dev, items, ps.shift[p], mask, rs, p, polls, s);
+      launch_scatter_any<K, 0>(ka, kb, nullptr, nullptr, n, n_dev, items, narrow, ps.shift[p], mask, rs, p, polls, s);
     std::swap(ka, kb);
     std::swap(va, vb);
   }
