@@ -875,6 +875,7 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
     GT_LAUNCH_CHECK();
     g->lvl_off.assign(size_t(lv) + 1, 0);
     GT_CUDA(cudaMemcpyAsync(g->lvl_off.data(), loff, size_t(lv + 1) * 8, cudaMemcpyDeviceToHost, s));
+    GT_CUDA(cudaStreamSynchronize(s));  // read below, level by level
     d.lvl_off = loff;
     d.level = level;
     d.lvl_order = order;
@@ -955,7 +956,7 @@ void load_build_dag(gt_grammar* g, cudaStream_t s) {
       max_u64_kernel<<<grid_for(F, threads, cap), threads, 0, s>>>(d.file_len, F, ctr + 14);
       GT_LAUNCH_CHECK();
     }
-    // one wait for every total (and for the level offsets copied above)
+    // one wait for every total (and for the edges' level offsets copied above)
     unsigned long long hv[9];
     GT_CUDA(cudaMemcpyAsync(hv, ctr + 6, 72, cudaMemcpyDeviceToHost, s));
     GT_CUDA(cudaStreamSynchronize(s));
