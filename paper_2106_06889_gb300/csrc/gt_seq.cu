@@ -25,11 +25,6 @@
 namespace gt {
 namespace {
 
-// Global counts, compacted: every owned window gets one row, in body
-// position order.  One CTA per tile of kTile symbols (4 per thread); each
-// tile's first row comes from the per-grammar tile offsets (the windows of
-// every tile counted and scanned once, seq_tile_offsets), and the emit pass
-// ranks the windows inside the tile.
 // Exclusive prefix of v over the CTA (kWinThreads threads); *total gets the sum.
 __device__ __forceinline__ int cta_excl_scan(int v, int* total) {
   __shared__ int warp_tot[kWinThreads / 32];
@@ -54,6 +49,11 @@ __device__ __forceinline__ int cta_excl_scan(int v, int* total) {
   return before + incl - v;
 }
 
+// Global counts, compacted: every owned window gets one row, in body
+// position order.  One CTA per tile of kTile symbols (4 per thread); each
+// tile's first row comes from the per-grammar tile offsets (the windows of
+// every tile counted and scanned once, seq_tile_offsets), and the emit pass
+// ranks the windows inside the tile.
 // Rows of rules nothing references (weight 0) get the pad key.  Rows past
 // `bound` are not written; the status word records it.  A warp takes 128
 // consecutive symbols, 32 at a time, so that two ballots give the rows' order;
