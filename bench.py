@@ -144,7 +144,9 @@ def kernel_bytes(workload: str, info: dict, out: dict) -> dict:
     writes the distinct 3-grams (16 B each).  Where the sort's rows hold their
     weight in the key's word (num_words up to 2^20 and at most three tokens per
     window), radix_downsweep_kernel<0> moves 16 B per row and reduce_runs_kernel
-    reads 8 B per row."""
+    reads 8 B per row; such a row holds one component of a weight, so a window
+    of weight 4 or more can take several: the windows counted here are the
+    fewest rows there can be."""
     G, V = info["num_syms"], info["num_words"]
     root_len = out["root_len"]
     if workload == "multi64_50m":
@@ -399,22 +401,28 @@ def measure(B, ctx, workload, g, steps, warmup, world, stream, autotune=True, e2
         h2d = sum(int(v.numel() * v.element_size()) for v in pinned.values())
         host_res = {}  # pinned host buffers for the result fields, sized by the untimed first step
 
-        def e2e_step(sizing):
+        def e2e_step(sizing, parts):
             """Load from the pinned host arrays, run the step's analytics, copy
-            every result back into pinned host memory; returns the bytes read back."""
+            every result back into pinned host memory; returns the bytes read
+            back.  parts: the wall time of the load (its upload included), of
+            the analytics until the first result is there, and of the rest."""
             nbytes = 0
+            t_start = time.perf_counter()
             gh2 = B.gt_load_grammar(ctx, HostG, stream)
+            t_load = time.perf_counter()
             q2 = step_queries(B, gh2, analytics, counts)
             res = [r for r in B.gt_run_batch(ctx, q2, stream) if r is not None]
             if "word_count" in analytics:
                 out_host.copy_(counts, non_blocking=True)
                 nbytes += out_host.numel() * out_host.element_size()
+            t_run = None
             for i, r in enumerate(res):  # every result field back to host memory
                 for fld in ("offsets", "word", "key", "count", "file"):
                     try:
                         t = B.result_tensor(r, fld)
                     except B.GtError:
                         continue
+                    t_run = t_run or time.perf_counter()  # the first field waits for its result
                     buf = host_res.get((i, fld))
                     if buf is None or buf.numel() < t.numel():
                         assert sizing, "result sizes change between steps"
@@ -426,18 +434,23 @@ def measure(B, ctx, workload, g, steps, warmup, world, stream, autotune=True, e2
             for r in res:
                 B.gt_free_result(r)
             B.gt_free_grammar(gh2)
+            t_end = time.perf_counter()
+            parts.append([1e3 * x for x in (t_end - t_start, t_load - t_start, t_run - t_load, t_end - t_run)])
             return nbytes
 
         with torch.cuda.stream(stream):
-            e2e_step(True)  # untimed: sizes the pinned result buffers
+            e2e_step(True, [])  # untimed: sizes the pinned result buffers
             torch.cuda.synchronize()
-            d2h_res = 0
+            d2h_res, parts = 0, []
             t0 = time.perf_counter()
             for _ in range(e2e_steps):
-                d2h_res += e2e_step(False)
+                d2h_res += e2e_step(False, parts)
             e2e_s = max_over_ranks((time.perf_counter() - t0) / e2e_steps, world)
         e2e = {"value": job_throughput(world, N, 1, e2e_s), "unit": "tokens/s", "h2d_bytes_per_step": h2d,
                "d2h_bytes_per_step": d2h_res // e2e_steps, "ms_per_step": 1e3 * e2e_s,
+               "steps_ms": [round(p[0], 3) for p in parts],
+               "median_ms": {k: round(float(np.median([p[i] for p in parts])), 3)
+                             for i, k in enumerate(("step", "load", "analytics", "copy_back"))},
                "note": "gt_load_grammar from pinned host arrays + the step's analytics + every result copied back "
                        "into pinned host memory (one untimed step first sizes those buffers)"}
     B.gt_free_grammar(gh)
@@ -924,7 +937,7 @@ def main():
     ctx = B.gt_create(local)
     stream = torch.cuda.Stream()
     m = measure(B, ctx, args.workload, g, args.steps, args.warmup, world, stream,
-                autotune=not args.no_autotune, e2e_steps=0 if args.no_e2e else max(2, min(args.steps, 5)),
+                autotune=not args.no_autotune, e2e_steps=0 if args.no_e2e else 10,
                 eager=args.eager)
     extras = {}
 
@@ -961,7 +974,7 @@ def main():
 
             def c3(c):
                 m3 = measure(B, c, other, g3, max(3, min(args.steps, 10)), 3, world, stream, autotune=False,
-                             e2e_steps=0 if args.no_e2e else 2, clocks=False)
+                             e2e_steps=0 if args.no_e2e else 10, clocks=False)
                 return {"m3": m3, "paths": sequence_paths(B, c, g3, stream)}
 
             r3 = fresh(c3)
