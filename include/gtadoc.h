@@ -365,8 +365,8 @@ gt_status gt_check_bounded_wait(gt_ctx* ctx, int publish, int64_t polls, int64_t
  *   "radix_prefetch" accepted, without effect: it selected a persistent
  *                   scatter that was slower than one CTA per tile.
  *   "radix_wide"    1: the radix sort's tiles exchange their counts in 64-bit
- *                   words at any size; 0 (default): from 2^30 rows on.  Same
- *                   results.
+ *                   words for up to 2^22 rows; 0 (default): from 2^30 rows on
+ *                   only.  Same results.
  *   "look_back_polls" polls of an unpublished total before a scan, sort,
  *                   reduction or root expansion works it out itself: 0 to 2^22
  *                   (default; at least 0.25 s).  GT_EINVAL otherwise.  Same

@@ -439,10 +439,11 @@ int radix_items(int64_t n, bool keys_only) {
   return p == 16 || n >= kRsLargeRows ? kRsLargeItems : kRsSmallItems;
 }
 
-// 32-bit look-back words hold the rows; "radix_wide" takes 64-bit ones at any size,
-// which otherwise start at 2^30 rows
+// 32-bit look-back words hold fewer than kRsNarrowRows rows; "radix_wide" takes the
+// 64-bit ones for up to kRsWideRows rows too
+constexpr int64_t kRsNarrowRows = int64_t(1) << 30, kRsWideRows = int64_t(1) << 22;
 bool radix_narrow(int64_t n) {
-  return n < (int64_t(1) << 30) && !(t_call_ctx && t_call_ctx->param("radix_wide", 0));
+  return n < kRsNarrowRows && !(n <= kRsWideRows && t_call_ctx && t_call_ctx->param("radix_wide", 0));
 }
 
 size_t radix_layout(int64_t n, int items, int passes, bool narrow, void* scratch, RadixScratch* out) {
@@ -523,12 +524,15 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, void* scratc
 }
 
 size_t radix_scratch_bytes(int64_t n, bool, int) {
-  // enough for a sort of any number of rows up to n: below kRsLargeRows the tiles
-  // are smaller and have more words
-  const bool narrow = radix_narrow(n);
-  auto bytes = [&](int64_t rows, int items) { return radix_layout(rows, items, kRsMaxPasses, narrow, nullptr, nullptr); };
-  const size_t small = bytes(std::min(n, kRsLargeRows - 1), kRsSmallItems);
-  return n < kRsLargeRows ? small : std::max(small, bytes(n, kRsLargeItems));
+  // enough for a sort of any number of rows up to n, whatever "radix_wide" says by
+  // then: below kRsLargeRows the tiles are smaller and have more words
+  auto bytes = [](int64_t rows, int items, bool narrow) {
+    return radix_layout(rows, items, kRsMaxPasses, narrow, nullptr, nullptr);
+  };
+  const size_t small = bytes(std::min(n, kRsLargeRows - 1), kRsSmallItems, false);
+  if (n < kRsLargeRows) return small;
+  return std::max({small, bytes(std::min(n, kRsWideRows), kRsLargeItems, false),
+                   bytes(n, kRsLargeItems, n < kRsNarrowRows)});
 }
 
 namespace {
