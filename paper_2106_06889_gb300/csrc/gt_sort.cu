@@ -287,7 +287,7 @@ __device__ __forceinline__ W rs_tile_word(const K* __restrict__ kin, int64_t til
 // scattered 8- and 4-byte staging stores, the read back) against the 34 cycles
 // its 24 bytes take at the measured copy rate.  The look-back is hidden: with
 // every word already published a pass over 49M rows is 6% shorter.  One such pass
-// takes 326 us, 173 at the copy rate; of 51M 8-byte keys alone 223 and 120, of 25M
+// takes 326 us, 173 at the copy rate; of 51M 8-byte keys alone 217 and 120, of 25M
 // 4-byte keys alone 85 and 30.
 template <class K, int VB, int ITEMS, class W>
 __global__ void __launch_bounds__(kRsThreads, ITEMS == kRsSmallItems ? 4 : 2)
